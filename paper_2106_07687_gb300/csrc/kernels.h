@@ -93,8 +93,8 @@ void launch_restrict_full64(const Grid& fine, const Grid& coarse, const double* 
                             int ncomp, cudaStream_t st);
 
 // Vanka (vanka.cu) -----------------------------------------------------------
-// inverse of the 12x12 restriction of A'(vbar) to every fluid cell, stored
-// inv[colour][144][slot], slot = tj * (nx/2 + 1) + ti, cell (2ti - ci, 2tj - cj)
+// inverse of the 12x12 restriction of A'(vbar) to every fluid cell, stored by
+// colour and slot as vanka_inv_index says
 template <typename T>
 void launch_vanka_setup(const Grid& g, const Sten<T>& s, const T* vb, T* inv, int* status,
                         cudaStream_t st);
@@ -108,11 +108,21 @@ void launch_vanka_pass(const Grid& g, const Sten<T>& s, int colour, const T* b, 
                        int shape = 0);
 // Slots of a colour's cells: slot (ti, tj) = cell (2 ti - cx, 2 tj - cy) of
 // colour (cx, cy), for ti < nx/2 + 1, tj < ny/2 + 1.  A row of slots is padded
-// to a multiple of 4 (16 bytes of FP32), so that a row of the inverse array
-// inv[colour][entry][tj][ti] starts on a 16-byte boundary (tensor-memory-
-// access copies need that); padding slots are never written or used.
+// to a multiple of 4; padding slots are never written or used.
 __host__ __device__ inline int vanka_pitch(const Grid& g) { return ((g.nx / 2 + 1) + 3) & ~3; }
 __host__ __device__ inline int vanka_slots(const Grid& g) { return vanka_pitch(g) * (g.ny / 2 + 1); }
+// Layout of the inverses: the 36 entries that node a of a cell needs (its
+// rows c * 4 + a, c = 0..2, entry e = c * 12 + k) as 36 / kVec16 vectors of
+// 16 bytes, inv[colour][vector][slot][a][kVec16].  A warp of a colour pass
+// (four consecutive lanes per cell) reads one vector of 8 cells as 512
+// consecutive bytes, 9 loads per thread in FP32 instead of 36 of 4 bytes.
+template <typename T>
+constexpr int kVec16 = 16 / (int)sizeof(T);
+template <typename T>
+__host__ __device__ inline size_t vanka_inv_index(int nslots, int colour, int slot, int a, int e) {
+  constexpr int V = kVec16<T>;
+  return ((((size_t)colour * (36 / V) + e / V) * nslots + slot) * 4 + a) * V + e % V;
+}
 // Streaming FP32 colour pass for large levels (vanka_stream.cu): the same
 // result as launch_vanka_pass, with the tile's inverses copied by TMA one
 // tile ahead.  map: a tensor map of the level's inverse array made by

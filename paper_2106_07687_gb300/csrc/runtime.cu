@@ -91,10 +91,22 @@ class Solver final : public SolverBase {
     // persistent sub-cycles: level table and one phase list per possible top level
     if (cfg.persistent_vcycle != 0) {
       std::vector<VLevel<T>> hv(K_ + 1);
-      for (int k = 0; k <= K_; ++k)
-        hv[k] = VLevel<T>{lv_[k].g, lv_[k].s, lv_[k].x, lv_[k].x2, lv_[k].b, lv_[k].d,
-                          lv_[k].vb, lv_[k].inv};
+      for (int k = 0; k <= K_; ++k) {
+        if (k > 0) {
+          const std::vector<uint16_t> pat = node_patterns(c_->lv[lv_[k].level]);
+          lv_[k].cf = c_->mem.alloc<T>(36 * (size_t)lv_[k].g.nn);
+          lv_[k].pat = c_->mem.alloc<uint16_t>(pat.size());
+          if (!c_->mem.ok()) return c_->fail(DNNMG_ERR_CUDA, "device allocation failed");
+          cudaMemcpyAsync(lv_[k].pat, pat.data(), sizeof(uint16_t) * pat.size(),
+                          cudaMemcpyHostToDevice, st_);
+          cudaStreamSynchronize(st_);
+        }
+        hv[k] = VLevel<T>{lv_[k].g, lv_[k].x, lv_[k].x2, lv_[k].b, lv_[k].d, lv_[k].inv,
+                          lv_[k].cf, lv_[k].pat};
+      }
       dlv_ = c_->mem.alloc<VLevel<T>>(K_ + 1);
+      dasm_ = c_->mem.alloc<AsmLevel<T>>(K_ + 1);
+      dtab_ = c_->mem.alloc<OpTable<T>>(1);
       std::vector<Phase> all;
       for (int k = 0; k <= K_; ++k) {
         const std::vector<Phase> p = vcycle_phases(k, cfg.nu1, cfg.nu2);
@@ -107,6 +119,7 @@ class Solver final : public SolverBase {
       cudaMemcpyAsync(dlv_, hv.data(), sizeof(VLevel<T>) * hv.size(), cudaMemcpyHostToDevice, st_);
       cudaMemcpyAsync(dph_, all.data(), sizeof(Phase) * all.size(), cudaMemcpyHostToDevice, st_);
       cudaStreamSynchronize(st_);
+      upload_operator();
       coarse_nd_ = 3 * lv_[0].g.nn;
       bool fits = true;
       for (int k = 0; k <= K_; ++k) fits = fits && vcycle_fits(ph_n_[k], k + 1);
@@ -156,13 +169,16 @@ class Solver final : public SolverBase {
     // idle: levels below the top run on side streams beside it
     const int p = c_->prof.begin(DNNMG_STAGE_VANKA_SETUP, lv_[K_].level, st_);
     const bool fork = !side_.empty() && !capturing();
-    if (fork) cudaEventRecord(fork_ev_, st_);
+    if (fork) {
+      cudaEventRecord(fork_ev_, st_);
+      for (cudaStream_t s : side_) cudaStreamWaitEvent(s, fork_ev_, 0);
+    }
+    // the first side stream is joined below, after level 1's setup
+    if (const int na = assembled_levels())
+      launch_assemble_blocks<T>(dasm_, na, asm_nodes_[na], fork ? side_[0] : st_);
     for (int k = K_; k > 0; --k) {
       cudaStream_t s = st_;
-      if (fork && k < K_) {
-        s = side_[k - 1];
-        cudaStreamWaitEvent(s, fork_ev_, 0);
-      }
+      if (fork && k < K_) s = side_[k - 1];
       launch_vanka_setup<T>(lv_[k].g, lv_[k].s, lv_[k].vb, lv_[k].inv, status_, s);
       if (s != st_) {
         cudaEventRecord(side_ev_[k - 1], s);
@@ -336,6 +352,8 @@ class Solver final : public SolverBase {
     Sten<T> s{};
     Sten<double> s64{};
     T *x = nullptr, *x2 = nullptr, *b = nullptr, *d = nullptr, *vb = nullptr, *inv = nullptr;
+    T* cf = nullptr;           // assembled velocity blocks (vnode.cuh)
+    uint16_t* pat = nullptr;   // node patterns
     double* vb64 = nullptr;
     alignas(64) unsigned char tmap[kTensorMapBytes] = {};  // TMA map of inv (FP32)
     bool stream_ok = false;  // the streaming colour pass can run on this level
@@ -376,16 +394,32 @@ class Solver final : public SolverBase {
       l.s64 = make_sten<double>(l.g.h, cfg);
     }
     if (part_solid_) pieces_ = make_patch_pieces(lv_[0].g.h, cfg);
-    if (dlv_) {
-      std::vector<VLevel<T>> hv(K_ + 1);
-      for (int k = 0; k <= K_; ++k)
-        hv[k] = VLevel<T>{lv_[k].g, lv_[k].s, lv_[k].x, lv_[k].x2, lv_[k].b, lv_[k].d,
-                          lv_[k].vb, lv_[k].inv};
-      cudaMemcpyAsync(dlv_, hv.data(), sizeof(VLevel<T>) * hv.size(), cudaMemcpyHostToDevice, st_);
-      cudaStreamSynchronize(st_);
-    }
+    if (dlv_) upload_operator();
     coarse_done_ = false;
     linearized_ = linearized_j_ = false;
+  }
+
+  // The constants of the persistent cycle's operator: every level's assembly
+  // record and the coefficient table of a mesh of width 1.
+  void upload_operator() {
+    std::vector<AsmLevel<T>> ha(K_ + 1);
+    asm_nodes_.assign(K_ + 1, 0);
+    for (int k = 1; k <= K_; ++k) {
+      ha[k - 1] = AsmLevel<T>{lv_[k].g, lv_[k].s, lv_[k].vb, lv_[k].cf, asm_nodes_[k - 1]};
+      asm_nodes_[k] = asm_nodes_[k - 1] + lv_[k].g.nn;
+    }
+    auto tab = std::make_unique<OpTable<T>>();
+    fill_op_table<T>(make_sten<double>(1.0, c_->cfg), *tab);
+    cudaMemcpyAsync(dasm_, ha.data(), sizeof(AsmLevel<T>) * ha.size(), cudaMemcpyHostToDevice, st_);
+    cudaMemcpyAsync(dtab_, tab.get(), sizeof(OpTable<T>), cudaMemcpyHostToDevice, st_);
+    cudaStreamSynchronize(st_);
+  }
+
+  // Levels whose part of the cycle the persistent launch runs (all while the
+  // split is not tuned yet): their velocity blocks are assembled.
+  int assembled_levels() const {
+    if (!dasm_ || split_ == 0 || (vgrid_ <= 0 && cluster_ <= 0)) return 0;
+    return split_ < 0 ? K_ : std::min(K_, std::max(0, split_ - lv_[0].level));
   }
 
   int split_level() const override { return split_ > 0 ? split_ : 0; }
@@ -464,11 +498,11 @@ class Solver final : public SolverBase {
           if (cand > 0 && ((mode == 0 && vgrid_ <= 0) || (mode == 1 && cluster_ <= 0))) continue;
           split_ = cand;
           split_mode_ = mode;
-          // cooperative grids: also fewer blocks than tiles (cheaper grid
-          // barriers, more tiles per block); 0 = one block per tile
-          for (int cap : {0, 2, 1}) {
+          // cooperative grids: also fewer blocks (cheaper grid barriers, more
+          // warps per block); 0 = one block per SM
+          for (int cap : {0, 2, 4}) {
             if (cap > 0 && (mode != 0 || cand == 0)) continue;
-            coop_cap_ = cap * sms_;
+            coop_cap_ = cap > 0 ? sms_ / cap : 0;
             persistent_failed_ = false;
             float ms = time_ms([&] { cycle(top, b, x); }, 5);
             if (persistent_failed_) ms = 1e30f;
@@ -514,15 +548,14 @@ class Solver final : public SolverBase {
       const int p = c_->prof.begin(DNNMG_STAGE_VCYCLE, lv_[k].level, st_);
       int rc;
       if (split_mode_ == 0) {
-        // one block per colour-pass tile of the sub-cycle's top level
-        int blocks = vcycle_coop_tiles(lv_[k].g);
-        blocks = blocks < 64 ? 64 : blocks;
+        // at most one block per warp tile of the sub-cycle's top level
+        int blocks = std::max(64, vcycle_warp_tiles(lv_[k].g));
         if (coop_cap_ > 0 && blocks > coop_cap_) blocks = coop_cap_;
         blocks = blocks > vgrid_ ? vgrid_ : blocks;
-        rc = launch_vcycle_persistent<T>(dlv_, dph_ + ph_off_[k], ph_n_[k], k, b, x, ainv_,
+        rc = launch_vcycle_persistent<T>(dlv_, dtab_, dph_ + ph_off_[k], ph_n_[k], k, b, x, ainv_,
                                          (T)c_->cfg.omega, blocks, coarse_nd_, st_, skip);
       } else {
-        rc = launch_vcycle_cluster<T>(dlv_, dph_ + ph_off_[k], ph_n_[k], k, b, x, ainv_,
+        rc = launch_vcycle_cluster<T>(dlv_, dtab_, dph_ + ph_off_[k], ph_n_[k], k, b, x, ainv_,
                                       (T)c_->cfg.omega, cluster_, coarse_nd_, st_);
       }
       c_->prof.end(p, st_);
@@ -573,6 +606,9 @@ class Solver final : public SolverBase {
   T* vbJ_ = nullptr;  // top-level linearisation of the FGMRES matvec
   LinLevels<T> lin_ = {};  // every level's linearisation buffers
   VLevel<T>* dlv_ = nullptr;
+  AsmLevel<T>* dasm_ = nullptr;    // levels 1..K of the assembly
+  OpTable<T>* dtab_ = nullptr;
+  std::vector<int> asm_nodes_;     // nodes of the first k assembled levels
   std::vector<cudaStream_t> side_;   // side_[k - 1]: setup of level k < K
   std::vector<cudaEvent_t> side_ev_;
   cudaEvent_t fork_ev_ = nullptr;

@@ -19,6 +19,8 @@ struct HostLevel {
 };
 
 HostLevel make_level(int ell, int oi0, int oj0, int olev);
+// patterns of the level's nodes (vnode.cuh)
+std::vector<uint16_t> node_patterns(const HostLevel& L);
 // whether some 2h stabilisation patch of the level is part solid
 bool part_solid_patches(const HostLevel& L);
 struct PatchPieces;

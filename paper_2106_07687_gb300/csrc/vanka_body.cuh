@@ -4,8 +4,8 @@
 // Setup: for every fluid cell, the restriction of the global Jacobian to the
 // cell's 12 DOFs (its 4 nodes x u, v, p), with identity rows/columns on
 // constrained DOFs, is inverted by Gauss-Jordan elimination with partial
-// pivoting and stored as inv[colour][entry][slot] so that the smoothing pass
-// streams it with coalesced loads.
+// pivoting and stored by node of the cell (vanka_inv_index) so that the
+// smoothing pass streams it with coalesced 16-byte loads.
 //
 // Tiled colour pass: a block owns kTCX x kTCY cells of the colour, i.e. the
 // (2 kTCX) x (2 kTCY) nodes they cover.  It stages the masked iterate, vbar
@@ -17,9 +17,46 @@
 // colour's fluid cells are copied, so x_out is complete and the next colour
 // reads it without races.
 #pragma once
-#include "common.cuh"
+#include "kernels.h"
 
 namespace dnnmg {
+
+// 16-byte vectors of T
+template <typename T>
+struct Vec16;
+template <>
+struct Vec16<float> {
+  using type = float4;
+};
+template <>
+struct Vec16<double> {
+  using type = double2;
+};
+__device__ __forceinline__ void vec_unpack(const float4& v, float* o) {
+  o[0] = v.x, o[1] = v.y, o[2] = v.z, o[3] = v.w;
+}
+__device__ __forceinline__ void vec_unpack(const double2& v, double* o) { o[0] = v.x, o[1] = v.y; }
+__device__ __forceinline__ float4 vec_pack(const float* o) {
+  return make_float4(o[0], o[1], o[2], o[3]);
+}
+__device__ __forceinline__ double2 vec_pack(const double* o) { return make_double2(o[0], o[1]); }
+
+// 36 entries stored as 16-byte vectors `stride` vectors apart, read only
+// during the kernel
+template <typename T>
+__device__ __forceinline__ void load36(const T* base, size_t first, size_t stride, T out[36]) {
+  using V = typename Vec16<T>::type;
+  const V* p = reinterpret_cast<const V*>(base) + first;
+#pragma unroll
+  for (int v = 0; v < 36 / kVec16<T>; ++v) vec_unpack(__ldg(p + v * stride), out + v * kVec16<T>);
+}
+// the rows c * 4 + a of the inverse of the cell of `slot` (see vanka_inv_index)
+template <typename T>
+__device__ __forceinline__ void load_inv_rows(const T* inv, int nslots, int colour, int slot, int a,
+                                              T iv[36]) {
+  load36<T>(inv, ((size_t)colour * (36 / kVec16<T>) * nslots + slot) * 4 + a, (size_t)nslots * 4,
+            iv);
+}
 
 template <typename T>
 __device__ __forceinline__ T vk_abs(T v) {
@@ -244,10 +281,10 @@ __device__ __forceinline__ void vanka_setup_cell(const Grid& g, const Sten<T>& s
   }
   if (lane >= 12) return;
   // row my_col of the inverse; entry j is its column pcol[j]
-  T* out = inv + (size_t)colour * 144 * nslots + slot;
 #pragma unroll
   for (int j = 0; j < 12; ++j)
-    out[(size_t)(my_col * 12 + pcol[j]) * nslots] = ok ? A[j] : T(0);
+    inv[vanka_inv_index<T>(nslots, colour, slot, my_col & 3, (my_col >> 2) * 12 + pcol[j])] =
+        ok ? A[j] : T(0);
 }
 
 // Resident blocks per SM the pass kernels ask the compiler for: FP32 passes
@@ -450,11 +487,7 @@ __device__ __forceinline__ void vanka_pass_tile(const Grid& g, const Sten<T>& s,
   if (node_ok) {
     xu = xin[n], xv = xin[nn + n], xp = xin[2 * nn + n];
     bu0 = b[n], bv0 = b[nn + n], bp0 = b[2 * nn + n];
-    const T* row0 = inv + (size_t)colour * 144 * nslots + slot;
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int k = 0; k < 12; ++k) iv[c * 12 + k] = row0[(size_t)((c * 4 + a) * 12 + k) * nslots];
+    load_inv_rows<T>(inv, nslots, colour, slot, a, iv);
   }
   pass_stage_rows<T, kTCX, kTCY, NTT>(g, s, xin, vb, i0, j0, t, S);
   // own cell (ci, cj) sits at staged index (ci - i0 + 2, cj - j0 + 2)
@@ -529,15 +562,13 @@ __device__ __forceinline__ void vanka_pass_zero_node(const Grid& g, int colour,
   }
   if (!node_ok) return;
   if (cell_ok) {
-    // one row of the inverse at a time (fewer live registers)
-    const T* row0 = inv + (size_t)colour * 144 * nslots + slot;
-    T acc[3];
+    T iv[36], acc[3];
+    load_inv_rows<T>(inv, nslots, colour, slot, a, iv);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       acc[c] = 0;
 #pragma unroll
-      for (int k = 0; k < 12; ++k)
-        acc[c] += row0[(size_t)((c * 4 + a) * 12 + k) * nslots] * d[k];
+      for (int k = 0; k < 12; ++k) acc[c] += iv[c * 12 + k] * d[k];
     }
     xout[n] = T(0) + omega * acc[0];
     xout[nn + n] = T(0) + omega * acc[1];

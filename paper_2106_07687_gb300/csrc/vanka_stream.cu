@@ -11,10 +11,10 @@
 // that of vanka_pass_tile (the same staging, rows, defect sums and 12 x 12
 // products in the same order), so the result is bitwise the tiled pass's.
 //
-// Thread layout: thread t owns node a = t / 64 of colour cell q = t % 64 of
-// the tile, so that a warp reads one inverse entry of 32 consecutive cells
-// (conflict-free in the [entry][cell] box); the four nodes of a cell pass
-// their defects through shared memory.
+// Thread layout: thread t owns node a = t % 4 of colour cell q = t / 4 of the
+// tile, so that a warp reads 512 consecutive bytes of a vector of the inverses
+// (vanka_inv_index); the four nodes of a cell pass their defects through
+// shared memory.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -39,7 +39,7 @@ constexpr uint32_t kStreamPolls = 1u << 24;
 constexpr int kBufs = 1;
 
 struct StreamSmem {
-  float inv[kBufs][144][kQ];  // inverse rows of the tile, [entry][qy * 16 + qx]
+  float4 inv[kBufs][9][kQ][4];  // inverse rows of the tile, [vector][qy * 16 + qx][node]
   PassSmem<float, kQX, kQY> p;
   float d[kQ][13];        // the 12 defects of each colour cell (padded row)
   uint64_t bar[2];
@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(kStreamThreads, kBufs == 1 ? 3 : 2)
   const int nbx = cdiv(sx, kQX), nt = nbx * cdiv(sy, kQY);
   const int nn = g.nn;
   const int t = threadIdx.x;
-  const int a = t / kQ, q = t % kQ, qx = q % kQX, qy = q / kQX;
+  const int a = t & 3, q = t >> 2, qx = q % kQX, qy = q / kQX;
   if (t == 0) {
     mbar_init(&S.bar[0], 1);
     mbar_init(&S.bar[1], 1);
@@ -81,8 +81,8 @@ __global__ void __launch_bounds__(kStreamThreads, kBufs == 1 ? 3 : 2)
   __syncthreads();
   auto issue = [&](int tile, int buf) {  // thread 0 only
     mbar_expect_tx(&S.bar[buf], kBoxBytes);
-    tma_load_3d(&S.inv[buf][0][0], &tmap, (tile % nbx) * kQX, (tile / nbx) * kQY, colour * 144,
-                &S.bar[buf]);
+    tma_load_3d(&S.inv[buf][0][0][0], &tmap, (tile % nbx) * kQX * 16, (tile / nbx) * kQY,
+                colour * 9, &S.bar[buf]);
   };
   uint32_t parity[2] = {0u, 0u};
   bool pending[2] = {(int)blockIdx.x < nt, false};  // a copy into the buffer is in flight
@@ -132,7 +132,12 @@ __global__ void __launch_bounds__(kStreamThreads, kBufs == 1 ? 3 : 2)
         for (int c = 0; c < 3; ++c) {
           acc[c] = 0;
 #pragma unroll
-          for (int k = 0; k < 12; ++k) acc[c] += S.inv[buf][(c * 4 + a) * 12 + k][q] * S.d[q][k];
+          for (int k4 = 0; k4 < 3; ++k4) {
+            float iv[4];
+            vec_unpack(S.inv[buf][3 * c + k4][q][a], iv);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) acc[c] += iv[k] * S.d[q][4 * k4 + k];
+          }
         }
         xout[n] = xu + omega * acc[0];
         xout[nn + n] = xv + omega * acc[1];
@@ -179,12 +184,12 @@ bool make_vanka_tensor_map(void* map, const float* inv, const Grid& g) {
   const PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
   if (!fn || !inv || (reinterpret_cast<uintptr_t>(inv) & 15)) return false;
   const int sx = g.nx / 2 + 1, sy = g.ny / 2 + 1, pitch = vanka_pitch(g);
-  // inv[colour][entry][tj][ti] as a 3-D array (ti, tj, colour * 144 + entry);
-  // rows of pitch floats, so every stride is a multiple of 16 bytes
-  const cuuint64_t dims[3] = {(cuuint64_t)sx, (cuuint64_t)sy, 4 * 144};
-  const cuuint64_t strides[2] = {(cuuint64_t)pitch * sizeof(float),
-                                 (cuuint64_t)pitch * sy * sizeof(float)};
-  const cuuint32_t box[3] = {kQX, kQY, 144};
+  // inv[colour][vector][tj][ti][node][4] as a 3-D array (16 floats per slot,
+  // tj, colour * 9 + vector); 64 bytes per slot, so every copy is aligned
+  const cuuint64_t dims[3] = {(cuuint64_t)sx * 16, (cuuint64_t)sy, 4 * 9};
+  const cuuint64_t strides[2] = {(cuuint64_t)pitch * 16 * sizeof(float),
+                                 (cuuint64_t)pitch * sy * 16 * sizeof(float)};
+  const cuuint32_t box[3] = {kQX * 16, kQY, 9};
   const cuuint32_t estr[3] = {1, 1, 1};
   return fn(reinterpret_cast<CUtensorMap*>(map), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3,
             const_cast<float*>(inv), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,

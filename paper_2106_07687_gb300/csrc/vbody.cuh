@@ -5,78 +5,6 @@
 
 namespace dnnmg {
 
-// One colour pass of the Vanka smoother for global thread `tid` (four
-// consecutive threads form the quad of one cell; every lane of a warp must
-// call this together because of the shuffles).  See vanka.cu.
-template <typename T>
-__device__ __forceinline__ void vanka_pass_thread(const Grid& g, const Sten<T>& s, int colour,
-                                                  const T* __restrict__ b,
-                                                  const T* __restrict__ xin,
-                                                  const T* __restrict__ vb,
-                                                  const T* __restrict__ inv, T omega,
-                                                  T* __restrict__ xout, int tid) {
-  const int cx = colour & 1, cy = colour >> 1;
-  const int sx = g.nx / 2 + 1, pitch = vanka_pitch(g);
-  const int nslots = vanka_slots(g);
-  const int slot = tid >> 2, a = tid & 3;
-  const bool slot_ok = slot < nslots && slot % pitch < sx;
-  const int ci = 2 * (slot % pitch) - cx, cj = 2 * (slot / pitch) - cy;
-  const int i = ci + (a & 1), j = cj + (a >> 1);
-  const bool node_ok = slot_ok && i >= 0 && j >= 0 && i <= g.nx && j <= g.ny;
-  const bool cell_ok = slot_ok && ci >= 0 && cj >= 0 && ci < g.nx && cj < g.ny &&
-                       !g.solid[(cj < 0 ? 0 : cj) * g.nx + (ci < 0 ? 0 : ci)];
-  const int nn = g.nn;
-  const int n = node_ok ? j * g.nnx + i : 0;
-  // loads independent of the defect first (latency overlaps the stencil)
-  T xu = 0, xv = 0, xp = 0, b0 = 0, b1 = 0, b2 = 0;
-  T iv[36];
-  if (node_ok) {
-    xu = xin[n], xv = xin[nn + n], xp = xin[2 * nn + n];
-    b0 = b[n], b1 = b[nn + n], b2 = b[2 * nn + n];
-  }
-  if (node_ok && cell_ok) {
-    const T* row0 = inv + (size_t)colour * 144 * nslots + slot;
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int k = 0; k < 12; ++k) iv[c * 12 + k] = row0[(size_t)((c * 4 + a) * 12 + k) * nslots];
-  }
-  T du = 0, dv = 0, dp = 0;
-  if (node_ok && cell_ok) {
-    T ru, rv, rp;
-    node_rows<T, false, true>(g, s, i, j, xin, vb, ru, rv, rp);
-    const uint8_t f = g.flags[n];
-    du = b0 - ((f & kVDir) ? xu : ru);
-    dv = b1 - ((f & kVDir) ? xv : rv);
-    dp = b2 - ((f & kPFix) ? xp : rp);
-  }
-  const int lane = threadIdx.x & 31, base = lane & ~3;
-  T d[12];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    d[k] = __shfl_sync(0xffffffffu, du, base + k);
-    d[4 + k] = __shfl_sync(0xffffffffu, dv, base + k);
-    d[8 + k] = __shfl_sync(0xffffffffu, dp, base + k);
-  }
-  if (!node_ok) return;
-  if (cell_ok) {
-    T acc[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      acc[c] = 0;
-#pragma unroll
-      for (int k = 0; k < 12; ++k) acc[c] += iv[c * 12 + k] * d[k];
-    }
-    xout[n] = xu + omega * acc[0];
-    xout[nn + n] = xv + omega * acc[1];
-    xout[2 * nn + n] = xp + omega * acc[2];
-  } else {
-    xout[n] = xu;
-    xout[nn + n] = xv;
-    xout[2 * nn + n] = xp;
-  }
-}
-
 // d = b - A'(vbar) x at node (i, j); constrained rows: b - x, or 0 if masked.
 template <typename T>
 __device__ __forceinline__ void defect_node(const Grid& g, const Sten<T>& s, const T* __restrict__ b,

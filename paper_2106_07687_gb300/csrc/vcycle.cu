@@ -6,15 +6,16 @@
 // coarse iterate zeroed), the coarse direct solve, prolongation -- built once
 // per top level on the host.  The kernel walks the phase list; all blocks
 // share every phase and meet at a barrier (grid-wide, or the hardware cluster
-// barrier) before the next.  Every phase runs the same per-thread bodies as
-// the one-launch-per-stage kernels, so the arithmetic is identical; only the
-// ~20 kernel launches per level and cycle disappear.
+// barrier) before the next.
+//
+// A phase is bound by its dependent chain (barrier, loads from L2, rows,
+// products, stores), not by bandwidth, on all but the largest levels.  Colour
+// passes and defects therefore work from assembled coefficients, one warp per
+// 8 x 4 nodes and without a block barrier (vnode.cuh).
 #include <algorithm>
 #include <cooperative_groups.h>
 
 #include "kernels.h"
-#include "optile_body.cuh"
-#include "vanka_body.cuh"
 #include "vbody.cuh"
 #include "vcycle.h"
 
@@ -24,32 +25,34 @@ namespace dnnmg {
 
 namespace {
 
-// Colour-pass tiles (colour cells).  The cooperative kernel takes 8 x 4
-// tiles, one per block at a time: on the small levels of a sub-cycle the
-// tile's cell rows (ALU-bound on one SM) are the longest part of a pass, and
-// smaller tiles spread a level over more SMs.  Its blocks have 256 threads:
-// 128 own the tile's nodes and 128 help stage it and compute its rows.  The
-// single-cluster kernel (16 blocks) keeps 16 x 4 tiles, two per block.
-constexpr int kCTX = 8, kCTY = 4;
-constexpr int kLTX = 16, kLTY = 4;
-constexpr int kCoopOwners = 4 * kCTX * kCTY;
-constexpr int kCoopThreads = 2 * kCoopOwners;
-constexpr int kClusterOwners = 4 * kLTX * kLTY;
-// threads per block of the single-cluster launch (FP64 needs more registers)
+// Threads per block, one block per SM: a pass holds 36 coefficients and 36
+// inverse entries per thread, so FP32 takes 16 warps of 128 registers and FP64
+// 8 warps of 255.
 template <typename T>
-constexpr int cluster_threads() {
-  return sizeof(T) == 4 ? 2 * kClusterOwners : kClusterOwners;
+constexpr int walk_threads() {
+  return sizeof(T) == 4 ? 512 : 256;
 }
 constexpr int kMaxPhases = 160;  // phases of one launch (a V(2,2) cycle from level 8)
 constexpr int kMaxVLevels = 10;
 
-// Shared-memory copies of the launch's phase list and level records, loaded
-// once so that no phase starts with a dependent global load.
+// Dynamic shared memory of a block: the launch's phase list, level records
+// and coefficient table, loaded once so that no phase starts with a dependent
+// global load, and a scratch area for the warp tiles or the coarse vector.
 template <typename T>
 struct WalkSmem {
+  OpTable<T> tab;
   VLevel<T> lv[kMaxVLevels];
   Phase ph[kMaxPhases];
+  alignas(16) WarpTile<T> tile[walk_threads<T>() / 32];
 };
+
+template <class S>
+__device__ __forceinline__ void copy_ints(S* dst, const S* src, int count) {
+  static_assert(sizeof(S) % sizeof(int) == 0, "record size");
+  const int* s = reinterpret_cast<const int*>(src);
+  int* d = reinterpret_cast<int*>(dst);
+  for (int e = threadIdx.x; e < (int)(count * sizeof(S) / sizeof(int)); e += blockDim.x) d[e] = s[e];
+}
 
 // Item n < count of a node-wise phase for every thread of the grid: chunks
 // of 32 consecutive items (one warp, coalesced) go round-robin over the
@@ -67,73 +70,47 @@ __device__ __forceinline__ void for_items(int count, F f) {
 
 // Walk the phase list; `sync` separates phases (a grid-wide barrier for the
 // cooperative launch, the cluster barrier for the single-cluster launch).
-// Threads of all blocks split every node-wise phase; a colour pass gives each
-// group of NTT threads of a block one TCX x TCY tile at a time.
-template <typename T, int TCX, int TCY, int NT, int NTT, class Sync>
-__device__ __forceinline__ void walk_phases(const VLevel<T>* __restrict__ glv,
-                                            const Phase* __restrict__ gph, int nph, int top,
-                                            const T* __restrict__ topb, T* __restrict__ topx,
-                                            const double* __restrict__ Ainv, T omega,
-                                            uint8_t* dyn, WalkSmem<T>& S, Sync sync) {
-  // dynamic shared memory: the pass tiles, the defect tile or the coarse vector
-  double* sbuf = reinterpret_cast<double*>(dyn);
-  PassSmem<T, TCX, TCY>* tsm = reinterpret_cast<PassSmem<T, TCX, TCY>*>(dyn);
-  constexpr int kDX = 16, kDY = 8;  // defect tile: owners plus helpers, as a pass tile
-  auto& dsm = *reinterpret_cast<OpSmem<T, kDX, kDY>*>(dyn);
-  {
-    const int nl = top + 1;
-    const int* src = reinterpret_cast<const int*>(glv);
-    int* dst = reinterpret_cast<int*>(S.lv);
-    for (int e = threadIdx.x; e < (int)(nl * sizeof(VLevel<T>) / sizeof(int)); e += NT)
-      dst[e] = src[e];
-    const int* ps = reinterpret_cast<const int*>(gph);
-    int* pd = reinterpret_cast<int*>(S.ph);
-    for (int e = threadIdx.x; e < (int)(nph * sizeof(Phase) / sizeof(int)); e += NT) pd[e] = ps[e];
-    __syncthreads();
-  }
-  constexpr int kTiles = NT / NTT;  // pass tiles in flight per block
-  const int sub = threadIdx.x / NTT;
+// Threads of all blocks split every node-wise phase; the warp tiles of a
+// colour pass or defect go round-robin over the blocks first.
+template <typename T, class Sync>
+__device__ __forceinline__ void walk_phases(const VLevel<T>* glv, const OpTable<T>* gtab,
+                                            const Phase* gph, int nph, int top, const T* topb,
+                                            T* topx, const double* __restrict__ Ainv, T omega,
+                                            WalkSmem<T>& S, Sync sync) {
+  constexpr int NT = walk_threads<T>();
+  double* sbuf = reinterpret_cast<double*>(S.tile);  // the coarse right-hand side
+  copy_ints(S.lv, glv, top + 1);
+  copy_ints(S.ph, gph, nph);
+  copy_ints(&S.tab, gtab, 1);
+  __syncthreads();
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int w0 = blockIdx.x + gridDim.x * w, nw = gridDim.x * (NT / 32);
   for (int p = 0; p < nph; ++p) {
     const Phase f = S.ph[p];
     const int k = f.level;
     const VLevel<T>& L = S.lv[k];
     const Grid& g = L.g;
-    const Sten<T>& ss = L.s;
     const T* b = k == top ? topb : L.b;
     T* x0 = k == top ? topx : L.x;
     switch (f.type) {
       case kPhasePass: {
-        // tiles of TCX x TCY colour cells, kTiles per block at a time
         const T* xin = f.in ? L.x2 : x0;
         T* xout = f.out ? L.x2 : x0;
-        const int nbx = cdiv(g.nx / 2 + 1, TCX);
-        const int nt = nbx * cdiv(g.ny / 2 + 1, TCY);
-        for (int t0 = blockIdx.x * kTiles; t0 < nt; t0 += gridDim.x * kTiles) {
-          const int t = t0 + sub;
-          vanka_pass_tile<T, TCX, TCY, NTT>(g, ss, f.colour, b, xin, L.vb, L.inv, omega, xout,
-                                            t % nbx, t / nbx, tsm[sub], t < nt);
-          __syncthreads();  // the tile's shared memory is reused by the next tile
-        }
+        const NodeLevel<T> N{g.nx, g.ny, g.nnx, g.nn, L.pat, L.cf, (T)g.h, (T)(g.h * g.h)};
+        const int pitch = vanka_pitch(g), nslots = vanka_slots(g);
+        const int nbx = cdiv(g.nx / 2 + 1, kWX / 2);
+        const int nt = nbx * cdiv(g.ny / 2 + 1, kWY / 2);
+        for (int t = w0; t < nt; t += nw)
+          warp_pass_tile<T>(N, S.tab, f.colour, b, xin, L.inv, pitch, nslots, omega, xout, t % nbx,
+                            t / nbx, lane, S.tile[w]);
         break;
       }
       case kPhaseDefect: {
-        // tiles of kDX x kDY nodes, each cell's rows computed once per tile
-        const T* x = f.in ? L.x2 : x0;
-        const int ntx = cdiv(g.nnx, kDX), ntiles = ntx * cdiv(g.nny, kDY);
-        const int nn = g.nn;
-        for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-          T ru, rv, rp;
-          int n;
-          op_tile_rows<T, false, true, kDX, kDY, NT>(g, ss, x, L.vb, t % ntx, t / ntx, dsm, ru, rv,
-                                                     rp, n);
-          if (n >= 0) {
-            const uint8_t fl = op_tile_flags<T, kDX, kDY>(dsm);
-            L.d[n] = (fl & kVDir) ? T(0) : b[n] - ru;
-            L.d[nn + n] = (fl & kVDir) ? T(0) : b[nn + n] - rv;
-            L.d[2 * nn + n] = (fl & kPFix) ? T(0) : b[2 * nn + n] - rp;
-          }
-          __syncthreads();  // the tile's shared memory is reused by the next tile
-        }
+        const NodeLevel<T> N{g.nx, g.ny, g.nnx, g.nn, L.pat, L.cf, (T)g.h, (T)(g.h * g.h)};
+        const int nbx = cdiv(g.nnx, kWX), nt = nbx * cdiv(g.nny, kWY);
+        for (int t = w0; t < nt; t += nw)
+          warp_defect_tile<T>(N, S.tab, b, f.in ? L.x2 : x0, L.d, t % nbx, t / nbx, lane,
+                              S.tile[w]);
         break;
       }
       case kPhaseRestrict: {
@@ -156,8 +133,7 @@ __device__ __forceinline__ void walk_phases(const VLevel<T>* __restrict__ glv,
         T* xout = f.out ? L.x2 : x0;
         const int count = 4 * vanka_slots(g);
         const int nchunks = (count + 31) >> 5;
-        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-        for (int c = blockIdx.x + gridDim.x * w; c < nchunks; c += gridDim.x * (NT / 32)) {
+        for (int c = w0; c < nchunks; c += nw) {
           const int e = (c << 5) + lane;
           vanka_pass_zero_node<T>(g, f.colour, b, L.inv, omega, xout, e, e < count);
         }
@@ -178,8 +154,7 @@ __device__ __forceinline__ void walk_phases(const VLevel<T>* __restrict__ glv,
         }
         __syncthreads();
         // one warp per row, rows round-robin over the blocks first
-        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-        for (int r = blockIdx.x + gridDim.x * w; r < nd; r += gridDim.x * (NT / 32)) {
+        for (int r = w0; r < nd; r += nw) {
           const double* row = Ainv + (size_t)r * nd;
           // chunks of 16 entries per lane: every load of a chunk is issued
           // before its products are summed, so that a row of up to 512
@@ -220,33 +195,41 @@ __device__ __forceinline__ void walk_phases(const VLevel<T>* __restrict__ glv,
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kCoopThreads)
-    vcycle_kernel(const VLevel<T>* __restrict__ lv, const Phase* __restrict__ ph, int nph, int top,
-                  const T* __restrict__ topb, T* __restrict__ topx, const double* __restrict__ Ainv,
-                  T omega, const int* skip) {
+__global__ void __launch_bounds__(walk_threads<T>(), 1)
+    vcycle_kernel(const VLevel<T>* lv, const OpTable<T>* tab, const Phase* ph, int nph, int top,
+                  const T* topb, T* topx, const double* __restrict__ Ainv, T omega,
+                  const int* skip) {
   // a speculative FGMRES iteration after the cycle stopped: every block
   // reads the same flag (set before this launch) and returns before any barrier
   if (skip && *skip) return;
-  extern __shared__ __align__(16) uint8_t dyn[];  // coarse vector or pass tiles
-  __shared__ WalkSmem<T> S;
+  extern __shared__ __align__(16) uint8_t dyn[];
   cg::grid_group grid = cg::this_grid();
-  walk_phases<T, kCTX, kCTY, kCoopThreads, kCoopThreads>(lv, ph, nph, top, topb, topx, Ainv,
-                                                         omega, dyn, S, [&] { grid.sync(); });
+  walk_phases<T>(lv, tab, ph, nph, top, topb, topx, Ainv, omega,
+                 *reinterpret_cast<WalkSmem<T>*>(dyn), [&] { grid.sync(); });
 }
 
 // The whole grid is one thread-block cluster; phases are separated by the
 // cluster barrier (release / acquire at cluster scope, so the global-memory
 // results of one phase are visible to every block of the cluster in the next).
 template <typename T>
-__global__ void __launch_bounds__(cluster_threads<T>())
-    vcycle_cluster_kernel(const VLevel<T>* __restrict__ lv, const Phase* __restrict__ ph, int nph,
-                          int top, const T* __restrict__ topb, T* __restrict__ topx,
-                          const double* __restrict__ Ainv, T omega) {
-  extern __shared__ __align__(16) uint8_t dyn[];  // coarse vector or pass tiles
-  __shared__ WalkSmem<T> S;
+__global__ void __launch_bounds__(walk_threads<T>(), 1)
+    vcycle_cluster_kernel(const VLevel<T>* lv, const OpTable<T>* tab, const Phase* ph, int nph,
+                          int top, const T* topb, T* topx, const double* __restrict__ Ainv,
+                          T omega) {
+  extern __shared__ __align__(16) uint8_t dyn[];
   cg::cluster_group cl = cg::this_cluster();
-  walk_phases<T, kLTX, kLTY, cluster_threads<T>(), kClusterOwners>(
-      lv, ph, nph, top, topb, topx, Ainv, omega, dyn, S, [&] { cl.sync(); });
+  walk_phases<T>(lv, tab, ph, nph, top, topb, topx, Ainv, omega,
+                 *reinterpret_cast<WalkSmem<T>*>(dyn), [&] { cl.sync(); });
+}
+
+template <typename T>
+__global__ void __launch_bounds__(128)
+    assemble_blocks_kernel(const AsmLevel<T>* __restrict__ lv, int nlev, int nodes) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= nodes) return;
+  int k = 0;
+  while (k + 1 < nlev && t >= lv[k + 1].first) ++k;
+  assemble_node<T>(lv[k].g, lv[k].s, lv[k].vb, lv[k].cf, t - lv[k].first);
 }
 
 void build_phases(int k, int top, int nu1, int nu2, std::vector<Phase>& out) {
@@ -277,20 +260,25 @@ void build_phases(int k, int top, int nu1, int nu2, std::vector<Phase>& out) {
 }  // namespace
 
 namespace {
-// dynamic shared memory of a block with `tiles_in_flight` TCX x TCY pass
-// tiles: the largest of the coarse right-hand side (FP64), the pass tiles and
-// the 16 x 8-node defect tile
-template <typename T, int TCX, int TCY>
-size_t walk_smem(int coarse_nd, int tiles_in_flight) {
-  size_t m = sizeof(PassSmem<T, TCX, TCY>) * tiles_in_flight;
-  m = std::max(m, sizeof(double) * coarse_nd);
-  m = std::max(m, sizeof(OpSmem<T, 16, 8>));
-  return m;
+// shared memory of a block: its tables and the larger of the warp tiles and
+// the coarse right-hand side (FP64)
+template <typename T>
+size_t walk_smem(int coarse_nd) {
+  const size_t tiles = sizeof(WarpTile<T>) * (walk_threads<T>() / 32);
+  const size_t head = offsetof(WalkSmem<T>, tile);
+  return head + std::max(tiles, sizeof(double) * coarse_nd);
 }
 }  // namespace
 
-int vcycle_coop_tiles(const Grid& g) {
-  return cdiv(g.nx / 2 + 1, kCTX) * cdiv(g.ny / 2 + 1, kCTY);
+template <typename T>
+void launch_assemble_blocks(const AsmLevel<T>* lv, int nlev, int nodes, cudaStream_t st) {
+  if (nodes <= 0) return;
+  note_launch();
+  assemble_blocks_kernel<T><<<cdiv(nodes, 128), 128, 0, st>>>(lv, nlev, nodes);
+}
+
+int vcycle_warp_tiles(const Grid& g) {
+  return cdiv(g.nx / 2 + 1, kWX / 2) * cdiv(g.ny / 2 + 1, kWY / 2);
 }
 
 bool vcycle_fits(int nphases, int nlevels) {
@@ -309,36 +297,35 @@ int vcycle_grid(int coarse_nd) {
   int dev = 0, sms = 0, per = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const size_t smem = walk_smem<T, kCTX, kCTY>(coarse_nd, 1);
+  const size_t smem = walk_smem<T>(coarse_nd);
   if (cudaFuncSetAttribute(vcycle_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)smem) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, vcycle_kernel<T>, kCoopThreads, smem) !=
-          cudaSuccess ||
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, vcycle_kernel<T>, walk_threads<T>(),
+                                                    smem) != cudaSuccess ||
       per <= 0)
     return 0;
-  if (per > 4) per = 4;
-  return per * sms;
+  return sms;  // one block per SM
 }
 
 template <typename T>
-int launch_vcycle_persistent(const VLevel<T>* lv, const Phase* ph, int nph, int top, const T* topb,
-                             T* topx, const double* Ainv, T omega, int grid, int coarse_nd,
-                             cudaStream_t st, const int* skip) {
-  void* args[] = {(void*)&lv,   (void*)&ph,   (void*)&nph,   (void*)&top, (void*)&topb,
-                  (void*)&topx, (void*)&Ainv, (void*)&omega, (void*)&skip};
+int launch_vcycle_persistent(const VLevel<T>* lv, const OpTable<T>* tab, const Phase* ph, int nph,
+                             int top, const T* topb, T* topx, const double* Ainv, T omega, int grid,
+                             int coarse_nd, cudaStream_t st, const int* skip) {
+  void* args[] = {(void*)&lv,   (void*)&tab,  (void*)&ph,   (void*)&nph,   (void*)&top,
+                  (void*)&topb, (void*)&topx, (void*)&Ainv, (void*)&omega, (void*)&skip};
   note_launch();
   const cudaError_t e =
-      cudaLaunchCooperativeKernel((void*)vcycle_kernel<T>, dim3(grid), dim3(kCoopThreads), args,
-                                  walk_smem<T, kCTX, kCTY>(coarse_nd, 1), st);
+      cudaLaunchCooperativeKernel((void*)vcycle_kernel<T>, dim3(grid), dim3(walk_threads<T>()),
+                                  args, walk_smem<T>(coarse_nd), st);
   return e == cudaSuccess ? 0 : 1;
 }
 
 template <typename T>
 int vcycle_cluster_size(int coarse_nd) {
-  const size_t smem = walk_smem<T, kLTX, kLTY>(coarse_nd, cluster_threads<T>() / kClusterOwners);
+  const size_t smem = walk_smem<T>(coarse_nd);
   if (cudaFuncSetAttribute(vcycle_cluster_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)smem) != cudaSuccess) {
     cudaGetLastError();
@@ -358,7 +345,7 @@ int vcycle_cluster_size(int coarse_nd) {
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3(cs);
-    cfg.blockDim = dim3(cluster_threads<T>());
+    cfg.blockDim = dim3(walk_threads<T>());
     cfg.dynamicSmemBytes = smem;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
@@ -372,9 +359,9 @@ int vcycle_cluster_size(int coarse_nd) {
 }
 
 template <typename T>
-int launch_vcycle_cluster(const VLevel<T>* lv, const Phase* ph, int nph, int top, const T* topb,
-                          T* topx, const double* Ainv, T omega, int cluster, int coarse_nd,
-                          cudaStream_t st) {
+int launch_vcycle_cluster(const VLevel<T>* lv, const OpTable<T>* tab, const Phase* ph, int nph,
+                          int top, const T* topb, T* topx, const double* Ainv, T omega,
+                          int cluster, int coarse_nd, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -382,32 +369,29 @@ int launch_vcycle_cluster(const VLevel<T>* lv, const Phase* ph, int nph, int top
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.gridDim = dim3(cluster);
-  cfg.blockDim = dim3(cluster_threads<T>());
-  cfg.dynamicSmemBytes = walk_smem<T, kLTX, kLTY>(coarse_nd, cluster_threads<T>() / kClusterOwners);
+  cfg.blockDim = dim3(walk_threads<T>());
+  cfg.dynamicSmemBytes = walk_smem<T>(coarse_nd);
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   note_launch();
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, vcycle_cluster_kernel<T>, lv, ph, nph, top, topb,
-                                           topx, Ainv, omega);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, vcycle_cluster_kernel<T>, lv, tab, ph, nph, top,
+                                           topb, topx, Ainv, omega);
   return e == cudaSuccess ? 0 : 1;
 }
 
-template int vcycle_grid<float>(int);
-template int vcycle_grid<double>(int);
-template int launch_vcycle_persistent<float>(const VLevel<float>*, const Phase*, int, int,
-                                             const float*, float*, const double*, float, int, int,
-                                             cudaStream_t, const int*);
-template int launch_vcycle_persistent<double>(const VLevel<double>*, const Phase*, int, int,
-                                              const double*, double*, const double*, double, int,
-                                              int, cudaStream_t, const int*);
-template int vcycle_cluster_size<float>(int);
-template int vcycle_cluster_size<double>(int);
-template int launch_vcycle_cluster<float>(const VLevel<float>*, const Phase*, int, int,
-                                          const float*, float*, const double*, float, int, int,
-                                          cudaStream_t);
-template int launch_vcycle_cluster<double>(const VLevel<double>*, const Phase*, int, int,
-                                           const double*, double*, const double*, double, int,
-                                           int, cudaStream_t);
+#define DNNMG_INST(T)                                                                            \
+  template void launch_assemble_blocks<T>(const AsmLevel<T>*, int, int, cudaStream_t);           \
+  template int vcycle_grid<T>(int);                                                              \
+  template int launch_vcycle_persistent<T>(const VLevel<T>*, const OpTable<T>*, const Phase*,    \
+                                           int, int, const T*, T*, const double*, T, int, int,   \
+                                           cudaStream_t, const int*);                            \
+  template int vcycle_cluster_size<T>(int);                                                      \
+  template int launch_vcycle_cluster<T>(const VLevel<T>*, const OpTable<T>*, const Phase*, int,  \
+                                        int, const T*, T*, const double*, T, int, int,           \
+                                        cudaStream_t);
+DNNMG_INST(float)
+DNNMG_INST(double)
+#undef DNNMG_INST
 
 }  // namespace dnnmg

@@ -3,6 +3,7 @@
 #include <vector>
 
 #include "kernels.h"
+#include "vnode.cuh"
 
 namespace dnnmg {
 
@@ -11,9 +12,25 @@ namespace dnnmg {
 template <typename T>
 struct VLevel {
   Grid g;
-  Sten<T> s;
-  T *x, *x2, *b, *d, *vb, *inv;
+  T *x, *x2, *b, *d, *inv;
+  const T* cf;           // assembled velocity blocks (null on the coarsest level)
+  const uint16_t* pat;   // node patterns
 };
+
+// A level's input to the assembly of its velocity blocks; `first` is its
+// first node in the concatenation of the levels of one launch.
+template <typename T>
+struct AsmLevel {
+  Grid g;
+  Sten<T> s;
+  const T* vb;
+  T* cf;
+  int first;
+};
+// velocity blocks of the first nlev levels of `lv` (device array), `nodes`
+// nodes in all, in one launch
+template <typename T>
+void launch_assemble_blocks(const AsmLevel<T>* lv, int nlev, int nodes, cudaStream_t st);
 
 enum PhaseType {
   kPhasePass,
@@ -37,8 +54,8 @@ std::vector<Phase> vcycle_phases(int top, int nu1, int nu2);
 // whether a launch of nphases phases over nlevels levels fits the kernels'
 // shared-memory tables
 bool vcycle_fits(int nphases, int nlevels);
-// colour-pass tiles of the cooperative kernel on a level (its natural grid)
-int vcycle_coop_tiles(const Grid& g);
+// warp tiles of a colour pass on a level
+int vcycle_warp_tiles(const Grid& g);
 // co-resident grid size for the cooperative launch (0 if not available)
 template <typename T>
 int vcycle_grid(int coarse_nd);
@@ -48,14 +65,14 @@ template <typename T>
 int vcycle_cluster_size(int coarse_nd);
 // the same cycle as one thread-block cluster of `cluster` blocks; 0 on success
 template <typename T>
-int launch_vcycle_cluster(const VLevel<T>* lv, const Phase* ph, int nph, int top, const T* topb,
-                          T* topx, const double* Ainv, T omega, int cluster, int coarse_nd,
-                          cudaStream_t st);
+int launch_vcycle_cluster(const VLevel<T>* lv, const OpTable<T>* tab, const Phase* ph, int nph,
+                          int top, const T* topb, T* topx, const double* Ainv, T omega,
+                          int cluster, int coarse_nd, cudaStream_t st);
 // returns 0 on success; with skip, nothing runs when *skip != 0 at the
 // launch's start
 template <typename T>
-int launch_vcycle_persistent(const VLevel<T>* lv, const Phase* ph, int nph, int top, const T* topb,
-                             T* topx, const double* Ainv, T omega, int grid, int coarse_nd,
-                             cudaStream_t st, const int* skip = nullptr);
+int launch_vcycle_persistent(const VLevel<T>* lv, const OpTable<T>* tab, const Phase* ph, int nph,
+                             int top, const T* topb, T* topx, const double* Ainv, T omega, int grid,
+                             int coarse_nd, cudaStream_t st, const int* skip = nullptr);
 
 }  // namespace dnnmg

@@ -1,0 +1,265 @@
+// Node-wise evaluation of the linearised operator from assembled
+// coefficients, and the colour pass and defect of the persistent V-cycle
+// built on it.
+//
+// The operator A'(vbar) of a level does not change during its cycles, while
+// every colour pass and defect applies it once (17 times per level and
+// cycle).  Evaluated cell by cell, with its Gauss points, a row costs about
+// 370 multiply-adds per node and three dependent stages with two block
+// barriers.  Here the 2x2 velocity blocks between a node and its 3x3
+// neighbours, which are all that depends on vbar, are assembled once per
+// linearisation (36 coefficients per node); the gradient, divergence and
+// stabilisation stencils depend only on which of the cells and patches around
+// the node are fluid, so their coefficients come from a small table in shared
+// memory.  A row is then 36 + 36 + 25 multiply-adds, and one warp does a tile
+// of 8 x 4 nodes by itself: no block barrier, and a level of few nodes still
+// spreads over all SMs.
+#pragma once
+#include "vanka_body.cuh"
+
+namespace dnnmg {
+
+// ---- node patterns ---------------------------------------------------------------
+// Bits of the pattern of node (i, j): the four cells around it that are fluid
+// (bit cx + 2 cy, cell (i - 1 + cx, j - 1 + cy)), the four stabilisation
+// patches that hold it and are fluid (bit dI + 2 dJ, patch ((i >> 1) - dI,
+// (j >> 1) - dJ)), and its constrained unknowns.
+constexpr int kPatPatch = 4, kPatVDir = 1 << 8, kPatPFix = 1 << 9;
+
+// ---- coefficient tables -----------------------------------------------------------
+// For a mesh of width 1 (a level scales them by h and h^2, powers of two):
+//   gd[cell mask][neighbour (di + 1) + 3 (dj + 1)] = coefficients of the
+//     neighbour's pressure in the u and v rows, and of its u and v in the
+//     pressure row;
+//   lps[patch mask][(i & 1) + 2 (j & 1)][(di + 2) + 5 (dj + 2)] = coefficients of
+//     the pressures around the node in its pressure row.
+template <typename T>
+struct OpTable {
+  T gd[16][9][4];
+  T lps[16][4][25];
+};
+
+// Fill a table from the constants s of a mesh of width 1 (host).
+template <typename T>
+void fill_op_table(const Sten<double>& s, OpTable<T>& t) {
+  for (int m = 0; m < 16; ++m) {
+    double gd[9][4] = {};
+    for (int c = 0; c < 4; ++c) {
+      if (!(m & (1 << c))) continue;
+      const int cx = c & 1, cy = c >> 1, a = (1 - cx) + 2 * (1 - cy);
+      for (int b = 0; b < 4; ++b) {
+        double* g = gd[(cx + (b & 1)) + 3 * (cy + (b >> 1))];
+        g[0] -= s.Dx[b * 4 + a];
+        g[1] -= s.Dy[b * 4 + a];
+        g[2] += s.Dx[a * 4 + b];
+        g[3] += s.Dy[a * 4 + b];
+      }
+    }
+    for (int e = 0; e < 9; ++e)
+      for (int k = 0; k < 4; ++k) t.gd[m][e][k] = (T)gd[e][k];
+    for (int cls = 0; cls < 4; ++cls) {
+      double l[25] = {};
+      for (int d = 0; d < 4; ++d) {
+        const int s0 = (cls & 1) + 2 * (d & 1), t0 = (cls >> 1) + 2 * (d >> 1);  // in the patch
+        if (!(m & (1 << d)) || s0 > 2 || t0 > 2) continue;
+        for (int q = 0; q < 9; ++q)
+          l[(q % 3 - s0 + 2) + 5 * (q / 3 - t0 + 2)] += s.S9[(s0 + 3 * t0) * 9 + q];
+      }
+      for (int e = 0; e < 25; ++e) t.lps[m][cls][e] = (T)l[e];
+    }
+  }
+}
+
+// ---- assembled velocity blocks -----------------------------------------------------
+// Coefficients of node (i, j): c[4 e + {0, 1, 2, 3}] = the uu, uv, vu and vv
+// entries towards neighbour e = (di + 1) + 3 (dj + 1), summed over the fluid
+// cells (rows of cells first).  Stored as 16-byte vectors of all nodes,
+// vector v of node n at v * nn + n.
+template <typename T>
+__device__ __forceinline__ void assemble_node(const Grid& g, const Sten<T>& s,
+                                              const T* __restrict__ vb, T* __restrict__ cf, int n) {
+  const int i = n % g.nnx, j = n / g.nnx;
+  T c[36];
+#pragma unroll
+  for (int k = 0; k < 36; ++k) c[k] = T(0);
+#pragma unroll
+  for (int cy = 0; cy < 2; ++cy)
+#pragma unroll
+    for (int cx = 0; cx < 2; ++cx) {
+      const int ci = i - 1 + cx, cj = j - 1 + cy;
+      if (ci < 0 || cj < 0 || ci >= g.nx || cj >= g.ny || g.solid[cj * g.nx + ci]) continue;
+      T bu[4], bv[4];
+      load_cell<T, false>(g, vb, ci, cj, 0, bu);
+      load_cell<T, false>(g, vb + g.nn, ci, cj, 0, bv);
+      GaussData<T> gd;
+      gauss_data<T>(bu, bv, gd);
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        T J[3][3];
+        elem_pair<T>(s, gd, (1 - cx) + 2 * (1 - cy), b, J);
+        T* q = c + 4 * ((cx + (b & 1)) + 3 * (cy + (b >> 1)));
+        q[0] += J[0][0], q[1] += J[0][1], q[2] += J[1][0], q[3] += J[1][1];
+      }
+    }
+  using V = typename Vec16<T>::type;
+  V* o = reinterpret_cast<V*>(cf) + n;
+#pragma unroll
+  for (int v = 0; v < 36 / kVec16<T>; ++v) o[(size_t)v * g.nn] = vec_pack(c + v * kVec16<T>);
+}
+
+// ---- one warp, 8 x 4 nodes -----------------------------------------------------------
+// Masked iterate of the warp's nodes plus a two-node halo: 12 x 8 nodes, rows
+// of 24 so that the four rows of a tile fall on different banks.
+constexpr int kWX = 8, kWY = 4, kWSX = kWX + 4, kWSY = kWY + 4, kWPitch = 24;
+template <typename T>
+struct WarpTile {
+  T w[3][kWSY][kWPitch];
+};
+
+// Level data of the node-wise kernels.
+template <typename T>
+struct NodeLevel {
+  int nx, ny, nnx, nn;
+  const uint16_t* pat;  // node patterns
+  const T* cf;          // assembled velocity blocks
+  T h, h2;              // mesh width and its square
+};
+
+// Stage the nodes around tile (i0, j0), three per lane; the iterate is read
+// through L2 (other SMs wrote it).
+template <typename T>
+__device__ __forceinline__ void stage_warp_tile(const NodeLevel<T>& L, const T* x, int i0, int j0,
+                                                int lane, WarpTile<T>& S) {
+  static_assert(kWSX * kWSY == 96, "three nodes per lane");
+  T u[3], v[3], p[3];
+  int pt[3];
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    const int e = lane + 32 * r, i = i0 - 2 + e % kWSX, j = j0 - 2 + e / kWSX;
+    const bool in = i >= 0 && j >= 0 && i <= L.nx && j <= L.ny;
+    const int n = in ? j * L.nnx + i : 0;
+    pt[r] = in ? (int)__ldg(L.pat + n) : (kPatVDir | kPatPFix);
+    u[r] = __ldcg(x + n);
+    v[r] = __ldcg(x + L.nn + n);
+    p[r] = __ldcg(x + 2 * L.nn + n);
+  }
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    const int e = lane + 32 * r, li = e % kWSX, lj = e / kWSX;
+    S.w[0][lj][li] = (pt[r] & kPatVDir) ? T(0) : u[r];
+    S.w[1][lj][li] = (pt[r] & kPatVDir) ? T(0) : v[r];
+    S.w[2][lj][li] = (pt[r] & kPatPFix) ? T(0) : p[r];
+  }
+}
+
+// Rows of A'(vbar) at the staged node (li, lj) with pattern pt, coefficients c
+// and class cls = (i & 1) + 2 (j & 1); constrained rows are the caller's.
+template <typename T>
+__device__ __forceinline__ void node_rows_assembled(const NodeLevel<T>& L, const OpTable<T>& tab,
+                                                    const WarpTile<T>& S, const T c[36], int li,
+                                                    int lj, int pt, int cls, T& ru, T& rv, T& rp) {
+  const T(*gd)[4] = tab.gd[pt & 15];
+  T u0 = 0, v0 = 0, u1 = 0, v1 = 0, d0 = 0, d1 = 0;
+#pragma unroll
+  for (int e = 0; e < 9; ++e) {
+    const T u = S.w[0][lj - 1 + e / 3][li - 1 + e % 3];
+    const T v = S.w[1][lj - 1 + e / 3][li - 1 + e % 3];
+    const T p = S.w[2][lj - 1 + e / 3][li - 1 + e % 3];
+    u0 += c[4 * e] * u + c[4 * e + 1] * v;
+    v0 += c[4 * e + 2] * u + c[4 * e + 3] * v;
+    u1 += gd[e][0] * p;
+    v1 += gd[e][1] * p;
+    d0 += gd[e][2] * u;
+    d1 += gd[e][3] * v;
+  }
+  const T* ls = tab.lps[(pt >> kPatPatch) & 15][cls];
+  T s[5];
+#pragma unroll
+  for (int dj = 0; dj < 5; ++dj) {
+    s[dj] = T(0);
+#pragma unroll
+    for (int di = 0; di < 5; ++di) s[dj] += ls[5 * dj + di] * S.w[2][lj - 2 + dj][li - 2 + di];
+  }
+  ru = u0 + L.h * u1;
+  rv = v0 + L.h * v1;
+  rp = L.h * (d0 + d1) + L.h2 * (((s[0] + s[1]) + (s[3] + s[4])) + s[2]);
+}
+
+// One colour pass (see vanka_body.cuh) on the warp's 4 x 2 colour cells (bx,
+// by).  Lane 4 q + a owns node a of cell q.
+template <typename T>
+__device__ __forceinline__ void warp_pass_tile(const NodeLevel<T>& L, const OpTable<T>& tab,
+                                               int colour, const T* b, const T* xin, const T* inv,
+                                               int pitch, int nslots, T omega, T* xout, int bx,
+                                               int by, int lane, WarpTile<T>& S) {
+  const int cx = colour & 1, cy = colour >> 1;
+  const int i0 = kWX * bx - cx, j0 = kWY * by - cy;
+  const int q = lane >> 2, a = lane & 3;
+  const int li = 2 * (q & 3) + (a & 1), lj = 2 * (q >> 2) + (a >> 1);
+  const int i = i0 + li, j = j0 + lj;
+  const bool node_ok = i >= 0 && j >= 0 && i <= L.nx && j <= L.ny;
+  const int n = node_ok ? j * L.nnx + i : 0;
+  const int slot = node_ok ? (2 * by + (q >> 2)) * pitch + 4 * bx + (q & 3) : 0;
+  // every load of the tile is issued before the first is used
+  T c[36], iv[36];
+  load36<T>(L.cf, n, L.nn, c);
+  load_inv_rows<T>(inv, nslots, colour, slot, a, iv);
+  const int pt = node_ok ? (int)__ldg(L.pat + n) : 0;
+  const T xu = __ldcg(xin + n), xv = __ldcg(xin + L.nn + n), xp = __ldcg(xin + 2 * L.nn + n);
+  const T bu = __ldcg(b + n), bv = __ldcg(b + L.nn + n), bp = __ldcg(b + 2 * L.nn + n);
+  stage_warp_tile<T>(L, xin, i0, j0, lane, S);
+  __syncwarp();
+  // the cell is fluid: its bit in the node's pattern
+  const bool cell_ok = node_ok && ((pt >> ((1 - (a & 1)) + 2 * (1 - (a >> 1)))) & 1);
+  T ru, rv, rp;
+  node_rows_assembled<T>(L, tab, S, c, li + 2, lj + 2, pt, (i & 1) + 2 * (j & 1), ru, rv, rp);
+  T du = bu - ((pt & kPatVDir) ? xu : ru), dv = bv - ((pt & kPatVDir) ? xv : rv),
+    dp = bp - ((pt & kPatPFix) ? xp : rp);
+  T d[12];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    d[k] = __shfl_sync(0xffffffffu, du, (lane & ~3) + k);
+    d[4 + k] = __shfl_sync(0xffffffffu, dv, (lane & ~3) + k);
+    d[8 + k] = __shfl_sync(0xffffffffu, dp, (lane & ~3) + k);
+  }
+  if (node_ok) {
+    T acc[3];
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      acc[r] = 0;
+#pragma unroll
+      for (int k = 0; k < 12; ++k) acc[r] += iv[r * 12 + k] * d[k];
+    }
+    xout[n] = cell_ok ? xu + omega * acc[0] : xu;
+    xout[L.nn + n] = cell_ok ? xv + omega * acc[1] : xv;
+    xout[2 * L.nn + n] = cell_ok ? xp + omega * acc[2] : xp;
+  }
+  __syncwarp();  // the tile's shared memory is reused
+}
+
+// d = b - A'(vbar) x, zero on constrained unknowns, on the warp's 8 x 4 nodes.
+template <typename T>
+__device__ __forceinline__ void warp_defect_tile(const NodeLevel<T>& L, const OpTable<T>& tab,
+                                                 const T* b, const T* x, T* d, int bx, int by,
+                                                 int lane, WarpTile<T>& S) {
+  const int i0 = kWX * bx, j0 = kWY * by, li = lane % kWX, lj = lane / kWX;
+  const int i = i0 + li, j = j0 + lj;
+  const bool ok = i <= L.nx && j <= L.ny;
+  const int n = ok ? j * L.nnx + i : 0;
+  T c[36];
+  load36<T>(L.cf, n, L.nn, c);
+  const int pt = ok ? (int)__ldg(L.pat + n) : 0;
+  const T bu = __ldcg(b + n), bv = __ldcg(b + L.nn + n), bp = __ldcg(b + 2 * L.nn + n);
+  stage_warp_tile<T>(L, x, i0, j0, lane, S);
+  __syncwarp();
+  T ru, rv, rp;
+  node_rows_assembled<T>(L, tab, S, c, li + 2, lj + 2, pt, (i & 1) + 2 * (j & 1), ru, rv, rp);
+  if (ok) {
+    d[n] = (pt & kPatVDir) ? T(0) : bu - ru;
+    d[L.nn + n] = (pt & kPatVDir) ? T(0) : bv - rv;
+    d[2 * L.nn + n] = (pt & kPatPFix) ? T(0) : bp - rp;
+  }
+  __syncwarp();
+}
+
+}  // namespace dnnmg
