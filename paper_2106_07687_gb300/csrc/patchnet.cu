@@ -2,14 +2,13 @@
 // cells with memory per patch, then dense layers; inputs and outputs per
 // patch as in the network evaluation of Algorithm 1).
 //
-// patchnet_forward_kernel<TRAIN, m, n>: persistent, one 128-patch tile at a
-// time per CTA, 512 threads in four warpgroups.  Patch row r of the tile is
-// TMEM lane r; warp w serves lanes 32 (w % 4) .. +31, and warpgroup w / 4
-// takes one quarter of every accumulator's columns in the epilogues (m / 4
-// hidden units of its row), so that the gate nonlinearities of a tile are
-// spread over 16 warps.  All weights live in shared memory as BF16 K-major
-// operands; per GRU layer the tensor core accumulates in TMEM (4m FP32
-// columns)
+// patchnet_forward_kernel<TRAIN, m, n, G>: persistent, 512 threads in G
+// groups that each take one 128-patch tile at a time.  Patch row r of a tile
+// is TMEM lane r; warp w serves lanes 32 (w % 4) .. +31, and the 4 / G
+// warpgroups of a group split every accumulator's columns in the epilogues
+// (m G / 4 hidden units per thread).  All weights live in shared memory as
+// BF16 K-major operands (one bulk copy per block); per GRU layer the tensor
+// core accumulates in TMEM (4m FP32 columns)
 //   [0,2m)   x W_ih[r,z]^T + h W_hh[r,z]^T      (gates r and z)
 //   [2m,3m)  x W_ih[n]^T                        (input part of gate n)
 //   [3m,4m)  h W_hh[n]^T                        (hidden part of gate n)
@@ -19,7 +18,14 @@
 // back from HBM (the thread's own earlier write), so no layer's state stays
 // in registers between layers.  The dense head reuses TMEM columns [0,128)
 // and [128,128+N2).
+//
+// A tile is a serial chain (loads, MMA, wait, gates, MMA, ...), so with more
+// tiles than SMs two groups run in each block, one computing gates while the
+// other waits for loads or MMAs; with at most one tile per SM a single group
+// gives the tile all 512 threads, which shortens the chain.
+#include "dfloat.cuh"
 #include "kernels.h"
+#include "krylov_body.cuh"
 #include "patchnet.cuh"
 #include "umma.cuh"
 
@@ -33,6 +39,7 @@ constexpr uint32_t kWaitPolls = 1u << 22;  // bound of every mbarrier wait
 constexpr int kTile = 128;
 constexpr int kFwdWG = 4;                      // warpgroups of the forward kernel
 constexpr int kFwdThreads = kTile * kFwdWG;
+constexpr size_t kSmemMax = 227 * 1024;
 
 __device__ __forceinline__ uint16_t f2bf(float v) {
   return __bfloat16_as_ushort(__float2bfloat16_rn(v));
@@ -76,33 +83,52 @@ __global__ void pack_bias_kernel(const float* __restrict__ w, NetDims d, float* 
 }
 
 // -- shared-memory plan of the forward kernel ---------------------------------
-// Operand regions are reused as soon as the MMA that reads them has
-// completed:
+// Weights and biases once per block, and an operand area per group.  Operand
+// regions are reused as soon as the MMA that reads them has completed:
 //   a: x_t (layer 0 input, kx0 columns), then each layer's new state (the
 //      next layer's input, m columns; the top layer's is the head's input);
 //   b: the previous state of the layer being evaluated (m columns), staged
 //      before that layer's MMAs;
 //   m: the dense head's hidden layer (128 columns), over a and b.
+// With two groups and a wide input (split), x_t lies over a and b too and the
+// first layer's previous state is staged after the MMAs of x_t.
 struct FwdSmem {
-  uint32_t w, bias, a, b, m, bar, tmem, total;
+  uint32_t w, bias, area, area_size, b, bar, tmem, total;
+  bool split;
   static __host__ __device__ uint32_t up(uint32_t v) { return (v + 127u) & ~127u; }
-  static __host__ __device__ FwdSmem of(const NetDims& d, size_t w_elems) {
+  static __host__ __device__ FwdSmem of(const NetDims& d, size_t w_elems, int groups) {
     FwdSmem s{};
     uint32_t o = 0;
     s.w = o;    o = up(o + (uint32_t)(w_elems * 2));
     s.bias = o; o = up(o + (uint32_t)((d.layers * 4 * d.hidden + d.mlp + d.nout()) * 4));
     const int ka = d.kx0() > d.hidden ? d.kx0() : d.hidden;
-    const uint32_t asz = kTile * ka * 2, bsz = kTile * d.hidden * 2, msz = kTile * 128 * 2;
-    s.a = o;
-    s.b = o + asz;
-    s.m = s.a;
-    o += asz + bsz > msz ? asz + bsz : msz;
-    s.bar = o;  o += 16;
+    s.split = groups > 1 && ka + d.hidden > 128;
+    s.b = kTile * (s.split ? d.hidden : ka) * 2;
+    const uint32_t absz = s.b + kTile * d.hidden * 2, msz = kTile * 128 * 2;
+    s.area = o;
+    s.area_size = absz > msz ? absz : msz;
+    o += groups * s.area_size;
+    s.bar = o;  o += 32;
     s.tmem = o; o += 16;
     s.total = o;
     return s;
   }
 };
+
+// barrier of one group's threads; group_any: whether p holds in any of them
+__device__ __forceinline__ void group_sync(int id, int n) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+__device__ __forceinline__ bool group_any(int id, int n, bool p) {
+  int r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\t"
+      "bar.red.or.pred q, %2, %3, p;\n\tselp.b32 %0, 1, 0, q;\n\t}\n"
+      : "=r"(r)
+      : "r"((int)p), "r"(id), "r"(n)
+      : "memory");
+  return r != 0;
+}
 
 // write U (8 or 16) consecutive values of row r (columns k0..) as BF16 operand
 template <int U>
@@ -129,17 +155,18 @@ __device__ __forceinline__ void mma_run(uint32_t d_tmem, uint32_t a_addr, int a_
   }
 }
 
+// U consecutive values as U / 4 groups of 16 bytes, `stride` groups apart
 template <int U>
-__device__ __forceinline__ void store_f32(float* dst, const float* v) {
+__device__ __forceinline__ void store_f32(float4* dst, size_t stride, const float* v) {
 #pragma unroll
   for (int q = 0; q < U / 4; ++q)
-    reinterpret_cast<float4*>(dst)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    dst[q * stride] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
 }
 template <int U>
-__device__ __forceinline__ void load_f32(const float* src, float* v) {
+__device__ __forceinline__ void load_f32(const float4* src, size_t stride, float* v) {
 #pragma unroll
   for (int q = 0; q < U / 4; ++q) {
-    const float4 u = reinterpret_cast<const float4*>(src)[q];
+    const float4 u = src[q * stride];
     v[4 * q] = u.x, v[4 * q + 1] = u.y, v[4 * q + 2] = u.z, v[4 * q + 3] = u.w;
   }
 }
@@ -148,36 +175,32 @@ __device__ __forceinline__ void load_f32(const float* src, float* v) {
 // gates from TMEM, new hidden state from hprev into `next` (BF16 operand)
 // and `hout` (FP32, HBM, the U units).  With `gsave` the gates r, z, n and
 // the hidden part of gate n (incl. bias) are stored for the backward pass
-// (row layout [r | z | n | hn], m each); with `hT` the new state is also
-// written transposed in BF16 (column `col`, row stride ldT).
+// ([r | z | n | hn], m each); hout and gsave are groups `stride` apart.  With
+// `hT` the new state is also written transposed in BF16 (rows `ldT` apart).
 template <int H, int U>
 __device__ __forceinline__ void gru_epilogue(uint32_t tm, const float* bias, const float* hprev,
-                                             uint8_t* next, int row, int u0, float* hout,
-                                             bool valid, float* gsave, uint16_t* hT, size_t ldT) {
-  float rp[U], zp[U], ip[U], hp[U];
-  tmem_ld<U>(tm + u0, rp);
-  tmem_ld<U>(tm + H + u0, zp);
-  tmem_ld<U>(tm + 2 * H + u0, ip);
-  tmem_ld<U>(tm + 3 * H + u0, hp);
+                                             uint8_t* next, int row, int u0, float4* hout,
+                                             bool valid, float4* gsave, size_t stride,
+                                             uint16_t* hT, size_t ldT) {
+  float g[4][U];
+  tmem_ld4(tm + u0, H, g);
   float hn[U];
 #pragma unroll
   for (int i = 0; i < U; ++i) {
     const int j = u0 + i;
-    const float r = sigmoidf_(rp[i] + bias[j]);
-    const float z = sigmoidf_(zp[i] + bias[H + j]);
-    const float ghn = hp[i] + bias[3 * H + j];
-    const float n = tanhf(ip[i] + bias[2 * H + j] + r * ghn);
+    const float r = sigmoidf_(g[0][i] + bias[j]);
+    const float z = sigmoidf_(g[1][i] + bias[H + j]);
+    const float ghn = g[3][i] + bias[3 * H + j];
+    const float n = tanhf(g[2][i] + bias[2 * H + j] + r * ghn);
     hn[i] = (1.0f - z) * n + z * hprev[i];
-    rp[i] = r, zp[i] = z, ip[i] = n, hp[i] = ghn;
+    g[0][i] = r, g[1][i] = z, g[2][i] = n, g[3][i] = ghn;
   }
   store_row<U>(next, row, u0, H, hn);
   if (!valid) return;
-  store_f32<U>(hout + u0, hn);
+  store_f32<U>(hout, stride, hn);
   if (gsave) {
-    store_f32<U>(gsave + u0, rp);
-    store_f32<U>(gsave + H + u0, zp);
-    store_f32<U>(gsave + 2 * H + u0, ip);
-    store_f32<U>(gsave + 3 * H + u0, hp);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) store_f32<U>(gsave + (k * H + u0) / 4 * stride, stride, g[k]);
   }
   if (hT)
 #pragma unroll
@@ -185,230 +208,346 @@ __device__ __forceinline__ void gru_epilogue(uint32_t tm, const float* bias, con
 }
 
 // Arguments of the forward kernel.  Inference: T = 1, hidden state read from
-// h_in and written to h_out.  Training: the hidden state starts at zero and
-// the kernel stores, per (t, p), the activations the backward pass needs
-// (act, FP32) and transposed BF16 copies of the GEMM inputs for the weight
-// gradients (column index t * P + p).
+// h_in and written to h_out, prediction to out.  Training: the hidden state
+// starts at zero and the kernel stores, per (t, p), the activations the
+// backward pass needs, the output gradients scale * (y - Y) and transposed
+// BF16 copies of the GEMM inputs for the weight gradients (column index
+// t * P + p), and per block the sum of (y - Y)^2.
 struct FwdArgs {
   const uint16_t* x;  // [P][T][C_in]
   int P, T;
   const float* h_in;  // [layers][P][m]
   float* h_out;       // [layers][P][m]
-  float* out;         // [P][T][C_out]
-  float* act;         // [T][P][act_size]
+  float* out;         // [P][C_out]
+  const float* Y;     // [P][T][C_out]
+  bool y_pairs;       // Y can be read in 8-byte pairs
+  float scale;
+  float4* act;        // [T][act_groups][P]
   uint16_t* xT;       // [kx0 + 16][T * P]
   uint16_t* hT[kMaxLayers];  // [m + 16][(T + 1) * P], state of step t at column (t + 1) * P + p
   uint16_t* y1T;      // [144][T * P]
+  uint16_t* dyT;      // [128][T * P]
+  double* loss_partial;
   int* status;
+  NetPost post;
 };
 
-template <bool TRAIN, int H, int NL>
+template <bool TRAIN, int H, int NL, int G>
 __global__ void __launch_bounds__(kFwdThreads, 1)
     patchnet_forward_kernel(NetDims d, PackLayout L, const uint16_t* __restrict__ wimg,
-                            const float* __restrict__ bias_g, FwdArgs a) {
-  constexpr int U = H / 4;  // hidden units of this thread's row
-  constexpr int KACT = act_size(H, NL);
+                            const float* __restrict__ bias_g, const __grid_constant__ FwdArgs a) {
+  constexpr int GT = kFwdThreads / G;     // threads of a group
+  constexpr int CQ = GT / kTile;          // column parts of an accumulator
+  constexpr int U = H / CQ;               // hidden units of this thread's row
+  constexpr int UC = U < 16 ? U : 16;     // of which one epilogue takes UC
+  constexpr int KG = act_groups(H, NL);
+  constexpr int NX = 4;                   // 16-byte chunks of x_t a thread loads at once
+  constexpr bool AHEAD = TRAIN && G == 1;  // x_t is loaded a step ahead (NX chunks hold it all)
   extern __shared__ __align__(1024) uint8_t sm[];
-  const FwdSmem S = FwdSmem::of(d, L.total);
+  __shared__ double red[kFwdThreads / 32];
+  const FwdSmem S = FwdSmem::of(d, L.total, G);
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int grp = t / GT, tg = t % GT;
   const int row = (warp & 3) * 32 + lane;  // patch row of the tile = TMEM lane
-  const int cq = warp >> 2;                // column quarter of the epilogues
-  uint64_t* bar = reinterpret_cast<uint64_t*>(sm + S.bar);
+  const int cq = tg / kTile;               // column part of the epilogues
+  uint64_t* wbar = reinterpret_cast<uint64_t*>(sm + S.bar);  // the weights' arrival
+  uint64_t* bar = wbar + 1 + grp;                            // this group's MMAs
   uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + S.tmem);
   float* bias = reinterpret_cast<float*>(sm + S.bias);
+  uint8_t* A = sm + S.area + (size_t)grp * S.area_size;      // regions a and m
+  uint8_t* Bh = A + S.b;                                     // region b
   const int P = a.P, T = a.T;
 
-  // weights and biases: one copy per CTA
-  {
-    const uint4* src = reinterpret_cast<const uint4*>(wimg);
-    uint4* dst = reinterpret_cast<uint4*>(sm + S.w);
-    for (size_t i = t; i < L.total / 8; i += kFwdThreads) dst[i] = src[i];
-    const int nb = NL * 4 * H + d.mlp + d.nout();
-    for (int i = t; i < nb; i += kFwdThreads) bias[i] = bias_g[i];
+  if (t == 0) {
+    for (int q = 0; q <= G; ++q) mbar_init(wbar + q, 1);
+    fence_async_smem();
+    const uint32_t bytes = (uint32_t)(L.total * 2);
+    mbar_expect_tx(wbar, bytes);
+    bulk_load(sm + S.w, wimg, bytes, wbar);
   }
-  if (warp == 0) tmem_alloc(tslot, 256);
-  if (t == 0) mbar_init(bar, 1);
-  fence_async_smem();
+  for (int i = t; i < NL * 4 * H + d.mlp + d.nout(); i += kFwdThreads) bias[i] = bias_g[i];
+  if (warp == 0) tmem_alloc(tslot, 256 * G);
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
-  const uint32_t tbase = *tslot;
+  const uint32_t tbase = *tslot + 256 * grp;
   const uint32_t tm = tbase + ((uint32_t)((warp & 3) * 32) << 16);  // this warp's lanes
-  const uint32_t sbase = smem_u32(sm);
+  const uint32_t sw = smem_u32(sm + S.w), sa = smem_u32(A), sbh = smem_u32(Bh);
   const int kx0 = d.kx0();
   const int u0 = U * cq;  // this thread's hidden units
   uint32_t phase = 0;
-  bool failed = false;
+  bool failed = false, weights = false;
+  double loss = 0.0;
   const int ntiles = (P + kTile - 1) / kTile;
   const size_t HP = (size_t)P * H;
   const size_t ld = (size_t)T * P, ldh = (size_t)(T + 1) * P;
 
-  for (int tile = blockIdx.x; tile < ntiles && !failed; tile += gridDim.x) {
+  // publish the group's operand writes, then one thread issues MMAs and the
+  // group waits for them; false when the wait hit its bound
+  auto run_mma = [&](auto issue) {
+    fence_async_smem();
+    fence_before_sync();
+    group_sync(1 + grp, GT);
+    if (tg == 0) {
+      fence_after_sync();
+      issue();
+      mma_commit(bar);
+    }
+    const bool late = !mbar_wait(bar, phase, kWaitPolls);
+    phase ^= 1;
+    failed = group_any(1 + grp, GT, late);
+    fence_after_sync();
+    return !failed;
+  };
+  // 16-byte chunks of x_t: chunk e of the tile is columns 8 q.. of row r.
+  // Inference: a thread's neighbours take the next chunks of the same row
+  // (coalesced loads); training: the same chunk of the next rows, so that the
+  // transposed copy is written coalesced
+  const int nq = kx0 / 8;
+  const bool vec = d.c_in % 8 == 0;  // input rows start on 16-byte boundaries
+  auto x_chunk = [&](int e, int& r, int& q) {
+    r = TRAIN ? e % kTile : e / nq;
+    q = TRAIN ? e / kTile : e % nq;
+  };
+  auto load_x = [&](int tile, int step, int e0, uint4* xr) {
+#pragma unroll
+    for (int c = 0; c < NX; ++c) {
+      const int e = e0 + c * GT;
+      int r, q;
+      x_chunk(e, r, q);
+      const int pr = tile * kTile + r;
+      xr[c] = make_uint4(0, 0, 0, 0);
+      if (e < kTile * nq && pr < P && q * 8 < d.c_in) {
+        const uint16_t* src = a.x + ((size_t)pr * T + step) * d.c_in;
+        if (vec) {
+          xr[c] = reinterpret_cast<const uint4*>(src)[q];
+        } else {  // element by element, zeros past C_in
+          uint32_t w[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int k = q * 8 + 2 * i;
+            w[i] = (k < d.c_in ? src[k] : 0u) | ((k + 1 < d.c_in ? (uint32_t)src[k + 1] : 0u) << 16);
+          }
+          xr[c] = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+      }
+    }
+  };
+  auto store_x = [&](int tile, int step, int e0, const uint4* xr) {
+#pragma unroll
+    for (int c = 0; c < NX; ++c) {
+      const int e = e0 + c * GT;
+      if (e >= kTile * nq) break;
+      int r, q;
+      x_chunk(e, r, q);
+      *reinterpret_cast<uint4*>(A + kmajor_offset(r, q * 8, kx0)) = xr[c];
+      const int pr = tile * kTile + r;
+      if (TRAIN && pr < P) {
+        const uint32_t w[4] = {xr[c].x, xr[c].y, xr[c].z, xr[c].w};
+        uint16_t* o = a.xT + (size_t)(q * 8) * ld + (size_t)step * P + pr;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          if (q * 8 + i < d.c_in) o[i * ld] = (uint16_t)(w[i >> 1] >> (16 * (i & 1)));
+      }
+    }
+  };
+
+  for (int tile = blockIdx.x + grp * gridDim.x; tile < ntiles && !failed;
+       tile += gridDim.x * G) {
     const int p = tile * kTile + row;
     const bool valid = p < P;
+    uint4 xr[NX];
+    if (AHEAD) load_x(tile, 0, tg, xr);
 #pragma unroll 1
     for (int step = 0; step < T && !failed; ++step) {
       const size_t col = (size_t)step * P + p;
-      float* act = TRAIN ? a.act + col * KACT : nullptr;
-      // previous state of layer l (this thread's units): zero at the start
-      // of a training sequence, else the thread's own earlier write
-      auto load_prev = [&](int l, float* hv) {
+      // saved groups of this step, and of the step before
+      float4* act = TRAIN ? a.act + (size_t)step * KG * P + p : nullptr;
+      const float4* actp = TRAIN ? act - (size_t)KG * P : nullptr;
+      // previous state of layer l, units u..u + UC: zero at the start of a
+      // training sequence, else the thread's own earlier write
+      auto load_prev = [&](int l, int u, float* hv) {
 #pragma unroll
-        for (int i = 0; i < U; ++i) hv[i] = 0.0f;
+        for (int i = 0; i < UC; ++i) hv[i] = 0.0f;
         if (!valid) return;
         if (TRAIN) {
-          if (step > 0) load_f32<U>(act - (size_t)P * KACT + act_h(H, l) + u0, hv);
+          if (step > 0) load_f32<UC>(actp + (size_t)(act_h(H, l) + u / 4) * P, P, hv);
         } else {
-          load_f32<U>(a.h_in + l * HP + (size_t)p * H + u0, hv);
+          load_f32<UC>(reinterpret_cast<const float4*>(a.h_in + l * HP + (size_t)p * H + u), 1, hv);
         }
       };
-      // ---- stage x_t (BF16, 16-byte chunks spread over the block) and the
-      // first layer's previous state (BF16 operand, this thread's units)
-      {
-        const int nq = kx0 / 8;
-        const bool vec = d.c_in % 8 == 0;  // input rows start on 16-byte boundaries
-        for (int e = t; e < kTile * nq; e += kFwdThreads) {
-          // inference: a thread's neighbours take the next chunks of the
-          // same row (coalesced loads); training: the same chunk of the next
-          // rows, so that the transposed copy is written coalesced
-          const int r = TRAIN ? e % kTile : e / nq, q = TRAIN ? e / kTile : e % nq;
-          const int pr = tile * kTile + r;
-          uint4 v = make_uint4(0, 0, 0, 0);
-          const bool in = pr < P && q * 8 < d.c_in;
-          const uint16_t* src = a.x + ((size_t)pr * T + step) * d.c_in;
-          if (in && vec) {
-            v = reinterpret_cast<const uint4*>(src)[q];
-          } else if (in) {  // element by element, zeros past C_in
-            uint16_t* ev = reinterpret_cast<uint16_t*>(&v);
-            for (int i = 0; i < 8; ++i) ev[i] = q * 8 + i < d.c_in ? src[q * 8 + i] : 0;
-          }
-          *reinterpret_cast<uint4*>(sm + S.a + kmajor_offset(r, q * 8, kx0)) = v;
-          if (TRAIN && in) {
-            const uint16_t* ev = reinterpret_cast<const uint16_t*>(&v);
-            const size_t cr = (size_t)step * P + pr;
-            for (int i = 0; i < 8 && q * 8 + i < d.c_in; ++i)
-              a.xT[(size_t)(q * 8 + i) * ld + cr] = ev[i];
-          }
+      // with one epilogue per layer the previous state stays in registers
+      // from its staging to the epilogue, else it is read again
+      float hprev[UC];
+      auto stage_prev = [&](int l) {
+#pragma unroll
+        for (int c = 0; c < U / UC; ++c) {
+          load_prev(l, u0 + c * UC, hprev);
+          store_row<UC>(Bh, row, u0 + c * UC, H, hprev);
+        }
+      };
+      if (AHEAD) {
+        store_x(tile, step, tg, xr);
+        if (step + 1 < T) load_x(tile, step + 1, tg, xr);
+      } else {
+        for (int e = tg; e < kTile * nq; e += NX * GT) {
+          load_x(tile, step, e, xr);
+          store_x(tile, step, e, xr);
         }
       }
-      float hprev[U];
-      load_prev(0, hprev);
-      store_row<U>(sm + S.b, row, u0, H, hprev);
+      if (!S.split) stage_prev(0);
+      if (!weights) {  // their copy, once
+        if ((failed = group_any(1 + grp, GT, !mbar_wait(wbar, 0, kWaitPolls)))) break;
+        weights = true;
+      }
       // ---- the GRU layers (unrolled); layer l reads its input from region
       // a and its previous state from region b and writes its new state into
       // region a
 #pragma unroll
       for (int l = 0; l < NL; ++l) {
-        fence_async_smem();
-        fence_before_sync();
-        __syncthreads();
-        const uint32_t ax = sbase + S.a, ah = sbase + S.b;
         const int kx = l == 0 ? kx0 : H;
-        if (t == 0) {
-          fence_after_sync();
-          mma_run(tbase + 0, ax, kx, sbase + S.w + 2 * L.rz[l], kx, 2 * H, kx, false);
-          mma_run(tbase + 0, ah, H, sbase + S.w + 2 * L.hrz[l], H, 2 * H, H, true);
-          mma_run(tbase + 2 * H, ax, kx, sbase + S.w + 2 * L.in[l], kx, H, kx, false);
-          mma_run(tbase + 3 * H, ah, H, sbase + S.w + 2 * L.hn[l], H, H, H, false);
-          mma_commit(bar);
+        auto mma_x = [&] {
+          mma_run(tbase + 0, sa, kx, sw + 2 * L.rz[l], kx, 2 * H, kx, false);
+        };
+        auto mma_n = [&] {
+          mma_run(tbase + 2 * H, sa, kx, sw + 2 * L.in[l], kx, H, kx, false);
+        };
+        auto mma_h = [&] {
+          mma_run(tbase + 0, sbh, H, sw + 2 * L.hrz[l], H, 2 * H, H, true);
+        };
+        auto mma_hn = [&] {
+          mma_run(tbase + 3 * H, sbh, H, sw + 2 * L.hn[l], H, H, H, false);
+        };
+        if (l == 0 && S.split) {
+          if (!run_mma([&] { mma_x(), mma_n(); })) break;
+          stage_prev(0);
+          if (!run_mma([&] { mma_h(), mma_hn(); })) break;
+        } else {
+          if (!run_mma([&] { mma_x(), mma_h(), mma_n(), mma_hn(); })) break;
         }
-        if (!mbar_wait(bar, phase, kWaitPolls)) failed = true;
-        phase ^= 1;
-        if (__syncthreads_or(failed)) {
-          failed = true;
-          break;
+#pragma unroll
+        for (int c = 0; c < U / UC; ++c) {
+          const int u = u0 + c * UC;
+          if (U > UC) load_prev(l, u, hprev);
+          float4* hout = TRAIN ? act + (size_t)(act_h(H, l) + u / 4) * P
+                               : reinterpret_cast<float4*>(a.h_out + l * HP + (size_t)p * H + u);
+          gru_epilogue<H, UC>(tm, bias + l * 4 * H, hprev, A, row, u, hout, valid,
+                              TRAIN ? act + (size_t)act_g(H, NL, l) * P : nullptr, TRAIN ? P : 1,
+                              TRAIN ? a.hT[l] + ldh - ld + col : nullptr, ldh);
         }
-        fence_after_sync();
-        float* hout = TRAIN ? act + act_h(H, l) : a.h_out + l * HP + (size_t)p * H;
-        uint16_t* hT = TRAIN ? a.hT[l] + ldh - ld + col : nullptr;
-        gru_epilogue<H, U>(tm, bias + l * 4 * H, hprev, sm + S.a, row, u0, hout, valid,
-                           TRAIN ? act + act_g(H, NL, l) : nullptr, hT, ldh);
-        if (l + 1 < NL) {  // region b is free: stage the next layer's previous state
-          load_prev(l + 1, hprev);
-          store_row<U>(sm + S.b, row, u0, H, hprev);
-        }
+        if (l + 1 < NL) stage_prev(l + 1);  // region b is free
       }
       if (failed) break;
       // ---- dense head: relu(h W1^T + b1) W2^T + b2 on the top layer's state,
       // or h W2^T + b2 without the hidden dense layer
       const float* b1 = bias + NL * 4 * H;
       if (d.mlp) {
-      fence_async_smem();
-      fence_before_sync();
-      __syncthreads();
-      if (t == 0) {
-        fence_after_sync();
-        mma_run(tbase + 0, sbase + S.a, H, sbase + S.w + 2 * L.w1, H, 128, H, false);
-        mma_commit(bar);
-      }
-      if (!mbar_wait(bar, phase, kWaitPolls)) failed = true;
-      phase ^= 1;
-      if (__syncthreads_or(failed)) {
-        failed = true;
-        break;
-      }
-      fence_after_sync();
+        if (!run_mma([&] { mma_run(tbase, sa, H, sw + 2 * L.w1, H, 128, H, false); })) break;
 #pragma unroll 1
-      for (int c = 2 * cq; c < 2 * cq + 2; ++c) {  // 32 of the 128 units
-        float v[16];
-        tmem_ld16(tm + c * 16, v);
-        if (TRAIN && valid) {
-          float pre[16];
+        for (int c2 = cq * (4 / CQ); c2 < (cq + 1) * (4 / CQ); ++c2) {  // 32 of the 128 units
+          uint32_t signs = 0;
 #pragma unroll
-          for (int i = 0; i < 16; ++i) pre[i] = v[i] + b1[c * 16 + i];
-          store_f32<16>(act + act_a1(H, NL) + c * 16, pre);
-        }
+          for (int c = 2 * c2; c < 2 * c2 + 2; ++c) {
+            float v[16];
+            tmem_ld16(tm + c * 16, v);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = fmaxf(v[i] + b1[c * 16 + i], 0.0f);
-        store_row<16>(sm + S.m, row, c * 16, 128, v);
-        if (TRAIN && valid)
+            for (int i = 0; i < 16; ++i) {
+              v[i] += b1[c * 16 + i];
+              signs |= (v[i] > 0.0f ? 1u : 0u) << ((c & 1) * 16 + i);
+              v[i] = fmaxf(v[i], 0.0f);
+            }
+            store_row<16>(A, row, c * 16, 128, v);
+            if (TRAIN && valid)
 #pragma unroll
-          for (int i = 0; i < 16; ++i) a.y1T[(size_t)(c * 16 + i) * ld + col] = f2bf(v[i]);
-      }
-      }
-      fence_async_smem();
-      fence_before_sync();
-      __syncthreads();
-      const int n2 = d.nout();
-      if (t == 0) {
-        fence_after_sync();
-        if (d.mlp)
-          mma_run(tbase + 128, sbase + S.m, 128, sbase + S.w + 2 * L.w2, 128, n2, 128, false);
-        else  // the single dense layer reads the top state in region a
-          mma_run(tbase + 128, sbase + S.a, H, sbase + S.w + 2 * L.w2, H, n2, H, false);
-        mma_commit(bar);
-      }
-      if (!mbar_wait(bar, phase, kWaitPolls)) failed = true;
-      phase ^= 1;
-      if (__syncthreads_or(failed)) {
-        failed = true;
-        break;
-      }
-      fence_after_sync();
-      const float* b2 = b1 + d.mlp;
-      if (cq < n2 / 16) {  // one 16-column chunk of the output per warpgroup
-        float v[16];
-        tmem_ld16(tm + 128 + cq * 16, v);
-        if (valid)
-          for (int i = 0; i < 16; ++i) {
-            const int j = cq * 16 + i;
-            if (j < d.c_out) a.out[((size_t)p * T + step) * d.c_out + j] = v[i] + b2[j];
+              for (int i = 0; i < 16; ++i) a.y1T[(size_t)(c * 16 + i) * ld + col] = f2bf(v[i]);
           }
+          if (TRAIN && valid)
+            reinterpret_cast<uint32_t*>(act + (size_t)act_sign(H, NL) * P)[c2] = signs;
+        }
+      }
+      const int n2 = d.nout();
+      if (!run_mma([&] {
+            if (d.mlp)
+              mma_run(tbase + 128, sa, 128, sw + 2 * L.w2, 128, n2, 128, false);
+            else  // the single dense layer reads the top state in region a
+              mma_run(tbase + 128, sa, H, sw + 2 * L.w2, H, n2, H, false);
+          }))
+        break;
+      const float* b2 = b1 + d.mlp;
+      for (int c = cq; c < n2 / 16; c += CQ) {  // 16-column chunks of the output
+        float v[16];
+        tmem_ld16(tm + 128 + c * 16, v);
+        if (!valid) continue;
+        if (!TRAIN) {
+          for (int i = 0; i < 16; ++i) {
+            const int j = c * 16 + i;
+            if (j < d.c_out) a.out[(size_t)p * d.c_out + j] = v[i] + b2[j];
+          }
+        } else {
+          // the step's squares in double-float, its sum added in FP64 (one
+          // conversion per chunk: FP64 runs at 1/64 of FP32 here)
+          const float* Y = a.Y + ((size_t)p * T + step) * d.c_out + c * 16;
+          float yv[16];
+#pragma unroll
+          for (int i = 0; i < 16; i += 2) {
+            const int left = d.c_out - (c * 16 + i);
+            if (a.y_pairs && left >= 2) {
+              const float2 q = *reinterpret_cast<const float2*>(Y + i);
+              yv[i] = q.x, yv[i + 1] = q.y;
+            } else {
+              yv[i] = left > 0 ? Y[i] : 0.0f;
+              yv[i + 1] = left > 1 ? Y[i + 1] : 0.0f;
+            }
+          }
+          dfloat sq;
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            const int j = c * 16 + i;
+            if (j < d.c_out) {
+              const float e = v[i] + b2[j] - yv[i];
+              sq += dfloat(e, 0.0f) * dfloat(e, 0.0f);
+              a.dyT[(size_t)j * ld + col] = f2bf(a.scale * e);
+            }
+          }
+          loss += (double)sq;
+        }
       }
       fence_before_sync();
-      __syncthreads();
+      group_sync(1 + grp, GT);
+      fence_after_sync();
     }
   }
+  if (TRAIN) {  // per-block sum of squares (fixed order)
+    for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+    if (lane == 0) red[warp] = loss;
+  }
   if (failed) {
-    if (t == 0) atomicOr(a.status, 4);
-    // let MMAs still in flight finish before the accumulator is released
+    if (tg == 0) atomicOr(a.status, 4);
+    // let copies and MMAs still in flight finish before their memory is released
+    mbar_wait(wbar, 0, kWaitPolls);
     mbar_wait(bar, phase, kWaitPolls);
   }
   fence_before_sync();
   __syncthreads();
   if (warp == 0) {
     fence_after_sync();
-    tmem_dealloc(tbase, 256);
+    tmem_dealloc(*tslot, 256 * G);
+  }
+  if (t != 0) return;
+  if (TRAIN) {
+    double s = 0.0;
+    for (int w = 0; w < kFwdThreads / 32; ++w) s += red[w];
+    a.loss_partial[blockIdx.x] = s;
+  } else if (a.post.mail) {
+    // every block's results are written before it counts itself, and the
+    // last one posts
+    __threadfence();
+    if (atomicAdd(a.post.counter, 1u) == gridDim.x - 1) {
+      __threadfence();
+      *a.post.counter = 0u;
+      a.post.mail->iv[0] = *reinterpret_cast<volatile int*>(a.status);
+      mail_post(a.post.mail, a.post.seq);
+    }
   }
 }
 
@@ -476,40 +615,50 @@ __global__ void __launch_bounds__(kTile, 1)
   }
 }
 
-template <bool TRAIN, int H, int NL>
-void launch_forward_shape(const NetDims& d, const PackedNet& pk, const FwdArgs& a,
+template <bool TRAIN, int H, int NL, int G>
+int launch_forward_groups(const NetDims& d, const PackedNet& pk, const FwdArgs& a, int blocks,
                           cudaStream_t st) {
   const PackLayout L = PackLayout::of(d);
-  const FwdSmem S = FwdSmem::of(d, L.total);
-  cudaFuncSetAttribute(patchnet_forward_kernel<TRAIN, H, NL>,
+  const FwdSmem S = FwdSmem::of(d, L.total, G);
+  cudaFuncSetAttribute(patchnet_forward_kernel<TRAIN, H, NL, G>,
                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S.total);
+  note_launch();
+  patchnet_forward_kernel<TRAIN, H, NL, G>
+      <<<blocks, kFwdThreads, S.total, st>>>(d, L, pk.w, pk.bias, a);
+  return blocks;
+}
+
+// Two groups per block when there are more tiles than SMs and the second
+// operand area fits beside the weights (not for 64 x 3), else one.
+template <bool TRAIN, int H, int NL>
+int launch_forward_shape(const NetDims& d, const PackedNet& pk, const FwdArgs& a, cudaStream_t st) {
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int ntiles = (a.P + kTile - 1) / kTile;
-  note_launch();
-  patchnet_forward_kernel<TRAIN, H, NL><<<ntiles < sms ? ntiles : sms, kFwdThreads, S.total, st>>>(
-      d, L, pk.w, pk.bias, a);
+  if (ntiles > sms && FwdSmem::of(d, PackLayout::of(d).total, 2).total + 256 <= kSmemMax)
+    return launch_forward_groups<TRAIN, H, NL, 2>(d, pk, a, sms, st);
+  return launch_forward_groups<TRAIN, H, NL, 1>(d, pk, a, ntiles < sms ? ntiles : sms, st);
 }
 
-// one instantiation per network size of Table 1
+// one instantiation per network size of Table 1; returns the blocks launched
 template <bool TRAIN>
-void launch_forward_impl(const NetDims& d, const PackedNet& pk, const FwdArgs& a, cudaStream_t st) {
+int launch_forward_impl(const NetDims& d, const PackedNet& pk, const FwdArgs& a, cudaStream_t st) {
   switch (d.hidden * 10 + d.layers) {
-    case 321: launch_forward_shape<TRAIN, 32, 1>(d, pk, a, st); break;
-    case 322: launch_forward_shape<TRAIN, 32, 2>(d, pk, a, st); break;
-    case 323: launch_forward_shape<TRAIN, 32, 3>(d, pk, a, st); break;
-    case 641: launch_forward_shape<TRAIN, 64, 1>(d, pk, a, st); break;
-    case 642: launch_forward_shape<TRAIN, 64, 2>(d, pk, a, st); break;
-    case 643: launch_forward_shape<TRAIN, 64, 3>(d, pk, a, st); break;
-    default: break;  // rejected by net_supported
+    case 321: return launch_forward_shape<TRAIN, 32, 1>(d, pk, a, st);
+    case 322: return launch_forward_shape<TRAIN, 32, 2>(d, pk, a, st);
+    case 323: return launch_forward_shape<TRAIN, 32, 3>(d, pk, a, st);
+    case 641: return launch_forward_shape<TRAIN, 64, 1>(d, pk, a, st);
+    case 642: return launch_forward_shape<TRAIN, 64, 2>(d, pk, a, st);
+    case 643: return launch_forward_shape<TRAIN, 64, 3>(d, pk, a, st);
+    default: return 0;  // rejected by net_supported
   }
 }
 
 }  // namespace
 
 size_t patchnet_forward_smem(const NetDims& d) {
-  return FwdSmem::of(d, PackLayout::of(d).total).total;
+  return FwdSmem::of(d, PackLayout::of(d).total, 1).total + 256;  // and the static part
 }
 
 bool net_supported(const NetDims& d) {
@@ -519,7 +668,6 @@ bool net_supported(const NetDims& d) {
       (d.mlp != 128 && d.mlp != 0) || d.c_in < 1 || d.c_in > 127 || d.c_out < 1 ||
       d.c_out > 64 || d.nout() > 16 * kFwdWG || (d.bias != 0 && d.bias != 1))
     return false;
-  constexpr size_t kSmemMax = 227 * 1024;
   return patchnet_forward_smem(d) <= kSmemMax && patchnet_backward_smem(d) <= kSmemMax;
 }
 
@@ -554,7 +702,7 @@ void launch_pack_weights(const NetDims& d, const float* w, PackedNet& pk, cudaSt
 
 void launch_patchnet_forward(const NetDims& d, const PackedNet& pk, const uint16_t* x,
                              const float* h, float* h_out, float* out, int P, int* status,
-                             cudaStream_t st) {
+                             cudaStream_t st, const NetPost& post) {
   if (P <= 0) return;
   FwdArgs a{};
   a.x = x;
@@ -564,24 +712,29 @@ void launch_patchnet_forward(const NetDims& d, const PackedNet& pk, const uint16
   a.h_out = h_out;
   a.out = out;
   a.status = status;
+  a.post = post;
   launch_forward_impl<false>(d, pk, a, st);
 }
 
-void launch_patchnet_train_forward(const NetDims& d, const PackedNet& pk, const uint16_t* x, int B,
-                                   int T, float* ypred, const TrainBufs& tb, int* status,
-                                   cudaStream_t st) {
-  if (B <= 0 || T <= 0) return;
+int launch_patchnet_train_forward(const NetDims& d, const PackedNet& pk, const uint16_t* x,
+                                  const float* Y, int B, int T, float scale, const TrainBufs& tb,
+                                  int* status, cudaStream_t st) {
+  if (B <= 0 || T <= 0) return 0;
   FwdArgs a{};
   a.x = x;
   a.P = B;
   a.T = T;
-  a.out = ypred;
+  a.Y = Y;
+  a.y_pairs = d.c_out % 2 == 0 && (reinterpret_cast<uintptr_t>(Y) & 7) == 0;
+  a.scale = scale;
   a.act = tb.act;
   a.xT = tb.xT;
   for (int l = 0; l < kMaxLayers; ++l) a.hT[l] = tb.hT[l];
   a.y1T = tb.y1T;
+  a.dyT = tb.dyT;
+  a.loss_partial = tb.loss_partial;
   a.status = status;
-  launch_forward_impl<true>(d, pk, a, st);
+  return launch_forward_impl<true>(d, pk, a, st);
 }
 
 int launch_umma_gemm(const uint16_t* A, const uint16_t* B, float* C, int M, int N, int K,

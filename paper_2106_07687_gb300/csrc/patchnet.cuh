@@ -18,6 +18,8 @@
 
 #include <cuda_runtime.h>
 
+#include "common.cuh"
+
 namespace dnnmg {
 
 constexpr int kMaxLayers = 3;
@@ -92,14 +94,17 @@ struct PackLayout {
   }
 };
 
-// Per (step, patch) activations saved by the training forward pass (FP32):
-// the new hidden state of every layer, the gates (r, z, n and the hidden
-// part of n incl. bias, m each) of every layer and the pre-activation of the
-// hidden dense layer.
-__host__ __device__ constexpr int act_h(int H, int l) { return l * H; }
-__host__ __device__ constexpr int act_g(int H, int NL, int l) { return NL * H + 4 * H * l; }
-__host__ __device__ constexpr int act_a1(int H, int NL) { return 5 * NL * H; }
-__host__ __device__ constexpr int act_size(int H, int NL) { return 5 * NL * H + 128; }
+// Per (step, sequence) activations saved by the training forward pass, in
+// 16-byte groups: the new hidden state of every layer and the gates (r, z, n
+// and the hidden part of n incl. bias, m each) of every layer in FP32, and the
+// 128 signs of the hidden dense layer's pre-activation (bit = positive).
+// Group q of sequence b at step t is at ((t * act_groups + q) * B + b): a
+// warp, which holds 32 consecutive sequences, writes and reads every group as
+// 512 consecutive bytes.
+__host__ __device__ constexpr int act_h(int H, int l) { return l * H / 4; }
+__host__ __device__ constexpr int act_g(int H, int NL, int l) { return (NL * H + 4 * H * l) / 4; }
+__host__ __device__ constexpr int act_sign(int H, int NL) { return 5 * NL * H / 4; }
+__host__ __device__ constexpr int act_groups(int H, int NL) { return 5 * NL * H / 4 + 1; }
 
 // Buffers of one training step for B sequences of T steps.  Columns of the
 // transposed BF16 streams are indexed t * B + b; every hT[l] holds a leading
@@ -107,10 +112,19 @@ __host__ __device__ constexpr int act_size(int H, int NL) { return 5 * NL * H + 
 // t * B + b is at the same column of the unshifted view.  Row C_in of xT,
 // row m of every hT[l] and row 128 of y1T hold ones (bias gradients).
 struct TrainBufs {
-  float* act = nullptr;                   // [T][B][act_size]
+  float4* act = nullptr;                  // [T][act_groups][B]
   uint16_t* xT = nullptr;                 // [kx0 + 16][T B]
   uint16_t* hT[kMaxLayers] = {};          // [m + 16][(T+1) B]
   uint16_t* y1T = nullptr;                // [144][T B]
+  uint16_t* dyT = nullptr;                // [128][T B] output gradients, rows >= C_out stay zero
+  double* loss_partial = nullptr;         // one per block of the forward kernel
+};
+// Where an inference launch posts its status word (iv[0]) when its last block
+// is done: mailbox, post number and a counter that is zero between launches.
+struct NetPost {
+  HostMail* mail = nullptr;
+  unsigned long long seq = 0;
+  unsigned* counter = nullptr;
 };
 
 // Shared-memory bytes of the forward and backward kernels (0 if the shape
@@ -124,11 +138,13 @@ void launch_pack_weights(const NetDims& d, const float* w, PackedNet& pk, cudaSt
 // in, h_out [layers][P][m] (may alias h), out [P][C_out] FP32
 void launch_patchnet_forward(const NetDims& d, const PackedNet& pk, const uint16_t* x,
                              const float* h, float* h_out, float* out, int P, int* status,
-                             cudaStream_t st);
-// training forward over T steps from a zero hidden state, saving activations
-void launch_patchnet_train_forward(const NetDims& d, const PackedNet& pk, const uint16_t* x, int B,
-                                   int T, float* ypred, const TrainBufs& tb, int* status,
-                                   cudaStream_t st);
+                             cudaStream_t st, const NetPost& post = NetPost{});
+// training forward over T steps from a zero hidden state: saves the
+// activations, the output gradients scale * (y - Y) and the loss's partial
+// sums, one per block; returns the number of blocks
+int launch_patchnet_train_forward(const NetDims& d, const PackedNet& pk, const uint16_t* x,
+                                  const float* Y, int B, int T, float scale, const TrainBufs& tb,
+                                  int* status, cudaStream_t st);
 // C[M x N] = A[M x K] * B[N x K]^T (BF16 row-major inputs, FP32 row-major out)
 int launch_umma_gemm(const uint16_t* A, const uint16_t* B, float* C, int M, int N, int K,
                      int* status, cudaStream_t st);

@@ -778,18 +778,17 @@ int dnnmg_ctx::init_train() {
   tr_blocks_max = sms;
   tr_splits_max = 160;
   const int H = nd.hidden, NL = nd.layers, MG = gate_rows(nd);
-  tb.act = mem.alloc<float>(K * act_size(H, NL));
+  tb.act = mem.alloc<float4>(K * act_groups(H, NL));
   tb.xT = mem.alloc<uint16_t>((size_t)(nd.kx0() + 16) * K);
   for (int l = 0; l < NL; ++l) tb.hT[l] = mem.alloc<uint16_t>((size_t)(H + 16) * Kh);
   tb.y1T = mem.alloc<uint16_t>(144 * K);
-  tr_ypred = mem.alloc<float>(K * nd.c_out);
-  dyT = mem.alloc<uint16_t>(128 * K);
+  tb.dyT = mem.alloc<uint16_t>(128 * K);
   da1T = mem.alloc<uint16_t>(128 * K);
   for (int l = 0; l < NL; ++l) {
     giT[l] = mem.alloc<uint16_t>((size_t)MG * K);
     ghT[l] = mem.alloc<uint16_t>((size_t)MG * K);
   }
-  loss_part = mem.alloc<double>(tr_blocks_max);
+  tb.loss_partial = mem.alloc<double>(tr_blocks_max);
   loss_dev = mem.alloc<float>(4);
   grad = mem.alloc<float>(nd.num_params());
   adam_m = mem.alloc<float>(nd.num_params());
@@ -831,7 +830,7 @@ int dnnmg_ctx::train_grad_impl(const uint16_t* Xd, const float* Yd, int B, int T
       fill_rows_one(tb.hT[l], Kh, H, H + 1, st);
     }
     cudaMemsetAsync(tb.y1T, 0, 2 * 144 * K, st);
-    cudaMemsetAsync(dyT, 0, 2 * 128 * K, st);
+    cudaMemsetAsync(tb.dyT, 0, 2 * 128 * K, st);
     fill_rows_one(tb.xT, K, nd.c_in, nd.c_in + 1, st);
     fill_rows_one(tb.y1T, K, 128, 129, st);
     tr_layout_B = B;
@@ -839,25 +838,21 @@ int dnnmg_ctx::train_grad_impl(const uint16_t* Xd, const float* Yd, int B, int T
   }
   const int p = prof.begin(DNNMG_STAGE_TRAIN, 0, st);
   launch_pack_backward(nd, w_master, wT, st);
-  launch_patchnet_train_forward(nd, pk, Xd, B, T, tr_ypred, tb, net_status, st);
+  const float scale = (float)(2.0 / ((double)B * T * nd.c_out));
+  const int nf = launch_patchnet_train_forward(nd, pk, Xd, Yd, B, T, scale, tb, net_status, st);
+  launch_loss(tb.loss_partial, nf, 1.0 / ((double)B * T * nd.c_out), loss_dev, st);
   BwdArgs a{};
   a.act = tb.act;
-  a.ypred = tr_ypred;
-  a.Y = Yd;
+  a.dyT = tb.dyT;
   a.B = B;
   a.T = T;
-  a.scale = (float)(2.0 / ((double)B * T * nd.c_out));
-  a.dyT = dyT;
   a.da1T = da1T;
   for (int l = 0; l < NL; ++l) {
     a.giT[l] = giT[l];
     a.ghT[l] = ghT[l];
   }
-  a.loss_partial = loss_part;
   a.status = net_status;
-  const int nb = std::min((B + 127) / 128, tr_blocks_max);
-  launch_patchnet_backward(nd, wT, a, nb, st);
-  launch_loss(loss_part, nb, 1.0 / ((double)B * T * nd.c_out), loss_dev, st);
+  launch_patchnet_backward(nd, wT, a, std::min((B + 127) / 128, tr_blocks_max), st);
   // weight gradients: dW = sum over columns of dG^T x (split-K), bias = ones
   // row; per layer W_ih against the layer's input (x, or the state of the
   // layer below at the same step: the shifted view of its stream) and W_hh
@@ -879,10 +874,10 @@ int dnnmg_ctx::train_grad_impl(const uint16_t* Xd, const float* Yd, int B, int T
   if (nd.mlp) {
     jobs[njobs++] = {da1T, tb.hT[NL - 1] + B, K, Kh, 128, H + 16, nd.mlp, H, H, grad + o.w1,
                      gb(o.b1)};
-    jobs[njobs++] = {dyT, tb.y1T, K, K, 128, 144, nd.c_out, nd.mlp, nd.mlp, grad + o.w2,
+    jobs[njobs++] = {tb.dyT, tb.y1T, K, K, 128, 144, nd.c_out, nd.mlp, nd.mlp, grad + o.w2,
                      gb(o.b2)};
   } else {  // a single dense layer: W2 against the top layer's new state
-    jobs[njobs++] = {dyT, tb.hT[NL - 1] + B, K, Kh, 128, H + 16, nd.c_out, H, H, grad + o.w2,
+    jobs[njobs++] = {tb.dyT, tb.hT[NL - 1] + B, K, Kh, 128, H + 16, nd.c_out, H, H, grad + o.w2,
                      gb(o.b2)};
   }
   // one wave: a block per SM at most (a block's 4-stage ring fills most of
@@ -1234,9 +1229,11 @@ int dnnmg_ctx::init_net() {
   pk.bias_elems = (size_t)nd.layers * 4 * nd.hidden + nd.mlp + nd.nout();
   pk.bias = mem.alloc<float>(pk.bias_elems);
   net_status = mem.alloc<int>(4);
+  net_counter = mem.alloc<unsigned>(1);
   if (!mem.ok()) return fail(DNNMG_ERR_CUDA, "device allocation failed");
   cudaMemsetAsync(w_master, 0, sizeof(float) * nd.num_params(), st);
   cudaMemsetAsync(net_status, 0, sizeof(int) * 4, st);
+  cudaMemsetAsync(net_counter, 0, sizeof(unsigned), st);
   launch_pack_weights(nd, w_master, pk, st);
   return check("network setup");
 }
@@ -1261,6 +1258,10 @@ int dnnmg_ctx::net_check(const char* what) {
   if (int rc = check(what)) return rc;
   const unsigned long long t = mail_ticket();
   launch_post(mail_d, t, nullptr, 0, 0, net_status, 0, 1, st);
+  return net_wait(t, what);
+}
+
+int dnnmg_ctx::net_wait(unsigned long long t, const char* what) {
   if (int rc = mail_wait(t, what)) return rc;
   const int s = mail_h->iv[0];
   if (s & 4) {
@@ -1290,9 +1291,11 @@ int dnnmg_ctx::patch_infer(const uint16_t* x, float* h, float* out, int P) {
   if (P < 0) return fail(DNNMG_ERR_ARG, "negative patch count");
   if (P == 0) return DNNMG_OK;
   const int p = prof.begin(DNNMG_STAGE_NETWORK, 0, st);
-  launch_patchnet_forward(nd, pk, x, h, h, out, P, net_status, st);
+  // the kernel's last block posts the status word itself
+  NetPost post{mail_d, mail_ticket(), net_counter};
+  launch_patchnet_forward(nd, pk, x, h, h, out, P, net_status, st, post);
   prof.end(p, st);
-  return net_check("patch_infer");
+  return net_wait(post.seq, "patch_infer");
 }
 
 void dnnmg_ctx::old_rhs(int level, const double* x_old, double* f, double* copy) {

@@ -195,6 +195,7 @@ struct dnnmg_ctx {
   float* w_master = nullptr;   // FP32 flat parameters
   dnnmg::PackedNet pk{};
   int* net_status = nullptr;
+  unsigned* net_counter = nullptr;  // finished blocks of an inference launch (0 between launches)
   // DNN-MG correction state (level L+1 fields)
   int P = 0;                       // patches = fluid cells of level L
   int* patch_cell = nullptr;       // [P] cell id of each patch
@@ -210,12 +211,11 @@ struct dnnmg_ctx {
   double* stat_partial = nullptr;  // [128][C_in][2] feature-statistics partials
   // training workspace (capacity cfg.train_batch x cfg.train_seq)
   dnnmg::TrainBufs tb{};
-  float *tr_ypred = nullptr, *loss_dev = nullptr, *grad = nullptr, *adam_m = nullptr,
+  float *loss_dev = nullptr, *grad = nullptr, *adam_m = nullptr,
         *adam_v = nullptr, *cpart = nullptr;
-  uint16_t *dyT = nullptr, *da1T = nullptr, *wT = nullptr;
+  uint16_t *da1T = nullptr, *wT = nullptr;
   uint16_t* giT[dnnmg::kMaxLayers] = {};  // gate gradients of each layer (input side)
   uint16_t* ghT[dnnmg::kMaxLayers] = {};  // (hidden side)
-  double* loss_part = nullptr;
   int tr_layout_B = -1, tr_layout_T = -1, adam_step = 0, tr_blocks_max = 0, tr_splits_max = 0;
   size_t cpart_floats = 0;
 
@@ -256,6 +256,7 @@ struct dnnmg_ctx {
   int get_weights(float* w_host);
   int patch_infer(const uint16_t* x, float* h, float* out, int P);
   int net_check(const char* what);
+  int net_wait(unsigned long long t, const char* what);  // for the status of post t
   int init_dnnmg();
   // f = old-time right-hand side of Eq. 5 from x_old on level `level`
   void old_rhs(int level, const double* x_old, double* f, double* copy = nullptr);

@@ -43,7 +43,7 @@ __global__ void pack_transpose_kernel(const float* __restrict__ src, int ld, int
 // both products of a layer (dG_h W_hh over [dr | dz] and r * dn, dG_i W_ih
 // over [dr | dz | dn]) read it.
 struct BwdSmem {
-  uint32_t w, r, bar, tmem, red, total;
+  uint32_t w, r, bar, tmem, total;
   static __host__ __device__ uint32_t up(uint32_t v) { return (v + 127u) & ~127u; }
   static __host__ __device__ BwdSmem of(const NetDims& d, size_t w_elems) {
     BwdSmem s{};
@@ -53,7 +53,6 @@ struct BwdSmem {
     s.r = o;    o += kTile * kr * 2;
     s.bar = o;  o += 16;
     s.tmem = o; o += 16;
-    s.red = o;  o += 16 * 8;  // one double per warp
     s.total = o;
     return s;
   }
@@ -72,11 +71,12 @@ __device__ __forceinline__ void store_row(uint8_t* buf, int r, int k0, int K, co
   }
 }
 
+// U consecutive values stored as U / 4 groups of 16 bytes, `stride` groups apart
 template <int U>
-__device__ __forceinline__ void load_f32(const float* src, float* v) {
+__device__ __forceinline__ void load_f32(const float4* src, size_t stride, float* v) {
 #pragma unroll
   for (int q = 0; q < U / 4; ++q) {
-    const float4 u = reinterpret_cast<const float4*>(src)[q];
+    const float4 u = src[q * stride];
     v[4 * q] = u.x, v[4 * q + 1] = u.y, v[4 * q + 2] = u.z, v[4 * q + 3] = u.w;
   }
 }
@@ -97,18 +97,18 @@ __device__ __forceinline__ void mma_run(uint32_t d_tmem, uint32_t a_addr, int a_
 // direct part dh * z of the previous state's gradient.  Rows past the batch
 // (valid false) read nothing and give zeros.
 template <int H, int U>
-__device__ __forceinline__ void gru_backward_chunk(int u0, const float* dh, const float* g,
-                                                   const float* hprev, float* dprev, uint8_t* R,
-                                                   int row, bool valid, uint16_t* giT,
+__device__ __forceinline__ void gru_backward_chunk(int u0, const float* dh, const float4* g,
+                                                   size_t stride, const float* hprev, float* dprev,
+                                                   uint8_t* R, int row, bool valid, uint16_t* giT,
                                                    uint16_t* ghT, size_t ld) {
   float gr[U], gz[U], gn[U], gh[U];
 #pragma unroll
   for (int i = 0; i < U; ++i) gr[i] = gz[i] = gn[i] = gh[i] = 0.0f;
   if (valid) {
-    load_f32<U>(g + u0, gr);
-    load_f32<U>(g + H + u0, gz);
-    load_f32<U>(g + 2 * H + u0, gn);
-    load_f32<U>(g + 3 * H + u0, gh);
+    load_f32<U>(g + (size_t)(u0 / 4) * stride, stride, gr);
+    load_f32<U>(g + (size_t)((H + u0) / 4) * stride, stride, gz);
+    load_f32<U>(g + (size_t)((2 * H + u0) / 4) * stride, stride, gn);
+    load_f32<U>(g + (size_t)((3 * H + u0) / 4) * stride, stride, gh);
   }
   float dar[U], daz[U], dan[U], dhn[U];
 #pragma unroll
@@ -142,6 +142,11 @@ __device__ __forceinline__ void gru_backward_chunk(int u0, const float* dh, cons
   }
 }
 
+// Prefetch contiguous bytes (a multiple of 16, from a 16-byte boundary) into L2.
+__device__ __forceinline__ void bulk_prefetch(const void* p, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
 constexpr int kBwdWG = 4;  // warpgroups: each takes a quarter of every accumulator's columns
 constexpr int kBwdThreads = kTile * kBwdWG;
 
@@ -153,7 +158,7 @@ constexpr int kBwdThreads = kTile * kBwdWG;
 template <int H, int NL>
 __global__ void __launch_bounds__(kBwdThreads, 1)
     patchnet_backward_kernel(NetDims d, BwdPack W, const uint16_t* __restrict__ wT, BwdArgs a) {
-  constexpr int U = H / 4, KACT = act_size(H, NL), KR = 4 * H;
+  constexpr int U = H / 4, KG = act_groups(H, NL), KR = 4 * H;
   extern __shared__ __align__(1024) uint8_t sm[];
   const BwdSmem S = BwdSmem::of(d, W.total);
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
@@ -161,7 +166,6 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
   const int cq = warp >> 2;                // column quarter
   uint64_t* bar = reinterpret_cast<uint64_t*>(sm + S.bar);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + S.tmem);
-  double* red = reinterpret_cast<double*>(sm + S.red);
   {
     const uint4* src = reinterpret_cast<const uint4*>(wT);
     uint4* dst = reinterpret_cast<uint4*>(sm + S.w);
@@ -183,7 +187,6 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
   const int u0 = U * cq;  // this thread's hidden units
   uint32_t phase = 0;
   bool failed = false;
-  double loss = 0.0;
   const int ntiles = (B + kTile - 1) / kTile;
 
   auto sync_mma = [&](auto issue) {
@@ -212,26 +215,29 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
 #pragma unroll 1
     for (int step = T - 1; step >= 0 && !failed; --step) {
       const size_t col = (size_t)step * B + p;
-      const float* act = a.act + col * KACT;
-      const float* actp = step > 0 ? act - (size_t)B * KACT : nullptr;
-      // ---- loss and dY (Eq. 7 as a mean): dY = 2 (y - Y) / (B T C); output
-      // columns 16 cq .. +15 (one 16-column chunk of the nout per warpgroup)
+      const float4* act = a.act + (size_t)step * KG * B + p;  // saved groups of this step
+      const float4* actp = step > 0 ? act - (size_t)KG * B : nullptr;
+      // the next step's groups (2 KB of the tile each) into L2 while this one runs
+      if (actp) {
+        const uint32_t bytes = 16u * min(kTile, B - tile * kTile);
+        for (int q = t; q < KG; q += kBwdThreads)
+          bulk_prefetch(a.act + ((size_t)(step - 1) * KG + q) * B + tile * kTile, bytes);
+      }
+      // ---- dY, output columns 16 cq .. +15 (one 16-column chunk of the nout
+      // per warpgroup), already rounded
       if (cq < NO / 16) {
-        float dy[16];
+        uint32_t w[8];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) dy[i] = 0.0f;
-        if (valid) {
-          const size_t o = ((size_t)p * T + step) * C;
-          for (int i = 0; i < 16; ++i) {
-            const int j = 16 * cq + i;
-            if (j >= C) break;
-            const float e = a.ypred[o + j] - a.Y[o + j];
-            loss += (double)e * e;
-            dy[i] = a.scale * e;
-            a.dyT[(size_t)j * ld + col] = f2bf(dy[i]);
-          }
+        for (int i = 0; i < 8; ++i) {
+          const int j = 16 * cq + 2 * i;
+          const uint32_t lo = valid && j < C ? a.dyT[(size_t)j * ld + col] : 0u;
+          const uint32_t hi = valid && j + 1 < C ? a.dyT[(size_t)(j + 1) * ld + col] : 0u;
+          w[i] = lo | (hi << 16);
         }
-        store_row<16>(R, row, 16 * cq, NO, dy);
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          *reinterpret_cast<uint4*>(R + kmajor_offset(row, 16 * cq + 8 * h, NO)) =
+              make_uint4(w[4 * h], w[4 * h + 1], w[4 * h + 2], w[4 * h + 3]);
       }
       sync_mma([&] { mma_run(tbase + 0, sb + S.r, NO, sw + 2 * W.w2t, NO, d.k2(), NO, false); });
       if (failed) break;
@@ -240,6 +246,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
         tmem_ld<U>(tm + u0, dtop);
       } else {
       // ---- dense head: da1 = (dY W2) * [a1 > 0], 32 of the 128 units
+      const uint32_t signs =
+          valid ? reinterpret_cast<const uint32_t*>(act + (size_t)act_sign(H, NL) * B)[cq] : 0u;
 #pragma unroll
       for (int c = 2 * cq; c < 2 * cq + 2; ++c) {
         float v[16];
@@ -247,7 +255,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
           const int j = c * 16 + i;
-          v[i] = (valid && act[act_a1(H, NL) + j] > 0.0f) ? v[i] : 0.0f;
+          v[i] = (signs >> ((c & 1) * 16 + i)) & 1u ? v[i] : 0.0f;
           if (valid) a.da1T[(size_t)j * ld + col] = f2bf(v[i]);
         }
         store_row<16>(R, row, c * 16, 128, v);
@@ -266,9 +274,9 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
           dh[i] = valid ? dtop[i] + dcar[l][i] : 0.0f;
           hp[i] = 0.0f;
         }
-        if (valid && actp) load_f32<U>(actp + act_h(H, l) + u0, hp);
-        gru_backward_chunk<H, U>(u0, dh, act + act_g(H, NL, l), hp, dp, R, row, valid,
-                                 a.giT[l] + col, a.ghT[l] + col, ld);
+        if (valid && actp) load_f32<U>(actp + (size_t)(act_h(H, l) + u0 / 4) * B, B, hp);
+        gru_backward_chunk<H, U>(u0, dh, act + (size_t)act_g(H, NL, l) * B, B, hp, dp, R, row,
+                                 valid, a.giT[l] + col, a.ghT[l] + col, ld);
         sync_mma([&] {
           const uint32_t r0 = sb + S.r, wh = sw + 2 * W.whh[l];
           mma_run(tbase + 0, r0, KR, wh, 3 * H, H, 2 * H, false);                 // [dr | dz]
@@ -286,15 +294,6 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
       fence_before_sync();
       __syncthreads();
     }
-  }
-  // per-CTA loss partial (fixed-order reduction)
-  for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
-  if (lane == 0) red[warp] = loss;
-  __syncthreads();
-  if (t == 0) {
-    double s = 0.0;
-    for (int w = 0; w < kBwdThreads / 32; ++w) s += red[w];
-    a.loss_partial[blockIdx.x] = s;
   }
   if (failed) {
     if (t == 0) atomicOr(a.status, 4);
@@ -446,11 +445,6 @@ struct WGradMaps {
   CUtensorMap a[kMaxWGradJobs], b[kMaxWGradJobs];
 };
 
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* mbar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(mbar)),
-               "r"(bytes)
-               : "memory");
-}
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y,
                                             uint64_t* mbar) {
   asm volatile(

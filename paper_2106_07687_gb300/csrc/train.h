@@ -37,16 +37,12 @@ struct BwdPack {
 inline int gate_rows(const NetDims& d) { return (3 * d.hidden + 127) / 128 * 128; }
 
 struct BwdArgs {
-  const float* act;      // [T][B][act_size] from the training forward
-  const float* ypred;    // [B][T][C_out]
-  const float* Y;        // [B][T][C_out] targets
+  const float4* act;     // [T][act_groups][B] from the training forward
+  const uint16_t* dyT;   // [128][T B] output gradients from the training forward
   int B, T;
-  float scale;           // 2 / (B T C_out)
-  uint16_t* dyT;         // [128][T B]   rows >= C_out stay zero
   uint16_t* da1T;        // [128][T B]
   uint16_t* giT[kMaxLayers];  // [gate_rows][T B]  dG_i of layer l (r, z, n)
   uint16_t* ghT[kMaxLayers];  // [gate_rows][T B]  dG_h of layer l (r, z, r * dn)
-  double* loss_partial;  // [gridDim]
   int* status;
 };
 

@@ -113,6 +113,24 @@ __device__ __forceinline__ void mbar_init(uint64_t* mbar, uint32_t count) {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 
+// Expect `bytes` of asynchronous copies in the barrier's current phase (and
+// arrive on it).
+__device__ __forceinline__ void mbar_expect_tx(uint64_t* mbar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(mbar)),
+               "r"(bytes)
+               : "memory");
+}
+// Asynchronous copy of `bytes` contiguous bytes (a multiple of 16, both
+// addresses on 16-byte boundaries) from global to shared memory.
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes,
+                                          uint64_t* mbar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+          smem_u32(dst)),
+      "l"(src), "r"(bytes), "r"(smem_u32(mbar))
+      : "memory");
+}
+
 // Wait until phase `parity` of the barrier completed.  Gives up after
 // `max_iter` polls and returns false (the caller records a timeout).
 __device__ __forceinline__ bool mbar_wait(uint64_t* mbar, uint32_t parity, uint32_t max_iter) {
@@ -162,6 +180,54 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float v[8]) {
       : "memory");
 #pragma unroll
   for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// Wait for this thread's tensor-memory loads.  The loaded registers pass
+// through the statement, so that no use of them is scheduled before it.
+template <int N>
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&r)[4][N]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int i = 0; i < N; ++i) asm volatile("" : "+r"(r[k][i]));
+}
+
+// Four such loads at column offsets 0, s, 2 s and 3 s, in flight together.
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t s, float (&v)[4][16]) {
+  uint32_t r[4][16];
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[k][0]), "=r"(r[k][1]), "=r"(r[k][2]), "=r"(r[k][3]), "=r"(r[k][4]),
+          "=r"(r[k][5]), "=r"(r[k][6]), "=r"(r[k][7]), "=r"(r[k][8]), "=r"(r[k][9]),
+          "=r"(r[k][10]), "=r"(r[k][11]), "=r"(r[k][12]), "=r"(r[k][13]), "=r"(r[k][14]),
+          "=r"(r[k][15])
+        : "r"(taddr + k * s)
+        : "memory");
+  tmem_wait_ld(r);
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[k][i] = __uint_as_float(r[k][i]);
+}
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t s, float (&v)[4][8]) {
+  uint32_t r[4][8];
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+        : "=r"(r[k][0]), "=r"(r[k][1]), "=r"(r[k][2]), "=r"(r[k][3]), "=r"(r[k][4]),
+          "=r"(r[k][5]), "=r"(r[k][6]), "=r"(r[k][7])
+        : "r"(taddr + k * s)
+        : "memory");
+  tmem_wait_ld(r);
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[k][i] = __uint_as_float(r[k][i]);
 }
 
 // U = 8 or 16 columns
