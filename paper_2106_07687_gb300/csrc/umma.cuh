@@ -230,6 +230,25 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t s, float (&v)[
     for (int i = 0; i < 8; ++i) v[k][i] = __uint_as_float(r[k][i]);
 }
 
+// Registers -> TMEM, 8 or 16 consecutive columns of this warp's lanes; complete
+// (for this thread's later loads) when it returns.
+__device__ __forceinline__ void tmem_st(uint32_t taddr, const float (&v)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+      "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};\n\t"
+      "tcgen05.wait::st.sync.aligned;" ::"r"(taddr),
+      "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]),
+      "f"(v[8]), "f"(v[9]), "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15])
+      : "memory");
+}
+__device__ __forceinline__ void tmem_st(uint32_t taddr, const float (&v)[8]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n\t"
+      "tcgen05.wait::st.sync.aligned;" ::"r"(taddr),
+      "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+      : "memory");
+}
+
 // U = 8 or 16 columns
 template <int U>
 __device__ __forceinline__ void tmem_ld(uint32_t taddr, float* v) {
