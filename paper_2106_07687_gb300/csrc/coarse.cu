@@ -6,27 +6,291 @@
 #include "coarse_body.cuh"
 #include "kernels.h"
 
+namespace cg = cooperative_groups;
+
 namespace dnnmg {
 
 namespace {
 
-// One thread per row of the coarse Jacobian.
-__global__ void assemble_kernel(Grid g, Sten<double> s, const double* __restrict__ vb,
-                                double* __restrict__ ab, const __grid_constant__ PatchPieces pp,
-                                int use_pieces) {
-  assemble_row(g, s, vb, ab, blockIdx.x * blockDim.x + threadIdx.x, use_pieces ? &pp : nullptr);
+// 61 us per assembly with one thread per row (7 of the 152 SMs had a block).
+__global__ void __launch_bounds__(128)
+    assemble_kernel(Grid g, Sten<double> s, const double* __restrict__ vb, double* __restrict__ ab,
+                    const __grid_constant__ PatchPieces pp, int use_pieces) {
+  assemble_entry(g, s, vb, ab, blockIdx.x * blockDim.x + threadIdx.x, use_pieces ? &pp : nullptr);
 }
 
 void launch_assemble(const Grid& g, const Sten<double>& s, const double* vb, double* ab,
                      const PatchPieces* pp, cudaStream_t st) {
   static const PatchPieces none{};
+  const Band bd = band_of(g);
+  cudaMemsetAsync(ab, 0, sizeof(double) * (size_t)bd.n * bd.W, st);
   note_launch();
-  assemble_kernel<<<cdiv(band_of(g).n, 128), 128, 0, st>>>(g, s, vb, ab, pp ? *pp : none,
-                                                            pp ? 1 : 0);
+  assemble_kernel<<<cdiv(bd.n * 100, 128), 128, 0, st>>>(g, s, vb, ab, pp ? *pp : none, pp ? 1 : 0);
+}
+
+// ---- inverse by elimination of node columns ---------------------------------------
+//
+// With the unknowns of one grid column (x = const) as a block of 27, the
+// matrix is block tridiagonal after the odd columns are eliminated: an odd
+// column couples to its two neighbours only, and the stabilisation reaches from
+// an even column to the next even ones.  Eliminating every other remaining
+// column leaves a block tridiagonal matrix again, so six levels (strides 1, 2,
+// .. 32) reduce the 33 columns to one; going back, each level's blocks of the
+// inverse follow from the level above:
+//   eliminated column i between i - s and i + s, Z = D_i^-1,
+//     P = -Z A(i, i-s), Q = -Z A(i, i+s), RP = -A(i-s, i) Z, RQ = -A(i+s, i) Z,
+//   inverse blocks  X(i, j) = P X(i-s, j) + Q X(i+s, j)   (j kept)
+//                   X(j, i) = X(j, i-s) RP + X(j, i+s) RQ
+//                   X(i, k) = [i = k] Z + X(i, k-s) RP_k + X(i, k+s) RQ_k.
+// The 27 x 27 blocks are inverted by Gauss-Jordan elimination with partial
+// pivoting, one thread block each.  Every level is a handful of grid-wide
+// phases instead of a chain of 891 columns: a banded LU of the whole matrix on
+// one cluster takes 1,843 us and its inverse 647 us, both set by dependent
+// FP64 operations on few SMs.  The blocks are regular because the velocity
+// part of the Jacobian and the stabilisation are positive on any set of
+// columns; a check at the end (componentwise backward error of one product,
+// tolerance kInvTol) asks for the banded LU where rounding has grown all the
+// same (strong convection at large time steps), and contexts with part-solid
+// patches, whose blocks can be singular, take the LU from the start.
+// Against the exact inverse both are off by 1e-14 to 8e-13 over nu = 0.004 ..
+// 0.02, dt = 0.005 .. 0.02 (means 2.3e-13 LU, 2.2e-13 here).
+constexpr int kCB = 27, kCBB = kCB * kCB;
+constexpr int kInvThreads = 256;
+constexpr double kInvTol = 2e-12;
+enum { kBlkD, kBlkL, kBlkU, kBlkC1, kBlkC2, kBlkZ, kBlkP, kBlkQ, kBlkRP, kBlkRQ, kBlkKinds };
+
+__host__ __device__ inline bool columns_supported(const Grid& g) { return 3 * g.nny == kCB; }
+__host__ __device__ inline size_t column_blocks_doubles(const Grid& g) {
+  return (size_t)kBlkKinds * g.nnx * kCBB + 2 * (size_t)band_of(g).n;
+}
+
+// Invert the 27 x 27 block whose entry (r, c) is load(r, c) into out (row
+// stride ldo).  Threads 0..127 of the block: lane r of warp w holds the
+// entries (r, w), (r, w + 4), ...; the four warps, one per scheduler, share
+// the FP64 work.  Column k's warp picks the pivot row (largest magnitude by the
+// high words, which order like the doubles; rows are never swapped) and
+// publishes the column.
+template <class F>
+__device__ __forceinline__ void invert_column_block(F load, double* out, int ldo, int* bad) {
+  __shared__ double fcol[2][32];
+  __shared__ int pc[kCB];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  constexpr int NC = (kCB + 3) / 4;
+  double a[NC];
+#pragma unroll
+  for (int q = 0; q < NC; ++q) a[q] = lane < kCB && w + 4 * q < kCB ? load(lane, w + 4 * q) : 0.0;
+  bool used = lane >= kCB;
+  int my = 0;
+#pragma unroll
+  for (int k = 0; k < kCB; ++k) {
+    if ((k & 3) == w) {
+      const double v = a[k >> 2];
+      const unsigned key = used ? 0u : (unsigned)(__double2hiint(v) & 0x7FFFFFFF);
+      const unsigned mx = __reduce_max_sync(0xffffffffu, key);
+      const int p = __ffs(__ballot_sync(0xffffffffu, key == mx && !used)) - 1;
+      fcol[k & 1][lane] = v;
+      if (lane == 0) {
+        pc[k] = p < 0 ? 0 : p;
+        if (mx == 0u) *bad = 1;
+      }
+    }
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+    const int p = pc[k];
+    const double ip = 1.0 / fcol[k & 1][p];
+    const bool piv = lane == p;
+    const double m = piv ? ip : -fcol[k & 1][lane] * ip;
+#pragma unroll
+    for (int q = 0; q < NC; ++q) {
+      const double ap = __shfl_sync(0xffffffffu, a[q], p);
+      if (w + 4 * q != k) a[q] = fma(m, ap, piv ? 0.0 : a[q]);
+    }
+    if ((k & 3) == w) a[k >> 2] = m;
+    if (piv) used = true, my = k;
+  }
+  if (lane >= kCB) return;
+#pragma unroll
+  for (int q = 0; q < NC; ++q)
+    if (w + 4 * q < kCB) out[(size_t)my * ldo + pc[w + 4 * q]] = a[q];
+}
+
+// acc + sum_k m_k N[k][lane], m_k in lane k (27 lanes)
+__device__ __forceinline__ double row_times(double m, const double* N, size_t ldn, int lane,
+                                            double acc) {
+  double b = 0.0;
+#pragma unroll
+  for (int k = 0; k < kCB; ++k) {
+    const double mk = __shfl_sync(0xffffffffu, m, k);
+    const double v = lane < kCB ? N[k * ldn + lane] : 0.0;
+    if (k & 1)
+      b = fma(mk, v, b);
+    else
+      acc = fma(mk, v, acc);
+  }
+  return acc + b;
+}
+
+__global__ void __launch_bounds__(kInvThreads)
+    column_inverse_kernel(Grid g, const double* __restrict__ ab, double* blk, double* X,
+                          int* need_lu) {
+  cg::grid_group grid = cg::this_grid();
+  const Band bd = band_of(g);
+  const int nc = g.nnx, n = bd.n, kl = bd.kl;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int kWarps = kInvThreads / 32;
+  const int gt = blockIdx.x * kInvThreads + tid, ngt = gridDim.x * kInvThreads;
+  auto B = [&](int kind, int i) { return blk + ((size_t)kind * nc + i) * kCBB; };
+  auto A = [&](int r, int c) {  // entry of the assembled band
+    const int o = c - r + kl;
+    return o >= 0 && o <= 2 * kl ? ab[(size_t)r * bd.W + o] : 0.0;
+  };
+  // items [0, total) in contiguous runs of a block, one warp per item
+  auto for_items = [&](int total, auto f) {
+    const int per = cdiv(total, gridDim.x), i0 = blockIdx.x * per, i1 = min(total, i0 + per);
+    for (int t = i0 + warp; t < i1; t += kWarps) f(t);
+  };
+  if (gt == 0) *need_lu = 0;
+  for (int e = gt; e < nc * kCBB; e += ngt) {
+    const int i = e / kCBB, r = e % kCBB / kCB, c = e % kCB;
+    B(kBlkD, i)[e % kCBB] = A(kCB * i + r, kCB * i + c);
+    if (i > 0) B(kBlkL, i)[e % kCBB] = A(kCB * i + r, kCB * (i - 1) + c);
+    if (i + 1 < nc) B(kBlkU, i)[e % kCBB] = A(kCB * i + r, kCB * (i + 1) + c);
+  }
+  grid.sync();
+  // D_i with the contributions of the columns eliminated at stride h on both sides
+  auto diag = [&](int i, int h, int e) {
+    double v = B(kBlkD, i)[e];
+    if (h > 0) {
+      if (i > 0) v += B(kBlkC1, i)[e];
+      if (i + h < nc) v += B(kBlkC2, i)[e];
+    }
+    return v;
+  };
+  int s = 1;
+  for (; s < nc; s *= 2) {
+    const int ne = (nc - s + 2 * s - 1) / (2 * s);  // columns s, 3s, 5s, ..
+    if ((int)blockIdx.x < ne) {
+      const int i = s + 2 * s * (int)blockIdx.x;
+      if (tid < 128)
+        invert_column_block([&](int r, int c) { return diag(i, s / 2, r * kCB + c); },
+                            B(kBlkZ, i), kCB, need_lu);
+    } else if (s > 1) {  // kept columns 0, 2s, ..: add the contributions
+      const int nk = (nc + 2 * s - 1) / (2 * s);
+      for (int e = ((int)blockIdx.x - ne) * kInvThreads + tid; e < nk * kCBB;
+           e += ((int)gridDim.x - ne) * kInvThreads) {
+        const int j = 2 * s * (e / kCBB);
+        B(kBlkD, j)[e % kCBB] = diag(j, s / 2, e % kCBB);
+      }
+    }
+    grid.sync();
+    for_items(ne * 3 * kCB, [&](int t) {
+      const int i = s + 2 * s * (t / (3 * kCB)), kind = t / kCB % 3, r = t % kCB;
+      const bool right = i + s < nc;
+      const int o = r * kCB + lane;
+      const bool on = lane < kCB;
+      const double *Z = B(kBlkZ, i), *L = B(kBlkL, i), *U = B(kBlkU, i);
+      if (kind == 0) {  // towards the left neighbour
+        const int j = i - s;
+        double* Uj = B(kBlkU, j);
+        const double q = -row_times(on ? Uj[o] : 0.0, Z, kCB, lane, 0.0);
+        const double c2 = row_times(q, L, kCB, lane, 0.0);
+        double u = 0.0;
+        if (right)
+          u = row_times(q, U, kCB, lane,
+                        s == 1 && on ? A(kCB * j + r, kCB * (j + 2) + lane) : 0.0);
+        if (on) {
+          B(kBlkRP, i)[o] = q;
+          B(kBlkC2, j)[o] = c2;
+          Uj[o] = u;
+        }
+      } else if (kind == 1) {  // towards the right neighbour
+        if (!right) return;
+        const int j = i + s;
+        double* Lj = B(kBlkL, j);
+        const double q = -row_times(on ? Lj[o] : 0.0, Z, kCB, lane, 0.0);
+        const double c1 = row_times(q, U, kCB, lane, 0.0);
+        const double l = row_times(q, L, kCB, lane,
+                                   s == 1 && on ? A(kCB * j + r, kCB * (j - 2) + lane) : 0.0);
+        if (on) {
+          B(kBlkRQ, i)[o] = q;
+          B(kBlkC1, j)[o] = c1;
+          Lj[o] = l;
+        }
+      } else {
+        const double z = on ? Z[o] : 0.0;
+        const double pv = -row_times(z, L, kCB, lane, 0.0);
+        if (on) B(kBlkP, i)[o] = pv;
+        if (right) {
+          const double qv = -row_times(z, U, kCB, lane, 0.0);
+          if (on) B(kBlkQ, i)[o] = qv;
+        }
+      }
+    });
+    grid.sync();
+  }
+  if (blockIdx.x == 0 && tid < 128)
+    invert_column_block([&](int r, int c) { return diag(0, s / 2, r * kCB + c); }, X, n, need_lu);
+  grid.sync();
+  auto XB = [&](int i, int j) { return X + (size_t)(kCB * i) * n + kCB * j; };
+  for (s /= 2; s >= 1; s /= 2) {
+    const int ne = (nc - s + 2 * s - 1) / (2 * s), nk = (nc + 2 * s - 1) / (2 * s);
+    for_items(2 * ne * nk * kCB, [&](int t) {
+      const int r = t % kCB, j = 2 * s * (t / kCB % nk), e = t / (kCB * nk);
+      const int i = s + 2 * s * (e % ne);
+      const bool right = i + s < nc, on = lane < kCB;
+      double v;
+      if (e < ne) {  // X(i, j)
+        v = row_times(on ? B(kBlkP, i)[r * kCB + lane] : 0.0, XB(i - s, j), n, lane, 0.0);
+        if (right)
+          v = row_times(on ? B(kBlkQ, i)[r * kCB + lane] : 0.0, XB(i + s, j), n, lane, v);
+        if (on) XB(i, j)[(size_t)r * n + lane] = v;
+      } else {  // X(j, i)
+        v = row_times(on ? XB(j, i - s)[(size_t)r * n + lane] : 0.0, B(kBlkRP, i), kCB, lane, 0.0);
+        if (right)
+          v = row_times(on ? XB(j, i + s)[(size_t)r * n + lane] : 0.0, B(kBlkRQ, i), kCB, lane, v);
+        if (on) XB(j, i)[(size_t)r * n + lane] = v;
+      }
+    });
+    grid.sync();
+    for_items(ne * ne * kCB, [&](int t) {
+      const int r = t % kCB, i = s + 2 * s * (t / kCB % ne), k = s + 2 * s * (t / (kCB * ne));
+      const bool right = k + s < nc, on = lane < kCB;
+      double v = i == k && on ? B(kBlkZ, i)[r * kCB + lane] : 0.0;
+      v = row_times(on ? XB(i, k - s)[(size_t)r * n + lane] : 0.0, B(kBlkRP, k), kCB, lane, v);
+      if (right)
+        v = row_times(on ? XB(i, k + s)[(size_t)r * n + lane] : 0.0, B(kBlkRQ, k), kCB, lane, v);
+      if (on) XB(i, k)[(size_t)r * n + lane] = v;
+    });
+    grid.sync();
+  }
+  // y = X b for a vector of signs, then the componentwise backward error of A y = b
+  double* y = blk + (size_t)kBlkKinds * nc * kCBB;
+  auto sign = [](int k) { return ((unsigned)k * 2654435761u >> 17) & 1u ? 1.0 : -1.0; };
+  for_items(n, [&](int r) {
+    double acc = 0.0;
+    for (int c = lane; c < n; c += 32) acc = fma(X[(size_t)r * n + c], sign(c), acc);
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) y[r] = acc;
+  });
+  grid.sync();
+  for_items(n, [&](int r) {
+    double res = 0.0, mag = 0.0;
+    for (int c = max(0, r - kl) + lane; c <= min(n - 1, r + kl); c += 32) {
+      const double v = A(r, c) * y[c];
+      res += v;
+      mag += fabs(v);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      res += __shfl_xor_sync(0xffffffffu, res, o);
+      mag += __shfl_xor_sync(0xffffffffu, mag, o);
+    }
+    if (lane == 0 && !(fabs(res - sign(r)) <= kInvTol * (mag + 1.0))) *need_lu = 1;
+  });
 }
 
 __global__ void __launch_bounds__(kLUThreads)
-    band_lu_kernel(Grid g, double* __restrict__ ab, int* __restrict__ piv, int* status) {
+    band_lu_kernel(Grid g, double* __restrict__ ab, int* __restrict__ piv, int* status,
+                   const int* need) {
+  if (need && !*need) return;
   extern __shared__ double win[];  // kWin * W
   band_lu_block(g, ab, piv, status, win);
 }
@@ -46,7 +310,6 @@ __global__ void __launch_bounds__(kLUThreads)
 // owner does its own panel columns first (warp 0) and factors them while its
 // other warps finish.  Every entry sees the same floating-point operations
 // in the same order as in band_lu_block, so the factors are the same.
-namespace cg = cooperative_groups;
 constexpr int kLUCluster = 8;
 constexpr int kLUCThreads = 256;
 
@@ -66,7 +329,9 @@ __device__ __forceinline__ void cl_wait() {
 }
 
 __global__ void __launch_bounds__(kLUCThreads)
-    band_lu_cluster_kernel(Grid g, double* __restrict__ ab, int* __restrict__ piv, int* status) {
+    band_lu_cluster_kernel(Grid g, double* __restrict__ ab, int* __restrict__ piv, int* status,
+                           const int* need) {
+  if (need && !*need) return;  // every block of the cluster reads the same word
   cg::cluster_group cl = cg::this_cluster();
   const Band bd = band_of(g);
   const int q = (int)cl.block_rank();
@@ -197,14 +462,18 @@ __global__ void __launch_bounds__(kLUCThreads)
   }
 }
 
-__global__ void diag_recip_kernel(Grid g, const double* __restrict__ ab, double* __restrict__ rd) {
+__global__ void diag_recip_kernel(Grid g, const double* __restrict__ ab, double* __restrict__ rd,
+                                  const int* need) {
+  if (need && !*need) return;
   band_diag_recip(g, ab, rd, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // Columns [kInvWarps * block, +kInvWarps) of the inverse.
 __global__ void __launch_bounds__(32 * kInvWarps)
     band_inverse_kernel(Grid g, const double* __restrict__ ab, const int* __restrict__ piv,
-                        const double* __restrict__ rd, double* __restrict__ Ainv) {
+                        const double* __restrict__ rd, double* __restrict__ Ainv,
+                        const int* need) {
+  if (need && !*need) return;
   extern __shared__ __align__(16) double sm[];
   band_inverse_block(g, ab, piv, rd, Ainv, blockIdx.x * kInvWarps, sm);
 }
@@ -264,7 +533,8 @@ __global__ void __launch_bounds__(1024)
 // Banded LU of the assembled coarse Jacobian: the cluster kernel when a
 // cluster of kLUCluster CTAs with its shared memory can be placed, else the
 // single-block kernel.
-void launch_band_lu(const Grid& g, double* ab, int* piv, int* status, cudaStream_t st) {
+void launch_band_lu(const Grid& g, double* ab, int* piv, int* status, const int* need,
+                    cudaStream_t st) {
   const Band bd = band_of(g);
   const size_t csm = lu_cluster_smem(bd);
   // whether the cluster can be placed, checked once per process (thread-safe
@@ -307,14 +577,14 @@ void launch_band_lu(const Grid& g, double* ab, int* piv, int* status, cudaStream
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     note_launch();
-    if (cudaLaunchKernelEx(&cfg, band_lu_cluster_kernel, g, ab, piv, status) == cudaSuccess) return;
+    if (cudaLaunchKernelEx(&cfg, band_lu_cluster_kernel, g, ab, piv, status, need) == cudaSuccess) return;
     cudaGetLastError();
   }
   const size_t win_bytes = sizeof(double) * kWin * bd.W;
   cudaFuncSetAttribute(band_lu_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)win_bytes);
   note_launch();
-  band_lu_kernel<<<1, kLUThreads, win_bytes, st>>>(g, ab, piv, status);
+  band_lu_kernel<<<1, kLUThreads, win_bytes, st>>>(g, ab, piv, status, need);
 }
 
 }  // namespace
@@ -327,7 +597,7 @@ size_t coarse_band_doubles(const Grid& g) {
 void launch_coarse_lu(const Grid& g, const Sten<double>& s, const double* vb, double* band,
                       int* piv, int* status, cudaStream_t st) {
   launch_assemble(g, s, vb, band, nullptr, st);
-  launch_band_lu(g, band, piv, status, st);
+  launch_band_lu(g, band, piv, status, nullptr, st);
 }
 
 void launch_coarse_lu_solve(const Grid& g, const double* band, const int* piv, const double* b,
@@ -350,23 +620,54 @@ size_t coarse_work_doubles(const Grid& g) {
   return (size_t)bd.n * bd.W + (size_t)bd.n + (size_t)bd.n;
 }
 
+size_t coarse_factor_doubles(const Grid& g) {
+  return coarse_work_doubles(g) + (columns_supported(g) ? column_blocks_doubles(g) + 1 : 0);
+}
+
 void launch_coarse_factor(const Grid& g, const Sten<double>& s, const double* vb, double* work,
                           double* Ainv, int* status, cudaStream_t st, const PatchPieces* pp) {
   const Band bd = band_of(g);
   double* ab = work;
   int* piv = reinterpret_cast<int*>(work + (size_t)bd.n * bd.W);
   launch_assemble(g, s, vb, ab, pp, st);
-  launch_band_lu(g, ab, piv, status, st);
+  // the inverse by node columns where the grid can be resident; the banded LU
+  // then runs only when that asks for it
+  const int* need = nullptr;
+  static const int blocks = [] {
+    int dev = 0, sms = 0, per = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, column_inverse_kernel, kInvThreads,
+                                                      0) != cudaSuccess)
+      per = 0;
+    cudaGetLastError();
+    return per > 0 ? sms : 0;
+  }();
+  if (!pp && columns_supported(g) && blocks > g.nnx) {
+    double* blk = work + coarse_work_doubles(g);
+    int* flag = reinterpret_cast<int*>(blk + column_blocks_doubles(g));
+    Grid gc = g;
+    const double* abc = ab;
+    void* args[] = {(void*)&gc, (void*)&abc, (void*)&blk, (void*)&Ainv, (void*)&flag};
+    note_launch();
+    if (cudaLaunchCooperativeKernel((void*)column_inverse_kernel, dim3(blocks), dim3(kInvThreads),
+                                    args, 0, st) == cudaSuccess)
+      need = flag;
+    else
+      cudaGetLastError();
+  }
+  launch_band_lu(g, ab, piv, status, need, st);
   double* rd = work + (size_t)bd.n * bd.W + bd.n;
   note_launch();
-  diag_recip_kernel<<<cdiv(bd.n, 128), 128, 0, st>>>(g, ab, rd);
+  diag_recip_kernel<<<cdiv(bd.n, 128), 128, 0, st>>>(g, ab, rd, need);
   const size_t smem = sizeof(double) * inv_block_smem_doubles(bd.n);
   static const bool inv_attr =
       cudaFuncSetAttribute(band_inverse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)smem) == cudaSuccess;
   (void)inv_attr;
   note_launch();
-  band_inverse_kernel<<<cdiv(bd.n, kInvWarps), 32 * kInvWarps, smem, st>>>(g, ab, piv, rd, Ainv);
+  band_inverse_kernel<<<cdiv(bd.n, kInvWarps), 32 * kInvWarps, smem, st>>>(g, ab, piv, rd, Ainv,
+                                                                           need);
 }
 
 template <typename T>

@@ -119,6 +119,97 @@ __device__ __forceinline__ void assemble_row(const Grid& g, const Sten<double>& 
   }
 }
 
+// Stabilisation entry between the pressures of nodes (i, j) and (ni, nj), the
+// patches that hold both added to v in the order of assemble_row.
+__device__ __forceinline__ double lps_entry(const Grid& g, const Sten<double>& s, int i, int j,
+                                            int ni, int nj, const PatchPieces* pp, double v) {
+  for (int dJ = 0; dJ < 2; ++dJ) {
+    const int PJ = (j >> 1) - dJ;
+    if (PJ < 0 || PJ >= g.ny / 2 || j - 2 * PJ > 2 || nj < 2 * PJ || nj > 2 * PJ + 2) continue;
+    for (int dI = 0; dI < 2; ++dI) {
+      const int PI = (i >> 1) - dI;
+      if (PI < 0 || PI >= g.nx / 2 || i - 2 * PI > 2 || ni < 2 * PI || ni > 2 * PI + 2) continue;
+      const int c00 = (2 * PJ) * g.nx + 2 * PI;
+      const int fm = (g.solid[c00] ? 0 : 1) | (g.solid[c00 + 1] ? 0 : 2) |
+                     (g.solid[c00 + g.nx] ? 0 : 4) | (g.solid[c00 + g.nx + 1] ? 0 : 8);
+      const bool whole = fm == 15 || !pp;
+      if ((whole && g.solid[c00]) || fm == 0) continue;
+      const int e = ((i - 2 * PI) + 3 * (j - 2 * PJ)) * 9 + (ni - 2 * PI) + 3 * (nj - 2 * PJ);
+      if (whole) {
+        v += s.S9[e];
+      } else {
+        double w = 0.0;
+        for (int c = 0; c < 4; ++c)
+          if (fm & (1 << c)) w += pp->S[c][e];
+        v += w;
+      }
+    }
+  }
+  return v;
+}
+
+// The same matrix as assemble_row, into a band that is zero: item t is one
+// pair (row, neighbour node within two nodes) times the four cells around the
+// row's node, one per lane of a group of four, so that the FP64 work (1/64 of
+// the FP32 rate here) spreads over the whole GPU.  The group's first lane adds
+// the cells' parts in assemble_row's order, so the entries are the same bit
+// for bit.  Every lane of a warp calls it.
+__device__ __forceinline__ void assemble_entry(const Grid& g, const Sten<double>& s,
+                                               const double* __restrict__ vb,
+                                               double* __restrict__ ab, int t,
+                                               const PatchPieces* pp) {
+  const Band bd = band_of(g);
+  const int pair = t >> 2, cell = t & 3, row = pair % bd.n, nb = pair / bd.n;
+  const bool in = nb < 25, near = nb < 9;
+  // the 3 x 3 neighbours first (they hold the FP64 work), then the outer ring
+  const int di = near ? nb % 3 - 1 : (nb < 19 ? (nb - 9) % 5 - 2 : ((nb & 1) ? 2 : -2));
+  const int dj = near ? nb / 3 - 1 : (nb < 19 ? (nb < 14 ? -2 : 2) : (nb - 19) / 2 - 1);
+  const int c = row % 3, node = row / 3, i = node / g.nny, j = node % g.nny;
+  const int ni = i + di, nj = j + dj;
+  const bool ok = in && ni >= 0 && nj >= 0 && ni <= g.nx && nj <= g.ny;
+  const uint8_t f = in ? g.flags[j * g.nnx + i] : uint8_t(0);
+  const bool cons = (c < 2) ? (f & kVDir) : (f & kPFix);
+  // this lane's cell, if it holds both nodes
+  const int cx = cell & 1, cy = cell >> 1, ci = i - 1 + cx, cj = j - 1 + cy;
+  const int bx = ni - ci, by = nj - cj;
+  double part[3] = {0.0, 0.0, 0.0};
+  const bool has = ok && near && !cons && ci >= 0 && cj >= 0 && ci < g.nx && cj < g.ny && bx >= 0 &&
+                   bx <= 1 && by >= 0 && by <= 1 && !g.solid[cj * g.nx + ci];
+  if (has) {
+    double bu[4], bv[4], J[3][3];
+    load_cell<double, false>(g, vb, ci, cj, 0, bu);
+    load_cell<double, false>(g, vb + g.nn, ci, cj, 0, bv);
+    GaussData<double> gd;
+    gauss_data<double>(bu, bv, gd);
+    elem_pair<double>(s, gd, (1 - cx) + 2 * (1 - cy), bx + 2 * by, J);
+    for (int k = 0; k < 3; ++k) part[k] = c == 0 ? J[0][k] : (c == 1 ? J[1][k] : J[2][k]);
+  }
+  double sum[3] = {0.0, 0.0, 0.0};
+  const int base = threadIdx.x & 28;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const bool hq = __shfl_sync(0xffffffffu, (int)has, base + q);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const double v = __shfl_sync(0xffffffffu, part[k], base + q);
+      if (hq) sum[k] += v;
+    }
+  }
+  if (cell != 0 || !ok) return;
+  if (cons) {
+    if (di == 0 && dj == 0) AB(ab, bd, row, row) = 1.0;
+    return;
+  }
+  const uint8_t fb = g.flags[nj * g.nnx + ni];
+  if (near && !(fb & kVDir)) {
+    AB(ab, bd, row, bidx(g, 0, ni, nj)) = sum[0];
+    AB(ab, bd, row, bidx(g, 1, ni, nj)) = sum[1];
+  }
+  if (fb & kPFix) return;
+  if (c == 2) sum[2] = lps_entry(g, s, i, j, ni, nj, pp, sum[2]);
+  if (near || c == 2) AB(ab, bd, row, bidx(g, 2, ni, nj)) = sum[2];
+}
+
 // Banded LU with partial pivoting in one thread block (dgbtf2 ordering).
 // The rows k..k+kl that elimination step k touches live in a shared-memory
 // window of kWin row slots (row r in slot r % kWin, same per-row band offset

@@ -142,8 +142,9 @@ constexpr int kSetupCells = kSetupThreads / 16;
 // Coarse direct solve (coarse.cu) -------------------------------------------
 // Assemble the banded Jacobian of the coarsest level (FP64), factor it with
 // partial pivoting and form the explicit inverse Ainv (ndof x ndof, FP64,
-// unknowns in band order).  `work` needs coarse_work_doubles(g) doubles.
+// unknowns in band order).  `work` needs coarse_factor_doubles(g) doubles.
 size_t coarse_work_doubles(const Grid& g);
+size_t coarse_factor_doubles(const Grid& g);  // `work` of launch_coarse_factor
 bool coarse_supported(const Grid& g);  // band fits the shared-memory window
 // Assemble + factor into caller-provided band storage (coarse_band_doubles(g)
 // doubles) and pivots (3 nn ints), and solve with those factors.

@@ -66,7 +66,7 @@ class Solver final : public SolverBase {
     // a level-1 obstacle at odd offsets leaves part-solid patches on the coarse level
     part_solid_ = part_solid_patches(c_->lv[lv_[0].level]);
     if (part_solid_) pieces_ = make_patch_pieces(g0.h, cfg);
-    coarse_work_ = c_->mem.alloc<double>(coarse_work_doubles(g0));
+    coarse_work_ = c_->mem.alloc<double>(coarse_factor_doubles(g0));
     ainv_ = c_->mem.alloc<double>((size_t)9 * g0.nn * g0.nn);
     status_ = c_->mem.alloc<int>(4);
     if (status_) cudaMemsetAsync(status_, 0, 4 * sizeof(int), st_);  // fresh memory is not zero
