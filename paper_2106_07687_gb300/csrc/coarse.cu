@@ -2,6 +2,7 @@
 // banded LU, explicit inverse and the dense solve (bodies in coarse_body.cuh).
 #include <cooperative_groups.h>
 #include <cstdio>
+#include <type_traits>
 
 #include "coarse_body.cuh"
 #include "kernels.h"
@@ -46,7 +47,8 @@ void launch_assemble(const Grid& g, const Sten<double>& s, const double* vb, dou
 // pivoting, one thread block each.  Every level is a handful of grid-wide
 // phases instead of a chain of 891 columns: a banded LU of the whole matrix on
 // one cluster takes 1,843 us and its inverse 647 us, both set by dependent
-// FP64 operations on few SMs.  The blocks are regular because the velocity
+// FP64 operations on few SMs; this takes 369 us, of which the seven levels of
+// block inverses 137 and the last level's products 90.  The blocks are regular because the velocity
 // part of the Jacobian and the stabilisation are positive on any set of
 // columns; a check at the end (componentwise backward error of one product,
 // tolerance kInvTol) asks for the banded LU where rounding has grown all the
@@ -55,81 +57,127 @@ void launch_assemble(const Grid& g, const Sten<double>& s, const double* vb, dou
 // Against the exact inverse both are off by 1e-14 to 8e-13 over nu = 0.004 ..
 // 0.02, dt = 0.005 .. 0.02 (means 2.3e-13 LU, 2.2e-13 here).
 constexpr int kCB = 27, kCBB = kCB * kCB;
-constexpr int kInvThreads = 256;
+constexpr int kInvThreads = 512;
+constexpr int kGjWarps = 8;   // warps that invert a block together
 constexpr double kInvTol = 2e-12;
-enum { kBlkD, kBlkL, kBlkU, kBlkC1, kBlkC2, kBlkZ, kBlkP, kBlkQ, kBlkRP, kBlkRQ, kBlkKinds };
+enum { kBlkD, kBlkL, kBlkU, kBlkL2, kBlkU2, kBlkC1, kBlkC2, kBlkZ, kBlkP, kBlkQ, kBlkRP, kBlkRQ, kBlkKinds };
 
 __host__ __device__ inline bool columns_supported(const Grid& g) { return 3 * g.nny == kCB; }
 __host__ __device__ inline size_t column_blocks_doubles(const Grid& g) {
   return (size_t)kBlkKinds * g.nnx * kCBB + 2 * (size_t)band_of(g).n;
 }
 
+// 1 / d by Newton's iteration from the hardware's approximation (about 20
+// bits): two steps reach the rounding error.
+__device__ __forceinline__ double recip64(double d) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+#pragma unroll
+  for (int k = 0; k < 2; ++k) y = fma(y, fma(-d, y, 1.0), y);
+  return y;
+}
+
 // Invert the 27 x 27 block whose entry (r, c) is load(r, c) into out (row
-// stride ldo).  Threads 0..127 of the block: lane r of warp w holds the
-// entries (r, w), (r, w + 4), ...; the four warps, one per scheduler, share
-// the FP64 work.  Column k's warp picks the pivot row (largest magnitude by the
+// stride ldo).  The first kGjWarps warps of the block: lane r of warp w holds
+// the entries (r, w), (r, w + kGjWarps), ...  Column k's warp picks the pivot row (largest magnitude by the
 // high words, which order like the doubles; rows are never swapped) and
-// publishes the column.
+// publishes the multipliers (every FP64 instruction of a warp takes 64 cycles
+// of its scheduler, so the reciprocal is formed once).
 template <class F>
 __device__ __forceinline__ void invert_column_block(F load, double* out, int ldo, int* bad) {
-  __shared__ double fcol[2][32];
+  __shared__ double mult[2][32];
   __shared__ int pc[kCB];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  constexpr int NC = (kCB + 3) / 4;
+  constexpr int NC = (kCB + kGjWarps - 1) / kGjWarps;
   double a[NC];
 #pragma unroll
-  for (int q = 0; q < NC; ++q) a[q] = lane < kCB && w + 4 * q < kCB ? load(lane, w + 4 * q) : 0.0;
+  for (int q = 0; q < NC; ++q)
+    a[q] = lane < kCB && w + kGjWarps * q < kCB ? load(lane, w + kGjWarps * q) : 0.0;
   bool used = lane >= kCB;
   int my = 0;
 #pragma unroll
-  for (int k = 0; k < kCB; ++k) {
-    if ((k & 3) == w) {
-      const double v = a[k >> 2];
-      const unsigned key = used ? 0u : (unsigned)(__double2hiint(v) & 0x7FFFFFFF);
-      const unsigned mx = __reduce_max_sync(0xffffffffu, key);
-      const int p = __ffs(__ballot_sync(0xffffffffu, key == mx && !used)) - 1;
-      fcol[k & 1][lane] = v;
-      if (lane == 0) {
-        pc[k] = p < 0 ? 0 : p;
-        if (mx == 0u) *bad = 1;
+  for (int kq = 0; kq < NC; ++kq)
+#pragma unroll 1
+    for (int kw = 0; kw < kGjWarps; ++kw) {
+      const int k = kGjWarps * kq + kw;
+      if (k >= kCB) break;
+      if (kw == w) {
+        const unsigned key = used ? 0u : (unsigned)(__double2hiint(a[kq]) & 0x7FFFFFFF);
+        const unsigned mx = __reduce_max_sync(0xffffffffu, key);
+        const int p = max(0, __ffs(__ballot_sync(0xffffffffu, key == mx && !used)) - 1);
+        const double ip = recip64(__shfl_sync(0xffffffffu, a[kq], p));
+        mult[k & 1][lane] = lane == p ? ip : -a[kq] * ip;
+        if (lane == 0) {
+          pc[k] = p;
+          if (mx == 0u) *bad = 1;
+        }
       }
-    }
-    asm volatile("bar.sync 1, 128;" ::: "memory");
-    const int p = pc[k];
-    const double ip = 1.0 / fcol[k & 1][p];
-    const bool piv = lane == p;
-    const double m = piv ? ip : -fcol[k & 1][lane] * ip;
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * kGjWarps) : "memory");
+      const int p = pc[k];
+      const bool piv = lane == p;
+      const double m = mult[k & 1][lane];
 #pragma unroll
-    for (int q = 0; q < NC; ++q) {
-      const double ap = __shfl_sync(0xffffffffu, a[q], p);
-      if (w + 4 * q != k) a[q] = fma(m, ap, piv ? 0.0 : a[q]);
+      for (int q = 0; q < NC; ++q) {
+        const double ap = __shfl_sync(0xffffffffu, a[q], p);
+        if (q != kq || kw != w) a[q] = fma(m, ap, piv ? 0.0 : a[q]);
+      }
+      if (kw == w) a[kq] = m;
+      if (piv) used = true, my = k;
     }
-    if ((k & 3) == w) a[k >> 2] = m;
-    if (piv) used = true, my = k;
-  }
   if (lane >= kCB) return;
 #pragma unroll
   for (int q = 0; q < NC; ++q)
-    if (w + 4 * q < kCB) out[(size_t)my * ldo + pc[w + 4 * q]] = a[q];
+    if (w + kGjWarps * q < kCB) out[(size_t)my * ldo + pc[w + kGjWarps * q]] = a[q];
 }
 
-// acc + sum_k m_k N[k][lane], m_k in lane k (27 lanes)
-__device__ __forceinline__ double row_times(double m, const double* N, size_t ldn, int lane,
-                                            double acc) {
-  double b = 0.0;
+// A product of blocks: out = sign (init + M N [+ M2 N2]) with the row strides
+// below (M2, init may be null).  One warp forms an 8 x 8 tile of it with FP64
+// tensor instructions, whose rate is that of the scalar ones here but which
+// take a twentieth of the instructions (with scalar multiply-adds and
+// shuffles a product's code did not fit the instruction cache beside the
+// rest, and its instructions took longer to arrive than its operands).  All
+// loads go out first: another SM has just written the blocks.
+struct Prod {
+  const double *M, *N, *M2, *N2, *init;
+  double* out;
+  int ldm, ldn, ldm2, ldn2, ldi, ldo;
+  double sign;
+};
+constexpr int kCT = (kCB + 7) / 8, kTiles = kCT * kCT, kCK = (kCB + 3) / 4;
+__device__ __forceinline__ void block_tile(const Prod& P, int tile, int lane) {
+  const int r = tile / kCT * 8 + (lane >> 2), c = tile % kCT * 8 + (lane >> 2), q = lane & 3;
+  double m[2][kCK], v[2][kCK];
 #pragma unroll
-  for (int k = 0; k < kCB; ++k) {
-    const double mk = __shfl_sync(0xffffffffu, m, k);
-    const double v = lane < kCB ? N[k * ldn + lane] : 0.0;
-    if (k & 1)
-      b = fma(mk, v, b);
-    else
-      acc = fma(mk, v, acc);
+  for (int h = 0; h < 2; ++h) {
+    const double *M = h ? P.M2 : P.M, *N = h ? P.N2 : P.N;
+    const size_t ldm = h ? P.ldm2 : P.ldm, ldn = h ? P.ldn2 : P.ldn;
+#pragma unroll
+    for (int k = 0; k < kCK; ++k) {
+      const int e = 4 * k + q;
+      m[h][k] = M && r < kCB && e < kCB ? M[r * ldm + e] : 0.0;
+      v[h][k] = M && c < kCB && e < kCB ? N[e * ldn + c] : 0.0;
+    }
   }
-  return acc + b;
+  const int co = tile % kCT * 8 + 2 * q;
+  double d[2];
+#pragma unroll
+  for (int e = 0; e < 2; ++e)
+    d[e] = P.init && r < kCB && co + e < kCB ? P.init[(size_t)r * P.ldi + co + e] : 0.0;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    if (h && !P.M2) break;
+#pragma unroll
+    for (int k = 0; k < kCK; ++k)
+      asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
+                   : "+d"(d[0]), "+d"(d[1])
+                   : "d"(m[h][k]), "d"(v[h][k]));
+  }
+#pragma unroll
+  for (int e = 0; e < 2; ++e)
+    if (r < kCB && co + e < kCB) P.out[(size_t)r * P.ldo + co + e] = P.sign * d[e];
 }
 
-__global__ void __launch_bounds__(kInvThreads)
+__global__ void __launch_bounds__(kInvThreads, 1)
     column_inverse_kernel(Grid g, const double* __restrict__ ab, double* blk, double* X,
                           int* need_lu) {
   cg::grid_group grid = cg::this_grid();
@@ -154,6 +202,8 @@ __global__ void __launch_bounds__(kInvThreads)
     B(kBlkD, i)[e % kCBB] = A(kCB * i + r, kCB * i + c);
     if (i > 0) B(kBlkL, i)[e % kCBB] = A(kCB * i + r, kCB * (i - 1) + c);
     if (i + 1 < nc) B(kBlkU, i)[e % kCBB] = A(kCB * i + r, kCB * (i + 1) + c);
+    if (i > 1) B(kBlkL2, i)[e % kCBB] = A(kCB * i + r, kCB * (i - 2) + c);
+    if (i + 2 < nc) B(kBlkU2, i)[e % kCBB] = A(kCB * i + r, kCB * (i + 2) + c);
   }
   grid.sync();
   // D_i with the contributions of the columns eliminated at stride h on both sides
@@ -166,14 +216,72 @@ __global__ void __launch_bounds__(kInvThreads)
     return v;
   };
   int s = 1;
-  for (; s < nc; s *= 2) {
-    const int ne = (nc - s + 2 * s - 1) / (2 * s);  // columns s, 3s, 5s, ..
+  auto XB = [&](int i, int j) { return X + (size_t)(kCB * i) * n + kCB * j; };
+  // The products of a phase of stride s, one 8 x 8 tile per warp:
+  //   0: P, Q, RP, RQ of the eliminated columns
+  //   1: the kept neighbours' contributions to D and couplings to the next kept
+  //   2: X(eliminated, kept), X(kept, eliminated)     3: X(eliminated, eliminated)
+  auto run_phase = [&](int phase) {
+    const int ne = (nc + s - 1) / (2 * s), nk = (nc + 2 * s - 1) / (2 * s);
+    const int total = phase < 2 ? 4 * ne : (phase == 2 ? 2 * ne * nk : ne * ne);
+    for_items(total * kTiles, [&](int t) {
+      const int u = t / kTiles;
+      Prod P{};
+      P.sign = 1.0;
+      P.ldm = P.ldn = P.ldm2 = P.ldn2 = P.ldi = P.ldo = kCB;
+      if (phase < 2) {
+        // even kinds towards the left neighbour j, odd kinds towards the right
+        const int i = s + 2 * s * (u >> 2), kind = u & 3, side = kind & 1;
+        const int j = side ? i + s : i - s;
+        if (side && j >= nc) return;
+        double *L = B(kBlkL, i), *U = B(kBlkU, i), *C = B(side ? kBlkL : kBlkU, j);
+        if (phase == 0) {
+          P.sign = -1.0;
+          if (kind < 2)
+            P.M = B(kBlkZ, i), P.N = side ? U : L, P.out = B(side ? kBlkQ : kBlkP, i);
+          else
+            P.M = C, P.N = B(kBlkZ, i), P.out = B(side ? kBlkRQ : kBlkRP, i);
+        } else {
+          P.M = B(side ? kBlkRQ : kBlkRP, i);
+          if (kind < 2) {
+            P.N = side ? U : L, P.out = B(side ? kBlkC1 : kBlkC2, j);
+          } else {
+            if (i + s >= nc) return;
+            P.N = side ? L : U, P.out = C;
+            // the coupling of two even columns that the matrix itself holds
+            if (s == 1) P.init = B(side ? kBlkL2 : kBlkU2, j);
+          }
+        }
+      } else {
+        P.ldo = n;
+        const int j = phase == 2 ? 2 * s * (u % nk) : 0, e = phase == 2 ? u / nk : u;
+        const int i = s + 2 * s * (e % ne);
+        if (phase == 2 && e < ne) {  // X(i, j)
+          P.M = B(kBlkP, i), P.N = XB(i - s, j), P.ldn = n;
+          if (i + s < nc) P.M2 = B(kBlkQ, i), P.N2 = XB(i + s, j), P.ldn2 = n;
+          P.out = XB(i, j);
+        } else {  // X(a, i), a kept or eliminated
+          const int a = phase == 2 ? j : s + 2 * s * (e / ne);
+          if (a == i) P.init = B(kBlkZ, i);
+          P.M = XB(a, i - s), P.N = B(kBlkRP, i), P.ldm = n;
+          if (i + s < nc) P.M2 = XB(a, i + s), P.N2 = B(kBlkRQ, i), P.ldm2 = n;
+          P.out = XB(a, i);
+        }
+      }
+      block_tile(P, t % kTiles, lane);
+    });
+    grid.sync();
+  };
+  // down: levels of stride 1, 2, ..; the last "level" is column 0 alone
+  for (;; s *= 2) {
+    const bool last = s >= nc;
+    const int ne = last ? 1 : (nc + s - 1) / (2 * s);  // columns s, 3 s, ..
     if ((int)blockIdx.x < ne) {
-      const int i = s + 2 * s * (int)blockIdx.x;
-      if (tid < 128)
+      const int i = last ? 0 : s + 2 * s * (int)blockIdx.x;
+      if (tid < 32 * kGjWarps)
         invert_column_block([&](int r, int c) { return diag(i, s / 2, r * kCB + c); },
-                            B(kBlkZ, i), kCB, need_lu);
-    } else if (s > 1) {  // kept columns 0, 2s, ..: add the contributions
+                            last ? X : B(kBlkZ, i), last ? n : kCB, need_lu);
+    } else if (s > 1 && !last) {  // kept columns 0, 2 s, ..: add the contributions
       const int nk = (nc + 2 * s - 1) / (2 * s);
       for (int e = ((int)blockIdx.x - ne) * kInvThreads + tid; e < nk * kCBB;
            e += ((int)gridDim.x - ne) * kInvThreads) {
@@ -182,85 +290,13 @@ __global__ void __launch_bounds__(kInvThreads)
       }
     }
     grid.sync();
-    for_items(ne * 3 * kCB, [&](int t) {
-      const int i = s + 2 * s * (t / (3 * kCB)), kind = t / kCB % 3, r = t % kCB;
-      const bool right = i + s < nc;
-      const int o = r * kCB + lane;
-      const bool on = lane < kCB;
-      const double *Z = B(kBlkZ, i), *L = B(kBlkL, i), *U = B(kBlkU, i);
-      if (kind == 0) {  // towards the left neighbour
-        const int j = i - s;
-        double* Uj = B(kBlkU, j);
-        const double q = -row_times(on ? Uj[o] : 0.0, Z, kCB, lane, 0.0);
-        const double c2 = row_times(q, L, kCB, lane, 0.0);
-        double u = 0.0;
-        if (right)
-          u = row_times(q, U, kCB, lane,
-                        s == 1 && on ? A(kCB * j + r, kCB * (j + 2) + lane) : 0.0);
-        if (on) {
-          B(kBlkRP, i)[o] = q;
-          B(kBlkC2, j)[o] = c2;
-          Uj[o] = u;
-        }
-      } else if (kind == 1) {  // towards the right neighbour
-        if (!right) return;
-        const int j = i + s;
-        double* Lj = B(kBlkL, j);
-        const double q = -row_times(on ? Lj[o] : 0.0, Z, kCB, lane, 0.0);
-        const double c1 = row_times(q, U, kCB, lane, 0.0);
-        const double l = row_times(q, L, kCB, lane,
-                                   s == 1 && on ? A(kCB * j + r, kCB * (j - 2) + lane) : 0.0);
-        if (on) {
-          B(kBlkRQ, i)[o] = q;
-          B(kBlkC1, j)[o] = c1;
-          Lj[o] = l;
-        }
-      } else {
-        const double z = on ? Z[o] : 0.0;
-        const double pv = -row_times(z, L, kCB, lane, 0.0);
-        if (on) B(kBlkP, i)[o] = pv;
-        if (right) {
-          const double qv = -row_times(z, U, kCB, lane, 0.0);
-          if (on) B(kBlkQ, i)[o] = qv;
-        }
-      }
-    });
-    grid.sync();
+    if (last) break;
+    run_phase(0);
+    run_phase(1);
   }
-  if (blockIdx.x == 0 && tid < 128)
-    invert_column_block([&](int r, int c) { return diag(0, s / 2, r * kCB + c); }, X, n, need_lu);
-  grid.sync();
-  auto XB = [&](int i, int j) { return X + (size_t)(kCB * i) * n + kCB * j; };
-  for (s /= 2; s >= 1; s /= 2) {
-    const int ne = (nc - s + 2 * s - 1) / (2 * s), nk = (nc + 2 * s - 1) / (2 * s);
-    for_items(2 * ne * nk * kCB, [&](int t) {
-      const int r = t % kCB, j = 2 * s * (t / kCB % nk), e = t / (kCB * nk);
-      const int i = s + 2 * s * (e % ne);
-      const bool right = i + s < nc, on = lane < kCB;
-      double v;
-      if (e < ne) {  // X(i, j)
-        v = row_times(on ? B(kBlkP, i)[r * kCB + lane] : 0.0, XB(i - s, j), n, lane, 0.0);
-        if (right)
-          v = row_times(on ? B(kBlkQ, i)[r * kCB + lane] : 0.0, XB(i + s, j), n, lane, v);
-        if (on) XB(i, j)[(size_t)r * n + lane] = v;
-      } else {  // X(j, i)
-        v = row_times(on ? XB(j, i - s)[(size_t)r * n + lane] : 0.0, B(kBlkRP, i), kCB, lane, 0.0);
-        if (right)
-          v = row_times(on ? XB(j, i + s)[(size_t)r * n + lane] : 0.0, B(kBlkRQ, i), kCB, lane, v);
-        if (on) XB(j, i)[(size_t)r * n + lane] = v;
-      }
-    });
-    grid.sync();
-    for_items(ne * ne * kCB, [&](int t) {
-      const int r = t % kCB, i = s + 2 * s * (t / kCB % ne), k = s + 2 * s * (t / (kCB * ne));
-      const bool right = k + s < nc, on = lane < kCB;
-      double v = i == k && on ? B(kBlkZ, i)[r * kCB + lane] : 0.0;
-      v = row_times(on ? XB(i, k - s)[(size_t)r * n + lane] : 0.0, B(kBlkRP, k), kCB, lane, v);
-      if (right)
-        v = row_times(on ? XB(i, k + s)[(size_t)r * n + lane] : 0.0, B(kBlkRQ, k), kCB, lane, v);
-      if (on) XB(i, k)[(size_t)r * n + lane] = v;
-    });
-    grid.sync();
+  for (s /= 2; s >= 1; s /= 2) {  // and back
+    run_phase(2);
+    run_phase(3);
   }
   // y = X b for a vector of signs, then the componentwise backward error of A y = b
   double* y = blk + (size_t)kBlkKinds * nc * kCBB;
