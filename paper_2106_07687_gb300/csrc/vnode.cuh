@@ -237,6 +237,161 @@ __device__ __forceinline__ void warp_pass_tile(const NodeLevel<T>& L, const OpTa
   __syncwarp();  // the tile's shared memory is reused
 }
 
+// ---- one warp, 4 x 2 nodes: four lanes per node -----------------------------------------
+// On a level with few tiles a warp's chain is all that a phase lasts, and in
+// FP64 every instruction of a warp takes 64 cycles of its scheduler.  Here lanes
+// 4 m + s, s = 0..3, share node m: each takes every fourth neighbour and every
+// fourth pressure of the stabilisation, then the columns of the inverse that
+// belong to node s of the cell; two butterfly sums join them.  A lane issues
+// about 60 instead of 180 multiply-adds, all lanes together a third more.
+constexpr int kSX = 4, kSY = 2, kSSX = kSX + 4, kSSY = kSY + 4;
+
+template <typename T>
+__device__ __forceinline__ T quad_sum(T v) {
+  v += __shfl_xor_sync(0xffffffffu, v, 1);
+  return v + __shfl_xor_sync(0xffffffffu, v, 2);
+}
+
+// Stage the 8 x 6 nodes around tile (i0, j0).
+template <typename T>
+__device__ __forceinline__ void stage_split_tile(const NodeLevel<T>& L, const T* x, int i0, int j0,
+                                                 int lane, WarpTile<T>& S) {
+  T u[2], v[2], p[2];
+  int pt[2];
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int e = lane + 32 * r, i = i0 - 2 + e % kSSX, j = j0 - 2 + e / kSSX;
+    const bool in = e < kSSX * kSSY && i >= 0 && j >= 0 && i <= L.nx && j <= L.ny;
+    const int n = in ? j * L.nnx + i : 0;
+    pt[r] = in ? (int)__ldg(L.pat + n) : (kPatVDir | kPatPFix);
+    u[r] = __ldcg(x + n);
+    v[r] = __ldcg(x + L.nn + n);
+    p[r] = __ldcg(x + 2 * L.nn + n);
+  }
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int e = lane + 32 * r, li = e % kSSX, lj = e / kSSX;
+    if (e >= kSSX * kSSY) break;
+    S.w[0][lj][li] = (pt[r] & kPatVDir) ? T(0) : u[r];
+    S.w[1][lj][li] = (pt[r] & kPatVDir) ? T(0) : v[r];
+    S.w[2][lj][li] = (pt[r] & kPatPFix) ? T(0) : p[r];
+  }
+}
+
+// this lane's coefficients: neighbours s, s + 4 and (s = 0) 8
+template <typename T>
+__device__ __forceinline__ void load_split_blocks(const NodeLevel<T>& L, int n, int s, T c[12]) {
+  using V = typename Vec16<T>::type;
+  constexpr int NV = 4 / kVec16<T>;
+  const V* p = reinterpret_cast<const V*>(L.cf);
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    const int e = s + 4 * r < 9 ? s + 4 * r : 8;
+#pragma unroll
+    for (int h = 0; h < NV; ++h)
+      vec_unpack(__ldg(p + (size_t)(e * NV + h) * L.nn + n), c + 4 * r + h * kVec16<T>);
+  }
+}
+
+template <typename T>
+__device__ __forceinline__ void node_rows_split(const NodeLevel<T>& L, const OpTable<T>& tab,
+                                                const WarpTile<T>& S, const T c[12], int li, int lj,
+                                                int pt, int cls, int s, T& ru, T& rv, T& rp) {
+  T u0 = 0, v0 = 0, u1 = 0, v1 = 0, d0 = 0, ls = 0;
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    const int e = s + 4 * r;
+    if (e >= 9) break;
+    const int dj = e / 3, di = e - 3 * dj;
+    const T* g = tab.gd[pt & 15][e];
+    const T u = S.w[0][lj - 1 + dj][li - 1 + di], v = S.w[1][lj - 1 + dj][li - 1 + di],
+            p = S.w[2][lj - 1 + dj][li - 1 + di];
+    u0 += c[4 * r] * u + c[4 * r + 1] * v;
+    v0 += c[4 * r + 2] * u + c[4 * r + 3] * v;
+    u1 += g[0] * p;
+    v1 += g[1] * p;
+    d0 += g[2] * u + g[3] * v;
+  }
+  const T* l = tab.lps[(pt >> kPatPatch) & 15][cls];
+#pragma unroll
+  for (int r = 0; r < 7; ++r) {
+    const int e = s + 4 * r;
+    if (e >= 25) break;
+    const int dj = e / 5, di = e - 5 * dj;
+    ls += l[e] * S.w[2][lj - 2 + dj][li - 2 + di];
+  }
+  ru = quad_sum(u0 + L.h * u1);
+  rv = quad_sum(v0 + L.h * v1);
+  rp = quad_sum(L.h * d0 + L.h2 * ls);
+}
+
+// One colour pass on the warp's 2 x 1 colour cells (bx, by).
+template <typename T>
+__device__ __forceinline__ void split_pass_tile(const NodeLevel<T>& L, const OpTable<T>& tab,
+                                                int colour, const T* b, const T* xin, const T* inv,
+                                                int pitch, int nslots, T omega, T* xout, int bx,
+                                                int by, int lane, WarpTile<T>& S) {
+  const int cx = colour & 1, cy = colour >> 1;
+  const int i0 = kSX * bx - cx, j0 = kSY * by - cy;
+  const int q = lane >> 4, a = (lane >> 2) & 3, s = lane & 3;
+  const int li = 2 * q + (a & 1), lj = a >> 1, i = i0 + li, j = j0 + lj;
+  const bool node_ok = i >= 0 && j >= 0 && i <= L.nx && j <= L.ny;
+  const int n = node_ok ? j * L.nnx + i : 0;
+  const int slot = node_ok ? by * pitch + 2 * bx + q : 0;
+  T c[12], iv[3][3];
+  load_split_blocks<T>(L, n, s, c);
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      iv[r][k] = __ldg(inv + vanka_inv_index<T>(nslots, colour, slot, a, r * 12 + 4 * k + s));
+  const int pt = node_ok ? (int)__ldg(L.pat + n) : 0;
+  const T xu = __ldcg(xin + n), xv = __ldcg(xin + L.nn + n), xp = __ldcg(xin + 2 * L.nn + n);
+  const T bu = __ldcg(b + n), bv = __ldcg(b + L.nn + n), bp = __ldcg(b + 2 * L.nn + n);
+  stage_split_tile<T>(L, xin, i0, j0, lane, S);
+  __syncwarp();
+  const bool cell_ok = node_ok && ((pt >> ((1 - (a & 1)) + 2 * (1 - (a >> 1)))) & 1);
+  T ru, rv, rp;
+  node_rows_split<T>(L, tab, S, c, li + 2, lj + 2, pt, (i & 1) + 2 * (j & 1), s, ru, rv, rp);
+  const T du = bu - ((pt & kPatVDir) ? xu : ru), dv = bv - ((pt & kPatVDir) ? xv : rv),
+          dp = bp - ((pt & kPatPFix) ? xp : rp);
+  const int src = (lane & 16) + 4 * s;  // node s of the cell
+  const T d0 = __shfl_sync(0xffffffffu, du, src), d1 = __shfl_sync(0xffffffffu, dv, src),
+          d2 = __shfl_sync(0xffffffffu, dp, src);
+  T acc[3];
+#pragma unroll
+  for (int r = 0; r < 3; ++r) acc[r] = quad_sum(iv[r][0] * d0 + iv[r][1] * d1 + iv[r][2] * d2);
+  if (node_ok && s < 3) {  // lane s writes component s
+    const T x = s == 0 ? xu : (s == 1 ? xv : xp), y = s == 0 ? acc[0] : (s == 1 ? acc[1] : acc[2]);
+    xout[s * L.nn + n] = cell_ok ? x + omega * y : x;
+  }
+  __syncwarp();
+}
+
+// d = b - A'(vbar) x, zero on constrained unknowns, on the warp's 4 x 2 nodes.
+template <typename T>
+__device__ __forceinline__ void split_defect_tile(const NodeLevel<T>& L, const OpTable<T>& tab,
+                                                  const T* b, const T* x, T* d, int bx, int by,
+                                                  int lane, WarpTile<T>& S) {
+  const int i0 = kSX * bx, j0 = kSY * by, m = lane >> 2, s = lane & 3;
+  const int li = m % kSX, lj = m / kSX, i = i0 + li, j = j0 + lj;
+  const bool ok = i <= L.nx && j <= L.ny;
+  const int n = ok ? j * L.nnx + i : 0;
+  T c[12];
+  load_split_blocks<T>(L, n, s, c);
+  const int pt = ok ? (int)__ldg(L.pat + n) : 0;
+  const T bb = __ldcg(b + (s < 3 ? s : 0) * L.nn + n);
+  stage_split_tile<T>(L, x, i0, j0, lane, S);
+  __syncwarp();
+  T ru, rv, rp;
+  node_rows_split<T>(L, tab, S, c, li + 2, lj + 2, pt, (i & 1) + 2 * (j & 1), s, ru, rv, rp);
+  if (ok && s < 3) {
+    const bool cons = pt & (s < 2 ? kPatVDir : kPatPFix);
+    d[s * L.nn + n] = cons ? T(0) : bb - (s == 0 ? ru : (s == 1 ? rv : rp));
+  }
+  __syncwarp();
+}
+
 // d = b - A'(vbar) x, zero on constrained unknowns, on the warp's 8 x 4 nodes.
 template <typename T>
 __device__ __forceinline__ void warp_defect_tile(const NodeLevel<T>& L, const OpTable<T>& tab,
