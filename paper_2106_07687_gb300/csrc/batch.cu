@@ -123,17 +123,14 @@ class Batch final : public BatchBase {
       for (int b = 0; b < cdiv(hl_[p][L_[p] + dl].g.nn, kNB); ++b) it.push_back(make_int2(p, b));
     return make_table(it);
   }
-  Table tile_table(int k, int shape) {
-    int tcx = 16, tcy = 4;
-    pass_shape_dims(shape, &tcx, &tcy);
+  // (problem, i), i < count(grid of level k), of the problems with the level
+  template <class F>
+  Work level_items(int k, F count) {
     std::vector<int2> it;
     for (int p = 0; p < n_; ++p)
-      if (L_[p] >= k) {
-        const Grid& g = hl_[p][k].g;
-        const int nt = cdiv(g.nx / 2 + 1, tcx) * cdiv(g.ny / 2 + 1, tcy);
-        for (int b = 0; b < nt; ++b) it.push_back(make_int2(p, b));
-      }
-    return make_table(it);
+      if (L_[p] >= k)
+        for (int b = 0; b < count(p); ++b) it.push_back(make_int2(p, b));
+    return make_table(it).w();
   }
   Table setup_table(int k) {
     std::vector<int2> it;
@@ -160,7 +157,6 @@ class Batch final : public BatchBase {
   }
 
   void vcycle_all(const T* b, T* x, const int* act);
-  void smooth(int k, const T* b, T* x, int sweeps, const int* act);
   void fgmres_iteration(int j);
   int linearize_masked(const int* act, bool coarse, bool precond);
   int solve(const int* nact_d, const std::vector<int>& nact, std::vector<int>& gits);
@@ -181,9 +177,11 @@ class Batch final : public BatchBase {
   std::vector<BLev<T>> hlev_;
   BView<T> v_{};
   // work lists
-  std::map<int, Table> node0_, node1_, tiles_, setup_;
+  std::map<int, Table> node0_, node1_, setup_;
   Table top_, fine_, mid_;
-  int shape_ = 0;
+  BWalk<T> walk_{};       // the cycle's records and items
+  Phase* ph_ = nullptr;   // its phases
+  int nph_ = 0;
   VecTab vt_{};
   // concatenated top-level vectors
   double *x64_ = nullptr, *xold64_ = nullptr, *f64_ = nullptr, *r64_ = nullptr;
@@ -325,7 +323,19 @@ int Batch<T>::init() {
       l.d = mem_.alloc<T>(n3);
       l.vb = mem_.alloc<T>(n2);
       l.vb64 = mem_.alloc<double>(n2);
-      if (k >= 2) l.inv = mem_.alloc<T>((size_t)4 * 144 * vanka_slots(g));
+      l.h = (T)g.h;
+      l.hs = (T)(g.h * g.h * c.alpha0 / c.nu);
+      l.mode = c.lps_mode;
+      if (k >= 2) {
+        l.inv = mem_.alloc<T>((size_t)4 * 144 * vanka_slots(g));
+        l.cf = mem_.alloc<T>((size_t)36 * g.nn);
+        const std::vector<uint16_t> pat = node_patterns(hl_[p][k]);
+        uint16_t* dp = mem_.alloc<uint16_t>(pat.size());
+        if (!mem_.ok()) return fail(DNNMG_ERR_CUDA, "device allocation failed");
+        cudaMemcpyAsync(dp, pat.data(), sizeof(uint16_t) * pat.size(), cudaMemcpyHostToDevice, st_);
+        cudaStreamSynchronize(st_);
+        l.pat = dp;
+      }
     }
     BPar& pr = hpar[p];
     pr.inv_k = 1.0 / c.dt;
@@ -401,7 +411,6 @@ int Batch<T>::init() {
     node0_[k] = node_table(k, 0);
     node1_[k] = node_table(k, 1);
     if (k >= 2) {
-      tiles_[k] = tile_table(k, shape_);
       setup_[k] = setup_table(k);
     }
   }
@@ -483,7 +492,51 @@ int Batch<T>::init() {
   cudaMemcpyAsync(ds64, hs64.data(), sizeof(Sten<double>) * hs64.size(), cudaMemcpyHostToDevice, st_);
   cudaMemcpyAsync(dsx, hsx.data(), sizeof(Sten<double>) * hsx.size(), cudaMemcpyHostToDevice, st_);
   cudaMemcpyAsync(dpar, hpar.data(), sizeof(BPar) * n_, cudaMemcpyHostToDevice, st_);
-  v_ = BView<T>{dl, dsT, ds64, dsx, dpar, nL_};
+  // coefficient tables of the stabilisation forms, and the cycle's items
+  OpTable<T>* dtab = mem_.alloc<OpTable<T>>(3);
+  if (!mem_.ok()) return fail(DNNMG_ERR_CUDA, "device allocation failed");
+  {
+    std::vector<OpTable<T>> tab(3);
+    for (int mode = 0; mode < 3; ++mode) {
+      dnnmg_config one = c0_;
+      one.nu = one.alpha0 = 1.0;
+      one.lps_mode = mode;
+      fill_op_table<T>(make_sten<double>(1.0, one), tab[mode]);
+    }
+    cudaMemcpyAsync(dtab, tab.data(), sizeof(OpTable<T>) * 3, cudaMemcpyHostToDevice, st_);
+    cudaStreamSynchronize(st_);
+  }
+  v_ = BView<T>{dl, dsT, ds64, dsx, dpar, dtab, nL_};
+  walk_.lev = dl;
+  walk_.tab = dtab;
+  walk_.nprob = n_;
+  walk_.nL = nL_;
+  walk_.mode = cf[0].lps_mode;
+  for (const dnnmg_config& c : cf)
+    if (c.lps_mode != cf[0].lps_mode) walk_.mode = -1;
+  walk_.n1 = n1_;
+  walk_.Ainv = Ainv_;
+  walk_.astride = astride_;
+  for (int k = 2; k <= Lmax_; ++k) {
+    auto g = [&](int p, int l) -> const Grid& { return hl_[p][l].g; };
+    walk_.pass[k] = level_items(k, [&](int p) { return vcycle_warp_tiles(g(p, k)); });
+    walk_.defect[k] = level_items(k, [&](int p) { return vcycle_defect_tiles(g(p, k)); });
+    walk_.zero[k] = level_items(k, [&](int p) { return cdiv(4 * vanka_slots(g(p, k)), 32); });
+    walk_.restr[k] = level_items(k, [&](int p) { return cdiv(g(p, k - 1).nn, 32); });
+    walk_.prol[k] = level_items(k, [&](int p) { return cdiv(g(p, k).nn, 32); });
+  }
+  {
+    // levels count from the coarsest (1); x is zeroed beforehand when no
+    // smoothing pass starts from zero
+    std::vector<Phase> ph = vcycle_phases(Lmax_ - 1, c0_.nu1, c0_.nu2);
+    if (!ph.empty() && ph[0].type == kPhaseZeroTop) ph.erase(ph.begin());
+    for (Phase& q : ph) q.level += 1;
+    nph_ = (int)ph.size();
+    ph_ = mem_.alloc<Phase>(ph.size());
+    if (!mem_.ok()) return fail(DNNMG_ERR_CUDA, "device allocation failed");
+    cudaMemcpyAsync(ph_, ph.data(), sizeof(Phase) * ph.size(), cudaMemcpyHostToDevice, st_);
+    cudaStreamSynchronize(st_);
+  }
   // ---- initial states (impulsive start) and zeroed Krylov storage
   cudaMemsetAsync(x64_, 0, sizeof(double) * N_, st_);
   cudaMemsetAsync(V_, 0, sizeof(T) * (size_t)(m_ + 1) * N_, st_);
@@ -508,40 +561,14 @@ int Batch<T>::init() {
   return check("batch setup");
 }
 
-template <typename T>
-void Batch<T>::smooth(int k, const T* b, T* x, int sweeps, const int* act) {
-  int cur = 0;
-  for (int s = 0; s < sweeps; ++s)
-    for (int colour = 0; colour < 4; ++colour) {
-      const int p = prof_.begin(DNNMG_STAGE_VANKA_PASS, k, st_);
-      bk_pass<T>(v_, k, colour, cur, 1 - cur, b, x, (T)c0_.omega, tiles_[k].w(), shape_, act, st_);
-      prof_.end(p, st_);
-      cur ^= 1;
-    }
-}
-
-// One V(nu1, nu2) cycle of every active problem on its own finest level with
-// x = 0 on entry (b, x in the top-level layout).
+// One V(nu1, nu2) cycle of every active problem on its own finest level (b, x
+// in the top-level layout); x is read only without pre-smoothing, and is then
+// zero on entry.
 template <typename T>
 void Batch<T>::vcycle_all(const T* b, T* x, const int* act) {
-  for (int k = Lmax_; k >= 2; --k) {
-    smooth(k, b, x, c0_.nu1, act);
-    int p = prof_.begin(DNNMG_STAGE_DEFECT, k, st_);
-    bk_defect<T>(v_, k, 0, b, x, node0_[k].w(), act, st_);
-    prof_.end(p, st_);
-    p = prof_.begin(DNNMG_STAGE_TRANSFER, k, st_);
-    bk_restrict<T>(v_, k, node1_[k - 1].w(), act, st_);
-    prof_.end(p, st_);
-  }
-  int p = prof_.begin(DNNMG_STAGE_COARSE_SOLVE, 1, st_);
-  bk_coarse_solve<T>(v_, n_, n1_, Ainv_, astride_, b, x, act, st_);
+  const int p = prof_.begin(DNNMG_STAGE_VCYCLE, Lmax_, st_);
+  bk_vcycle<T>(walk_, ph_, nph_, b, x, (T)c0_.omega, act, st_);
   prof_.end(p, st_);
-  for (int k = 2; k <= Lmax_; ++k) {
-    p = prof_.begin(DNNMG_STAGE_TRANSFER, k, st_);
-    bk_prolong<T>(v_, k, 0, x, node0_[k].w(), act, st_);
-    prof_.end(p, st_);
-    smooth(k, b, x, c0_.nu2, act);
-  }
 }
 
 // Linearise the active problems at their current state: the FGMRES matvec
@@ -558,6 +585,7 @@ int Batch<T>::linearize_masked(const int* act, bool coarse, bool precond) {
     bk_cast_vb<T>(v_, k, node0_[k].w(), act, st_);
     if (k >= 2) {
       const int p = prof_.begin(DNNMG_STAGE_VANKA_SETUP, k, st_);
+      bk_assemble<T>(v_, k, node0_[k].w(), act, st_);
       bk_setup<T>(v_, k, status_, setup_[k].w(), act, st_);
       prof_.end(p, st_);
     }
@@ -605,7 +633,7 @@ void Batch<T>::fgmres_iteration(int j) {
   T* zj = Z_ + (size_t)j * N_;
   T* w = V_ + (size_t)(j + 1) * N_;
   const int hs = 2 * m_ + 4;
-  launch_fill<T>(zj, T(0), N_, st_);
+  if (c0_.nu1 == 0) launch_fill<T>(zj, T(0), N_, st_);
   vcycle_all(vj, zj, gact_);
   int p = prof_.begin(DNNMG_STAGE_APPLY, Lmax_, st_);
   bk_apply<T>(v_, zj, vbJ_, w, top_.w(), gact_, st_);

@@ -22,6 +22,7 @@
 
 #include "../../include/dnnmg.h"
 #include "common.cuh"
+#include "vcycle.h"
 
 namespace dnnmg {
 
@@ -35,9 +36,12 @@ struct BLev {
   Grid g;
   T *x, *x2, *b, *d, *vb, *inv;  // multigrid buffers (x, b unused on the top level)
   double* vb64;                  // FP64 linearisation point (velocity)
+  T* cf;                         // assembled velocity blocks (vnode.cuh)
+  const uint16_t* pat;           // node patterns
+  T h, hs;                       // mesh width; h^2 alpha0 / nu, the stabilisation's scale
   long long off;                 // offset of the problem in the top-level vectors
   int top;                       // 1 on the problem's finest solved level
-  int pad;
+  int mode;                      // stabilisation form (index of the coefficient table)
 };
 
 // Per-problem scalars read by the batched kernels.
@@ -60,6 +64,7 @@ struct BView {
   const Sten<double>* s64;   // FP64 constants (residual, coarse assembly)
   const Sten<double>* sx;    // explicit theta-scheme bracket (FP64)
   const BPar* par;           // [problem]
+  const OpTable<T>* tab;     // per stabilisation form, for h = nu = alpha0 = 1
   int nL;
 };
 
@@ -68,6 +73,25 @@ struct Work {
   const int2* d = nullptr;
   int n = 0;
 };
+
+// Items of the batched cycle's phases on every level: (problem, warp tile) of
+// the passes and defects, (problem, chunk of 32) of the first pass from zero
+// (four items per slot), the restriction from the level (nodes of the level
+// below) and the prolongation to it.
+constexpr int kBLevels = 11;
+template <typename T>
+struct BWalk {
+  const BLev<T>* lev;
+  const OpTable<T>* tab;
+  int nprob, nL, mode, n1;  // mode: every problem's stabilisation form, -1 if they differ
+  const double* Ainv;       // coarse inverses, `astride` doubles apart, n1 unknowns
+  long long astride;
+  Work pass[kBLevels], defect[kBLevels], zero[kBLevels], restr[kBLevels], prol[kBLevels];
+};
+// one cycle over nph phases (build_batch_phases) of every active problem
+template <typename T>
+void bk_vcycle(const BWalk<T>& W, const Phase* ph, int nph, const T* topb, T* topx, T omega,
+               const int* act, cudaStream_t st);
 
 // Blocks of the concatenated top-level vectors: the problem of every block
 // and every problem's first block and block count.
@@ -82,20 +106,6 @@ struct VecTab {
 // a problem with act[problem] == 0 returns at once.  dl selects the level of
 // the node kernels that run on a problem's own levels: 0 = finest solved
 // level L, 1 = level L + 1 (the DNN-MG fine level).
-template <typename T>
-void bk_pass(const BView<T>& v, int k, int colour, int in, int out, const T* topb, T* topx,
-             T omega, Work w, int shape, const int* act, cudaStream_t st);
-template <typename T>
-void bk_defect(const BView<T>& v, int k, int in, const T* topb, T* topx, Work w, const int* act,
-               cudaStream_t st);
-template <typename T>
-void bk_restrict(const BView<T>& v, int k, Work w, const int* act, cudaStream_t st);
-template <typename T>
-void bk_prolong(const BView<T>& v, int k, int in, T* topx, Work w, const int* act,
-                cudaStream_t st);
-template <typename T>
-void bk_coarse_solve(const BView<T>& v, int nprob, int n1, const double* Ainv, long long astride,
-                     const T* topb, T* topx, const int* act, cudaStream_t st);
 template <typename T>
 void bk_apply(const BView<T>& v, const T* w, const T* vbJ, T* y, Work wk, const int* act,
               cudaStream_t st);
@@ -117,6 +127,9 @@ template <typename T>
 void bk_inject_vb(const BView<T>& v, int k, Work wk, const int* act, cudaStream_t st);
 template <typename T>
 void bk_cast_vb(const BView<T>& v, int k, Work wk, const int* act, cudaStream_t st);
+// velocity blocks of level k (work: node blocks), then the local inverses
+template <typename T>
+void bk_assemble(const BView<T>& v, int k, Work wk, const int* act, cudaStream_t st);
 template <typename T>
 void bk_setup(const BView<T>& v, int k, int* status, Work wk, const int* act, cudaStream_t st);
 template <typename T>
@@ -164,9 +177,6 @@ void bk_gather(const BView<T>& v, int K, int P, const int* pinst, const int* pce
 template <typename T>
 void bk_scatter(const BView<T>& v, int K, const int* cell_patch, const float* out, int c_out,
                 const double* xt, double* vcorr, Work wk, const int* act, cudaStream_t st);
-// tile shape (cells per block) of pass shape s
-void pass_shape_dims(int s, int* tcx, int* tcy);
-
 class BatchBase {
  public:
   virtual ~BatchBase() = default;

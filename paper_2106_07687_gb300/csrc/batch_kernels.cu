@@ -10,7 +10,7 @@
 #include "dnnmg_body.cuh"
 #include "kernels.h"
 #include "krylov_body.cuh"
-#include "vanka_body.cuh"
+#include "vnode.cuh"
 #include "vbody.cuh"
 
 namespace dnnmg {
@@ -32,88 +32,6 @@ __device__ __forceinline__ void load_const(S& dst, const S& src) {
 template <typename T>
 __device__ __forceinline__ const BLev<T>& lev_of(const BView<T>& v, int p, int k) {
   return v.lev[(size_t)p * v.nL + k];
-}
-
-// ---------------------------------------------------------------- V-cycle
-
-template <typename T, int TCX, int TCY>
-__global__ void __launch_bounds__(4 * TCX * TCY, pass_min_blocks<T>(4 * TCX * TCY))
-    bpass_kernel(BView<T> v, int k, int colour, int in, int out, const T* __restrict__ topb,
-                 T* __restrict__ topx, T omega, const int2* __restrict__ work,
-                 const int* __restrict__ act) {
-  const int2 w = work[blockIdx.x];
-  if (masked(act, w.x)) return;
-  __shared__ Sten<T> ss;
-  extern __shared__ __align__(16) uint8_t smraw[];
-  const BLev<T> L = lev_of(v, w.x, k);
-  load_const(ss, v.sT[(size_t)w.x * v.nL + k]);
-  T* x0 = L.top ? topx + L.off : L.x;
-  const T* b = L.top ? topb + L.off : L.b;
-  const T* xin = in ? L.x2 : x0;
-  T* xout = out ? L.x2 : x0;
-  const int nbx = cdiv(L.g.nx / 2 + 1, TCX);
-  vanka_pass_tile<T, TCX, TCY>(L.g, ss, colour, b, xin, L.vb, L.inv, omega, xout, w.y % nbx,
-                               w.y / nbx, *reinterpret_cast<PassSmem<T, TCX, TCY>*>(smraw));
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kNB)
-    bdefect_kernel(BView<T> v, int k, int in, const T* __restrict__ topb, T* __restrict__ topx,
-                   const int2* __restrict__ work, const int* __restrict__ act) {
-  const int2 w = work[blockIdx.x];
-  if (masked(act, w.x)) return;
-  __shared__ Sten<T> ss;
-  const BLev<T> L = lev_of(v, w.x, k);
-  load_const(ss, v.sT[(size_t)w.x * v.nL + k]);
-  const int n = w.y * kNB + threadIdx.x;
-  if (n >= L.g.nn) return;
-  const T* x0 = L.top ? topx + L.off : L.x;
-  const T* b = L.top ? topb + L.off : L.b;
-  defect_node<T>(L.g, ss, b, in ? L.x2 : x0, L.vb, L.d, true, n % L.g.nnx, n / L.g.nnx);
-}
-
-// work: node blocks of level k - 1 of the problems that have level k
-template <typename T>
-__global__ void __launch_bounds__(kNB)
-    brestrict_kernel(BView<T> v, int k, const int2* __restrict__ work,
-                     const int* __restrict__ act) {
-  const int2 w = work[blockIdx.x];
-  if (masked(act, w.x)) return;
-  const BLev<T> F = lev_of(v, w.x, k), C = lev_of(v, w.x, k - 1);
-  const int n = w.y * kNB + threadIdx.x;
-  if (n >= C.g.nn) return;
-  restrict_node<T, true>(F.g, C.g, F.d, C.b, 3, n % C.g.nnx, n / C.g.nnx);
-  C.x[n] = T(0);
-  C.x[C.g.nn + n] = T(0);
-  C.x[2 * C.g.nn + n] = T(0);
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kNB)
-    bprolong_kernel(BView<T> v, int k, int in, T* __restrict__ topx, const int2* __restrict__ work,
-                    const int* __restrict__ act) {
-  const int2 w = work[blockIdx.x];
-  if (masked(act, w.x)) return;
-  const BLev<T> F = lev_of(v, w.x, k), C = lev_of(v, w.x, k - 1);
-  const int n = w.y * kNB + threadIdx.x;
-  if (n >= F.g.nn) return;
-  T* x0 = F.top ? topx + F.off : F.x;
-  prolong_add_node<T>(F.g, C.g, C.x, in ? F.x2 : x0, n % F.g.nnx, n / F.g.nnx);
-}
-
-// grid (row blocks, problems); the coarsest level is level 1 for every problem
-template <typename T>
-__global__ void __launch_bounds__(32 * kSolveWarps)
-    bcoarse_solve_kernel(BView<T> v, const double* __restrict__ Ainv, long long astride,
-                         const T* __restrict__ topb, T* __restrict__ topx,
-                         const int* __restrict__ act) {
-  const int p = blockIdx.y;
-  if (masked(act, p)) return;
-  extern __shared__ double sb[];
-  const BLev<T> C = lev_of(v, p, 1);
-  const T* b = C.top ? topb + C.off : C.b;
-  T* x = C.top ? topx + C.off : C.x;
-  coarse_solve_rows<T>(C.g, Ainv + (size_t)p * astride, b, x, blockIdx.x, sb);
 }
 
 // ------------------------------------------------- top- and fine-level nodes
@@ -251,6 +169,18 @@ __global__ void __launch_bounds__(kNB)
   L.vb[L.g.nn + n] = (T)L.vb64[L.g.nn + n];
 }
 
+template <typename T>
+__global__ void __launch_bounds__(kNB)
+    bblocks_kernel(BView<T> v, int k, const int2* __restrict__ work, const int* __restrict__ act) {
+  const int2 wk = work[blockIdx.x];
+  if (masked(act, wk.x)) return;
+  __shared__ Sten<T> ss;
+  const BLev<T> L = lev_of(v, wk.x, k);
+  load_const(ss, v.sT[(size_t)wk.x * v.nL + k]);
+  const int n = wk.y * kNB + threadIdx.x;
+  if (n < L.g.nn) assemble_node<T>(L.g, ss, L.vb, L.cf, n);
+}
+
 // work: (problem, colour * slot_blocks + slot_block)
 template <typename T>
 __global__ void __launch_bounds__(kSetupThreads)
@@ -258,13 +188,10 @@ __global__ void __launch_bounds__(kSetupThreads)
                   const int* __restrict__ act) {
   const int2 wk = work[blockIdx.x];
   if (masked(act, wk.x)) return;
-  __shared__ Sten<T> ss;
   const BLev<T> L = lev_of(v, wk.x, k);
-  load_const(ss, v.sT[(size_t)wk.x * v.nL + k]);
   const int nsb = cdiv(vanka_slots(L.g), kSetupCells);
-  __shared__ SetupSmem<T> W[kSetupCells];
-  vanka_setup_cell<T>(L.g, ss, L.vb, L.inv, status + wk.x, wk.y / nsb,
-                      (wk.y % nsb) * kSetupCells + threadIdx.x / 16, W[threadIdx.x / 16]);
+  vanka_setup_cell<T>(L.g, L.pat, L.cf, v.tab[L.mode], L.h, L.hs, L.inv, status + wk.x, wk.y / nsb,
+                      (wk.y % nsb) * kSetupCells + threadIdx.x / 16);
 }
 
 template <typename T>
@@ -531,43 +458,9 @@ __global__ void __launch_bounds__(kNB)
                   n % F.g.nnx, n / F.g.nnx);
 }
 
-template <typename T, int TCX, int TCY>
-void pass_launch(const BView<T>& v, int k, int colour, int in, int out, const T* topb, T* topx,
-                 T omega, Work w, const int* act, cudaStream_t st) {
-  const size_t smem = sizeof(PassSmem<T, TCX, TCY>);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(bpass_kernel<T, TCX, TCY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
-    attr = true;
-  }
-  note_launch();
-  bpass_kernel<T, TCX, TCY><<<w.n, 4 * TCX * TCY, smem, st>>>(v, k, colour, in, out, topb, topx,
-                                                              omega, w.d, act);
-}
-
 inline int vblocks(const VecTab& vt) { return vt.nblk; }
 
 }  // namespace
-
-void pass_shape_dims(int s, int* tcx, int* tcy) {
-  switch (s) {
-    case 1: *tcx = 8, *tcy = 4; break;
-    case 2: *tcx = 8, *tcy = 8; break;
-    default: *tcx = 16, *tcy = 4; break;
-  }
-}
-
-template <typename T>
-void bk_pass(const BView<T>& v, int k, int colour, int in, int out, const T* topb, T* topx,
-             T omega, Work w, int shape, const int* act, cudaStream_t st) {
-  if (w.n <= 0) return;
-  switch (shape) {
-    case 1: pass_launch<T, 8, 4>(v, k, colour, in, out, topb, topx, omega, w, act, st); break;
-    case 2: pass_launch<T, 8, 8>(v, k, colour, in, out, topb, topx, omega, w, act, st); break;
-    default: pass_launch<T, 16, 4>(v, k, colour, in, out, topb, topx, omega, w, act, st); break;
-  }
-}
 
 #define NODE_LAUNCH(kernel, ...)                                  \
   do {                                                            \
@@ -575,31 +468,6 @@ void bk_pass(const BView<T>& v, int k, int colour, int in, int out, const T* top
     note_launch();                                                \
     kernel<<<w.n, kNB, 0, st>>>(__VA_ARGS__, w.d, act);           \
   } while (0)
-
-template <typename T>
-void bk_defect(const BView<T>& v, int k, int in, const T* topb, T* topx, Work w, const int* act,
-               cudaStream_t st) {
-  NODE_LAUNCH(bdefect_kernel<T>, v, k, in, topb, topx);
-}
-
-template <typename T>
-void bk_restrict(const BView<T>& v, int k, Work w, const int* act, cudaStream_t st) {
-  NODE_LAUNCH(brestrict_kernel<T>, v, k);
-}
-
-template <typename T>
-void bk_prolong(const BView<T>& v, int k, int in, T* topx, Work w, const int* act,
-                cudaStream_t st) {
-  NODE_LAUNCH(bprolong_kernel<T>, v, k, in, topx);
-}
-
-template <typename T>
-void bk_coarse_solve(const BView<T>& v, int nprob, int n1, const double* Ainv, long long astride,
-                     const T* topb, T* topx, const int* act, cudaStream_t st) {
-  note_launch();
-  bcoarse_solve_kernel<T><<<dim3(cdiv(n1, kSolveWarps), nprob), 32 * kSolveWarps,
-                            sizeof(double) * n1, st>>>(v, Ainv, astride, topb, topx, act);
-}
 
 template <typename T>
 void bk_apply(const BView<T>& v, const T* wv, const T* vbJ, T* y, Work w, const int* act,
@@ -644,6 +512,11 @@ void bk_inject_vb(const BView<T>& v, int k, Work w, const int* act, cudaStream_t
 template <typename T>
 void bk_cast_vb(const BView<T>& v, int k, Work w, const int* act, cudaStream_t st) {
   NODE_LAUNCH(bcast_vb_kernel<T>, v, k);
+}
+
+template <typename T>
+void bk_assemble(const BView<T>& v, int k, Work w, const int* act, cudaStream_t st) {
+  NODE_LAUNCH(bblocks_kernel<T>, v, k);
 }
 
 template <typename T>
@@ -777,14 +650,6 @@ void bk_scatter(const BView<T>& v, int K, const int* cell_patch, const float* ou
 #undef NODE_LAUNCH
 
 #define BK_INST(T)                                                                              \
-  template void bk_pass<T>(const BView<T>&, int, int, int, int, const T*, T*, T, Work, int,     \
-                           const int*, cudaStream_t);                                           \
-  template void bk_defect<T>(const BView<T>&, int, int, const T*, T*, Work, const int*,         \
-                             cudaStream_t);                                                     \
-  template void bk_restrict<T>(const BView<T>&, int, Work, const int*, cudaStream_t);           \
-  template void bk_prolong<T>(const BView<T>&, int, int, T*, Work, const int*, cudaStream_t);   \
-  template void bk_coarse_solve<T>(const BView<T>&, int, int, const double*, long long,         \
-                                   const T*, T*, const int*, cudaStream_t);                     \
   template void bk_apply<T>(const BView<T>&, const T*, const T*, T*, Work, const int*,          \
                             cudaStream_t);                                                      \
   template void bk_defect_top<T>(const BView<T>&, const T*, const T*, const T*, T*, Work,       \
@@ -798,6 +663,7 @@ void bk_scatter(const BView<T>& v, int K, const int* cell_patch, const float* ou
   template void bk_top_vb<T>(const BView<T>&, const double*, Work, const int*, cudaStream_t);   \
   template void bk_inject_vb<T>(const BView<T>&, int, Work, const int*, cudaStream_t);          \
   template void bk_cast_vb<T>(const BView<T>&, int, Work, const int*, cudaStream_t);            \
+  template void bk_assemble<T>(const BView<T>&, int, Work, const int*, cudaStream_t);          \
   template void bk_setup<T>(const BView<T>&, int, int*, Work, const int*, cudaStream_t);        \
   template void bk_coarse_factor<T>(const BView<T>&, int, int, double*, long long, long long,   \
                                     double*, long long, int*, const int*, cudaStream_t);        \

@@ -1,0 +1,194 @@
+// The V(nu1, nu2) cycle of all problems of a batch as one cooperative launch.
+//
+// The phases are those of the single problem's cycle (vcycle.cu) from the
+// largest level of the batch down: a phase of level k works on every problem
+// that has the level, over a list of (problem, tile) or (problem, chunk of 32
+// nodes) items, one warp each, with the same warp bodies (vnode.cuh).  One FP32
+// cycle of twelve channels on levels 3 to 5: 77 launches with cell-by-cell tiles
+// 1,338 us, this 713 us, near the bandwidth of the inverses and blocks on the
+// top level (265 k nodes, 80 MB per pass).
+// Where the grid cannot be resident the same kernel is launched once per phase.
+#include <algorithm>
+#include <cooperative_groups.h>
+
+#include "batch.h"
+#include "coarse_body.cuh"
+#include "vbody.cuh"
+#include "vcycle.h"
+
+namespace cg = cooperative_groups;
+
+namespace dnnmg {
+
+namespace {
+
+constexpr int kRecBytes = 96 * 1024;  // level records kept in shared memory, at most
+
+template <typename T>
+struct BWalkSmem {
+  OpTable<T> tab;
+  alignas(16) WarpTile<T> tile[walk_threads<T>() / 32];  // or the coarse right-hand side
+};
+
+template <typename T>
+__global__ void __launch_bounds__(walk_threads<T>(), 1)
+    bvcycle_kernel(const __grid_constant__ BWalk<T> W, const Phase* __restrict__ ph, int p0, int p1,
+                   const T* topb, T* topx, T omega, const int* act) {
+  constexpr int NT = walk_threads<T>(), NW = NT / 32;
+  extern __shared__ __align__(16) uint8_t dyn[];
+  BWalkSmem<T>& S = *reinterpret_cast<BWalkSmem<T>*>(dyn);
+  BLev<T>* srec = reinterpret_cast<BLev<T>*>(dyn + sizeof(BWalkSmem<T>));
+  const int nrec = W.nprob * W.nL;
+  const bool in_smem = nrec * (int)sizeof(BLev<T>) <= kRecBytes;
+  if (in_smem) copy_ints(srec, W.lev, nrec);
+  copy_ints(&S.tab, W.tab + (W.mode >= 0 ? W.mode : 0), 1);
+  __syncthreads();
+  const BLev<T>* rec = in_smem ? srec : W.lev;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int w0 = blockIdx.x + gridDim.x * w, nw = gridDim.x * NW;
+  for (int p = p0; p < p1; ++p) {
+    const Phase f{__ldg(&ph[p].type), __ldg(&ph[p].level), __ldg(&ph[p].colour), __ldg(&ph[p].in),
+                  __ldg(&ph[p].out)};
+    const int k = f.level;
+    // item t of a list: its problem's record of level k and its index there
+    auto items = [&](const Work& list, auto body) {
+      for (int t = w0; t < list.n; t += nw) {
+        const int2 it = __ldg(list.d + t);
+        if (act && !act[it.x]) continue;
+        body(rec[it.x * W.nL + k], it.x, it.y);
+      }
+    };
+    auto table = [&](const BLev<T>& L) -> const OpTable<T>& {
+      return W.mode >= 0 ? S.tab : W.tab[L.mode];
+    };
+    auto node_level = [&](const BLev<T>& L) {
+      return NodeLevel<T>{L.g.nx, L.g.ny, L.g.nnx, L.g.nn, L.pat, L.cf, L.h, L.hs};
+    };
+    switch (f.type) {
+      case kPhasePass:
+        items(W.pass[k], [&](const BLev<T>& L, int, int t) {
+          T* x0 = L.top ? topx + L.off : L.x;
+          const int nbx = cdiv(L.g.nx / 2 + 1, kWX / 2);
+          warp_pass_tile<T>(node_level(L), table(L), f.colour, L.top ? topb + L.off : L.b,
+                            f.in ? L.x2 : x0, L.inv, vanka_pitch(L.g), vanka_slots(L.g), omega,
+                            f.out ? L.x2 : x0, t % nbx, t / nbx, lane, S.tile[w]);
+        });
+        break;
+      case kPhasePassZero:
+        items(W.zero[k], [&](const BLev<T>& L, int, int c) {
+          const int e = (c << 5) + lane;
+          vanka_pass_zero_node<T>(L.g, f.colour, L.top ? topb + L.off : L.b, L.inv, omega,
+                                  f.out ? L.x2 : (L.top ? topx + L.off : L.x), e,
+                                  e < 4 * vanka_slots(L.g));
+        });
+        break;
+      case kPhaseDefect:
+        items(W.defect[k], [&](const BLev<T>& L, int, int t) {
+          const int nbx = cdiv(L.g.nnx, kWX);
+          warp_defect_tile<T>(node_level(L), table(L), L.top ? topb + L.off : L.b,
+                              f.in ? L.x2 : (L.top ? topx + L.off : L.x), L.d, t % nbx, t / nbx,
+                              lane, S.tile[w]);
+        });
+        break;
+      case kPhaseRestrict:
+        items(W.restr[k], [&](const BLev<T>& F, int prob, int c) {
+          const BLev<T>& C = rec[prob * W.nL + k - 1];
+          const int n = (c << 5) + lane;
+          if (n >= C.g.nn) return;
+          restrict_node<T, true>(F.g, C.g, F.d, C.b, 3, n % C.g.nnx, n / C.g.nnx);
+          if (f.colour == 1)
+            for (int q = 0; q < 3; ++q) C.x[q * C.g.nn + n] = T(0);
+        });
+        break;
+      case kPhaseProlong:
+        items(W.prol[k], [&](const BLev<T>& F, int prob, int c) {
+          const BLev<T>& C = rec[prob * W.nL + k - 1];
+          const int n = (c << 5) + lane;
+          if (n >= F.g.nn) return;
+          prolong_add_node<T>(F.g, C.g, C.x, f.in ? F.x2 : (F.top ? topx + F.off : F.x),
+                              n % F.g.nnx, n / F.g.nnx);
+        });
+        break;
+      case kPhaseCoarse: {
+        // the blocks share the problems out, and a problem's blocks its rows
+        double* sb = reinterpret_cast<double*>(S.tile);
+        const int per = max(1, (int)gridDim.x / W.nprob);  // blocks per problem
+        for (int prob = (int)blockIdx.x / per; prob < W.nprob;
+             prob += max(1, (int)gridDim.x / per)) {
+          if (act && !act[prob]) continue;  // the same for the whole block
+          const BLev<T>& L = rec[prob * W.nL + k];
+          const T* b = L.top ? topb + L.off : L.b;
+          T* x = L.top ? topx + L.off : L.x;
+          const int nd = 3 * L.g.nn;
+          __syncthreads();
+          for (int q = threadIdx.x; q < nd; q += NT) sb[q] = (double)__ldcg(b + band_to_level(L.g, q));
+          __syncthreads();
+          for (int r = (int)blockIdx.x % per + per * w; r < nd; r += per * NW) {
+            const double* row = W.Ainv + (size_t)prob * W.astride + (size_t)r * nd;
+            double acc[4] = {0.0, 0.0, 0.0, 0.0};
+            for (int c0 = lane; c0 < nd; c0 += 16 * 32) {
+              double rv[16];
+#pragma unroll
+              for (int u = 0; u < 16; ++u) rv[u] = c0 + 32 * u < nd ? row[c0 + 32 * u] : 0.0;
+#pragma unroll
+              for (int u = 0; u < 16; ++u)
+                if (c0 + 32 * u < nd) acc[u & 3] += rv[u] * sb[c0 + 32 * u];
+            }
+            double a = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+            if (lane == 0) x[band_to_level(L.g, r)] = (T)a;
+          }
+          __syncthreads();
+        }
+        break;
+      }
+      default: break;
+    }
+    if (p + 1 < p1) cg::this_grid().sync();
+  }
+}
+
+template <typename T>
+size_t walk_bytes(int nprob, int nL, int n1) {
+  const size_t rec = (size_t)nprob * nL * sizeof(BLev<T>);
+  const size_t head = std::max(sizeof(BWalkSmem<T>),
+                               offsetof(BWalkSmem<T>, tile) + sizeof(double) * n1);
+  return std::max(head, sizeof(BWalkSmem<T>)) + (rec <= (size_t)kRecBytes ? rec : 0);
+}
+
+}  // namespace
+
+template <typename T>
+void bk_vcycle(const BWalk<T>& W, const Phase* ph, int nph, const T* topb, T* topx, T omega,
+               const int* act, cudaStream_t st) {
+  const size_t smem = walk_bytes<T>(W.nprob, W.nL, W.n1);
+  int dev = 0, sms = 0, per = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaFuncSetAttribute(bvcycle_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, bvcycle_kernel<T>, walk_threads<T>(),
+                                                    smem) != cudaSuccess)
+    per = 0;
+  if (per > 0) {
+    BWalk<T> w = W;
+    int p0 = 0;
+    void* args[] = {(void*)&w,    (void*)&ph,   (void*)&p0,    (void*)&nph,
+                    (void*)&topb, (void*)&topx, (void*)&omega, (void*)&act};
+    note_launch();
+    if (cudaLaunchCooperativeKernel((void*)bvcycle_kernel<T>, dim3(sms), dim3(walk_threads<T>()),
+                                    args, smem, st) == cudaSuccess)
+      return;
+    cudaGetLastError();
+  }
+  for (int p = 0; p < nph; ++p) {
+    note_launch();
+    bvcycle_kernel<T><<<sms, walk_threads<T>(), smem, st>>>(W, ph, p, p + 1, topb, topx, omega, act);
+  }
+}
+
+template void bk_vcycle<float>(const BWalk<float>&, const Phase*, int, const float*, float*, float,
+                               const int*, cudaStream_t);
+template void bk_vcycle<double>(const BWalk<double>&, const Phase*, int, const double*, double*,
+                                double, const int*, cudaStream_t);
+
+}  // namespace dnnmg

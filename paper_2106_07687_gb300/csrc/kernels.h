@@ -94,10 +94,13 @@ void launch_restrict_full64(const Grid& fine, const Grid& coarse, const double* 
 
 // Vanka (vanka.cu) -----------------------------------------------------------
 // inverse of the 12x12 restriction of A'(vbar) to every fluid cell, stored by
-// colour and slot as vanka_inv_index says
+// colour and slot as vanka_inv_index says, from the level's node patterns,
+// assembled blocks and the coefficient table (vnode.cuh)
 template <typename T>
-void launch_vanka_setup(const Grid& g, const Sten<T>& s, const T* vb, T* inv, int* status,
-                        cudaStream_t st);
+struct OpTable;
+template <typename T>
+void launch_vanka_setup(const Grid& g, const uint16_t* pat, const T* cf, const OpTable<T>* tab,
+                        T* inv, int* status, cudaStream_t st);
 // one colour pass: xout = xin + omega A_c^{-1} (b - A xin)_c on the colour's cells;
 // `shape` picks the tile of colour cells a block owns: 0 = 16x4, 1 = 8x4, 2 = 8x8
 constexpr int kPassShapes = 3;

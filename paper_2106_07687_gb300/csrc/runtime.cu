@@ -44,8 +44,19 @@ class Solver final : public SolverBase {
       l.d = c_->mem.alloc<T>(n3);
       l.vb = c_->mem.alloc<T>(n2);
       l.vb64 = c_->mem.alloc<double>(n2);
-      if (k > 0) l.inv = c_->mem.alloc<T>((size_t)4 * 144 * vanka_slots(l.g));
+      if (k > 0) {
+        l.inv = c_->mem.alloc<T>((size_t)4 * 144 * vanka_slots(l.g));
+        const std::vector<uint16_t> pat = node_patterns(c_->lv[l.level]);
+        l.cf = c_->mem.alloc<T>(36 * (size_t)l.g.nn);
+        l.pat = c_->mem.alloc<uint16_t>(pat.size());
+        if (!c_->mem.ok()) return c_->fail(DNNMG_ERR_CUDA, "device allocation failed");
+        cudaMemcpyAsync(l.pat, pat.data(), sizeof(uint16_t) * pat.size(), cudaMemcpyHostToDevice,
+                        st_);
+        cudaStreamSynchronize(st_);
+      }
     }
+    dasm_ = c_->mem.alloc<AsmLevel<T>>(K_ + 1);
+    dtab_ = c_->mem.alloc<OpTable<T>>(1);
     // streaming colour passes (FP32): a tensor map of every level's inverses
     if constexpr (sizeof(T) == 4) {
       for (int k = 1; k <= K_; ++k)
@@ -88,25 +99,15 @@ class Solver final : public SolverBase {
     skip_ = c_->mem.alloc<int>(1);
     target_dev_ = c_->mem.alloc<double>(1);
     if (!c_->mem.ok()) return c_->fail(DNNMG_ERR_CUDA, "device allocation failed");
+    upload_operator();
     // persistent sub-cycles: level table and one phase list per possible top level
     if (cfg.persistent_vcycle != 0) {
       std::vector<VLevel<T>> hv(K_ + 1);
       for (int k = 0; k <= K_; ++k) {
-        if (k > 0) {
-          const std::vector<uint16_t> pat = node_patterns(c_->lv[lv_[k].level]);
-          lv_[k].cf = c_->mem.alloc<T>(36 * (size_t)lv_[k].g.nn);
-          lv_[k].pat = c_->mem.alloc<uint16_t>(pat.size());
-          if (!c_->mem.ok()) return c_->fail(DNNMG_ERR_CUDA, "device allocation failed");
-          cudaMemcpyAsync(lv_[k].pat, pat.data(), sizeof(uint16_t) * pat.size(),
-                          cudaMemcpyHostToDevice, st_);
-          cudaStreamSynchronize(st_);
-        }
         hv[k] = VLevel<T>{lv_[k].g, lv_[k].x, lv_[k].x2, lv_[k].b, lv_[k].d, lv_[k].inv,
                           lv_[k].cf, lv_[k].pat};
       }
       dlv_ = c_->mem.alloc<VLevel<T>>(K_ + 1);
-      dasm_ = c_->mem.alloc<AsmLevel<T>>(K_ + 1);
-      dtab_ = c_->mem.alloc<OpTable<T>>(1);
       std::vector<Phase> all;
       for (int k = 0; k <= K_; ++k) {
         const std::vector<Phase> p = vcycle_phases(k, cfg.nu1, cfg.nu2);
@@ -119,7 +120,6 @@ class Solver final : public SolverBase {
       cudaMemcpyAsync(dlv_, hv.data(), sizeof(VLevel<T>) * hv.size(), cudaMemcpyHostToDevice, st_);
       cudaMemcpyAsync(dph_, all.data(), sizeof(Phase) * all.size(), cudaMemcpyHostToDevice, st_);
       cudaStreamSynchronize(st_);
-      upload_operator();
       coarse_nd_ = 3 * lv_[0].g.nn;
       bool fits = true;
       for (int k = 0; k <= K_; ++k) fits = fits && vcycle_fits(ph_n_[k], k + 1);
@@ -134,11 +134,11 @@ class Solver final : public SolverBase {
       cudaGetDevice(&dev);
       cudaDeviceGetAttribute(&sms_, cudaDevAttrMultiProcessorCount, dev);
     }
-    // side streams and events of the concurrent Vanka setups (levels 1..K-1)
-    if (K_ > 1) {
+    // side streams and events of the concurrent Vanka setups (levels 1..K)
+    if (K_ > 0) {
       if (cudaEventCreateWithFlags(&fork_ev_, cudaEventDisableTiming) != cudaSuccess)
         return c_->fail(DNNMG_ERR_CUDA, "event creation failed");
-      for (int k = 1; k < K_; ++k) {
+      for (int k = 1; k <= K_; ++k) {
         cudaStream_t s = nullptr;
         cudaEvent_t e = nullptr;
         if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess ||
@@ -165,34 +165,37 @@ class Solver final : public SolverBase {
     // every level's point (injection down the hierarchy, FP64 and T copies)
     // and the matvec's, in one launch
     launch_linearize_levels<T>(lin_, x64, vbJ_, report || !tuned_ ? status_ : nullptr, st_);
-    // the levels' setups are independent and each leaves most of the GPU
-    // idle: levels below the top run on side streams beside it
-    const int p = c_->prof.begin(DNNMG_STAGE_VANKA_SETUP, lv_[K_].level, st_);
+    // every level's velocity blocks in one launch, then the levels' setups,
+    // which are independent and leave much of the GPU idle on the small levels:
+    // those below the top run on side streams beside it, or all of them beside
+    // the coarse factorisation (dependent phases of few warps), unless the
+    // stages are being timed
+    const bool factor = coarse || !coarse_done_;
+    int p = c_->prof.begin(DNNMG_STAGE_VANKA_SETUP, lv_[K_].level, st_);
+    launch_assemble_blocks<T>(dasm_, K_, asm_nodes_[K_], st_);
     const bool fork = !side_.empty() && !capturing();
-    if (fork) {
-      cudaEventRecord(fork_ev_, st_);
-      for (cudaStream_t s : side_) cudaStreamWaitEvent(s, fork_ev_, 0);
-    }
-    // the first side stream is joined below, after level 1's setup
-    if (const int na = assembled_levels())
-      launch_assemble_blocks<T>(dasm_, na, asm_nodes_[na], fork ? side_[0] : st_);
+    const bool beside = fork && factor && !c_->prof.on();
+    if (fork) cudaEventRecord(fork_ev_, st_);
+    if (beside) factor_coarse();
     for (int k = K_; k > 0; --k) {
       cudaStream_t s = st_;
-      if (fork && k < K_) s = side_[k - 1];
-      launch_vanka_setup<T>(lv_[k].g, lv_[k].s, lv_[k].vb, lv_[k].inv, status_, s);
+      if (fork && (k < K_ || beside)) {
+        s = side_[k - 1];
+        cudaStreamWaitEvent(s, fork_ev_, 0);
+      }
+      launch_vanka_setup<T>(lv_[k].g, lv_[k].pat, lv_[k].cf, dtab_, lv_[k].inv, status_, s);
       if (s != st_) {
         cudaEventRecord(side_ev_[k - 1], s);
         cudaStreamWaitEvent(st_, side_ev_[k - 1], 0);
       }
     }
     c_->prof.end(p, st_);
-    if (coarse || !coarse_done_) {
-      const int p = c_->prof.begin(DNNMG_STAGE_COARSE_FACTOR, lv_[0].level, st_);
-      launch_coarse_factor(lv_[0].g, lv_[0].s64, lv_[0].vb64, coarse_work_, ainv_, status_, st_,
-                           part_solid_ ? &pieces_ : nullptr);
+    if (factor && !beside) {
+      p = c_->prof.begin(DNNMG_STAGE_COARSE_FACTOR, lv_[0].level, st_);
+      factor_coarse();
       c_->prof.end(p, st_);
-      coarse_done_ = true;
     }
+    if (factor) coarse_done_ = true;
     if (!report && tuned_) {
       linearized_ = true;
       return c_->check("linearize");
@@ -394,13 +397,18 @@ class Solver final : public SolverBase {
       l.s64 = make_sten<double>(l.g.h, cfg);
     }
     if (part_solid_) pieces_ = make_patch_pieces(lv_[0].g.h, cfg);
-    if (dlv_) upload_operator();
+    upload_operator();
     coarse_done_ = false;
     linearized_ = linearized_j_ = false;
   }
 
-  // The constants of the persistent cycle's operator: every level's assembly
-  // record and the coefficient table of a mesh of width 1.
+  void factor_coarse() {
+    launch_coarse_factor(lv_[0].g, lv_[0].s64, lv_[0].vb64, coarse_work_, ainv_, status_, st_,
+                         part_solid_ ? &pieces_ : nullptr);
+  }
+
+  // The constants of the assembled operator: every level's assembly record and
+  // the coefficient table of a mesh of width 1.
   void upload_operator() {
     std::vector<AsmLevel<T>> ha(K_ + 1);
     asm_nodes_.assign(K_ + 1, 0);
@@ -413,13 +421,6 @@ class Solver final : public SolverBase {
     cudaMemcpyAsync(dasm_, ha.data(), sizeof(AsmLevel<T>) * ha.size(), cudaMemcpyHostToDevice, st_);
     cudaMemcpyAsync(dtab_, tab.get(), sizeof(OpTable<T>), cudaMemcpyHostToDevice, st_);
     cudaStreamSynchronize(st_);
-  }
-
-  // Levels whose part of the cycle the persistent launch runs (all while the
-  // split is not tuned yet): their velocity blocks are assembled.
-  int assembled_levels() const {
-    if (!dasm_ || split_ == 0 || (vgrid_ <= 0 && cluster_ <= 0)) return 0;
-    return split_ < 0 ? K_ : std::min(K_, std::max(0, split_ - lv_[0].level));
   }
 
   int split_level() const override { return split_ > 0 ? split_ : 0; }
@@ -609,7 +610,7 @@ class Solver final : public SolverBase {
   AsmLevel<T>* dasm_ = nullptr;    // levels 1..K of the assembly
   OpTable<T>* dtab_ = nullptr;
   std::vector<int> asm_nodes_;     // nodes of the first k assembled levels
-  std::vector<cudaStream_t> side_;   // side_[k - 1]: setup of level k < K
+  std::vector<cudaStream_t> side_;   // side_[k - 1]: setup of level k
   std::vector<cudaEvent_t> side_ev_;
   cudaEvent_t fork_ev_ = nullptr;
   bool capturing() const {

@@ -1,22 +1,21 @@
 // Cell-wise Vanka smoother (Sec. 2.2 names multigrid as the preconditioner;
 // the smoother is cell-wise Vanka with 12x12 local solves): the launchers of
-// the setup and of one colour pass.  The per-cell and per-tile arithmetic is
-// in vanka_body.cuh.
+// the setup and of one colour pass.  The arithmetic is in vnode.cuh (setup) and
+// vanka_body.cuh (passes by tiles).
 #include "kernels.h"
 #include "vanka_body.cuh"
+#include "vnode.cuh"
 
 namespace dnnmg {
 
 namespace {
 
-
 template <typename T>
 __global__ void __launch_bounds__(kSetupThreads)
-    vanka_setup_kernel(Grid g, Sten<T> s, const T* __restrict__ vb, T* __restrict__ inv,
-                       int* status) {
-  __shared__ SetupSmem<T> W[kSetupCells];
-  vanka_setup_cell<T>(g, s, vb, inv, status, blockIdx.y,
-                      blockIdx.x * kSetupCells + threadIdx.x / 16, W[threadIdx.x / 16]);
+    vanka_setup_kernel(Grid g, const uint16_t* __restrict__ pat, const T* __restrict__ cf,
+                       const OpTable<T>* __restrict__ tab, T* __restrict__ inv, int* status) {
+  vanka_setup_cell<T>(g, pat, cf, *tab, (T)g.h, (T)(g.h * g.h), inv, status, blockIdx.y,
+                      blockIdx.x * kSetupCells + threadIdx.x / 16);
 }
 
 template <typename T, int TCX, int TCY>
@@ -49,11 +48,11 @@ void pass_shape(const Grid& g, const Sten<T>& s, int colour, const T* b, const T
 }  // namespace
 
 template <typename T>
-void launch_vanka_setup(const Grid& g, const Sten<T>& s, const T* vb, T* inv, int* status,
-                        cudaStream_t st) {
+void launch_vanka_setup(const Grid& g, const uint16_t* pat, const T* cf, const OpTable<T>* tab,
+                        T* inv, int* status, cudaStream_t st) {
   dim3 grid(cdiv(vanka_slots(g), kSetupCells), 4);
   note_launch();
-  vanka_setup_kernel<T><<<grid, kSetupThreads, 0, st>>>(g, s, vb, inv, status);
+  vanka_setup_kernel<T><<<grid, kSetupThreads, 0, st>>>(g, pat, cf, tab, inv, status);
 }
 
 template <typename T>
@@ -72,10 +71,10 @@ void launch_vanka_pass(const Grid& g, const Sten<T>& s, int colour, const T* b, 
   }
 }
 
-template void launch_vanka_setup<float>(const Grid&, const Sten<float>&, const float*, float*,
-                                        int*, cudaStream_t);
-template void launch_vanka_setup<double>(const Grid&, const Sten<double>&, const double*,
-                                         double*, int*, cudaStream_t);
+template void launch_vanka_setup<float>(const Grid&, const uint16_t*, const float*,
+                                        const OpTable<float>*, float*, int*, cudaStream_t);
+template void launch_vanka_setup<double>(const Grid&, const uint16_t*, const double*,
+                                         const OpTable<double>*, double*, int*, cudaStream_t);
 template void launch_vanka_pass<float>(const Grid&, const Sten<float>&, int, const float*,
                                        const float*, const float*, const float*, float, float*,
                                        cudaStream_t, int);

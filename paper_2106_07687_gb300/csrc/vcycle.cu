@@ -25,13 +25,6 @@ namespace dnnmg {
 
 namespace {
 
-// Threads per block, one block per SM: a pass holds 36 coefficients and 36
-// inverse entries per thread, so FP32 takes 16 warps of 128 registers and FP64
-// 8 warps of 255.
-template <typename T>
-constexpr int walk_threads() {
-  return sizeof(T) == 4 ? 512 : 256;
-}
 constexpr int kMaxPhases = 160;  // phases of one launch (a V(2,2) cycle from level 8)
 constexpr int kMaxVLevels = 10;
 
@@ -45,14 +38,6 @@ struct WalkSmem {
   Phase ph[kMaxPhases];
   alignas(16) WarpTile<T> tile[walk_threads<T>() / 32];
 };
-
-template <class S>
-__device__ __forceinline__ void copy_ints(S* dst, const S* src, int count) {
-  static_assert(sizeof(S) % sizeof(int) == 0, "record size");
-  const int* s = reinterpret_cast<const int*>(src);
-  int* d = reinterpret_cast<int*>(dst);
-  for (int e = threadIdx.x; e < (int)(count * sizeof(S) / sizeof(int)); e += blockDim.x) d[e] = s[e];
-}
 
 // Item n < count of a node-wise phase for every thread of the grid: chunks
 // of 32 consecutive items (one warp, coalesced) go round-robin over the
@@ -302,6 +287,8 @@ void launch_assemble_blocks(const AsmLevel<T>* lv, int nlev, int nodes, cudaStre
 int vcycle_warp_tiles(const Grid& g) {
   return cdiv(g.nx / 2 + 1, kWX / 2) * cdiv(g.ny / 2 + 1, kWY / 2);
 }
+
+int vcycle_defect_tiles(const Grid& g) { return cdiv(g.nnx, kWX) * cdiv(g.nny, kWY); }
 
 bool vcycle_fits(int nphases, int nlevels) {
   return nphases <= kMaxPhases && nlevels <= kMaxVLevels;

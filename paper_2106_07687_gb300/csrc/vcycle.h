@@ -56,6 +56,8 @@ std::vector<Phase> vcycle_phases(int top, int nu1, int nu2);
 bool vcycle_fits(int nphases, int nlevels);
 // warp tiles of a colour pass on a level
 int vcycle_warp_tiles(const Grid& g);
+// warp tiles of a defect
+int vcycle_defect_tiles(const Grid& g);
 // co-resident grid size for the cooperative launch (0 if not available)
 template <typename T>
 int vcycle_grid(int coarse_nd);

@@ -107,6 +107,143 @@ __device__ __forceinline__ void assemble_node(const Grid& g, const Sten<T>& s,
   for (int v = 0; v < 36 / kVec16<T>; ++v) o[(size_t)v * g.nn] = vec_pack(c + v * kVec16<T>);
 }
 
+// ---- setup of the local inverses -------------------------------------------------------
+// 1 / d; in FP64 by Newton's iteration from the hardware's approximation
+// (about 20 bits; two steps reach the rounding error), because every FP64
+// instruction takes 64 cycles of a warp's scheduler
+__device__ __forceinline__ float pivot_recip(float d) { return 1.0f / d; }
+__device__ __forceinline__ double pivot_recip(double d) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+#pragma unroll
+  for (int k = 0; k < 2; ++k) y = fma(y, fma(-d, y, 1.0), y);
+  return y;
+}
+
+// Inverse of the restriction of the level's Jacobian to the 12 unknowns of
+// the fluid cell of `slot` in `colour` (its 4 nodes x u, v, p), with identity
+// rows and columns on constrained unknowns, by a group of 16 consecutive lanes
+// (a half-warp; every lane of it calls this with the same cell).  Lane r < 12
+// gathers row r = (component c, node a) from the assembled blocks of node a
+// and the coefficient table and keeps it in registers.  Gauss-Jordan
+// elimination with partial pivoting then runs across the lanes, in place: at
+// step k the unused lane with the largest |A[.][k]| (lowest lane on ties) is
+// the pivot row p, and every lane adds a multiple of it,
+//   A[.][j] = m A[p][j] + (0 on the pivot row, A[.][j] elsewhere),
+// m = 1 / A[p][k] there and -A[.][k] / A[p][k] elsewhere, which column k then
+// holds.  Rows are never swapped; the lane that pivoted on column k ends with
+// row k of the inverse, whose column pcol[j] sits in column j.
+// Assembling the 12 x 12 matrix cell by cell took most of the former setup
+// (Gauss-point data of nine cells and 36 element blocks per cell): per launch,
+// mean over levels 2 .. 5 in FP32 48.7 -> 28.1 us, levels 2 and 3 in FP64 137
+// -> 44 us.
+template <typename T>
+__device__ __forceinline__ void vanka_setup_cell(const Grid& g, const uint16_t* pat, const T* cf,
+                                                 const OpTable<T>& tab, T h, T h2,
+                                                 T* __restrict__ inv, int* status, int colour,
+                                                 int slot) {
+  const int cx = colour & 1, cy = colour >> 1;
+  const int sx = g.nx / 2 + 1, pitch = vanka_pitch(g);
+  const int nslots = vanka_slots(g);
+  if (slot >= nslots || slot % pitch >= sx) return;
+  const int ci = 2 * (slot % pitch) - cx, cj = 2 * (slot / pitch) - cy;
+  if (ci < 0 || cj < 0 || ci >= g.nx || cj >= g.ny || g.solid[cj * g.nx + ci]) return;
+  const int lane = threadIdx.x & 15;
+  const unsigned mask = 0xFFFFu << (threadIdx.x & 16);  // this half-warp
+  const int r = lane < 12 ? lane : 0;                   // lanes 12..15 shadow row 0
+  const int c = r >> 2, ax = r & 1, ay = (r >> 1) & 1;
+  const int n0 = cj * g.nnx + ci, na = n0 + ay * g.nnx + ax;
+  int pt[4];
+#pragma unroll
+  for (int b = 0; b < 4; ++b) pt[b] = __ldg(pat + n0 + (b >> 1) * g.nnx + (b & 1));
+  const int pa = __ldg(pat + na);
+  const int cls = ((ci + ax) & 1) + 2 * ((cj + ay) & 1);
+  T A[12];
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    const int di = (b & 1) - ax, dj = (b >> 1) - ay, e = (di + 1) + 3 * (dj + 1);
+    const T* gd = tab.gd[pa & 15][e];
+    if (c < 2) {
+      // the uu, uv (c = 0) or vu, vv (c = 1) entries of the block
+      const int k = 4 * e + 2 * c;
+      constexpr int V = kVec16<T>;
+      const T* q = cf + ((size_t)(k / V) * g.nn + na) * V + k % V;
+      A[b] = __ldg(q);
+      A[4 + b] = __ldg(q + 1);
+      A[8 + b] = h * __ldg(gd + c);
+    } else {
+      A[b] = h * __ldg(gd + 2);
+      A[4 + b] = h * __ldg(gd + 3);
+      A[8 + b] = h2 * __ldg(tab.lps[(pa >> kPatPatch) & 15][cls] + (di + 2) + 5 * (dj + 2));
+    }
+  }
+  // identity rows and zero columns on constrained unknowns
+  const bool own_cons = pa & (c < 2 ? kPatVDir : kPatPFix);
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    const bool col_cons = pt[k & 3] & (k < 8 ? kPatVDir : kPatPFix);
+    if (own_cons) A[k] = k == r ? T(1) : T(0);
+    else if (col_cons) A[k] = T(0);
+  }
+  bool used = lane >= 12, ok = true;
+  int my_col = 0;
+  int pcol[12];
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    // the bit patterns of non-negative numbers order like the numbers: one
+    // maximum over the half-warp (FP64: of the high words), then the lowest
+    // unused lane that holds it
+    unsigned key;
+    if constexpr (sizeof(T) == 4)
+      key = __float_as_uint(A[k]) & 0x7FFFFFFFu;
+    else
+      key = (unsigned)__double2hiint(A[k]) & 0x7FFFFFFFu;
+    if (used) key = 0u;
+    const unsigned mx = __reduce_max_sync(mask, key);
+    const int p = (__ffs(__ballot_sync(mask, key == mx && !used) & mask) - 1) & 15;
+    pcol[k] = p;
+    ok = ok && mx != 0u;  // the same in every lane of the group
+    if (ok) {
+      const bool piv = lane == p;
+      const T ip = pivot_recip(__shfl_sync(mask, A[k], p, 16));
+      const T m = piv ? ip : -A[k] * ip;
+#pragma unroll
+      for (int cc = 0; cc < 12; ++cc) {
+        if (cc == k) continue;
+        const T ap = __shfl_sync(mask, A[cc], p, 16);
+        A[cc] = m * ap + (piv ? T(0) : A[cc]);
+      }
+      A[k] = m;
+      if (piv) used = true, my_col = k;
+    }
+  }
+  if (!ok) {
+    if (lane == 0) atomicOr(status, 1);
+  }
+  if (lane >= 12) return;
+#pragma unroll
+  for (int j = 0; j < 12; ++j)
+    inv[vanka_inv_index<T>(nslots, colour, slot, my_col & 3, (my_col >> 2) * 12 + pcol[j])] =
+        ok ? A[j] : T(0);
+}
+
+// ---- persistent kernels -----------------------------------------------------------------
+// Threads per block, one block per SM: a pass holds 36 coefficients and 36
+// inverse entries per thread, so FP32 takes 16 warps of 128 registers and FP64
+// 8 warps of 255.
+template <typename T>
+constexpr int walk_threads() {
+  return sizeof(T) == 4 ? 512 : 256;
+}
+// count records from global to shared memory, by the whole block
+template <class S>
+__device__ __forceinline__ void copy_ints(S* dst, const S* src, int count) {
+  static_assert(sizeof(S) % sizeof(int) == 0, "record size");
+  const int* s = reinterpret_cast<const int*>(src);
+  int* d = reinterpret_cast<int*>(dst);
+  for (int e = threadIdx.x; e < (int)(count * sizeof(S) / sizeof(int)); e += blockDim.x) d[e] = s[e];
+}
+
 // ---- one warp, 8 x 4 nodes -----------------------------------------------------------
 // Masked iterate of the warp's nodes plus a two-node halo: 12 x 8 nodes, rows
 // of 24 so that the four rows of a tile fall on different banks.
