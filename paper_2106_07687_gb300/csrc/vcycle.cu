@@ -70,11 +70,12 @@ __device__ __forceinline__ void walk_phases(const VLevel<T>* glv, const OpTable<
   __syncthreads();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int w0 = blockIdx.x + gridDim.x * w, nw = gridDim.x * (NT / 32);
-  // Four lanes per node while that gives every scheduler (four per block) at
-  // most little more than one warp.  On 152 blocks that is up to level 3 (612
-  // warps).  One cycle, one -> four lanes per node on levels 2 and 3: FP64 287 ->
-  // 191 us on 128x32, 435 -> 339 us on 256x64; FP32 117 -> 115 and 174 -> 172 us.
-  // With level 4 (2,244 warps) as well: FP64 401, FP32 180 us.
+  // FP64: four lanes per node while that gives every scheduler (four per block)
+  // at most little more than one warp.  On 152 blocks that is up to level 3
+  // (612 warps): one cycle, one -> four lanes per node on levels 2 and 3, 287 ->
+  // 191 us on 128x32, 435 -> 339 us on 256x64; with level 4 (2,244 warps) as well
+  // 401 us.  In FP32 the same gains 2 us a cycle, but the larger kernel loses 15
+  // (its instructions come through the cache once per phase).
   auto split_level = [&](const Grid& g) {
     return 4 * cdiv(g.nnx, kWX) * cdiv(g.nny, kWY) <= 5 * (int)gridDim.x;
   };
@@ -91,13 +92,14 @@ __device__ __forceinline__ void walk_phases(const VLevel<T>* glv, const OpTable<
         T* xout = f.out ? L.x2 : x0;
         const NodeLevel<T> N{g.nx, g.ny, g.nnx, g.nn, L.pat, L.cf, (T)g.h, (T)(g.h * g.h)};
         const int pitch = vanka_pitch(g), nslots = vanka_slots(g);
-        if (split_level(g)) {
-          const int nbx = cdiv(g.nx / 2 + 1, kSX / 2), nt = nbx * cdiv(g.ny / 2 + 1, kSY / 2);
-          for (int t = w0; t < nt; t += nw)
-            split_pass_tile<T>(N, S.tab, f.colour, b, xin, L.inv, pitch, nslots, omega, xout,
-                               t % nbx, t / nbx, lane, S.tile[w]);
-          break;
-        }
+        if constexpr (sizeof(T) == 8)
+          if (split_level(g)) {
+            const int nbx = cdiv(g.nx / 2 + 1, kSX / 2), nt = nbx * cdiv(g.ny / 2 + 1, kSY / 2);
+            for (int t = w0; t < nt; t += nw)
+              split_pass_tile<T>(N, S.tab, f.colour, b, xin, L.inv, pitch, nslots, omega, xout,
+                                 t % nbx, t / nbx, lane, S.tile[w]);
+            break;
+          }
         const int nbx = cdiv(g.nx / 2 + 1, kWX / 2);
         const int nt = nbx * cdiv(g.ny / 2 + 1, kWY / 2);
         for (int t = w0; t < nt; t += nw)
@@ -107,13 +109,14 @@ __device__ __forceinline__ void walk_phases(const VLevel<T>* glv, const OpTable<
       }
       case kPhaseDefect: {
         const NodeLevel<T> N{g.nx, g.ny, g.nnx, g.nn, L.pat, L.cf, (T)g.h, (T)(g.h * g.h)};
-        if (split_level(g)) {
-          const int nbx = cdiv(g.nnx, kSX), nt = nbx * cdiv(g.nny, kSY);
-          for (int t = w0; t < nt; t += nw)
-            split_defect_tile<T>(N, S.tab, b, f.in ? L.x2 : x0, L.d, t % nbx, t / nbx, lane,
-                                 S.tile[w]);
-          break;
-        }
+        if constexpr (sizeof(T) == 8)
+          if (split_level(g)) {
+            const int nbx = cdiv(g.nnx, kSX), nt = nbx * cdiv(g.nny, kSY);
+            for (int t = w0; t < nt; t += nw)
+              split_defect_tile<T>(N, S.tab, b, f.in ? L.x2 : x0, L.d, t % nbx, t / nbx, lane,
+                                   S.tile[w]);
+            break;
+          }
         const int nbx = cdiv(g.nnx, kWX), nt = nbx * cdiv(g.nny, kWY);
         for (int t = w0; t < nt; t += nw)
           warp_defect_tile<T>(N, S.tab, b, f.in ? L.x2 : x0, L.d, t % nbx, t / nbx, lane,
