@@ -528,7 +528,7 @@ int Batch<T>::init() {
   {
     // levels count from the coarsest (1); x is zeroed beforehand when no
     // smoothing pass starts from zero
-    std::vector<Phase> ph = vcycle_phases(Lmax_ - 1, c0_.nu1, c0_.nu2);
+    std::vector<Phase> ph = vcycle_phases(Lmax_ - 1, c0_.nu1, c0_.nu2, false);
     if (!ph.empty() && ph[0].type == kPhaseZeroTop) ph.erase(ph.begin());
     for (Phase& q : ph) q.level += 1;
     nph_ = (int)ph.size();

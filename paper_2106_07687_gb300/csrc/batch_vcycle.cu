@@ -46,9 +46,11 @@ __global__ void __launch_bounds__(walk_threads<T>(), 1)
   const BLev<T>* rec = in_smem ? srec : W.lev;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int w0 = blockIdx.x + gridDim.x * w, nw = gridDim.x * NW;
+  int budget = 1;  // nothing waits on tags here
   for (int p = p0; p < p1; ++p) {
-    const Phase f{__ldg(&ph[p].type), __ldg(&ph[p].level), __ldg(&ph[p].colour), __ldg(&ph[p].in),
-                  __ldg(&ph[p].out)};
+    Phase f{};
+    f.type = __ldg(&ph[p].type), f.level = __ldg(&ph[p].level), f.colour = __ldg(&ph[p].colour);
+    f.in = __ldg(&ph[p].in), f.out = __ldg(&ph[p].out);
     const int k = f.level;
     // item t of a list: its problem's record of level k and its index there
     auto items = [&](const Work& list, auto body) {
@@ -70,24 +72,27 @@ __global__ void __launch_bounds__(walk_threads<T>(), 1)
           T* x0 = L.top ? topx + L.off : L.x;
           const int nbx = cdiv(L.g.nx / 2 + 1, kWX / 2);
           warp_pass_tile<T>(node_level(L), table(L), f.colour, L.top ? topb + L.off : L.b,
-                            f.in ? L.x2 : x0, L.inv, vanka_pitch(L.g), vanka_slots(L.g), omega,
-                            f.out ? L.x2 : x0, t % nbx, t / nbx, lane, S.tile[w]);
+                            PlanarX<T>{f.in ? L.x2 : x0, f.out ? L.x2 : x0, L.g.nn}, L.inv,
+                            vanka_pitch(L.g), vanka_slots(L.g), omega, t % nbx, t / nbx, lane,
+                            S.tile[w], budget);
         });
         break;
       case kPhasePassZero:
         items(W.zero[k], [&](const BLev<T>& L, int, int c) {
           const int e = (c << 5) + lane;
-          vanka_pass_zero_node<T>(L.g, f.colour, L.top ? topb + L.off : L.b, L.inv, omega,
-                                  f.out ? L.x2 : (L.top ? topx + L.off : L.x), e,
-                                  e < 4 * vanka_slots(L.g));
+          T* out = f.out ? L.x2 : (L.top ? topx + L.off : L.x);
+          zero_pass_node<T>(L.g, f.colour, L.top ? topb + L.off : L.b,
+                            PlanarX<T>{nullptr, out, L.g.nn}, L.inv, omega, e,
+                            e < 4 * vanka_slots(L.g));
         });
         break;
       case kPhaseDefect:
         items(W.defect[k], [&](const BLev<T>& L, int, int t) {
           const int nbx = cdiv(L.g.nnx, kWX);
           warp_defect_tile<T>(node_level(L), table(L), L.top ? topb + L.off : L.b,
-                              f.in ? L.x2 : (L.top ? topx + L.off : L.x), L.d, t % nbx, t / nbx,
-                              lane, S.tile[w]);
+                              PlanarX<T>{f.in ? L.x2 : (L.top ? topx + L.off : L.x), nullptr,
+                                         L.g.nn},
+                              L.d, t % nbx, t / nbx, lane, S.tile[w], budget);
         });
         break;
       case kPhaseRestrict:

@@ -80,7 +80,11 @@ class Solver final : public SolverBase {
     coarse_work_ = c_->mem.alloc<double>(coarse_factor_doubles(g0));
     ainv_ = c_->mem.alloc<double>((size_t)9 * g0.nn * g0.nn);
     status_ = c_->mem.alloc<int>(4);
-    if (status_) cudaMemsetAsync(status_, 0, 4 * sizeof(int), st_);  // fresh memory is not zero
+    // setup status (0, 1), wait status (2) and the number of the next cycle (3)
+    if (status_) {
+      cudaMemsetAsync(status_, 0, 3 * sizeof(int), st_);  // fresh memory is not zero
+      cudaMemsetAsync(status_ + 3, 1, sizeof(int), st_);
+    }
     m_ = cfg.gmres_m;
     n_ = 3 * (size_t)lv_[K_].g.nn;
     V_ = c_->mem.alloc<T>((m_ + 1) * n_);
@@ -104,13 +108,17 @@ class Solver final : public SolverBase {
     if (cfg.persistent_vcycle != 0) {
       std::vector<VLevel<T>> hv(K_ + 1);
       for (int k = 0; k <= K_; ++k) {
-        hv[k] = VLevel<T>{lv_[k].g, lv_[k].x, lv_[k].x2, lv_[k].b, lv_[k].d, lv_[k].inv,
-                          lv_[k].cf, lv_[k].pat};
+        // the iterate's tagged buffers; no cycle has the number 0 they start with
+        const size_t words = 2 * (size_t)kTagWords<T> * lv_[k].g.nn;
+        ulonglong2* xt = k > 0 ? c_->mem.alloc<ulonglong2>(words) : nullptr;
+        if (xt) cudaMemsetAsync(xt, 0, words * sizeof(ulonglong2), st_);
+        hv[k] = VLevel<T>{lv_[k].g, lv_[k].x, lv_[k].b, lv_[k].d, lv_[k].inv, lv_[k].cf,
+                          lv_[k].pat, xt};
       }
       dlv_ = c_->mem.alloc<VLevel<T>>(K_ + 1);
       std::vector<Phase> all;
       for (int k = 0; k <= K_; ++k) {
-        const std::vector<Phase> p = vcycle_phases(k, cfg.nu1, cfg.nu2);
+        const std::vector<Phase> p = vcycle_phases(k, cfg.nu1, cfg.nu2, true);
         ph_off_.push_back((int)all.size());
         ph_n_.push_back((int)p.size());
         all.insert(all.end(), p.begin(), p.end());
@@ -554,10 +562,12 @@ class Solver final : public SolverBase {
         if (coop_cap_ > 0 && blocks > coop_cap_) blocks = coop_cap_;
         blocks = blocks > vgrid_ ? vgrid_ : blocks;
         rc = launch_vcycle_persistent<T>(dlv_, dtab_, dph_ + ph_off_[k], ph_n_[k], k, b, x, ainv_,
-                                         (T)c_->cfg.omega, blocks, coarse_nd_, st_, skip);
+                                         (T)c_->cfg.omega, status_ + 2, blocks, coarse_nd_, st_,
+                                         skip);
       } else {
         rc = launch_vcycle_cluster<T>(dlv_, dtab_, dph_ + ph_off_[k], ph_n_[k], k, b, x, ainv_,
-                                      (T)c_->cfg.omega, cluster_, coarse_nd_, st_);
+                                      (T)c_->cfg.omega, status_ + 2, cluster_, coarse_nd_,
+                                      st_);
       }
       c_->prof.end(p, st_);
       if (rc == 0) return;

@@ -5,13 +5,18 @@
 // sequence of phases -- Vanka colour passes, defect, restriction (with the
 // coarse iterate zeroed), the coarse direct solve, prolongation -- built once
 // per top level on the host.  The kernel walks the phase list; all blocks
-// share every phase and meet at a barrier (grid-wide, or the hardware cluster
-// barrier) before the next.
+// share every phase.
 //
 // A phase is bound by its dependent chain (barrier, loads from L2, rows,
 // products, stores), not by bandwidth, on all but the largest levels.  Colour
 // passes and defects therefore work from assembled coefficients, one warp per
-// 8 x 4 nodes and without a block barrier (vnode.cuh).
+// 8 x 4 nodes and without a block barrier, and the iterate's values carry the
+// number of their update, so that a tile waits for its own inputs only
+// (vnode.cuh).  Barriers (grid-wide, or the hardware cluster barrier) remain
+// after the defect, the restriction and the coarse solve, whose outputs are
+// plain arrays.  One cycle, barriers after every phase -> numbered updates: FP32
+// on levels 3 / 5 / 6 (128x32, 512x128, 1024x256 cells) 92 -> 82, 244 -> 185,
+// 528 -> 430 us, FP64 on level 3 191 -> 154 us.
 #include <algorithm>
 #include <cooperative_groups.h>
 
@@ -53,29 +58,32 @@ __device__ __forceinline__ void for_items(int count, F f) {
   }
 }
 
-// Walk the phase list; `sync` separates phases (a grid-wide barrier for the
-// cooperative launch, the cluster barrier for the single-cluster launch).
-// Threads of all blocks split every node-wise phase; the warp tiles of a
-// colour pass or defect go round-robin over the blocks first.
+// Walk the phase list; `sync` separates the phases whose outputs are plain
+// arrays (a grid-wide barrier for the cooperative launch, the cluster barrier for
+// the single-cluster launch).  Threads of all blocks split every node-wise
+// phase; the warp tiles of a colour pass or defect go round-robin over the
+// blocks first.  state: the status word and the cycle's number.
 template <typename T, class Sync>
 __device__ __forceinline__ void walk_phases(const VLevel<T>* glv, const OpTable<T>* gtab,
                                             const Phase* gph, int nph, int top, const T* topb,
                                             T* topx, const double* __restrict__ Ainv, T omega,
-                                            WalkSmem<T>& S, Sync sync) {
+                                            int* state, WalkSmem<T>& S, Sync sync) {
   constexpr int NT = walk_threads<T>();
   double* sbuf = reinterpret_cast<double*>(S.tile);  // the coarse right-hand side
   copy_ints(S.lv, glv, top + 1);
   copy_ints(S.ph, gph, nph);
   copy_ints(&S.tab, gtab, 1);
+  const unsigned cycle = __ldcg(reinterpret_cast<unsigned*>(state) + 1), tag0 = cycle << 8;
   __syncthreads();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int w0 = blockIdx.x + gridDim.x * w, nw = gridDim.x * (NT / 32);
+  int budget = kTagPolls;
   // FP64: four lanes per node while that gives every scheduler (four per block)
   // at most little more than one warp.  On 152 blocks that is up to level 3
-  // (612 warps): one cycle, one -> four lanes per node on levels 2 and 3, 287 ->
-  // 191 us on 128x32, 435 -> 339 us on 256x64; with level 4 (2,244 warps) as well
-  // 401 us.  In FP32 the same gains 2 us a cycle, but the larger kernel loses 15
-  // (its instructions come through the cache once per phase).
+  // (612 warps): one cycle with barriers, one -> four lanes per node on levels 2
+  // and 3, 287 -> 191 us on 128x32, 435 -> 339 us on 256x64; with level 4 (2,244
+  // warps) as well 401 us.  In FP32 the same gains 2 us a cycle, but the larger
+  // kernel loses 15 (its instructions come through the cache once per phase).
   auto split_level = [&](const Grid& g) {
     return 4 * cdiv(g.nnx, kWX) * cdiv(g.nny, kWY) <= 5 * (int)gridDim.x;
   };
@@ -85,71 +93,67 @@ __device__ __forceinline__ void walk_phases(const VLevel<T>* glv, const OpTable<
     const VLevel<T>& L = S.lv[k];
     const Grid& g = L.g;
     const T* b = k == top ? topb : L.b;
-    T* x0 = k == top ? topx : L.x;
+    const size_t words = (size_t)kTagWords<T> * g.nn;
+    const TaggedX<T> x{L.xt + f.in * words, L.xt + f.out * words, f.last ? topx : nullptr, g.nn,
+                       tag0 + f.tin,        tag0 + f.tout,        state};
+    const NodeLevel<T> N{g.nx, g.ny, g.nnx, g.nn, L.pat, L.cf, (T)g.h, (T)(g.h * g.h)};
+    bool barrier = false;
     switch (f.type) {
       case kPhasePass: {
-        const T* xin = f.in ? L.x2 : x0;
-        T* xout = f.out ? L.x2 : x0;
-        const NodeLevel<T> N{g.nx, g.ny, g.nnx, g.nn, L.pat, L.cf, (T)g.h, (T)(g.h * g.h)};
         const int pitch = vanka_pitch(g), nslots = vanka_slots(g);
         if constexpr (sizeof(T) == 8)
           if (split_level(g)) {
             const int nbx = cdiv(g.nx / 2 + 1, kSX / 2), nt = nbx * cdiv(g.ny / 2 + 1, kSY / 2);
             for (int t = w0; t < nt; t += nw)
-              split_pass_tile<T>(N, S.tab, f.colour, b, xin, L.inv, pitch, nslots, omega, xout,
-                                 t % nbx, t / nbx, lane, S.tile[w]);
+              split_pass_tile<T>(N, S.tab, f.colour, b, x, L.inv, pitch, nslots, omega, t % nbx,
+                                 t / nbx, lane, S.tile[w], budget);
             break;
           }
         const int nbx = cdiv(g.nx / 2 + 1, kWX / 2);
         const int nt = nbx * cdiv(g.ny / 2 + 1, kWY / 2);
         for (int t = w0; t < nt; t += nw)
-          warp_pass_tile<T>(N, S.tab, f.colour, b, xin, L.inv, pitch, nslots, omega, xout, t % nbx,
-                            t / nbx, lane, S.tile[w]);
+          warp_pass_tile<T>(N, S.tab, f.colour, b, x, L.inv, pitch, nslots, omega, t % nbx, t / nbx,
+                            lane, S.tile[w], budget);
         break;
       }
       case kPhaseDefect: {
-        const NodeLevel<T> N{g.nx, g.ny, g.nnx, g.nn, L.pat, L.cf, (T)g.h, (T)(g.h * g.h)};
+        barrier = true;
         if constexpr (sizeof(T) == 8)
           if (split_level(g)) {
             const int nbx = cdiv(g.nnx, kSX), nt = nbx * cdiv(g.nny, kSY);
             for (int t = w0; t < nt; t += nw)
-              split_defect_tile<T>(N, S.tab, b, f.in ? L.x2 : x0, L.d, t % nbx, t / nbx, lane,
-                                   S.tile[w]);
+              split_defect_tile<T>(N, S.tab, b, x, L.d, t % nbx, t / nbx, lane, S.tile[w], budget);
             break;
           }
         const int nbx = cdiv(g.nnx, kWX), nt = nbx * cdiv(g.nny, kWY);
         for (int t = w0; t < nt; t += nw)
-          warp_defect_tile<T>(N, S.tab, b, f.in ? L.x2 : x0, L.d, t % nbx, t / nbx, lane,
-                              S.tile[w]);
+          warp_defect_tile<T>(N, S.tab, b, x, L.d, t % nbx, t / nbx, lane, S.tile[w], budget);
         break;
       }
       case kPhaseRestrict: {
+        barrier = true;
         const VLevel<T>& C = S.lv[k - 1];
         const Grid& c = C.g;
-        const bool zero = f.colour == 1;
+        const TaggedX<T> xc{C.xt, C.xt, nullptr, c.nn, tag0, tag0, state};
         for_items<NT>(c.nn, [&](int n) {
           restrict_node<T, true>(g, c, L.d, C.b, 3, n % c.nnx, n / c.nnx);
-          if (zero) {
-            C.x[n] = T(0);
-            C.x[c.nn + n] = T(0);
-            C.x[2 * c.nn + n] = T(0);
-          }
+          if (f.colour == 1 && k > 1) xc.store(n, T(0), T(0), T(0));
         });
         break;
       }
       case kPhasePassZero: {
         // four items per colour cell, warp-sized chunks round-robin over the
         // blocks; every lane of a warp takes part in the cell's shuffles
-        T* xout = f.out ? L.x2 : x0;
-        const int count = 4 * vanka_slots(g);
-        const int nchunks = (count + 31) >> 5;
+        const int count = 4 * vanka_slots(g), nchunks = (count + 31) >> 5;
         for (int c = w0; c < nchunks; c += nw) {
           const int e = (c << 5) + lane;
-          vanka_pass_zero_node<T>(g, f.colour, b, L.inv, omega, xout, e, e < count);
+          zero_pass_node<T>(g, f.colour, b, x, L.inv, omega, e, e < count);
         }
         break;
       }
       case kPhaseCoarse: {
+        barrier = true;
+        T* x0 = k == top ? topx : L.x;
         const int nd = 3 * g.nn;
         for (int q0 = threadIdx.x; q0 < nd; q0 += 4 * NT) {  // four loads in flight
           double v[4];
@@ -189,46 +193,58 @@ __device__ __forceinline__ void walk_phases(const VLevel<T>* glv, const OpTable<
       }
       case kPhaseProlong: {
         const VLevel<T>& C = S.lv[k - 1];
-        T* x = f.in ? L.x2 : x0;
-        for_items<NT>(g.nn, [&](int n) {
-          prolong_add_node<T>(g, C.g, C.x, x, n % g.nnx, n / g.nnx);
-        });
+        const Grid& c = C.g;
+        const TaggedX<T> xc{C.xt + f.cin * (size_t)kTagWords<T> * c.nn, nullptr, nullptr, c.nn,
+                            tag0 + f.tcin, 0u, state};
+        const int nchunks = (g.nn + 31) >> 5;  // whole warps wait together
+        for (int q = w0; q < nchunks; q += nw) {
+          const bool valid = (q << 5) + lane < g.nn;
+          const int n = valid ? (q << 5) + lane : 0, i = n % g.nnx, j = n / g.nnx;
+          if (f.tcin)
+            prolong_node<T>(g, c, xc, x, i, j, valid, budget);
+          else
+            prolong_node<T>(g, c, PlanarX<T>{C.x, nullptr, c.nn}, x, i, j, valid, budget);
+        }
         break;
       }
       case kPhaseZeroTop: {
-        for_items<NT>(3 * g.nn, [&](int n) { topx[n] = T(0); });
+        if (k > 0) for_items<NT>(g.nn, [&](int n) { x.store(n, T(0), T(0), T(0)); });
         break;
       }
     }
-    sync();
+    if (barrier && p + 1 < nph) sync();
   }
+  // every block has read the number before its first barrier (a cycle with a
+  // phase that uses it has one)
+  if (blockIdx.x == 0 && threadIdx.x == 0)
+    *(reinterpret_cast<volatile unsigned*>(state) + 1) = cycle + 1;
 }
 
 template <typename T>
 __global__ void __launch_bounds__(walk_threads<T>(), 1)
     vcycle_kernel(const VLevel<T>* lv, const OpTable<T>* tab, const Phase* ph, int nph, int top,
-                  const T* topb, T* topx, const double* __restrict__ Ainv, T omega,
+                  const T* topb, T* topx, const double* __restrict__ Ainv, T omega, int* state,
                   const int* skip) {
   // a speculative FGMRES iteration after the cycle stopped: every block
   // reads the same flag (set before this launch) and returns before any barrier
   if (skip && *skip) return;
   extern __shared__ __align__(16) uint8_t dyn[];
   cg::grid_group grid = cg::this_grid();
-  walk_phases<T>(lv, tab, ph, nph, top, topb, topx, Ainv, omega,
+  walk_phases<T>(lv, tab, ph, nph, top, topb, topx, Ainv, omega, state,
                  *reinterpret_cast<WalkSmem<T>*>(dyn), [&] { grid.sync(); });
 }
 
-// The whole grid is one thread-block cluster; phases are separated by the
-// cluster barrier (release / acquire at cluster scope, so the global-memory
-// results of one phase are visible to every block of the cluster in the next).
+// The whole grid is one thread-block cluster; the barriers are the cluster's
+// (release / acquire at cluster scope, so the global-memory results of one phase
+// are visible to every block of the cluster in the next).
 template <typename T>
 __global__ void __launch_bounds__(walk_threads<T>(), 1)
     vcycle_cluster_kernel(const VLevel<T>* lv, const OpTable<T>* tab, const Phase* ph, int nph,
                           int top, const T* topb, T* topx, const double* __restrict__ Ainv,
-                          T omega) {
+                          T omega, int* state) {
   extern __shared__ __align__(16) uint8_t dyn[];
   cg::cluster_group cl = cg::this_cluster();
-  walk_phases<T>(lv, tab, ph, nph, top, topb, topx, Ainv, omega,
+  walk_phases<T>(lv, tab, ph, nph, top, topb, topx, Ainv, omega, state,
                  *reinterpret_cast<WalkSmem<T>*>(dyn), [&] { cl.sync(); });
 }
 
@@ -242,29 +258,35 @@ __global__ void __launch_bounds__(128)
   assemble_node<T>(lv[k].g, lv[k].s, lv[k].vb, lv[k].cf, t - lv[k].first);
 }
 
-void build_phases(int k, int top, int nu1, int nu2, std::vector<Phase>& out) {
+// phases of the cycle of level k; returns the buffer and number of its final
+// iterate (0: the coarsest level's solution).  In the tagged form a prolongation
+// writes the other buffer, otherwise it works in place.
+std::pair<int, int> build_phases(int k, int nu1, int nu2, bool tagged, std::vector<Phase>& out) {
   if (k == 0) {
     out.push_back({kPhaseCoarse, 0, 0, 0, 0});
-    return;
+    return {0, 0};
   }
   // with pre-smoothing, the first pass starts from the zero iterate and
   // writes every node, so no level needs zeroing beforehand
-  int cur = 0;
+  int cur = 0, tag = 0;
+  auto push = [&](int type, int colour, bool flip, bool update) {
+    Phase f{type, k, colour, cur, flip ? 1 - cur : 0};
+    f.tin = tag;
+    cur = flip ? f.out : cur;
+    f.tout = tag += update;
+    out.push_back(f);
+  };
   for (int s = 0; s < nu1; ++s)
-    for (int c = 0; c < 4; ++c) {
-      out.push_back({s == 0 && c == 0 ? kPhasePassZero : kPhasePass, k, c, cur, 1 - cur});
-      cur ^= 1;
-    }
-  out.push_back({kPhaseDefect, k, 0, cur, 0});
-  out.push_back({kPhaseRestrict, k, nu1 > 0 ? 0 : 1, 0, 0});
-  build_phases(k - 1, top, nu1, nu2, out);
-  out.push_back({kPhaseProlong, k, 0, cur, 0});
+    for (int c = 0; c < 4; ++c) push(s == 0 && c == 0 ? kPhasePassZero : kPhasePass, c, true, true);
+  push(kPhaseDefect, 0, false, false);
+  push(kPhaseRestrict, nu1 > 0 ? 0 : 1, false, false);
+  const std::pair<int, int> coarse = build_phases(k - 1, nu1, nu2, tagged, out);
+  push(kPhaseProlong, 0, tagged, true);
+  out.back().cin = coarse.first;
+  out.back().tcin = coarse.second;
   for (int s = 0; s < nu2; ++s)
-    for (int c = 0; c < 4; ++c) {
-      out.push_back({kPhasePass, k, c, cur, 1 - cur});
-      cur ^= 1;
-    }
-  (void)top;
+    for (int c = 0; c < 4; ++c) push(kPhasePass, c, true, true);
+  return {cur, tag};
 }
 
 }  // namespace
@@ -297,10 +319,11 @@ bool vcycle_fits(int nphases, int nlevels) {
   return nphases <= kMaxPhases && nlevels <= kMaxVLevels;
 }
 
-std::vector<Phase> vcycle_phases(int top, int nu1, int nu2) {
+std::vector<Phase> vcycle_phases(int top, int nu1, int nu2, bool tagged) {
   std::vector<Phase> out;
   if (nu1 == 0 || top == 0) out.push_back({kPhaseZeroTop, top, 0, 0, 0});
-  build_phases(top, top, nu1, nu2, out);
+  build_phases(top, nu1, nu2, tagged, out);
+  out.back().last = 1;
   return out;
 }
 
@@ -324,10 +347,12 @@ int vcycle_grid(int coarse_nd) {
 
 template <typename T>
 int launch_vcycle_persistent(const VLevel<T>* lv, const OpTable<T>* tab, const Phase* ph, int nph,
-                             int top, const T* topb, T* topx, const double* Ainv, T omega, int grid,
-                             int coarse_nd, cudaStream_t st, const int* skip) {
+                             int top, const T* topb, T* topx, const double* Ainv, T omega,
+                             int* state, int grid, int coarse_nd, cudaStream_t st,
+                             const int* skip) {
   void* args[] = {(void*)&lv,   (void*)&tab,  (void*)&ph,   (void*)&nph,   (void*)&top,
-                  (void*)&topb, (void*)&topx, (void*)&Ainv, (void*)&omega, (void*)&skip};
+                  (void*)&topb, (void*)&topx, (void*)&Ainv, (void*)&omega, (void*)&state,
+                  (void*)&skip};
   note_launch();
   const cudaError_t e =
       cudaLaunchCooperativeKernel((void*)vcycle_kernel<T>, dim3(grid), dim3(walk_threads<T>()),
@@ -373,7 +398,7 @@ int vcycle_cluster_size(int coarse_nd) {
 template <typename T>
 int launch_vcycle_cluster(const VLevel<T>* lv, const OpTable<T>* tab, const Phase* ph, int nph,
                           int top, const T* topb, T* topx, const double* Ainv, T omega,
-                          int cluster, int coarse_nd, cudaStream_t st) {
+                          int* state, int cluster, int coarse_nd, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -388,7 +413,7 @@ int launch_vcycle_cluster(const VLevel<T>* lv, const OpTable<T>* tab, const Phas
   cfg.numAttrs = 1;
   note_launch();
   const cudaError_t e = cudaLaunchKernelEx(&cfg, vcycle_cluster_kernel<T>, lv, tab, ph, nph, top,
-                                           topb, topx, Ainv, omega);
+                                           topb, topx, Ainv, omega, state);
   return e == cudaSuccess ? 0 : 1;
 }
 
@@ -396,11 +421,11 @@ int launch_vcycle_cluster(const VLevel<T>* lv, const OpTable<T>* tab, const Phas
   template void launch_assemble_blocks<T>(const AsmLevel<T>*, int, int, cudaStream_t);           \
   template int vcycle_grid<T>(int);                                                              \
   template int launch_vcycle_persistent<T>(const VLevel<T>*, const OpTable<T>*, const Phase*,    \
-                                           int, int, const T*, T*, const double*, T, int, int,   \
-                                           cudaStream_t, const int*);                            \
+                                           int, int, const T*, T*, const double*, T, int*, int,  \
+                                           int, cudaStream_t, const int*);                       \
   template int vcycle_cluster_size<T>(int);                                                      \
   template int launch_vcycle_cluster<T>(const VLevel<T>*, const OpTable<T>*, const Phase*, int,  \
-                                        int, const T*, T*, const double*, T, int, int,           \
+                                        int, const T*, T*, const double*, T, int*, int, int,     \
                                         cudaStream_t);
 DNNMG_INST(float)
 DNNMG_INST(double)

@@ -12,9 +12,10 @@ namespace dnnmg {
 template <typename T>
 struct VLevel {
   Grid g;
-  T *x, *x2, *b, *d, *inv;
+  T *x, *b, *d, *inv;    // x: the coarsest level's solution
   const T* cf;           // assembled velocity blocks (null on the coarsest level)
   const uint16_t* pat;   // node patterns
+  ulonglong2* xt;        // the iterate: two tagged buffers of kTagWords nn words (vnode.cuh)
 };
 
 // A level's input to the assembly of its velocity blocks; `first` is its
@@ -42,15 +43,21 @@ enum PhaseType {
   kPhasePassZero  // first pass of a sweep from x = 0 (the input is not read)
 };
 
-// in / out select the level's iterate (0: x, the caller's buffer on the top
-// level; 1: the second buffer x2); a restriction with colour = 1 also zeroes
-// the coarse iterate (needed when no pre-smoothing pass starts from zero)
+// in / out select the level's iterate (two buffers); a restriction with colour
+// = 1 also starts the coarse iterate from zero (needed when no pre-smoothing pass
+// does).  tin / tout: number, within the cycle, of the level's update that the
+// phase reads and writes; cin / tcin: buffer and number of the coarse level's
+// iterate that a prolongation reads (tcin 0: the coarsest level's solution).
+// last: the phase writes the cycle's result.
 struct Phase {
   int type, level, colour, in, out;
+  int tin = 0, tout = 0, cin = 0, tcin = 0, last = 0;
 };
 
-// phase list of one V(nu1, nu2) cycle with top level `top`, x zeroed first
-std::vector<Phase> vcycle_phases(int top, int nu1, int nu2);
+// phase list of one V(nu1, nu2) cycle with top level `top`, x zeroed first.
+// tagged: for the single problem's kernel; otherwise a prolongation works in
+// place and the top level's result is in buffer 0.
+std::vector<Phase> vcycle_phases(int top, int nu1, int nu2, bool tagged);
 // whether a launch of nphases phases over nlevels levels fits the kernels'
 // shared-memory tables
 bool vcycle_fits(int nphases, int nlevels);
@@ -69,12 +76,15 @@ int vcycle_cluster_size(int coarse_nd);
 template <typename T>
 int launch_vcycle_cluster(const VLevel<T>* lv, const OpTable<T>* tab, const Phase* ph, int nph,
                           int top, const T* topb, T* topx, const double* Ainv, T omega,
-                          int cluster, int coarse_nd, cudaStream_t st);
+                          int* state, int cluster, int coarse_nd, cudaStream_t st);
+// state: two device words, a status word (8: a wait for an update hit its bound)
+// and the cycle's number, which the launch counts up (starts above 0).
 // returns 0 on success; with skip, nothing runs when *skip != 0 at the
 // launch's start
 template <typename T>
 int launch_vcycle_persistent(const VLevel<T>* lv, const OpTable<T>* tab, const Phase* ph, int nph,
-                             int top, const T* topb, T* topx, const double* Ainv, T omega, int grid,
-                             int coarse_nd, cudaStream_t st, const int* skip = nullptr);
+                             int top, const T* topb, T* topx, const double* Ainv, T omega,
+                             int* state, int grid, int coarse_nd, cudaStream_t st,
+                             const int* skip = nullptr);
 
 }  // namespace dnnmg

@@ -262,24 +262,140 @@ struct NodeLevel {
   T h, h2;              // mesh width and its square
 };
 
-// Stage the nodes around tile (i0, j0), three per lane; the iterate is read
-// through L2 (other SMs wrote it).
+// ---- the iterate of a level ------------------------------------------------------------
+// PlanarX: [3][nn] arrays; a grid-wide barrier separates the phases that write
+// and read it.
+// TaggedX: every node's values carry the number of the update that wrote them,
+// in the same 16-byte word (FP32: u, v, p, tag; FP64: three words of a value and
+// a tag), which is stored and loaded as one access.  A reader waits until the
+// tag is the one it needs, so that consecutive phases need no grid-wide barrier:
+// the barrier's chain (stores acknowledged, an atomic, a poll) and the load
+// behind it become one store and one polled load.  Two buffers suffice: the
+// tile that overwrites a node has waited for the values of every tile that read
+// the node's previous ones (they lie within its own two-node halo).  Tags never
+// repeat: they hold the cycle's number, kept on the device.  The wait is
+// bounded (kTagPolls rounds over a warp's whole run; then bit 8 of *status is
+// set and the warp stops waiting).  All lanes of the warp call load.
+constexpr int kTagPolls = 1 << 21;
+
 template <typename T>
-__device__ __forceinline__ void stage_warp_tile(const NodeLevel<T>& L, const T* x, int i0, int j0,
-                                                int lane, WarpTile<T>& S) {
+struct PlanarX {
+  const T* in;
+  T* out;
+  int nn;
+  template <int N>
+  __device__ __forceinline__ void load(const int (&n)[N], const bool (&)[N], T (&u)[N], T (&v)[N],
+                                       T (&p)[N], int&) const {
+#pragma unroll
+    for (int r = 0; r < N; ++r)
+      u[r] = __ldcg(in + n[r]), v[r] = __ldcg(in + nn + n[r]), p[r] = __ldcg(in + 2 * nn + n[r]);
+  }
+  __device__ __forceinline__ void store(int n, T u, T v, T p) const {
+    out[n] = u, out[nn + n] = v, out[2 * nn + n] = p;
+  }
+  __device__ __forceinline__ void store_one(int n, int c, T v) const { out[c * nn + n] = v; }
+};
+
+__device__ __forceinline__ void ld_pair(const ulonglong2* p, unsigned long long& a,
+                                        unsigned long long& b) {
+  asm volatile("{ .reg .b128 t; ld.relaxed.gpu.global.b128 t, [%2]; mov.b128 {%0, %1}, t; }"
+               : "=l"(a), "=l"(b)
+               : "l"(p)
+               : "memory");
+}
+__device__ __forceinline__ void st_pair(ulonglong2* p, unsigned long long a, unsigned long long b) {
+  asm volatile("{ .reg .b128 t; mov.b128 t, {%1, %2}; st.relaxed.gpu.global.b128 [%0], t; }" ::"l"(p),
+               "l"(a), "l"(b)
+               : "memory");
+}
+
+// words of a node in a tagged buffer
+template <typename T>
+constexpr int kTagWords = sizeof(T) == 4 ? 1 : 3;
+
+template <typename T>
+struct TaggedX {
+  const ulonglong2* in;
+  ulonglong2* out;
+  T* planar;  // when set, the values go there instead (the cycle's result)
+  int nn;
+  unsigned tin, tout;
+  int* status;
+  template <int N>
+  __device__ __forceinline__ void load(const int (&n)[N], const bool (&need)[N], T (&u)[N],
+                                       T (&v)[N], T (&p)[N], int& budget) const {
+    bool ready;
+    do {
+      ready = true;
+#pragma unroll
+      for (int r = 0; r < N; ++r) {
+        unsigned long long a, b;
+        if constexpr (sizeof(T) == 4) {
+          ld_pair(in + n[r], a, b);
+          u[r] = __uint_as_float((unsigned)a);
+          v[r] = __uint_as_float((unsigned)(a >> 32));
+          p[r] = __uint_as_float((unsigned)b);
+          ready = ready && (!need[r] || (unsigned)(b >> 32) == tin);
+        } else {
+          T* const o[3] = {&u[r], &v[r], &p[r]};
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            ld_pair(in + c * nn + n[r], a, b);
+            *o[c] = __longlong_as_double((long long)a);
+            ready = ready && (!need[r] || (unsigned)b == tin);
+          }
+        }
+      }
+      // the warp stays together: lanes that left one by one would run what
+      // follows in turn (FP64 tiles 13.6 k instead of 5.9 k cycles)
+      ready = __all_sync(0xffffffffu, ready);
+    } while (!ready && --budget > 0);
+    if (!ready) {
+      budget = 1;
+      atomicOr(status, 8);
+    }
+  }
+  __device__ __forceinline__ void store(int n, T u, T v, T p) const {
+    if (planar) {
+      planar[n] = u, planar[nn + n] = v, planar[2 * nn + n] = p;
+    } else if constexpr (sizeof(T) == 4) {
+      st_pair(out + n,
+              (unsigned long long)__float_as_uint(u) |
+                  ((unsigned long long)__float_as_uint(v) << 32),
+              (unsigned long long)__float_as_uint(p) | ((unsigned long long)tout << 32));
+    } else {
+      store_one(n, 0, u), store_one(n, 1, v), store_one(n, 2, p);
+    }
+  }
+  __device__ __forceinline__ void store_one(int n, int c, T v) const {  // FP64
+    if (planar)
+      planar[c * nn + n] = v;
+    else
+      st_pair(out + c * nn + n, (unsigned long long)__double_as_longlong((double)v), tout);
+  }
+};
+
+// Stage the nodes around tile (i0, j0), three per lane, and load this lane's own
+// node `own` (its unmasked values; -1: none).
+template <typename T, bool OWN, class X>
+__device__ __forceinline__ void stage_warp_tile(const NodeLevel<T>& L, const X& x, int i0, int j0,
+                                                int lane, int own, WarpTile<T>& S, T& xu, T& xv,
+                                                T& xp, int& budget) {
   static_assert(kWSX * kWSY == 96, "three nodes per lane");
-  T u[3], v[3], p[3];
-  int pt[3];
+  constexpr int N = OWN ? 4 : 3;
+  T u[N], v[N], p[N];
+  int pt[3], n[N];
+  bool in[N];
 #pragma unroll
   for (int r = 0; r < 3; ++r) {
     const int e = lane + 32 * r, i = i0 - 2 + e % kWSX, j = j0 - 2 + e / kWSX;
-    const bool in = i >= 0 && j >= 0 && i <= L.nx && j <= L.ny;
-    const int n = in ? j * L.nnx + i : 0;
-    pt[r] = in ? (int)__ldg(L.pat + n) : (kPatVDir | kPatPFix);
-    u[r] = __ldcg(x + n);
-    v[r] = __ldcg(x + L.nn + n);
-    p[r] = __ldcg(x + 2 * L.nn + n);
+    in[r] = i >= 0 && j >= 0 && i <= L.nx && j <= L.ny;
+    n[r] = in[r] ? j * L.nnx + i : 0;
+    pt[r] = in[r] ? (int)__ldg(L.pat + n[r]) : (kPatVDir | kPatPFix);
   }
+  if constexpr (OWN) in[3] = own >= 0, n[3] = in[3] ? own : 0;
+  x.template load<N>(n, in, u, v, p, budget);
+  if constexpr (OWN) xu = u[3], xv = v[3], xp = p[3];
 #pragma unroll
   for (int r = 0; r < 3; ++r) {
     const int e = lane + 32 * r, li = e % kWSX, lj = e / kWSX;
@@ -324,11 +440,11 @@ __device__ __forceinline__ void node_rows_assembled(const NodeLevel<T>& L, const
 
 // One colour pass (see vanka_body.cuh) on the warp's 4 x 2 colour cells (bx,
 // by).  Lane 4 q + a owns node a of cell q.
-template <typename T>
+template <typename T, class X>
 __device__ __forceinline__ void warp_pass_tile(const NodeLevel<T>& L, const OpTable<T>& tab,
-                                               int colour, const T* b, const T* xin, const T* inv,
-                                               int pitch, int nslots, T omega, T* xout, int bx,
-                                               int by, int lane, WarpTile<T>& S) {
+                                               int colour, const T* b, const X& x, const T* inv,
+                                               int pitch, int nslots, T omega, int bx, int by,
+                                               int lane, WarpTile<T>& S, int& budget) {
   const int cx = colour & 1, cy = colour >> 1;
   const int i0 = kWX * bx - cx, j0 = kWY * by - cy;
   const int q = lane >> 2, a = lane & 3;
@@ -338,13 +454,12 @@ __device__ __forceinline__ void warp_pass_tile(const NodeLevel<T>& L, const OpTa
   const int n = node_ok ? j * L.nnx + i : 0;
   const int slot = node_ok ? (2 * by + (q >> 2)) * pitch + 4 * bx + (q & 3) : 0;
   // every load of the tile is issued before the first is used
-  T c[36], iv[36];
+  T c[36], iv[36], xu, xv, xp;
   load36<T>(L.cf, n, L.nn, c);
   load_inv_rows<T>(inv, nslots, colour, slot, a, iv);
   const int pt = node_ok ? (int)__ldg(L.pat + n) : 0;
-  const T xu = __ldcg(xin + n), xv = __ldcg(xin + L.nn + n), xp = __ldcg(xin + 2 * L.nn + n);
   const T bu = __ldcg(b + n), bv = __ldcg(b + L.nn + n), bp = __ldcg(b + 2 * L.nn + n);
-  stage_warp_tile<T>(L, xin, i0, j0, lane, S);
+  stage_warp_tile<T, true>(L, x, i0, j0, lane, node_ok ? n : -1, S, xu, xv, xp, budget);
   __syncwarp();
   // the cell is fluid: its bit in the node's pattern
   const bool cell_ok = node_ok && ((pt >> ((1 - (a & 1)) + 2 * (1 - (a >> 1)))) & 1);
@@ -367,11 +482,87 @@ __device__ __forceinline__ void warp_pass_tile(const NodeLevel<T>& L, const OpTa
 #pragma unroll
       for (int k = 0; k < 12; ++k) acc[r] += iv[r * 12 + k] * d[k];
     }
-    xout[n] = cell_ok ? xu + omega * acc[0] : xu;
-    xout[L.nn + n] = cell_ok ? xv + omega * acc[1] : xv;
-    xout[2 * L.nn + n] = cell_ok ? xp + omega * acc[2] : xp;
+    x.store(n, cell_ok ? xu + omega * acc[0] : xu, cell_ok ? xv + omega * acc[1] : xv,
+            cell_ok ? xp + omega * acc[2] : xp);
   }
   __syncwarp();  // the tile's shared memory is reused
+}
+
+// The first colour pass of a smoothing sweep that starts from x = 0, for
+// item e = 4 * slot + a (node a of the colour cell of `slot`): the defect is
+// then b on every row (b - A 0 = b, and b - x = b on constrained rows), so
+// the pass needs neither the iterate nor any operator rows:
+// x_out = omega A_c^-1 b on the colour's fluid cells and 0 on every other
+// node, bitwise what the tiled pass computes from x = 0, and every node of the
+// level is written.  The four items of a cell are consecutive lanes of one
+// warp; all 32 lanes call this (valid = false for padding items).
+template <typename T, class X>
+__device__ __forceinline__ void zero_pass_node(const Grid& g, int colour, const T* b, const X& x,
+                                               const T* inv, T omega, int e, bool valid) {
+  const int cx = colour & 1, cy = colour >> 1;
+  const int sx = g.nx / 2 + 1, pitch = vanka_pitch(g), nslots = vanka_slots(g), nn = g.nn;
+  const int slot = e >> 2, a = e & 3;
+  const bool slot_ok = valid && slot < nslots && slot % pitch < sx;
+  const int ci = 2 * (slot % pitch) - cx, cj = 2 * (slot / pitch) - cy;
+  const int i = ci + (a & 1), j = cj + (a >> 1);
+  const bool node_ok = slot_ok && i >= 0 && j >= 0 && i <= g.nx && j <= g.ny;
+  const bool cell_ok = slot_ok && ci >= 0 && cj >= 0 && ci < g.nx && cj < g.ny &&
+                       !g.solid[cj * g.nx + ci];
+  const int n = node_ok ? j * g.nnx + i : 0;
+  T du = 0, dv = 0, dp = 0;
+  if (node_ok) du = __ldcg(b + n), dv = __ldcg(b + nn + n), dp = __ldcg(b + 2 * nn + n);
+  const int base = (threadIdx.x & 31) & ~3;
+  T d[12];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    d[k] = __shfl_sync(0xffffffffu, du, base + k);
+    d[4 + k] = __shfl_sync(0xffffffffu, dv, base + k);
+    d[8 + k] = __shfl_sync(0xffffffffu, dp, base + k);
+  }
+  if (!node_ok) return;
+  T acc[3] = {T(0), T(0), T(0)};
+  if (cell_ok) {
+    T iv[36];
+    load_inv_rows<T>(inv, nslots, colour, slot, a, iv);
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int k = 0; k < 12; ++k) acc[c] += iv[c * 12 + k] * d[k];
+  }
+  x.store(n, omega * acc[0], omega * acc[1], omega * acc[2]);
+}
+
+// x += P xc at fine node (i, j) on free unknowns (prolong_add_node of vbody.cuh).
+// All lanes of a warp call it.
+template <typename T, class XC, class XF>
+__device__ __forceinline__ void prolong_node(const Grid& f, const Grid& c, const XC& xc,
+                                             const XF& x, int i, int j, bool valid, int& budget) {
+  const int I0 = i >> 1, J0 = j >> 1, nI = (i & 1) ? 2 : 1, nJ = (j & 1) ? 2 : 1;
+  int m[4], n[1] = {j * f.nnx + i};
+  bool use[4], one[1] = {valid};
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    use[e] = valid && (e & 1) < nI && (e >> 1) < nJ;
+    m[e] = use[e] ? (J0 + (e >> 1)) * c.nnx + I0 + (e & 1) : J0 * c.nnx + I0;
+  }
+  const uint8_t fl = f.flags[n[0]];
+  uint8_t cfl[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) cfl[e] = use[e] ? c.flags[m[e]] : uint8_t(0xFF);
+  T xv[3][1], cv[3][4];
+  x.template load<1>(n, one, xv[0], xv[1], xv[2], budget);
+  xc.template load<4>(m, use, cv[0], cv[1], cv[2], budget);
+  const T w = T(1) / T(nI * nJ);
+#pragma unroll
+  for (int comp = 0; comp < 3; ++comp) {
+    const uint8_t bit = comp < 2 ? kVDir : kPFix;
+    T acc = 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (!(cfl[e] & bit)) acc += cv[comp][e];
+    if (!(fl & bit)) xv[comp][0] += w * acc;
+  }
+  if (valid) x.store(n[0], xv[0][0], xv[1][0], xv[2][0]);
 }
 
 // ---- one warp, 4 x 2 nodes: four lanes per node -----------------------------------------
@@ -389,22 +580,25 @@ __device__ __forceinline__ T quad_sum(T v) {
   return v + __shfl_xor_sync(0xffffffffu, v, 2);
 }
 
-// Stage the 8 x 6 nodes around tile (i0, j0).
-template <typename T>
-__device__ __forceinline__ void stage_split_tile(const NodeLevel<T>& L, const T* x, int i0, int j0,
-                                                 int lane, WarpTile<T>& S) {
-  T u[2], v[2], p[2];
-  int pt[2];
+// Stage the 8 x 6 nodes around tile (i0, j0) and load this lane's own node.
+template <typename T, bool OWN, class X>
+__device__ __forceinline__ void stage_split_tile(const NodeLevel<T>& L, const X& x, int i0, int j0,
+                                                 int lane, int own, WarpTile<T>& S, T& xu, T& xv,
+                                                 T& xp, int& budget) {
+  constexpr int N = OWN ? 3 : 2;
+  T u[N], v[N], p[N];
+  int pt[2], n[N];
+  bool in[N];
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
     const int e = lane + 32 * r, i = i0 - 2 + e % kSSX, j = j0 - 2 + e / kSSX;
-    const bool in = e < kSSX * kSSY && i >= 0 && j >= 0 && i <= L.nx && j <= L.ny;
-    const int n = in ? j * L.nnx + i : 0;
-    pt[r] = in ? (int)__ldg(L.pat + n) : (kPatVDir | kPatPFix);
-    u[r] = __ldcg(x + n);
-    v[r] = __ldcg(x + L.nn + n);
-    p[r] = __ldcg(x + 2 * L.nn + n);
+    in[r] = e < kSSX * kSSY && i >= 0 && j >= 0 && i <= L.nx && j <= L.ny;
+    n[r] = in[r] ? j * L.nnx + i : 0;
+    pt[r] = in[r] ? (int)__ldg(L.pat + n[r]) : (kPatVDir | kPatPFix);
   }
+  if constexpr (OWN) in[2] = own >= 0, n[2] = in[2] ? own : 0;
+  x.template load<N>(n, in, u, v, p, budget);
+  if constexpr (OWN) xu = u[2], xv = v[2], xp = p[2];
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
     const int e = lane + 32 * r, li = e % kSSX, lj = e / kSSX;
@@ -463,11 +657,11 @@ __device__ __forceinline__ void node_rows_split(const NodeLevel<T>& L, const OpT
 }
 
 // One colour pass on the warp's 2 x 1 colour cells (bx, by).
-template <typename T>
+template <typename T, class X>
 __device__ __forceinline__ void split_pass_tile(const NodeLevel<T>& L, const OpTable<T>& tab,
-                                                int colour, const T* b, const T* xin, const T* inv,
-                                                int pitch, int nslots, T omega, T* xout, int bx,
-                                                int by, int lane, WarpTile<T>& S) {
+                                                int colour, const T* b, const X& x, const T* inv,
+                                                int pitch, int nslots, T omega, int bx, int by,
+                                                int lane, WarpTile<T>& S, int& budget) {
   const int cx = colour & 1, cy = colour >> 1;
   const int i0 = kSX * bx - cx, j0 = kSY * by - cy;
   const int q = lane >> 4, a = (lane >> 2) & 3, s = lane & 3;
@@ -483,9 +677,9 @@ __device__ __forceinline__ void split_pass_tile(const NodeLevel<T>& L, const OpT
     for (int k = 0; k < 3; ++k)
       iv[r][k] = __ldg(inv + vanka_inv_index<T>(nslots, colour, slot, a, r * 12 + 4 * k + s));
   const int pt = node_ok ? (int)__ldg(L.pat + n) : 0;
-  const T xu = __ldcg(xin + n), xv = __ldcg(xin + L.nn + n), xp = __ldcg(xin + 2 * L.nn + n);
   const T bu = __ldcg(b + n), bv = __ldcg(b + L.nn + n), bp = __ldcg(b + 2 * L.nn + n);
-  stage_split_tile<T>(L, xin, i0, j0, lane, S);
+  T xu, xv, xp;
+  stage_split_tile<T, true>(L, x, i0, j0, lane, node_ok ? n : -1, S, xu, xv, xp, budget);
   __syncwarp();
   const bool cell_ok = node_ok && ((pt >> ((1 - (a & 1)) + 2 * (1 - (a >> 1)))) & 1);
   T ru, rv, rp;
@@ -499,17 +693,17 @@ __device__ __forceinline__ void split_pass_tile(const NodeLevel<T>& L, const OpT
 #pragma unroll
   for (int r = 0; r < 3; ++r) acc[r] = quad_sum(iv[r][0] * d0 + iv[r][1] * d1 + iv[r][2] * d2);
   if (node_ok && s < 3) {  // lane s writes component s
-    const T x = s == 0 ? xu : (s == 1 ? xv : xp), y = s == 0 ? acc[0] : (s == 1 ? acc[1] : acc[2]);
-    xout[s * L.nn + n] = cell_ok ? x + omega * y : x;
+    const T o = s == 0 ? xu : (s == 1 ? xv : xp), y = s == 0 ? acc[0] : (s == 1 ? acc[1] : acc[2]);
+    x.store_one(n, s, cell_ok ? o + omega * y : o);
   }
   __syncwarp();
 }
 
 // d = b - A'(vbar) x, zero on constrained unknowns, on the warp's 4 x 2 nodes.
-template <typename T>
+template <typename T, class X>
 __device__ __forceinline__ void split_defect_tile(const NodeLevel<T>& L, const OpTable<T>& tab,
-                                                  const T* b, const T* x, T* d, int bx, int by,
-                                                  int lane, WarpTile<T>& S) {
+                                                  const T* b, const X& x, T* d, int bx, int by,
+                                                  int lane, WarpTile<T>& S, int& budget) {
   const int i0 = kSX * bx, j0 = kSY * by, m = lane >> 2, s = lane & 3;
   const int li = m % kSX, lj = m / kSX, i = i0 + li, j = j0 + lj;
   const bool ok = i <= L.nx && j <= L.ny;
@@ -518,7 +712,8 @@ __device__ __forceinline__ void split_defect_tile(const NodeLevel<T>& L, const O
   load_split_blocks<T>(L, n, s, c);
   const int pt = ok ? (int)__ldg(L.pat + n) : 0;
   const T bb = __ldcg(b + (s < 3 ? s : 0) * L.nn + n);
-  stage_split_tile<T>(L, x, i0, j0, lane, S);
+  T xu, xv, xp;
+  stage_split_tile<T, false>(L, x, i0, j0, lane, -1, S, xu, xv, xp, budget);
   __syncwarp();
   T ru, rv, rp;
   node_rows_split<T>(L, tab, S, c, li + 2, lj + 2, pt, (i & 1) + 2 * (j & 1), s, ru, rv, rp);
@@ -530,10 +725,10 @@ __device__ __forceinline__ void split_defect_tile(const NodeLevel<T>& L, const O
 }
 
 // d = b - A'(vbar) x, zero on constrained unknowns, on the warp's 8 x 4 nodes.
-template <typename T>
+template <typename T, class X>
 __device__ __forceinline__ void warp_defect_tile(const NodeLevel<T>& L, const OpTable<T>& tab,
-                                                 const T* b, const T* x, T* d, int bx, int by,
-                                                 int lane, WarpTile<T>& S) {
+                                                 const T* b, const X& x, T* d, int bx, int by,
+                                                 int lane, WarpTile<T>& S, int& budget) {
   const int i0 = kWX * bx, j0 = kWY * by, li = lane % kWX, lj = lane / kWX;
   const int i = i0 + li, j = j0 + lj;
   const bool ok = i <= L.nx && j <= L.ny;
@@ -542,7 +737,8 @@ __device__ __forceinline__ void warp_defect_tile(const NodeLevel<T>& L, const Op
   load36<T>(L.cf, n, L.nn, c);
   const int pt = ok ? (int)__ldg(L.pat + n) : 0;
   const T bu = __ldcg(b + n), bv = __ldcg(b + L.nn + n), bp = __ldcg(b + 2 * L.nn + n);
-  stage_warp_tile<T>(L, x, i0, j0, lane, S);
+  T xu, xv, xp;
+  stage_warp_tile<T, false>(L, x, i0, j0, lane, -1, S, xu, xv, xp, budget);
   __syncwarp();
   T ru, rv, rp;
   node_rows_assembled<T>(L, tab, S, c, li + 2, lj + 2, pt, (i & 1) + 2 * (j & 1), ru, rv, rp);
