@@ -328,7 +328,7 @@ int Batch<T>::init() {
       l.mode = c.lps_mode;
       if (k >= 2) {
         l.inv = mem_.alloc<T>((size_t)4 * 144 * vanka_slots(g));
-        l.cf = mem_.alloc<T>((size_t)36 * g.nn);
+        l.cf = mem_.alloc<T>((size_t)kCoefs<T> * g.nn);
         const std::vector<uint16_t> pat = node_patterns(hl_[p][k]);
         uint16_t* dp = mem_.alloc<uint16_t>(pat.size());
         if (!mem_.ok()) return fail(DNNMG_ERR_CUDA, "device allocation failed");

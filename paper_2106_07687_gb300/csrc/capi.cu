@@ -114,6 +114,7 @@ Sten<T> make_sten(double h, const dnnmg_config& c) {
       Dy[a][b] = m1[ax][bx] * c1[ay][by];
     }
   Sten<T> s;
+  s.Es = (T)(h * h / 4 / c.dt);  // K has zero row sums
   for (int a = 0; a < 4; ++a)
     for (int b = 0; b < 4; ++b) {
       s.E[a * 4 + b] = (T)(M[a][b] / c.dt + c.theta * c.nu * K[a][b]);

@@ -32,6 +32,7 @@ struct Grid {
 template <typename T>
 struct Sten {
   T E[16];    // (1/k) M + theta nu K  (row a, column b)
+  T Es;       // the sum of a row of E
   T Dx[16];   // int xi_a d/dx phi_b
   T Dy[16];   // int xi_a d/dy phi_b
   T S9[81];   // alpha kappa^T K9 kappa on the 3x3 nodes of a patch

@@ -47,7 +47,7 @@ class Solver final : public SolverBase {
       if (k > 0) {
         l.inv = c_->mem.alloc<T>((size_t)4 * 144 * vanka_slots(l.g));
         const std::vector<uint16_t> pat = node_patterns(c_->lv[l.level]);
-        l.cf = c_->mem.alloc<T>(36 * (size_t)l.g.nn);
+        l.cf = c_->mem.alloc<T>(kCoefs<T> * (size_t)l.g.nn);
         l.pat = c_->mem.alloc<uint16_t>(pat.size());
         if (!c_->mem.ok()) return c_->fail(DNNMG_ERR_CUDA, "device allocation failed");
         cudaMemcpyAsync(l.pat, pat.data(), sizeof(uint16_t) * pat.size(), cudaMemcpyHostToDevice,

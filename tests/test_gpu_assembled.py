@@ -40,3 +40,22 @@ def test_assembled_cycle_matches_cell_by_cell_cycle(precision, tol, mode, L, ob,
     # the tiles wait for each other's updates one by one: the same values whatever the order
     for _ in range(20):
         assert (walk.vcycle(L, b).double().cpu().numpy() == out[1]).all()
+
+
+@pytest.mark.parametrize("L,nu,dt", [(2, 0.004, 0.02), (3, 0.01, 0.005), (5, 0.0065, 0.005)])
+def test_fp32_rows_act_on_differences(L, nu, dt):
+    """FP32 rows are applied to differences of the iterate, so that a cycle's
+    error against FP64 stays at a few of the result's own roundings (6e-8)
+    instead of their amplification by a smooth pressure (1e-6 and more)."""
+    dn = lib()
+    lev = mesh.Level(L, obstacle=(2, 1))
+    x = torch.from_numpy(seeded_state(lev, 7)).cuda()
+    g = torch.Generator().manual_seed(17 + L)
+    b = torch.randn(lev.ndof, generator=g, dtype=torch.float64).float()
+    out = []
+    for precision in (0, 1):
+        c = dn.Context(level_solve=L, precision=precision, obstacle_i0=2, obstacle_j0=1, nu=nu,
+                       dt=dt, persistent_vcycle=L, persistent_mode=0)
+        c.linearize(x)
+        out.append(c.vcycle(L, b.to(c.vdtype).cuda()).double().cpu().numpy())
+    assert rel(out[1], out[0]) < 1e-6, rel(out[1], out[0])
