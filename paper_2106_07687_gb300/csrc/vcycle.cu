@@ -16,7 +16,7 @@
 // after the defect, the restriction and the coarse solve, whose outputs are
 // plain arrays.  One cycle, barriers after every phase -> numbered updates: FP32
 // on levels 3 / 5 / 6 (128x32, 512x128, 1024x256 cells) 92 -> 82, 244 -> 185,
-// 528 -> 430 us, FP64 on level 3 191 -> 154 us.
+// 528 -> 430 us (72, 168, 407 us since), FP64 on level 3 191 -> 154 us (151).
 #include <algorithm>
 #include <cooperative_groups.h>
 
@@ -33,6 +33,26 @@ namespace {
 constexpr int kMaxPhases = 160;  // phases of one launch (a V(2,2) cycle from level 8)
 constexpr int kMaxVLevels = 10;
 
+// What a colour pass or defect reads of its phase and level, resolved once per
+// launch: a phase is a chain of dependent steps, and looking its level up,
+// dividing by its tile counts and rounding its mesh width took 700 of its 4,400
+// cycles (FP32; one cycle on 512x128 cells 180 -> 168 us).
+template <typename T>
+struct alignas(16) PassRec {
+  int type, colour;
+  int nx, ny, nnx, nn, pitch, nslots;
+  int tiles, nbx;      // warp tiles, and how many in a row
+  unsigned inv_nbx;    // 2^32 / nbx, rounded up (nbx > 1): t / nbx for t nbx < 2^32
+  int split;           // four lanes per node
+  unsigned tin, tout;
+  T h, h2;
+  const T *b, *inv, *cf;
+  const uint16_t* pat;
+  const ulonglong2* in;
+  ulonglong2* out;
+  T *planar, *d;
+};
+
 // Dynamic shared memory of a block: the launch's phase list, level records
 // and coefficient table, loaded once so that no phase starts with a dependent
 // global load, and a scratch area for the warp tiles or the coarse vector.
@@ -41,6 +61,7 @@ struct WalkSmem {
   OpTable<T> tab;
   VLevel<T> lv[kMaxVLevels];
   Phase ph[kMaxPhases];
+  PassRec<T> rec[kMaxPhases];
   alignas(16) WarpTile<T> tile[walk_threads<T>() / 32];
 };
 
@@ -75,19 +96,71 @@ __device__ __forceinline__ void walk_phases(const VLevel<T>* glv, const OpTable<
   copy_ints(&S.tab, gtab, 1);
   const unsigned cycle = __ldcg(reinterpret_cast<unsigned*>(state) + 1), tag0 = cycle << 8;
   __syncthreads();
+  for (int p = threadIdx.x; p < nph; p += NT) {
+    const Phase f = S.ph[p];
+    const VLevel<T>& L = S.lv[f.level];
+    const Grid& g = L.g;
+    PassRec<T> r;
+    r.type = f.type, r.colour = f.colour;
+    r.nx = g.nx, r.ny = g.ny, r.nnx = g.nnx, r.nn = g.nn;
+    r.pitch = vanka_pitch(g), r.nslots = vanka_slots(g);
+    // FP64: four lanes per node while that gives every scheduler (four per
+    // block) at most little more than one warp.  On 152 blocks that is up to
+    // level 3 (612 warps): one cycle with barriers, one -> four lanes per node on
+    // levels 2 and 3, 287 -> 191 us on 128x32, 435 -> 339 us on 256x64; with level
+    // 4 (2,244 warps) as well 401 us.  In FP32 the same gains 2 us a cycle, but
+    // the larger kernel loses 15 (its instructions come through the cache once
+    // per phase).
+    r.split = sizeof(T) == 8 && 4 * cdiv(g.nnx, kWX) * cdiv(g.nny, kWY) <= 5 * (int)gridDim.x;
+    const int sx = r.split ? kSX : kWX, sy = r.split ? kSY : kWY;
+    if (f.type == kPhasePass) {
+      r.nbx = cdiv(g.nx / 2 + 1, sx / 2);
+      r.tiles = r.nbx * cdiv(g.ny / 2 + 1, sy / 2);
+    } else {
+      r.nbx = cdiv(g.nnx, sx);
+      r.tiles = r.nbx * cdiv(g.nny, sy);
+    }
+    r.inv_nbx = 0xFFFFFFFFu / r.nbx + 1u;
+    r.tin = tag0 + f.tin, r.tout = tag0 + f.tout;
+    r.h = (T)g.h, r.h2 = (T)(g.h * g.h);
+    r.b = f.level == top ? topb : L.b;
+    r.inv = L.inv, r.cf = L.cf, r.pat = L.pat;
+    const size_t words = (size_t)kTagWords<T> * g.nn;
+    r.in = L.xt + f.in * words, r.out = L.xt + f.out * words;
+    r.planar = f.last ? topx : nullptr;
+    r.d = L.d;
+    S.rec[p] = r;
+  }
+  __syncthreads();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int w0 = blockIdx.x + gridDim.x * w, nw = gridDim.x * (NT / 32);
   int budget = kTagPolls;
-  // FP64: four lanes per node while that gives every scheduler (four per block)
-  // at most little more than one warp.  On 152 blocks that is up to level 3
-  // (612 warps): one cycle with barriers, one -> four lanes per node on levels 2
-  // and 3, 287 -> 191 us on 128x32, 435 -> 339 us on 256x64; with level 4 (2,244
-  // warps) as well 401 us.  In FP32 the same gains 2 us a cycle, but the larger
-  // kernel loses 15 (its instructions come through the cache once per phase).
-  auto split_level = [&](const Grid& g) {
-    return 4 * cdiv(g.nnx, kWX) * cdiv(g.nny, kWY) <= 5 * (int)gridDim.x;
-  };
   for (int p = 0; p < nph; ++p) {
+    const PassRec<T>& R = S.rec[p];
+    const int type = R.type;
+    if (type == kPhasePass || type == kPhaseDefect) {
+      const TaggedX<T> x{R.in, R.out, R.planar, R.nn, R.tin, R.tout, state};
+      const NodeLevel<T> N{R.nx, R.ny, R.nnx, R.nn, R.pat, R.cf, R.h, R.h2};
+      for (int t = w0; t < R.tiles; t += nw) {
+        const int by = __umulhi(t, R.inv_nbx), bx = t - by * R.nbx;
+        if constexpr (sizeof(T) == 8)
+          if (R.split) {
+            if (type == kPhasePass)
+              split_pass_tile<T>(N, S.tab, R.colour, R.b, x, R.inv, R.pitch, R.nslots, omega, bx,
+                                 by, lane, S.tile[w], budget);
+            else
+              split_defect_tile<T>(N, S.tab, R.b, x, R.d, bx, by, lane, S.tile[w], budget);
+            continue;
+          }
+        if (type == kPhasePass)
+          warp_pass_tile<T>(N, S.tab, R.colour, R.b, x, R.inv, R.pitch, R.nslots, omega, bx, by,
+                            lane, S.tile[w], budget);
+        else
+          warp_defect_tile<T>(N, S.tab, R.b, x, R.d, bx, by, lane, S.tile[w], budget);
+      }
+      if (type == kPhaseDefect) sync();
+      continue;
+    }
     const Phase f = S.ph[p];
     const int k = f.level;
     const VLevel<T>& L = S.lv[k];
@@ -96,40 +169,8 @@ __device__ __forceinline__ void walk_phases(const VLevel<T>* glv, const OpTable<
     const size_t words = (size_t)kTagWords<T> * g.nn;
     const TaggedX<T> x{L.xt + f.in * words, L.xt + f.out * words, f.last ? topx : nullptr, g.nn,
                        tag0 + f.tin,        tag0 + f.tout,        state};
-    const NodeLevel<T> N{g.nx, g.ny, g.nnx, g.nn, L.pat, L.cf, (T)g.h, (T)(g.h * g.h)};
     bool barrier = false;
     switch (f.type) {
-      case kPhasePass: {
-        const int pitch = vanka_pitch(g), nslots = vanka_slots(g);
-        if constexpr (sizeof(T) == 8)
-          if (split_level(g)) {
-            const int nbx = cdiv(g.nx / 2 + 1, kSX / 2), nt = nbx * cdiv(g.ny / 2 + 1, kSY / 2);
-            for (int t = w0; t < nt; t += nw)
-              split_pass_tile<T>(N, S.tab, f.colour, b, x, L.inv, pitch, nslots, omega, t % nbx,
-                                 t / nbx, lane, S.tile[w], budget);
-            break;
-          }
-        const int nbx = cdiv(g.nx / 2 + 1, kWX / 2);
-        const int nt = nbx * cdiv(g.ny / 2 + 1, kWY / 2);
-        for (int t = w0; t < nt; t += nw)
-          warp_pass_tile<T>(N, S.tab, f.colour, b, x, L.inv, pitch, nslots, omega, t % nbx, t / nbx,
-                            lane, S.tile[w], budget);
-        break;
-      }
-      case kPhaseDefect: {
-        barrier = true;
-        if constexpr (sizeof(T) == 8)
-          if (split_level(g)) {
-            const int nbx = cdiv(g.nnx, kSX), nt = nbx * cdiv(g.nny, kSY);
-            for (int t = w0; t < nt; t += nw)
-              split_defect_tile<T>(N, S.tab, b, x, L.d, t % nbx, t / nbx, lane, S.tile[w], budget);
-            break;
-          }
-        const int nbx = cdiv(g.nnx, kWX), nt = nbx * cdiv(g.nny, kWY);
-        for (int t = w0; t < nt; t += nw)
-          warp_defect_tile<T>(N, S.tab, b, x, L.d, t % nbx, t / nbx, lane, S.tile[w], budget);
-        break;
-      }
       case kPhaseRestrict: {
         barrier = true;
         const VLevel<T>& C = S.lv[k - 1];

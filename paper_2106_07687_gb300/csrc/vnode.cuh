@@ -309,7 +309,9 @@ struct NodeLevel {
 // the node's previous ones (they lie within its own two-node halo).  Tags never
 // repeat: they hold the cycle's number, kept on the device.  The wait is
 // bounded (kTagPolls rounds over a warp's whole run; then bit 8 of *status is
-// set and the warp stops waiting).  All lanes of the warp call load.
+// set and the warp stops waiting).  All lanes of the warp call load; other_loads
+// is run once, behind the first round's loads, to issue what the tile reads
+// besides the iterate: the tags are then mostly there when it is through.
 constexpr int kTagPolls = 1 << 21;
 
 template <typename T>
@@ -317,12 +319,13 @@ struct PlanarX {
   const T* in;
   T* out;
   int nn;
-  template <int N>
+  template <int N, class F>
   __device__ __forceinline__ void load(const int (&n)[N], const bool (&)[N], T (&u)[N], T (&v)[N],
-                                       T (&p)[N], int&) const {
+                                       T (&p)[N], int&, F other_loads) const {
 #pragma unroll
     for (int r = 0; r < N; ++r)
       u[r] = __ldcg(in + n[r]), v[r] = __ldcg(in + nn + n[r]), p[r] = __ldcg(in + 2 * nn + n[r]);
+    other_loads();
   }
   __device__ __forceinline__ void store(int n, T u, T v, T p) const {
     out[n] = u, out[nn + n] = v, out[2 * nn + n] = p;
@@ -330,17 +333,17 @@ struct PlanarX {
   __device__ __forceinline__ void store_one(int n, int c, T v) const { out[c * nn + n] = v; }
 };
 
+// (no clobber of memory: nothing but these two touches a tagged buffer, and a
+// tag vouches for the values beside it only)
 __device__ __forceinline__ void ld_pair(const ulonglong2* p, unsigned long long& a,
                                         unsigned long long& b) {
   asm volatile("{ .reg .b128 t; ld.relaxed.gpu.global.b128 t, [%2]; mov.b128 {%0, %1}, t; }"
                : "=l"(a), "=l"(b)
-               : "l"(p)
-               : "memory");
+               : "l"(p));
 }
 __device__ __forceinline__ void st_pair(ulonglong2* p, unsigned long long a, unsigned long long b) {
   asm volatile("{ .reg .b128 t; mov.b128 t, {%1, %2}; st.relaxed.gpu.global.b128 [%0], t; }" ::"l"(p),
-               "l"(a), "l"(b)
-               : "memory");
+               "l"(a), "l"(b));
 }
 
 // words of a node in a tagged buffer
@@ -355,39 +358,53 @@ struct TaggedX {
   int nn;
   unsigned tin, tout;
   int* status;
-  template <int N>
+  template <int N, class F>
   __device__ __forceinline__ void load(const int (&n)[N], const bool (&need)[N], T (&u)[N],
-                                       T (&v)[N], T (&p)[N], int& budget) const {
-    bool ready;
-    do {
-      ready = true;
-#pragma unroll
-      for (int r = 0; r < N; ++r) {
-        unsigned long long a, b;
-        if constexpr (sizeof(T) == 4) {
-          ld_pair(in + n[r], a, b);
-          u[r] = __uint_as_float((unsigned)a);
-          v[r] = __uint_as_float((unsigned)(a >> 32));
-          p[r] = __uint_as_float((unsigned)b);
-          ready = ready && (!need[r] || (unsigned)(b >> 32) == tin);
-        } else {
-          T* const o[3] = {&u[r], &v[r], &p[r]};
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            ld_pair(in + c * nn + n[r], a, b);
-            *o[c] = __longlong_as_double((long long)a);
-            ready = ready && (!need[r] || (unsigned)b == tin);
-          }
-        }
-      }
-      // the warp stays together: lanes that left one by one would run what
-      // follows in turn (FP64 tiles 13.6 k instead of 5.9 k cycles)
-      ready = __all_sync(0xffffffffu, ready);
-    } while (!ready && --budget > 0);
-    if (!ready) {
-      budget = 1;
+                                       T (&v)[N], T (&p)[N], int& budget, F other_loads) const {
+    unsigned long long q[N][sizeof(T) == 4 ? 2 : 6];
+    if constexpr (sizeof(T) == 8) other_loads();  // FP64 has no registers to spare for the tags
+    round(n, q);
+    if constexpr (sizeof(T) == 4) other_loads();
+    // the warp stays together: lanes that left one by one would run what
+    // follows in turn (FP64 tiles 13.6 k instead of 5.9 k cycles)
+    while (!__all_sync(0xffffffffu, ready(need, q)) && --budget > 0) round(n, q);
+    if (budget <= 0) {
+      budget = 0;
       atomicOr(status, 8);
     }
+#pragma unroll
+    for (int r = 0; r < N; ++r) {
+      if constexpr (sizeof(T) == 4) {
+        u[r] = __uint_as_float((unsigned)q[r][0]);
+        v[r] = __uint_as_float((unsigned)(q[r][0] >> 32));
+        p[r] = __uint_as_float((unsigned)q[r][1]);
+      } else {
+        u[r] = __longlong_as_double((long long)q[r][0]);
+        v[r] = __longlong_as_double((long long)q[r][2]);
+        p[r] = __longlong_as_double((long long)q[r][4]);
+      }
+    }
+  }
+  template <int N, int W>
+  __device__ __forceinline__ void round(const int (&n)[N], unsigned long long (&q)[N][W]) const {
+#pragma unroll
+    for (int r = 0; r < N; ++r)
+#pragma unroll
+      for (int c = 0; c < W / 2; ++c) ld_pair(in + c * nn + n[r], q[r][2 * c], q[r][2 * c + 1]);
+  }
+  template <int N, int W>
+  __device__ __forceinline__ bool ready(const bool (&need)[N],
+                                        const unsigned long long (&q)[N][W]) const {
+    bool ok = true;
+#pragma unroll
+    for (int r = 0; r < N; ++r)
+#pragma unroll
+      for (int c = 0; c < W / 2; ++c) {
+        const unsigned tag =
+            sizeof(T) == 4 ? (unsigned)(q[r][2 * c + 1] >> 32) : (unsigned)q[r][2 * c + 1];
+        ok = ok && (!need[r] || tag == tin);
+      }
+    return ok;
   }
   __device__ __forceinline__ void store(int n, T u, T v, T p) const {
     if (planar) {
@@ -411,10 +428,10 @@ struct TaggedX {
 
 // Stage the nodes around tile (i0, j0), three per lane, and load this lane's own
 // node `own` (its unmasked values; -1: none).
-template <typename T, bool OWN, class X>
+template <typename T, bool OWN, class X, class F>
 __device__ __forceinline__ void stage_warp_tile(const NodeLevel<T>& L, const X& x, int i0, int j0,
                                                 int lane, int own, WarpTile<T>& S, T& xu, T& xv,
-                                                T& xp, int& budget) {
+                                                T& xp, int& budget, F other_loads) {
   static_assert(kWSX * kWSY == 96, "three nodes per lane");
   constexpr int N = OWN ? 4 : 3;
   T u[N], v[N], p[N];
@@ -425,10 +442,14 @@ __device__ __forceinline__ void stage_warp_tile(const NodeLevel<T>& L, const X& 
     const int e = lane + 32 * r, i = i0 - 2 + e % kWSX, j = j0 - 2 + e / kWSX;
     in[r] = i >= 0 && j >= 0 && i <= L.nx && j <= L.ny;
     n[r] = in[r] ? j * L.nnx + i : 0;
-    pt[r] = in[r] ? (int)__ldg(L.pat + n[r]) : (kPatVDir | kPatPFix);
   }
   if constexpr (OWN) in[3] = own >= 0, n[3] = in[3] ? own : 0;
-  x.template load<N>(n, in, u, v, p, budget);
+  x.template load<N>(n, in, u, v, p, budget, [&] {
+    other_loads();
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+      pt[r] = in[r] ? (int)__ldg(L.pat + n[r]) : (kPatVDir | kPatPFix);
+  });
   if constexpr (OWN) xu = u[3], xv = v[3], xp = p[3];
 #pragma unroll
   for (int r = 0; r < 3; ++r) {
@@ -497,13 +518,16 @@ __device__ __forceinline__ void warp_pass_tile(const NodeLevel<T>& L, const OpTa
   const bool node_ok = i >= 0 && j >= 0 && i <= L.nx && j <= L.ny;
   const int n = node_ok ? j * L.nnx + i : 0;
   const int slot = node_ok ? (2 * by + (q >> 2)) * pitch + 4 * bx + (q & 3) : 0;
-  // every load of the tile is issued before the first is used
-  T c[36], iv[36], xu, xv, xp;
-  load36<T>(L.cf, n, L.nn, c);
-  load_inv_rows<T>(inv, nslots, colour, slot, a, iv);
-  const int pt = node_ok ? (int)__ldg(L.pat + n) : 0;
-  const T bu = __ldcg(b + n), bv = __ldcg(b + L.nn + n), bp = __ldcg(b + 2 * L.nn + n);
-  stage_warp_tile<T, true>(L, x, i0, j0, lane, node_ok ? n : -1, S, xu, xv, xp, budget);
+  // every load of the tile is issued before the first is used, the iterate's
+  // (behind which the others' latency hides) first
+  T c[36], iv[36], xu, xv, xp, bu, bv, bp;
+  int pt;
+  stage_warp_tile<T, true>(L, x, i0, j0, lane, node_ok ? n : -1, S, xu, xv, xp, budget, [&] {
+    load36<T>(L.cf, n, L.nn, c);
+    pt = node_ok ? (int)__ldg(L.pat + n) : 0;
+    bu = __ldcg(b + n), bv = __ldcg(b + L.nn + n), bp = __ldcg(b + 2 * L.nn + n);
+    load_inv_rows<T>(inv, nslots, colour, slot, a, iv);
+  });
   __syncwarp();
   // the cell is fluid: its bit in the node's pattern
   const bool cell_ok = node_ok && ((pt >> ((1 - (a & 1)) + 2 * (1 - (a >> 1)))) & 1);
@@ -589,13 +613,15 @@ __device__ __forceinline__ void prolong_node(const Grid& f, const Grid& c, const
     use[e] = valid && (e & 1) < nI && (e >> 1) < nJ;
     m[e] = use[e] ? (J0 + (e >> 1)) * c.nnx + I0 + (e & 1) : J0 * c.nnx + I0;
   }
-  const uint8_t fl = f.flags[n[0]];
-  uint8_t cfl[4];
-#pragma unroll
-  for (int e = 0; e < 4; ++e) cfl[e] = use[e] ? c.flags[m[e]] : uint8_t(0xFF);
+  uint8_t fl, cfl[4];
   T xv[3][1], cv[3][4];
-  x.template load<1>(n, one, xv[0], xv[1], xv[2], budget);
-  xc.template load<4>(m, use, cv[0], cv[1], cv[2], budget);
+  xc.template load<4>(m, use, cv[0], cv[1], cv[2], budget, [&] {
+    x.template load<1>(n, one, xv[0], xv[1], xv[2], budget, [&] {
+      fl = f.flags[n[0]];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) cfl[e] = use[e] ? c.flags[m[e]] : uint8_t(0xFF);
+    });
+  });
   const T w = T(1) / T(nI * nJ);
 #pragma unroll
   for (int comp = 0; comp < 3; ++comp) {
@@ -625,10 +651,10 @@ __device__ __forceinline__ T quad_sum(T v) {
 }
 
 // Stage the 8 x 6 nodes around tile (i0, j0) and load this lane's own node.
-template <typename T, bool OWN, class X>
+template <typename T, bool OWN, class X, class F>
 __device__ __forceinline__ void stage_split_tile(const NodeLevel<T>& L, const X& x, int i0, int j0,
                                                  int lane, int own, WarpTile<T>& S, T& xu, T& xv,
-                                                 T& xp, int& budget) {
+                                                 T& xp, int& budget, F other_loads) {
   constexpr int N = OWN ? 3 : 2;
   T u[N], v[N], p[N];
   int pt[2], n[N];
@@ -638,10 +664,14 @@ __device__ __forceinline__ void stage_split_tile(const NodeLevel<T>& L, const X&
     const int e = lane + 32 * r, i = i0 - 2 + e % kSSX, j = j0 - 2 + e / kSSX;
     in[r] = e < kSSX * kSSY && i >= 0 && j >= 0 && i <= L.nx && j <= L.ny;
     n[r] = in[r] ? j * L.nnx + i : 0;
-    pt[r] = in[r] ? (int)__ldg(L.pat + n[r]) : (kPatVDir | kPatPFix);
   }
   if constexpr (OWN) in[2] = own >= 0, n[2] = in[2] ? own : 0;
-  x.template load<N>(n, in, u, v, p, budget);
+  x.template load<N>(n, in, u, v, p, budget, [&] {
+    other_loads();
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+      pt[r] = in[r] ? (int)__ldg(L.pat + n[r]) : (kPatVDir | kPatPFix);
+  });
   if constexpr (OWN) xu = u[2], xv = v[2], xp = p[2];
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
@@ -713,17 +743,18 @@ __device__ __forceinline__ void split_pass_tile(const NodeLevel<T>& L, const OpT
   const bool node_ok = i >= 0 && j >= 0 && i <= L.nx && j <= L.ny;
   const int n = node_ok ? j * L.nnx + i : 0;
   const int slot = node_ok ? by * pitch + 2 * bx + q : 0;
-  T c[12], iv[3][3];
-  load_split_blocks<T>(L, n, s, c);
+  T c[12], iv[3][3], bu, bv, bp, xu, xv, xp;
+  int pt;
+  stage_split_tile<T, true>(L, x, i0, j0, lane, node_ok ? n : -1, S, xu, xv, xp, budget, [&] {
+    load_split_blocks<T>(L, n, s, c);
+    pt = node_ok ? (int)__ldg(L.pat + n) : 0;
+    bu = __ldcg(b + n), bv = __ldcg(b + L.nn + n), bp = __ldcg(b + 2 * L.nn + n);
 #pragma unroll
-  for (int r = 0; r < 3; ++r)
+    for (int r = 0; r < 3; ++r)
 #pragma unroll
-    for (int k = 0; k < 3; ++k)
-      iv[r][k] = __ldg(inv + vanka_inv_index<T>(nslots, colour, slot, a, r * 12 + 4 * k + s));
-  const int pt = node_ok ? (int)__ldg(L.pat + n) : 0;
-  const T bu = __ldcg(b + n), bv = __ldcg(b + L.nn + n), bp = __ldcg(b + 2 * L.nn + n);
-  T xu, xv, xp;
-  stage_split_tile<T, true>(L, x, i0, j0, lane, node_ok ? n : -1, S, xu, xv, xp, budget);
+      for (int k = 0; k < 3; ++k)
+        iv[r][k] = __ldg(inv + vanka_inv_index<T>(nslots, colour, slot, a, r * 12 + 4 * k + s));
+  });
   __syncwarp();
   const bool cell_ok = node_ok && ((pt >> ((1 - (a & 1)) + 2 * (1 - (a >> 1)))) & 1);
   T ru, rv, rp;
@@ -752,12 +783,13 @@ __device__ __forceinline__ void split_defect_tile(const NodeLevel<T>& L, const O
   const int li = m % kSX, lj = m / kSX, i = i0 + li, j = j0 + lj;
   const bool ok = i <= L.nx && j <= L.ny;
   const int n = ok ? j * L.nnx + i : 0;
-  T c[12];
-  load_split_blocks<T>(L, n, s, c);
-  const int pt = ok ? (int)__ldg(L.pat + n) : 0;
-  const T bb = __ldcg(b + (s < 3 ? s : 0) * L.nn + n);
-  T xu, xv, xp;
-  stage_split_tile<T, false>(L, x, i0, j0, lane, -1, S, xu, xv, xp, budget);
+  T c[12], bb, xu, xv, xp;
+  int pt;
+  stage_split_tile<T, false>(L, x, i0, j0, lane, -1, S, xu, xv, xp, budget, [&] {
+    load_split_blocks<T>(L, n, s, c);
+    pt = ok ? (int)__ldg(L.pat + n) : 0;
+    bb = __ldcg(b + (s < 3 ? s : 0) * L.nn + n);
+  });
   __syncwarp();
   T ru, rv, rp;
   node_rows_split<T>(L, tab, S, c, li + 2, lj + 2, pt, (i & 1) + 2 * (j & 1), s, ru, rv, rp);
@@ -777,12 +809,13 @@ __device__ __forceinline__ void warp_defect_tile(const NodeLevel<T>& L, const Op
   const int i = i0 + li, j = j0 + lj;
   const bool ok = i <= L.nx && j <= L.ny;
   const int n = ok ? j * L.nnx + i : 0;
-  T c[36];
-  load36<T>(L.cf, n, L.nn, c);
-  const int pt = ok ? (int)__ldg(L.pat + n) : 0;
-  const T bu = __ldcg(b + n), bv = __ldcg(b + L.nn + n), bp = __ldcg(b + 2 * L.nn + n);
-  T xu, xv, xp;
-  stage_warp_tile<T, false>(L, x, i0, j0, lane, -1, S, xu, xv, xp, budget);
+  T c[36], bu, bv, bp, xu, xv, xp;
+  int pt;
+  stage_warp_tile<T, false>(L, x, i0, j0, lane, -1, S, xu, xv, xp, budget, [&] {
+    load36<T>(L.cf, n, L.nn, c);
+    pt = ok ? (int)__ldg(L.pat + n) : 0;
+    bu = __ldcg(b + n), bv = __ldcg(b + L.nn + n), bp = __ldcg(b + 2 * L.nn + n);
+  });
   __syncwarp();
   T ru, rv, rp;
   node_rows_assembled<T>(L, tab, S, c, li + 2, lj + 2, pt, (i & 1) + 2 * (j & 1), ru, rv, rp);
