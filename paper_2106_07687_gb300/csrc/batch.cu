@@ -157,6 +157,7 @@ class Batch final : public BatchBase {
   }
 
   void vcycle_all(const T* b, T* x, const int* act);
+  int read_status(std::vector<int>& status);
   void fgmres_iteration(int j);
   int linearize_masked(const int* act, bool coarse, bool precond);
   int solve(const int* nact_d, const std::vector<int>& nact, std::vector<int>& gits);
@@ -319,7 +320,6 @@ int Batch<T>::init() {
         l.x = mem_.alloc<T>(n3);
         l.b = mem_.alloc<T>(n3);
       }
-      l.x2 = mem_.alloc<T>(n3);
       l.d = mem_.alloc<T>(n3);
       l.vb = mem_.alloc<T>(n2);
       l.vb64 = mem_.alloc<double>(n2);
@@ -329,6 +329,10 @@ int Batch<T>::init() {
       if (k >= 2) {
         l.inv = mem_.alloc<T>((size_t)4 * 144 * vanka_slots(g));
         l.cf = mem_.alloc<T>((size_t)kCoefs<T> * g.nn);
+        // no cycle has the number 0 the tags start with
+        const size_t words = 2 * (size_t)kTagWords<T> * g.nn;
+        l.xt = mem_.alloc<ulonglong2>(words);
+        if (l.xt) cudaMemsetAsync(l.xt, 0, words * sizeof(ulonglong2), st_);
         const std::vector<uint16_t> pat = node_patterns(hl_[p][k]);
         uint16_t* dp = mem_.alloc<uint16_t>(pat.size());
         if (!mem_.ok()) return fail(DNNMG_ERR_CUDA, "device allocation failed");
@@ -389,7 +393,7 @@ int Batch<T>::init() {
   cact_ = mem_.alloc<int>(n_);
   nact_ = mem_.alloc<int>(n_);
   sel_ = mem_.alloc<int>(n_);
-  status_ = mem_.alloc<int>(n_);
+  status_ = mem_.alloc<int>(n_ + 2);  // and the cycles' state words
   // vector blocks
   std::vector<int> vinst(nblk), vfirst(n_), vcount(n_);
   for (int p = 0; p < n_; ++p) {
@@ -517,19 +521,26 @@ int Batch<T>::init() {
   walk_.n1 = n1_;
   walk_.Ainv = Ainv_;
   walk_.astride = astride_;
+  walk_.state = status_ + n_;
   for (int k = 2; k <= Lmax_; ++k) {
     auto g = [&](int p, int l) -> const Grid& { return hl_[p][l].g; };
-    walk_.pass[k] = level_items(k, [&](int p) { return vcycle_warp_tiles(g(p, k)); });
     walk_.defect[k] = level_items(k, [&](int p) { return vcycle_defect_tiles(g(p, k)); });
+    {
+      std::vector<int2> it;
+      for (int p = 0; p < n_; ++p)
+        if (L_[p] >= k) {
+          const int nbx = vcycle_tile_columns(g(p, k)), nt = vcycle_warp_tiles(g(p, k));
+          for (int t = 0; t < nt; ++t) it.push_back(make_int2(p, t % nbx + (t / nbx << 16)));
+        }
+      walk_.pass[k] = make_table(it).w();
+    }
     walk_.zero[k] = level_items(k, [&](int p) { return cdiv(4 * vanka_slots(g(p, k)), 32); });
     walk_.restr[k] = level_items(k, [&](int p) { return cdiv(g(p, k - 1).nn, 32); });
     walk_.prol[k] = level_items(k, [&](int p) { return cdiv(g(p, k).nn, 32); });
   }
   {
-    // levels count from the coarsest (1); x is zeroed beforehand when no
-    // smoothing pass starts from zero
-    std::vector<Phase> ph = vcycle_phases(Lmax_ - 1, c0_.nu1, c0_.nu2, false);
-    if (!ph.empty() && ph[0].type == kPhaseZeroTop) ph.erase(ph.begin());
+    // levels count from the coarsest (1)
+    std::vector<Phase> ph = vcycle_phases(Lmax_ - 1, c0_.nu1, c0_.nu2);
     for (Phase& q : ph) q.level += 1;
     nph_ = (int)ph.size();
     ph_ = mem_.alloc<Phase>(ph.size());
@@ -551,6 +562,8 @@ int Batch<T>::init() {
     cudaStreamSynchronize(st_);
   }
   for (int* a : {kcnt_, its_, gact_, cact_, nact_, sel_, status_}) cudaMemsetAsync(a, 0, sizeof(int) * n_, st_);
+  cudaMemsetAsync(status_ + n_, 0, sizeof(int), st_);
+  cudaMemsetAsync(status_ + n_ + 1, 1, sizeof(int), st_);
   for (double* a : {resid_, target_, nrm_}) cudaMemsetAsync(a, 0, sizeof(double) * n_, st_);
   const double one = 1.0;
   cudaMemcpyAsync(one_, &one, sizeof(double), cudaMemcpyHostToDevice, st_);
@@ -569,6 +582,16 @@ void Batch<T>::vcycle_all(const T* b, T* x, const int* act) {
   const int p = prof_.begin(DNNMG_STAGE_VCYCLE, Lmax_, st_);
   bk_vcycle<T>(walk_, ph_, nph_, b, x, (T)c0_.omega, act, st_);
   prof_.end(p, st_);
+}
+
+// The setups' status words, and an error when a wait of an earlier cycle hit its
+// bound (reported once).
+template <typename T>
+int Batch<T>::read_status(std::vector<int>& status) {
+  if (int rc = sync_read(status_, status.data(), sizeof(int) * (n_ + 1))) return rc;
+  if (!status[n_]) return DNNMG_OK;
+  cudaMemsetAsync(status_ + n_, 0, sizeof(int), st_);
+  return fail(DNNMG_ERR_TIMEOUT, "a wait for an update of the cycle timed out");
 }
 
 // Linearise the active problems at their current state: the FGMRES matvec
@@ -605,8 +628,8 @@ int Batch<T>::linearize(const double* x64) {
   (void)x64;
   sync_in();
   if (int rc = linearize_masked(nullptr, true, true)) return rc;
-  std::vector<int> status(n_);
-  if (int rc = sync_read(status_, status.data(), sizeof(int) * n_)) return rc;
+  std::vector<int> status(n_ + 1);
+  if (int rc = read_status(status)) return rc;
   for (int p = 0; p < n_; ++p) {
     if (status[p] & 1) return fail(DNNMG_ERR_NUMERICAL, "singular local Vanka matrix");
     if (status[p] & 2) return fail(DNNMG_ERR_NUMERICAL, "singular coarse-level matrix");
@@ -620,7 +643,8 @@ int Batch<T>::vcycle(const void* b, void* x) {
   sync_in();
   launch_fill<T>(static_cast<T*>(x), T(0), N_, st_);
   vcycle_all(static_cast<const T*>(b), static_cast<T*>(x), nullptr);
-  cudaStreamSynchronize(st_);
+  std::vector<int> status(n_ + 1);
+  if (int rc = read_status(status)) return rc;
   return check("vcycle");
 }
 
@@ -782,8 +806,8 @@ int Batch<T>::newton(const std::vector<int>& mask, std::vector<dnnmg_step_stats>
     const bool precond = it == 0 || !c0_.precond_lag;
     if (int rc = linearize_masked(act_d, refresh, precond)) return rc;
     if (precond) {
-      std::vector<int> status(n_);
-      if (int rc = sync_read(status_, status.data(), sizeof(int) * n_)) return rc;
+      std::vector<int> status(n_ + 1);
+      if (int rc = read_status(status)) return rc;
       bool changed = false;
       for (int q = 0; q < n_; ++q)
         if (act[q] && status[q]) {

@@ -34,7 +34,9 @@ constexpr int kVB = kVT * kVE;  // elements per vector block (padding unit)
 template <typename T>
 struct BLev {
   Grid g;
-  T *x, *x2, *b, *d, *vb, *inv;  // multigrid buffers (x, b unused on the top level)
+  T *x, *b, *d, *vb, *inv;       // multigrid buffers (x: the coarsest level's solution; x, b
+                                 // unused on the top level)
+  ulonglong2* xt;                // the iterate: two tagged buffers (vnode.cuh)
   double* vb64;                  // FP64 linearisation point (velocity)
   T* cf;                         // assembled velocity blocks (vnode.cuh)
   const uint16_t* pat;           // node patterns
@@ -74,8 +76,8 @@ struct Work {
   int n = 0;
 };
 
-// Items of the batched cycle's phases on every level: (problem, warp tile) of
-// the passes and defects, (problem, chunk of 32) of the first pass from zero
+// Items of the batched cycle's phases on every level: (problem, warp tile bx +
+// 65536 by) of the passes, (problem, tile) of the defects, (problem, chunk of 32) of the first pass from zero
 // (four items per slot), the restriction from the level (nodes of the level
 // below) and the prolongation to it.
 constexpr int kBLevels = 11;
@@ -86,6 +88,7 @@ struct BWalk {
   int nprob, nL, mode, n1;  // mode: every problem's stabilisation form, -1 if they differ
   const double* Ainv;       // coarse inverses, `astride` doubles apart, n1 unknowns
   long long astride;
+  int* state;               // a status word and the cycle's number (see launch_vcycle_persistent)
   Work pass[kBLevels], defect[kBLevels], zero[kBLevels], restr[kBLevels], prol[kBLevels];
 };
 // one cycle over nph phases (build_batch_phases) of every active problem

@@ -3,10 +3,11 @@
 // The phases are those of the single problem's cycle (vcycle.cu) from the
 // largest level of the batch down: a phase of level k works on every problem
 // that has the level, over a list of (problem, tile) or (problem, chunk of 32
-// nodes) items, one warp each, with the same warp bodies (vnode.cuh).  One FP32
-// cycle of twelve channels on levels 3 to 5: 77 launches with cell-by-cell tiles
-// 1,338 us, this 713 us, near the bandwidth of the inverses and blocks on the
-// top level (265 k nodes, 80 MB per pass).
+// nodes) items, one warp each, with the same warp bodies and the same numbered
+// updates of the iterate instead of barriers (vnode.cuh).  One FP32 cycle of
+// twelve channels on levels 3 to 5: 77 launches with cell-by-cell tiles 1,338
+// us, this with a barrier per phase 704 us, with numbered updates 577 us; a pass
+// of the top level moves 80 MB of inverses and blocks (265 k nodes, 12 us).
 // Where the grid cannot be resident the same kernel is launched once per phase.
 #include <algorithm>
 #include <cooperative_groups.h>
@@ -33,7 +34,7 @@ struct BWalkSmem {
 template <typename T>
 __global__ void __launch_bounds__(walk_threads<T>(), 1)
     bvcycle_kernel(const __grid_constant__ BWalk<T> W, const Phase* __restrict__ ph, int p0, int p1,
-                   const T* topb, T* topx, T omega, const int* act) {
+                   const T* topb, T* topx, T omega, const int* act, int bump) {
   constexpr int NT = walk_threads<T>(), NW = NT / 32;
   extern __shared__ __align__(16) uint8_t dyn[];
   BWalkSmem<T>& S = *reinterpret_cast<BWalkSmem<T>*>(dyn);
@@ -46,11 +47,14 @@ __global__ void __launch_bounds__(walk_threads<T>(), 1)
   const BLev<T>* rec = in_smem ? srec : W.lev;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int w0 = blockIdx.x + gridDim.x * w, nw = gridDim.x * NW;
-  int budget = 1;  // nothing waits on tags here
+  const unsigned cycle = __ldcg(reinterpret_cast<unsigned*>(W.state) + 1), tag0 = cycle << 8;
+  int budget = kTagPolls;
   for (int p = p0; p < p1; ++p) {
     Phase f{};
     f.type = __ldg(&ph[p].type), f.level = __ldg(&ph[p].level), f.colour = __ldg(&ph[p].colour);
     f.in = __ldg(&ph[p].in), f.out = __ldg(&ph[p].out);
+    f.tin = __ldg(&ph[p].tin), f.tout = __ldg(&ph[p].tout), f.cin = __ldg(&ph[p].cin);
+    f.tcin = __ldg(&ph[p].tcin), f.last = __ldg(&ph[p].last);
     const int k = f.level;
     // item t of a list: its problem's record of level k and its index there
     auto items = [&](const Work& list, auto body) {
@@ -66,33 +70,32 @@ __global__ void __launch_bounds__(walk_threads<T>(), 1)
     auto node_level = [&](const BLev<T>& L) {
       return NodeLevel<T>{L.g.nx, L.g.ny, L.g.nnx, L.g.nn, L.pat, L.cf, L.h, L.hs};
     };
+    auto iterate = [&](const BLev<T>& L) {
+      const size_t words = (size_t)kTagWords<T> * L.g.nn;
+      return TaggedX<T>{L.xt + f.in * words, L.xt + f.out * words,
+                        f.last && L.top ? topx + L.off : nullptr, L.g.nn, tag0 + f.tin,
+                        tag0 + f.tout,       W.state};
+    };
     switch (f.type) {
       case kPhasePass:
         items(W.pass[k], [&](const BLev<T>& L, int, int t) {
-          T* x0 = L.top ? topx + L.off : L.x;
-          const int nbx = cdiv(L.g.nx / 2 + 1, kWX / 2);
           warp_pass_tile<T>(node_level(L), table(L), f.colour, L.top ? topb + L.off : L.b,
-                            PlanarX<T>{f.in ? L.x2 : x0, f.out ? L.x2 : x0, L.g.nn}, L.inv,
-                            vanka_pitch(L.g), vanka_slots(L.g), omega, t % nbx, t / nbx, lane,
-                            S.tile[w], budget);
+                            iterate(L), L.inv, vanka_pitch(L.g), vanka_slots(L.g), omega,
+                            t & 0xFFFF, t >> 16, lane, S.tile[w], budget);
         });
         break;
       case kPhasePassZero:
         items(W.zero[k], [&](const BLev<T>& L, int, int c) {
           const int e = (c << 5) + lane;
-          T* out = f.out ? L.x2 : (L.top ? topx + L.off : L.x);
-          zero_pass_node<T>(L.g, f.colour, L.top ? topb + L.off : L.b,
-                            PlanarX<T>{nullptr, out, L.g.nn}, L.inv, omega, e,
+          zero_pass_node<T>(L.g, f.colour, L.top ? topb + L.off : L.b, iterate(L), L.inv, omega, e,
                             e < 4 * vanka_slots(L.g));
         });
         break;
       case kPhaseDefect:
         items(W.defect[k], [&](const BLev<T>& L, int, int t) {
           const int nbx = cdiv(L.g.nnx, kWX);
-          warp_defect_tile<T>(node_level(L), table(L), L.top ? topb + L.off : L.b,
-                              PlanarX<T>{f.in ? L.x2 : (L.top ? topx + L.off : L.x), nullptr,
-                                         L.g.nn},
-                              L.d, t % nbx, t / nbx, lane, S.tile[w], budget);
+          warp_defect_tile<T>(node_level(L), table(L), L.top ? topb + L.off : L.b, iterate(L), L.d,
+                              t % nbx, t / nbx, lane, S.tile[w], budget);
         });
         break;
       case kPhaseRestrict:
@@ -101,17 +104,23 @@ __global__ void __launch_bounds__(walk_threads<T>(), 1)
           const int n = (c << 5) + lane;
           if (n >= C.g.nn) return;
           restrict_node<T, true>(F.g, C.g, F.d, C.b, 3, n % C.g.nnx, n / C.g.nnx);
-          if (f.colour == 1)
-            for (int q = 0; q < 3; ++q) C.x[q * C.g.nn + n] = T(0);
+          if (f.colour == 1 && C.xt)
+            TaggedX<T>{C.xt, C.xt, nullptr, C.g.nn, tag0, tag0, W.state}.store(n, T(0), T(0), T(0));
         });
         break;
       case kPhaseProlong:
         items(W.prol[k], [&](const BLev<T>& F, int prob, int c) {
           const BLev<T>& C = rec[prob * W.nL + k - 1];
-          const int n = (c << 5) + lane;
-          if (n >= F.g.nn) return;
-          prolong_add_node<T>(F.g, C.g, C.x, f.in ? F.x2 : (F.top ? topx + F.off : F.x),
-                              n % F.g.nnx, n / F.g.nnx);
+          const bool valid = (c << 5) + lane < F.g.nn;  // whole warps wait together
+          const int n = valid ? (c << 5) + lane : 0, i = n % F.g.nnx, j = n / F.g.nnx;
+          if (f.tcin)
+            prolong_node<T>(F.g, C.g,
+                            TaggedX<T>{C.xt + f.cin * (size_t)kTagWords<T> * C.g.nn, nullptr,
+                                       nullptr, C.g.nn, tag0 + f.tcin, 0u, W.state},
+                            iterate(F), i, j, valid, budget);
+          else
+            prolong_node<T>(F.g, C.g, PlanarX<T>{C.x, nullptr, C.g.nn}, iterate(F), i, j, valid,
+                            budget);
         });
         break;
       case kPhaseCoarse: {
@@ -147,11 +156,31 @@ __global__ void __launch_bounds__(walk_threads<T>(), 1)
         }
         break;
       }
+      case kPhaseZeroTop:  // every problem's own top level
+        for (int l = 2; l < W.nL && l < kBLevels; ++l)
+          for (int t = w0; t < W.prol[l].n; t += nw) {
+            const int2 it = __ldg(W.prol[l].d + t);
+            const BLev<T>& L = rec[it.x * W.nL + l];
+            const int n = (it.y << 5) + lane;
+            if ((!act || act[it.x]) && L.top && n < L.g.nn)
+              TaggedX<T>{L.xt, L.xt, nullptr, L.g.nn, tag0, tag0, W.state}.store(n, T(0), T(0),
+                                                                              T(0));
+          }
+        break;
       default: break;
     }
-    if (p + 1 < p1) cg::this_grid().sync();
+    // the defect, the restricted one and the coarse solution are plain arrays
+    const bool plain =
+        f.type == kPhaseDefect || f.type == kPhaseRestrict || f.type == kPhaseCoarse;
+    if (plain && p + 1 < p1) cg::this_grid().sync();
   }
+  // every block has read the number before its first barrier (a cycle with a
+  // phase that uses it has one)
+  if (bump && blockIdx.x == 0 && threadIdx.x == 0)
+    *(reinterpret_cast<volatile unsigned*>(W.state) + 1) = cycle + 1;
 }
+
+__global__ void next_cycle_kernel(int* state) { state[1] += 1; }
 
 template <typename T>
 size_t walk_bytes(int nprob, int nL, int n1) {
@@ -176,9 +205,10 @@ void bk_vcycle(const BWalk<T>& W, const Phase* ph, int nph, const T* topb, T* to
     per = 0;
   if (per > 0) {
     BWalk<T> w = W;
-    int p0 = 0;
+    int p0 = 0, bump = 1;
     void* args[] = {(void*)&w,    (void*)&ph,   (void*)&p0,    (void*)&nph,
-                    (void*)&topb, (void*)&topx, (void*)&omega, (void*)&act};
+                    (void*)&topb, (void*)&topx, (void*)&omega, (void*)&act,
+                    (void*)&bump};
     note_launch();
     if (cudaLaunchCooperativeKernel((void*)bvcycle_kernel<T>, dim3(sms), dim3(walk_threads<T>()),
                                     args, smem, st) == cudaSuccess)
@@ -187,8 +217,11 @@ void bk_vcycle(const BWalk<T>& W, const Phase* ph, int nph, const T* topb, T* to
   }
   for (int p = 0; p < nph; ++p) {
     note_launch();
-    bvcycle_kernel<T><<<sms, walk_threads<T>(), smem, st>>>(W, ph, p, p + 1, topb, topx, omega, act);
+    bvcycle_kernel<T><<<sms, walk_threads<T>(), smem, st>>>(W, ph, p, p + 1, topb, topx, omega, act,
+                                                     0);
   }
+  note_launch();
+  next_cycle_kernel<<<1, 1, 0, st>>>(W.state);
 }
 
 template void bk_vcycle<float>(const BWalk<float>&, const Phase*, int, const float*, float*, float,

@@ -118,7 +118,7 @@ class Solver final : public SolverBase {
       dlv_ = c_->mem.alloc<VLevel<T>>(K_ + 1);
       std::vector<Phase> all;
       for (int k = 0; k <= K_; ++k) {
-        const std::vector<Phase> p = vcycle_phases(k, cfg.nu1, cfg.nu2, true);
+        const std::vector<Phase> p = vcycle_phases(k, cfg.nu1, cfg.nu2);
         ph_off_.push_back((int)all.size());
         ph_n_.push_back((int)p.size());
         all.insert(all.end(), p.begin(), p.end());

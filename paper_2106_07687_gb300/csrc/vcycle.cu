@@ -127,7 +127,7 @@ __device__ __forceinline__ void walk_phases(const VLevel<T>* glv, const OpTable<
     r.inv = L.inv, r.cf = L.cf, r.pat = L.pat;
     const size_t words = (size_t)kTagWords<T> * g.nn;
     r.in = L.xt + f.in * words, r.out = L.xt + f.out * words;
-    r.planar = f.last ? topx : nullptr;
+    r.planar = f.last && f.level == top ? topx : nullptr;
     r.d = L.d;
     S.rec[p] = r;
   }
@@ -167,7 +167,7 @@ __device__ __forceinline__ void walk_phases(const VLevel<T>* glv, const OpTable<
     const Grid& g = L.g;
     const T* b = k == top ? topb : L.b;
     const size_t words = (size_t)kTagWords<T> * g.nn;
-    const TaggedX<T> x{L.xt + f.in * words, L.xt + f.out * words, f.last ? topx : nullptr, g.nn,
+    const TaggedX<T> x{L.xt + f.in * words, L.xt + f.out * words, f.last && k == top ? topx : nullptr, g.nn,
                        tag0 + f.tin,        tag0 + f.tout,        state};
     bool barrier = false;
     switch (f.type) {
@@ -300,9 +300,8 @@ __global__ void __launch_bounds__(128)
 }
 
 // phases of the cycle of level k; returns the buffer and number of its final
-// iterate (0: the coarsest level's solution).  In the tagged form a prolongation
-// writes the other buffer, otherwise it works in place.
-std::pair<int, int> build_phases(int k, int nu1, int nu2, bool tagged, std::vector<Phase>& out) {
+// iterate (0: the coarsest level's solution)
+std::pair<int, int> build_phases(int k, int nu1, int nu2, std::vector<Phase>& out) {
   if (k == 0) {
     out.push_back({kPhaseCoarse, 0, 0, 0, 0});
     return {0, 0};
@@ -310,23 +309,24 @@ std::pair<int, int> build_phases(int k, int nu1, int nu2, bool tagged, std::vect
   // with pre-smoothing, the first pass starts from the zero iterate and
   // writes every node, so no level needs zeroing beforehand
   int cur = 0, tag = 0;
-  auto push = [&](int type, int colour, bool flip, bool update) {
-    Phase f{type, k, colour, cur, flip ? 1 - cur : 0};
+  auto push = [&](int type, int colour, bool update) {
+    Phase f{type, k, colour, cur, update ? 1 - cur : 0};
     f.tin = tag;
-    cur = flip ? f.out : cur;
-    f.tout = tag += update;
+    if (update) cur = f.out, ++tag;
+    f.tout = tag;
     out.push_back(f);
   };
   for (int s = 0; s < nu1; ++s)
-    for (int c = 0; c < 4; ++c) push(s == 0 && c == 0 ? kPhasePassZero : kPhasePass, c, true, true);
-  push(kPhaseDefect, 0, false, false);
-  push(kPhaseRestrict, nu1 > 0 ? 0 : 1, false, false);
-  const std::pair<int, int> coarse = build_phases(k - 1, nu1, nu2, tagged, out);
-  push(kPhaseProlong, 0, tagged, true);
+    for (int c = 0; c < 4; ++c) push(s == 0 && c == 0 ? kPhasePassZero : kPhasePass, c, true);
+  push(kPhaseDefect, 0, false);
+  push(kPhaseRestrict, nu1 > 0 ? 0 : 1, false);
+  const std::pair<int, int> coarse = build_phases(k - 1, nu1, nu2, out);
+  push(kPhaseProlong, 0, true);
   out.back().cin = coarse.first;
   out.back().tcin = coarse.second;
   for (int s = 0; s < nu2; ++s)
-    for (int c = 0; c < 4; ++c) push(kPhasePass, c, true, true);
+    for (int c = 0; c < 4; ++c) push(kPhasePass, c, true);
+  out.back().last = 1;
   return {cur, tag};
 }
 
@@ -350,6 +350,8 @@ void launch_assemble_blocks(const AsmLevel<T>* lv, int nlev, int nodes, cudaStre
   assemble_blocks_kernel<T><<<cdiv(nodes, 128), 128, 0, st>>>(lv, nlev, nodes);
 }
 
+int vcycle_tile_columns(const Grid& g) { return cdiv(g.nx / 2 + 1, kWX / 2); }
+
 int vcycle_warp_tiles(const Grid& g) {
   return cdiv(g.nx / 2 + 1, kWX / 2) * cdiv(g.ny / 2 + 1, kWY / 2);
 }
@@ -360,11 +362,10 @@ bool vcycle_fits(int nphases, int nlevels) {
   return nphases <= kMaxPhases && nlevels <= kMaxVLevels;
 }
 
-std::vector<Phase> vcycle_phases(int top, int nu1, int nu2, bool tagged) {
+std::vector<Phase> vcycle_phases(int top, int nu1, int nu2) {
   std::vector<Phase> out;
   if (nu1 == 0 || top == 0) out.push_back({kPhaseZeroTop, top, 0, 0, 0});
-  build_phases(top, nu1, nu2, tagged, out);
-  out.back().last = 1;
+  build_phases(top, nu1, nu2, out);
   return out;
 }
 

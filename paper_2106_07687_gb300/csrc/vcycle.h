@@ -48,21 +48,21 @@ enum PhaseType {
 // does).  tin / tout: number, within the cycle, of the level's update that the
 // phase reads and writes; cin / tcin: buffer and number of the coarse level's
 // iterate that a prolongation reads (tcin 0: the coarsest level's solution).
-// last: the phase writes the cycle's result.
+// last: the level's final update (on the top level it goes to the result).
 struct Phase {
   int type, level, colour, in, out;
   int tin = 0, tout = 0, cin = 0, tcin = 0, last = 0;
 };
 
-// phase list of one V(nu1, nu2) cycle with top level `top`, x zeroed first.
-// tagged: for the single problem's kernel; otherwise a prolongation works in
-// place and the top level's result is in buffer 0.
-std::vector<Phase> vcycle_phases(int top, int nu1, int nu2, bool tagged);
+// phase list of one V(nu1, nu2) cycle with top level `top`, x zeroed first
+std::vector<Phase> vcycle_phases(int top, int nu1, int nu2);
 // whether a launch of nphases phases over nlevels levels fits the kernels'
 // shared-memory tables
 bool vcycle_fits(int nphases, int nlevels);
 // warp tiles of a colour pass on a level
 int vcycle_warp_tiles(const Grid& g);
+// and how many of them lie side by side
+int vcycle_tile_columns(const Grid& g);
 // warp tiles of a defect
 int vcycle_defect_tiles(const Grid& g);
 // co-resident grid size for the cooperative launch (0 if not available)

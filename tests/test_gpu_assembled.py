@@ -59,3 +59,35 @@ def test_fp32_rows_act_on_differences(L, nu, dt):
         c.linearize(x)
         out.append(c.vcycle(L, b.to(c.vdtype).cuda()).double().cpu().numpy())
     assert rel(out[1], out[0]) < 1e-6, rel(out[1], out[0])
+
+
+@pytest.mark.parametrize("nu1,nu2,modes", [(2, 2, (0,)), (0, 2, (0, 1)), (1, 0, (1,))])
+@pytest.mark.parametrize("precision,tol", [(0, 1e-12), (1, 1e-5)])
+def test_batched_cycle_matches_single_cycles(precision, tol, nu1, nu2, modes):
+    """Problems whose finest levels differ wait for each other's updates of no
+    level but their own: every problem's cycle is that of its own context."""
+    dn = lib()
+    levels = (1, 3, 2, 4, 3)
+    kw = [dict(level_solve=L, precision=precision, obstacle_i0=2, obstacle_j0=1, nu=0.006 + 0.001 * p,
+               dt=0.01, nu1=nu1, nu2=nu2, lps_mode=modes[p % len(modes)]) for p, L in enumerate(levels)]
+    B = dn.Batch([dn.default_config(**k) for k in kw])
+    g = torch.Generator().manual_seed(3)
+    bvec = torch.zeros(B.length, dtype=B.vdtype, device="cuda")
+    single = []
+    for p, L in enumerate(levels):
+        lev = mesh.Level(L, obstacle=(2, 1))
+        x = torch.from_numpy(seeded_state(lev, 40 + p)).cuda()
+        b = torch.randn(lev.ndof, generator=g, dtype=torch.float64).to(B.vdtype).cuda()
+        off = B.layout(p)[1]
+        bvec[off:off + lev.ndof] = b
+        B.set_state(p, x)
+        c = dn.Context(persistent_vcycle=max(L, 2), persistent_mode=0, **kw[p])
+        c.linearize(x)
+        single.append((off, lev.ndof, c.vcycle(L, b).double().cpu().numpy()))
+    B.linearize()
+    first = B.vcycle(bvec).clone()
+    for off, n, ref in single:
+        got = first[off:off + n].double().cpu().numpy()
+        assert rel(got, ref) < tol, rel(got, ref)
+    for _ in range(10):
+        assert torch.equal(B.vcycle(bvec), first)
