@@ -247,6 +247,29 @@ __device__ __forceinline__ void gauss_data(const T bu[4], const T bv[4], GaussDa
   }
 }
 
+// The same with what the Gauss points share computed once: a derivative along
+// one axis depends on the point's other coordinate only, and the values come
+// from interpolations along x and then y.  56 operations instead of 96, for the
+// types whose arithmetic bounds the operator kernels (FP64, double-float).
+template <typename T>
+__device__ __forceinline__ void gauss_data_shared(const T bu[4], const T bv[4], GaussData<T>& gd) {
+  const T G[2] = {T(kG0), T(kG1)}, F[2] = {T(1) - T(kG0), T(1) - T(kG1)};
+  auto field = [&](const T b[4], T v[4], T vx[4], T vy[4]) {
+    const T d0 = b[1] - b[0], d1 = b[3] - b[2], e0 = b[2] - b[0], e1 = b[3] - b[1];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const T x = F[k] * d0 + G[k] * d1, y = F[k] * e0 + G[k] * e1;
+      const T lo = F[k] * b[0] + G[k] * b[1], hi = F[k] * b[2] + G[k] * b[3];
+      vx[2 * k] = vx[2 * k + 1] = x;  // points of one height
+      vy[k] = vy[2 + k] = y;          // points of one abscissa
+      v[k] = F[0] * lo + G[0] * hi;
+      v[2 + k] = F[1] * lo + G[1] * hi;
+    }
+  };
+  field(bu, gd.Bu, gd.Bux, gd.Buy);
+  field(bv, gd.Bv, gd.Bvx, gd.Bvy);
+}
+
 // Element Jacobian A'_T(vbar) entries between local nodes al (row) and be
 // (column): J[c][c'] for components (u, v, p) (Eq. 6, before LPS).
 template <typename T>
@@ -298,37 +321,25 @@ __device__ __forceinline__ void cell_all_rows(const Sten<T>& s, const T wu[4], c
     r[a] = ru, r[4 + a] = rv, r[8 + a] = rp;
   }
   const T sc = s.wq * s.ih;
+  GaussData<T> W, B;
+  if constexpr (sizeof(T) == 8) {
+    gauss_data_shared<T>(wu, wv, W);
+    if (!NONLIN) gauss_data_shared<T>(bu, bv, B);
+  } else {
+    gauss_data<T>(wu, wv, W);
+    if (!NONLIN) gauss_data<T>(bu, bv, B);
+  }
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     T phi[4], dx[4], dy[4];
     shape_at<T>(q, phi, dx, dy);
-    T Wu = 0, Wv = 0, Wux = 0, Wuy = 0, Wvx = 0, Wvy = 0;
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      Wu += phi[b] * wu[b];
-      Wv += phi[b] * wv[b];
-      Wux += dx[b] * wu[b];
-      Wuy += dy[b] * wu[b];
-      Wvx += dx[b] * wv[b];
-      Wvy += dy[b] * wv[b];
-    }
     T cu, cv;
     if (NONLIN) {
-      cu = Wu * Wux + Wv * Wuy;
-      cv = Wu * Wvx + Wv * Wvy;
+      cu = W.Bu[q] * W.Bux[q] + W.Bv[q] * W.Buy[q];
+      cv = W.Bu[q] * W.Bvx[q] + W.Bv[q] * W.Bvy[q];
     } else {
-      T Bu = 0, Bv = 0, Bux = 0, Buy = 0, Bvx = 0, Bvy = 0;
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        Bu += phi[b] * bu[b];
-        Bv += phi[b] * bv[b];
-        Bux += dx[b] * bu[b];
-        Buy += dy[b] * bu[b];
-        Bvx += dx[b] * bv[b];
-        Bvy += dy[b] * bv[b];
-      }
-      cu = Bu * Wux + Bv * Wuy + Wu * Bux + Wv * Buy;
-      cv = Bu * Wvx + Bv * Wvy + Wu * Bvx + Wv * Bvy;
+      cu = B.Bu[q] * W.Bux[q] + B.Bv[q] * W.Buy[q] + W.Bu[q] * B.Bux[q] + W.Bv[q] * B.Buy[q];
+      cv = B.Bu[q] * W.Bvx[q] + B.Bv[q] * W.Bvy[q] + W.Bu[q] * B.Bvx[q] + W.Bv[q] * B.Bvy[q];
     }
     cu *= sc;
     cv *= sc;

@@ -101,8 +101,10 @@ __device__ __forceinline__ void op_tile_rows(const Grid& g, const Sten<T>& s,
     for (int k = 0; k < 12; ++k) S.cres[e][k] = r[k];
   }
   // the patches start where the cells left off, on the threads that the
-  // cell loop leaves idle (a rotation of the thread index)
-  constexpr int kOff = (kCX * kCY) % NTT;
+  // cell loop leaves idle (a rotation of the thread index), or on the next warp
+  // if the block has one to spare
+  constexpr int kEnd = (kCX * kCY) % NTT, kNext = (kEnd + 31) / 32 * 32;
+  constexpr int kOff = kNext + kPX * kPY <= NTT ? kNext : kEnd;
   for (int e = (t + NTT - kOff) % NTT; e < kPX * kPY; e += NTT) {
     const int pi = PI0 + e % kPX, pj = PJ0 + e / kPX;
     const bool ok = pi >= 0 && pj >= 0 && pi < g.nx / 2 && pj < g.ny / 2 &&

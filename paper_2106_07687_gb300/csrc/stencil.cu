@@ -1,8 +1,8 @@
 // Matrix-free operator kernels: Jacobian apply, defect, FP64 nonlinear
 // residual and the old-time right-hand side (Sec. 2.1, Eqs. 3-6).
 //
-// Apply, defect and residual run tiled (32 x 8 nodes per block, cell and
-// patch rows computed once per tile, optile_body.cuh); the right-hand-side
+// Apply, defect and residual run tiled (cell and patch rows computed once per
+// tile, optile_body.cuh); the right-hand-side
 // kernels run one thread per node with 32 x 4 blocks, x fastest, so each
 // warp reads contiguous rows of the SoA fields.
 #include "kernels.h"
@@ -39,19 +39,35 @@ __global__ void __launch_bounds__(kBX* kBY)
 
 inline dim3 node_grid(const Grid& g) { return dim3(cdiv(g.nnx, kBX), cdiv(g.nny, kBY)); }
 
-// Tiled variants (optile_body.cuh): one block per TX x TY nodes.
-constexpr int kTX = 32, kTY = 8;
+// Tiled variants (optile_body.cuh): one block per TX x TY nodes.  In FP32, 32 x 8
+// nodes by 256 threads.  In FP64 and double-float, where the arithmetic of a
+// tile's cells bounds the kernel, 8 x 6 by three warps: 63 cells (two warps, a
+// node's worth of 1.3 lanes; 32 x 8 has 297 cells for 256 threads, two rounds,
+// 2.0) and 20 patches (the third).  The levels that run in FP64 also have too few
+// large tiles for 152 SMs (25 on 128x32 cells, 81 on 256x64).
+// With the shared Gauss-point sums (gauss_data_shared): FP64 Jacobian apply on
+// 128x32 cells 31.8 -> 10.8 us, residual 38.5 -> 15.8 us; double-float residual on
+// 512x128 39.5 -> 33.4 us.
+template <typename T>
+struct TileOf {
+  static constexpr int X = 8, Y = 6, NT = 96;
+};
+template <>
+struct TileOf<float> {
+  static constexpr int X = 32, Y = 8, NT = 256;
+};
 
 template <typename T>
-__global__ void __launch_bounds__(kTX* kTY)
+__global__ void __launch_bounds__(TileOf<T>::NT)
     apply_tiled_kernel(Grid g, Sten<T> s, const T* __restrict__ w, const T* __restrict__ vb,
                        T* __restrict__ y, const int* skip) {
   if (skip && *skip) return;  // a speculative FGMRES iteration after the cycle stopped
+  constexpr int kTX = TileOf<T>::X, kTY = TileOf<T>::Y, kNT = TileOf<T>::NT;
   extern __shared__ __align__(16) uint8_t smraw[];
   auto& S = *reinterpret_cast<OpSmem<T, kTX, kTY>*>(smraw);
   T ru, rv, rp;
   int n;
-  op_tile_rows<T, false, true, kTX, kTY>(g, s, w, vb, blockIdx.x, blockIdx.y, S, ru, rv, rp, n);
+  op_tile_rows<T, false, true, kTX, kTY, kNT>(g, s, w, vb, blockIdx.x, blockIdx.y, S, ru, rv, rp, n);
   if (n < 0) return;
   const uint8_t f = op_tile_flags<T, kTX, kTY>(S);
   y[n] = (f & kVDir) ? w[n] : ru;
@@ -60,14 +76,15 @@ __global__ void __launch_bounds__(kTX* kTY)
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kTX* kTY)
+__global__ void __launch_bounds__(TileOf<T>::NT)
     defect_tiled_kernel(Grid g, Sten<T> s, const T* __restrict__ b, const T* __restrict__ x,
                         const T* __restrict__ vb, T* __restrict__ d, bool masked) {
+  constexpr int kTX = TileOf<T>::X, kTY = TileOf<T>::Y, kNT = TileOf<T>::NT;
   extern __shared__ __align__(16) uint8_t smraw[];
   auto& S = *reinterpret_cast<OpSmem<T, kTX, kTY>*>(smraw);
   T ru, rv, rp;
   int n;
-  op_tile_rows<T, false, true, kTX, kTY>(g, s, x, vb, blockIdx.x, blockIdx.y, S, ru, rv, rp, n);
+  op_tile_rows<T, false, true, kTX, kTY, kNT>(g, s, x, vb, blockIdx.x, blockIdx.y, S, ru, rv, rp, n);
   if (n < 0) return;
   const uint8_t f = op_tile_flags<T, kTX, kTY>(S);
   const int nn = g.nn;
@@ -114,15 +131,16 @@ __device__ __forceinline__ void norm_reduce(double sq, const NormOut& no) {
   }
 }
 
-__global__ void __launch_bounds__(kTX* kTY)
+__global__ void __launch_bounds__(TileOf<double>::NT)
     residual64_tiled_kernel(Grid g, Sten<double> s, const double* __restrict__ x,
                             const double* __restrict__ f, double* __restrict__ r,
                             const NormOut no) {
+  constexpr int kTX = TileOf<double>::X, kTY = TileOf<double>::Y, kNT = TileOf<double>::NT;
   extern __shared__ __align__(16) uint8_t smraw[];
   auto& S = *reinterpret_cast<OpSmem<double, kTX, kTY>*>(smraw);
   double ru, rv, rp;
   int n;
-  op_tile_rows<double, true, false, kTX, kTY>(g, s, x, nullptr, blockIdx.x, blockIdx.y, S, ru, rv,
+  op_tile_rows<double, true, false, kTX, kTY, kNT>(g, s, x, nullptr, blockIdx.x, blockIdx.y, S, ru, rv,
                                               rp, n);
   double sq = 0.0;
   if (n >= 0) {
@@ -140,14 +158,15 @@ __global__ void __launch_bounds__(kTX* kTY)
 // The same residual with the operator evaluated in FP32 (the state rounded
 // to FP32, the subtraction from f in FP64): the fine-level residual whose
 // only use is the network's input features, which are rounded to BF16.
-__global__ void __launch_bounds__(kTX* kTY)
+__global__ void __launch_bounds__(TileOf<float>::NT)
     residual32_tiled_kernel(Grid g, Sten<float> s, const double* __restrict__ x,
                             const double* __restrict__ f, double* __restrict__ r) {
+  constexpr int kTX = TileOf<float>::X, kTY = TileOf<float>::Y, kNT = TileOf<float>::NT;
   extern __shared__ __align__(16) uint8_t smraw[];
   auto& S = *reinterpret_cast<OpSmem<float, kTX, kTY>*>(smraw);
   float ru, rv, rp;
   int n;
-  op_tile_rows<float, true, false, kTX, kTY, kTX * kTY, double>(g, s, x, nullptr, blockIdx.x,
+  op_tile_rows<float, true, false, kTX, kTY, kNT, double>(g, s, x, nullptr, blockIdx.x,
                                                                blockIdx.y, S, ru, rv, rp, n);
   if (n < 0) return;
   const uint8_t fl = op_tile_flags<float, kTX, kTY>(S);
@@ -160,15 +179,16 @@ __global__ void __launch_bounds__(kTX* kTY)
 // The same residual with the operator evaluated in double-float arithmetic
 // (about 48 significant bits; the subtraction from f in FP64), for
 // mixed-precision contexts.
-__global__ void __launch_bounds__(kTX* kTY)
+__global__ void __launch_bounds__(TileOf<dfloat>::NT)
     residual_df_tiled_kernel(Grid g, Sten<dfloat> s, const double* __restrict__ x,
                              const double* __restrict__ f, double* __restrict__ r,
                              const NormOut no) {
+  constexpr int kTX = TileOf<dfloat>::X, kTY = TileOf<dfloat>::Y, kNT = TileOf<dfloat>::NT;
   extern __shared__ __align__(16) uint8_t smraw[];
   auto& S = *reinterpret_cast<OpSmem<dfloat, kTX, kTY>*>(smraw);
   dfloat ru, rv, rp;
   int n;
-  op_tile_rows<dfloat, true, false, kTX, kTY, kTX * kTY, double>(
+  op_tile_rows<dfloat, true, false, kTX, kTY, kNT, double>(
       g, s, x, nullptr, blockIdx.x, blockIdx.y, S, ru, rv, rp, n);
   double sq = 0.0;
   if (n >= 0) {
@@ -183,7 +203,12 @@ __global__ void __launch_bounds__(kTX* kTY)
   if (no.partials) norm_reduce(sq, no);
 }
 
-inline dim3 tile_grid(const Grid& g) { return dim3(cdiv(g.nnx, kTX), cdiv(g.nny, kTY)); }
+template <typename T>
+dim3 tile_grid(const Grid& g) {
+  return dim3(cdiv(g.nnx, TileOf<T>::X), cdiv(g.nny, TileOf<T>::Y));
+}
+template <typename T>
+using TileSmem = OpSmem<T, TileOf<T>::X, TileOf<T>::Y>;
 
 // opt a kernel in to `bytes` of dynamic shared memory; callers keep the
 // result in a function-local static, so each launcher does it once
@@ -200,19 +225,21 @@ template <typename T>
 void launch_apply(const Grid& g, const Sten<T>& s, const T* w, const T* vb, T* y, cudaStream_t st,
                   const int* skip) {
   note_launch();
-  static const size_t sm = smem_attr(apply_tiled_kernel<T>, sizeof(OpSmem<T, kTX, kTY>));
-  apply_tiled_kernel<T><<<tile_grid(g), kTX * kTY, sm, st>>>(g, s, w, vb, y, skip);
+  static const size_t sm = smem_attr(apply_tiled_kernel<T>, sizeof(TileSmem<T>));
+  apply_tiled_kernel<T><<<tile_grid<T>(g), TileOf<T>::NT, sm, st>>>(g, s, w, vb, y, skip);
 }
 
 template <typename T>
 void launch_defect(const Grid& g, const Sten<T>& s, const T* b, const T* x, const T* vb, T* d,
                    bool masked, cudaStream_t st) {
   note_launch();
-  static const size_t sm = smem_attr(defect_tiled_kernel<T>, sizeof(OpSmem<T, kTX, kTY>));
-  defect_tiled_kernel<T><<<tile_grid(g), kTX * kTY, sm, st>>>(g, s, b, x, vb, d, masked);
+  static const size_t sm = smem_attr(defect_tiled_kernel<T>, sizeof(TileSmem<T>));
+  defect_tiled_kernel<T><<<tile_grid<T>(g), TileOf<T>::NT, sm, st>>>(g, s, b, x, vb, d, masked);
 }
 
-int residual_blocks(const Grid& g) { return cdiv(g.nnx, kTX) * cdiv(g.nny, kTY); }
+int residual_blocks(const Grid& g) {  // the double-float and FP64 kernels' tiles
+  return cdiv(g.nnx, TileOf<double>::X) * cdiv(g.nny, TileOf<double>::Y);
+}
 
 void launch_residual64(const Grid& g, const Sten<double>& s, const double* x, const double* f,
                        double* r, cudaStream_t st, bool dfloat_ops, const NormOut& no) {
@@ -228,13 +255,13 @@ void launch_residual64(const Grid& g, const Sten<double>& s, const double* x, co
     sd.ih = dfloat(s.ih);
     note_launch();
     static const size_t smd =
-        smem_attr(residual_df_tiled_kernel, sizeof(OpSmem<dfloat, kTX, kTY>));
-    residual_df_tiled_kernel<<<tile_grid(g), kTX * kTY, smd, st>>>(g, sd, x, f, r, no);
+        smem_attr(residual_df_tiled_kernel, sizeof(TileSmem<dfloat>));
+    residual_df_tiled_kernel<<<tile_grid<dfloat>(g), TileOf<dfloat>::NT, smd, st>>>(g, sd, x, f, r, no);
     return;
   }
   note_launch();
-  static const size_t sm = smem_attr(residual64_tiled_kernel, sizeof(OpSmem<double, kTX, kTY>));
-  residual64_tiled_kernel<<<tile_grid(g), kTX * kTY, sm, st>>>(g, s, x, f, r, no);
+  static const size_t sm = smem_attr(residual64_tiled_kernel, sizeof(TileSmem<double>));
+  residual64_tiled_kernel<<<tile_grid<double>(g), TileOf<double>::NT, sm, st>>>(g, s, x, f, r, no);
 }
 
 void launch_residual_features(const Grid& g, const Sten<double>& s, const double* x,
@@ -253,8 +280,8 @@ void launch_residual_features(const Grid& g, const Sten<double>& s, const double
   sf.wq = (float)s.wq;
   sf.ih = (float)s.ih;
   note_launch();
-  static const size_t sm = smem_attr(residual32_tiled_kernel, sizeof(OpSmem<float, kTX, kTY>));
-  residual32_tiled_kernel<<<tile_grid(g), kTX * kTY, sm, st>>>(g, sf, x, f, r);
+  static const size_t sm = smem_attr(residual32_tiled_kernel, sizeof(TileSmem<float>));
+  residual32_tiled_kernel<<<tile_grid<float>(g), TileOf<float>::NT, sm, st>>>(g, sf, x, f, r);
 }
 
 void launch_old_time_rhs64(const Grid& g, double inv_k, const double* x_old, double* f,
