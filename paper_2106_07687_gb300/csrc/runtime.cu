@@ -175,21 +175,28 @@ class Solver final : public SolverBase {
     launch_linearize_levels<T>(lin_, x64, vbJ_, report || !tuned_ ? status_ : nullptr, st_);
     // every level's velocity blocks in one launch, then the levels' setups,
     // which are independent and leave much of the GPU idle on the small levels:
-    // those below the top run on side streams beside it, or all of them beside
-    // the coarse factorisation (dependent phases of few warps), unless the
-    // stages are being timed
+    // those below the top run on side streams beside it, or the blocks and all
+    // of them beside the coarse factorisation (dependent phases of few warps),
+    // unless the stages are being timed.  FP64 Newton step on 256x64 cells, blocks
+    // before -> beside the factorisation: 972 -> 880 us.
     const bool factor = coarse || !coarse_done_;
-    int p = c_->prof.begin(DNNMG_STAGE_VANKA_SETUP, lv_[K_].level, st_);
-    launch_assemble_blocks<T>(dasm_, K_, asm_nodes_[K_], st_);
     const bool fork = !side_.empty() && !capturing();
     const bool beside = fork && factor && !c_->prof.on();
-    if (fork) cudaEventRecord(fork_ev_, st_);
+    int p = c_->prof.begin(DNNMG_STAGE_VANKA_SETUP, lv_[K_].level, st_);
+    cudaStream_t blocks = st_;
+    if (beside) {
+      blocks = side_[K_ - 1];
+      cudaEventRecord(fork_ev_, st_);
+      cudaStreamWaitEvent(blocks, fork_ev_, 0);
+    }
+    launch_assemble_blocks<T>(dasm_, K_, asm_nodes_[K_], blocks);
+    if (fork) cudaEventRecord(fork_ev_, blocks);
     if (beside) factor_coarse();
     for (int k = K_; k > 0; --k) {
       cudaStream_t s = st_;
       if (fork && (k < K_ || beside)) {
         s = side_[k - 1];
-        cudaStreamWaitEvent(s, fork_ev_, 0);
+        if (s != blocks) cudaStreamWaitEvent(s, fork_ev_, 0);
       }
       launch_vanka_setup<T>(lv_[k].g, lv_[k].pat, lv_[k].cf, dtab_, lv_[k].inv, status_, s);
       if (s != st_) {
