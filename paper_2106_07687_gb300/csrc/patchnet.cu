@@ -70,17 +70,9 @@ __device__ __forceinline__ uint32_t bf16_pair(float lo, float hi) {
 }
 
 // -- packing -----------------------------------------------------------------
-__global__ void pack_block_kernel(const float* __restrict__ src, int ld, int row0, int rows_valid,
-                                  int cols_valid, int R, int K, uint16_t* __restrict__ dst) {
-  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < R * K; idx += gridDim.x * blockDim.x) {
-    const int r = idx / K, k = idx % K;
-    const float v = (r < rows_valid && k < cols_valid) ? src[(size_t)(row0 + r) * ld + k] : 0.0f;
-    dst[kmajor_offset(r, k, K) >> 1] = f2bf(v);
-  }
-}
-
 // fused biases; a network without biases gets zeros
-__global__ void pack_bias_kernel(const float* __restrict__ w, NetDims d, float* __restrict__ bias) {
+__device__ __forceinline__ void pack_bias(const float* __restrict__ w, const NetDims& d,
+                                          float* __restrict__ bias) {
   const int H = d.hidden;
   const NetOffsets o = d.offsets();
   for (int l = 0; l < d.layers; ++l) {
@@ -102,6 +94,32 @@ __global__ void pack_bias_kernel(const float* __restrict__ w, NetDims d, float* 
   for (int j = threadIdx.x; j < d.mlp; j += blockDim.x) ob[j] = d.bias ? w[o.b1 + j] : 0.0f;
   for (int j = threadIdx.x; j < d.nout(); j += blockDim.x)
     ob[d.mlp + j] = d.bias && j < d.c_out ? w[o.b2 + j] : 0.0f;
+}
+
+// All operands of a network in one launch, a job per blockIdx.y, and the biases
+// (bias != null) as one more.  For 2 x 64 units fifteen launches of 1.5 us before;
+// with one host wait per call instead of two, a training step of 19,456 sequences
+// x 10 steps 689 -> 630 us, a gradient of 32 x 2 units 233 -> 215 us.
+struct PackArgs {
+  PackJob job[kMaxPackJobs];
+  int n;
+  const float* w;
+  float* bias;
+};
+__global__ void __launch_bounds__(256)
+    pack_kernel(const __grid_constant__ PackArgs a, const NetDims d) {
+  if ((int)blockIdx.y == a.n) {
+    if (blockIdx.x == 0) pack_bias(a.w, d, a.bias);
+    return;
+  }
+  const PackJob& J = a.job[blockIdx.y];
+  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < J.R * J.K;
+       idx += gridDim.x * blockDim.x) {
+    const int r = idx / J.K, k = idx % J.K;
+    const float v = r < J.rows && k < J.cols ? J.src[(size_t)r * J.rstride + (size_t)k * J.kstride]
+                                             : 0.0f;
+    J.dst[kmajor_offset(r, k, J.K) >> 1] = f2bf(v);
+  }
 }
 
 // -- shared-memory plan of the forward kernel ---------------------------------
@@ -741,33 +759,36 @@ bool net_supported(const NetDims& d) {
   return patchnet_forward_smem(d) <= kSmemMax && patchnet_backward_smem(d) <= kSmemMax;
 }
 
+void launch_pack(const NetDims& d, const PackJob* jobs, int n, const float* w, float* bias,
+                 cudaStream_t st) {
+  PackArgs a{};
+  for (int q = 0; q < n; ++q) a.job[q] = jobs[q];
+  a.n = n;
+  a.w = w;
+  a.bias = bias;
+  note_launch();
+  pack_kernel<<<dim3(32, n + (bias ? 1 : 0)), 256, 0, st>>>(a, d);
+}
+
 void launch_pack_weights(const NetDims& d, const float* w, PackedNet& pk, cudaStream_t st) {
   const PackLayout L = PackLayout::of(d);
   const NetOffsets o = d.offsets();
   const int H = d.hidden;
+  PackJob jobs[kMaxPackJobs];
+  int n = 0;
   for (int l = 0; l < d.layers; ++l) {
-    const int c = l == 0 ? d.c_in : H;
+    const int c = l == 0 ? d.c_in : H, kx = L.kx[l];
     const float* Wih = w + o.wih[l];
     const float* Whh = w + o.whh[l];
-    const int kx = L.kx[l];
-    note_launch();
-    pack_block_kernel<<<64, 256, 0, st>>>(Wih, c, 0, 2 * H, c, 2 * H, kx, pk.w + L.rz[l]);
-    note_launch();
-    pack_block_kernel<<<64, 256, 0, st>>>(Wih, c, 2 * H, H, c, H, kx, pk.w + L.in[l]);
-    note_launch();
-    pack_block_kernel<<<64, 256, 0, st>>>(Whh, H, 0, 2 * H, H, 2 * H, H, pk.w + L.hrz[l]);
-    note_launch();
-    pack_block_kernel<<<64, 256, 0, st>>>(Whh, H, 2 * H, H, H, H, H, pk.w + L.hn[l]);
+    jobs[n++] = {Wih, pk.w + L.rz[l], c, 1, 2 * H, c, 2 * H, kx};
+    jobs[n++] = {Wih + (size_t)2 * H * c, pk.w + L.in[l], c, 1, H, c, H, kx};
+    jobs[n++] = {Whh, pk.w + L.hrz[l], H, 1, 2 * H, H, 2 * H, H};
+    jobs[n++] = {Whh + (size_t)2 * H * H, pk.w + L.hn[l], H, 1, H, H, H, H};
   }
-  if (d.mlp) {
-    note_launch();
-    pack_block_kernel<<<64, 256, 0, st>>>(w + o.w1, H, 0, 128, H, 128, H, pk.w + L.w1);
-  }
+  if (d.mlp) jobs[n++] = {w + o.w1, pk.w + L.w1, H, 1, 128, H, 128, H};
   const int k2 = d.k2();
-  note_launch();
-  pack_block_kernel<<<64, 256, 0, st>>>(w + o.w2, k2, 0, d.c_out, k2, d.nout(), k2, pk.w + L.w2);
-  note_launch();
-  pack_bias_kernel<<<1, 128, 0, st>>>(w, d, pk.bias);
+  jobs[n++] = {w + o.w2, pk.w + L.w2, k2, 1, d.c_out, k2, d.nout(), k2};
+  launch_pack(d, jobs, n, w, pk.bias, st);
 }
 
 void launch_patchnet_forward(const NetDims& d, const PackedNet& pk, const uint16_t* x,

@@ -132,6 +132,17 @@ struct NetPost {
 size_t patchnet_forward_smem(const NetDims& d);
 size_t patchnet_backward_smem(const NetDims& d);
 bool net_supported(const NetDims& d);
+// A BF16 operand of R rows and K columns in the core-matrix layout: element (r, k)
+// = src[r rstride + k kstride] for r < rows and k < cols, else 0.
+struct PackJob {
+  const float* src;
+  uint16_t* dst;
+  int rstride, kstride, rows, cols, R, K;
+};
+constexpr int kMaxPackJobs = 4 * kMaxLayers + 2;
+// the jobs, and with bias the fused biases of the parameters w, in one launch
+void launch_pack(const NetDims& d, const PackJob* jobs, int n, const float* w, float* bias,
+                 cudaStream_t st);
 // master FP32 flat weights -> packed BF16 operands + fused biases
 void launch_pack_weights(const NetDims& d, const float* w, PackedNet& pk, cudaStream_t st);
 // one recurrent step for P patches: x [P][C_in] BF16, h [layers][P][m] FP32

@@ -907,27 +907,30 @@ int dnnmg_ctx::train_grad_impl(const uint16_t* Xd, const float* Yd, int B, int T
   if (launch_wgrad(jobs, njobs, (int)K, splits, cpart, net_status, st))
     return fail(DNNMG_ERR_ARG, "weight-gradient GEMM shape");
   prof.end(p, st);
-  return net_check("train");
+  return check("train");
+}
+
+// The loss and the status with one wait, behind everything the call launched.
+int dnnmg_ctx::train_finish(const char* what, float* loss) {
+  cudaMemcpyAsync(h_scalars, loss_dev, sizeof(float), cudaMemcpyDeviceToHost, st);
+  if (int rc = net_check(what)) return rc;
+  if (loss) std::memcpy(loss, h_scalars, sizeof(float));
+  return check(what);
 }
 
 int dnnmg_ctx::train_grad(const uint16_t* X, const float* Y, int B, int T, float* g, float* loss) {
   if (int rc = train_grad_impl(X, Y, B, T)) return rc;
   if (g) cudaMemcpyAsync(g, grad, sizeof(float) * nd.num_params(), cudaMemcpyDeviceToDevice, st);
-  cudaMemcpyAsync(h_scalars, loss_dev, sizeof(float), cudaMemcpyDeviceToHost, st);
-  cudaStreamSynchronize(st);
-  if (loss) std::memcpy(loss, h_scalars, sizeof(float));
-  return check("train_grad");
+  return train_finish("train_grad", loss);
 }
 
 int dnnmg_ctx::train_step(const uint16_t* X, const float* Y, int B, int T, float lr, float* loss) {
   if (int rc = train_grad_impl(X, Y, B, T)) return rc;
-  ++adam_step;
-  launch_adam(w_master, grad, adam_m, adam_v, nd.num_params(), lr, adam_step, st);
+  launch_adam(w_master, grad, adam_m, adam_v, nd.num_params(), lr, adam_step + 1, net_status, st);
   launch_pack_weights(nd, w_master, pk, st);
-  cudaMemcpyAsync(h_scalars, loss_dev, sizeof(float), cudaMemcpyDeviceToHost, st);
-  cudaStreamSynchronize(st);
-  if (loss) std::memcpy(loss, h_scalars, sizeof(float));
-  return check("train_step");
+  const int rc = train_finish("train_step", loss);
+  if (rc == DNNMG_OK) ++adam_step;  // otherwise the weights are as they were
+  return rc;
 }
 
 // Patch lists and level L+1 buffers of the DNN-MG correction.

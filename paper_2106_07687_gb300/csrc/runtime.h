@@ -272,6 +272,7 @@ struct dnnmg_ctx {
   int get_patch_inputs(uint16_t* x);
   int init_train();
   int train_grad_impl(const uint16_t* X, const float* Y, int B, int T);
+  int train_finish(const char* what, float* loss);
   int train_grad(const uint16_t* X, const float* Y, int B, int T, float* g, float* loss);
   int train_step(const uint16_t* X, const float* Y, int B, int T, float lr, float* loss);
   int reset_optimizer();

@@ -27,16 +27,6 @@ __device__ __forceinline__ uint16_t f2bf(float v) {
   return __bfloat16_as_ushort(__float2bfloat16_rn(v));
 }
 
-// transposed operand: element (n, k) = src[k * ld + n] for k < K_valid
-__global__ void pack_transpose_kernel(const float* __restrict__ src, int ld, int N, int K,
-                                      int K_valid, uint16_t* __restrict__ dst) {
-  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < N * K; idx += gridDim.x * blockDim.x) {
-    const int n = idx / K, k = idx % K;
-    const float v = k < K_valid ? src[(size_t)k * ld + n] : 0.0f;
-    dst[kmajor_offset(n, k, K) >> 1] = f2bf(v);
-  }
-}
-
 // Shared memory of the backward kernel: the transposed weights and one
 // operand region R of 128 rows, which holds in turn dY (nout columns), dA1
 // (128) and the gate gradients [dr | dz | dn | r * dn] of a layer (4m);
@@ -635,7 +625,9 @@ __global__ void loss_kernel(const double* __restrict__ part, int n, double inv, 
 // Adam with bias correction: w -= lr * mhat / (sqrt(vhat) + eps)
 __global__ void adam_kernel(float* __restrict__ w, const float* __restrict__ g,
                             float* __restrict__ m, float* __restrict__ v, size_t n, float lr,
-                            float b1, float b2, float c1, float c2, float eps) {
+                            float b1, float b2, float c1, float c2, float eps,
+                            const int* skip) {
+  if (*skip) return;  // the gradient is not valid: a wait of its kernels hit its bound
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
        i += (size_t)gridDim.x * blockDim.x) {
     const float gi = g[i];
@@ -659,19 +651,16 @@ void launch_pack_backward(const NetDims& d, const float* w, uint16_t* wT, cudaSt
     Wih[l] = w + o.wih[l];
     Whh[l] = w + o.whh[l];
   }
-  note_launch();
-  pack_transpose_kernel<<<64, 256, 0, st>>>(w + o.w2, k2, k2, d.nout(), d.c_out, wT + W.w2t);
-  if (d.mlp) {
-    note_launch();
-    pack_transpose_kernel<<<64, 256, 0, st>>>(w + o.w1, H, H, 128, 128, wT + W.w1t);
-  }
+  // transposed operands: element (n, k) = src[k ld + n]
+  PackJob jobs[kMaxPackJobs];
+  int n = 0;
+  jobs[n++] = {w + o.w2, wT + W.w2t, 1, k2, k2, d.c_out, k2, d.nout()};
+  if (d.mlp) jobs[n++] = {w + o.w1, wT + W.w1t, 1, H, H, 128, H, 128};
   for (int l = 0; l < d.layers; ++l) {
-    note_launch();
-    pack_transpose_kernel<<<64, 256, 0, st>>>(Whh[l], H, H, 3 * H, 3 * H, wT + W.whh[l]);
-    if (l == 0) continue;
-    note_launch();
-    pack_transpose_kernel<<<64, 256, 0, st>>>(Wih[l], H, H, 3 * H, 3 * H, wT + W.wih[l]);
+    jobs[n++] = {Whh[l], wT + W.whh[l], 1, H, H, 3 * H, H, 3 * H};
+    if (l > 0) jobs[n++] = {Wih[l], wT + W.wih[l], 1, H, H, 3 * H, H, 3 * H};
   }
+  launch_pack(d, jobs, n, nullptr, nullptr, st);
 }
 
 size_t patchnet_backward_smem(const NetDims& d) {
@@ -776,11 +765,11 @@ void launch_loss(const double* part, int n, double inv, float* out, cudaStream_t
 }
 
 void launch_adam(float* w, const float* g, float* m, float* v, size_t n, float lr, int step,
-                 cudaStream_t st) {
+                 const int* skip, cudaStream_t st) {
   const float b1 = 0.9f, b2 = 0.999f;
   const float c1 = 1.0f - powf(b1, (float)step), c2 = 1.0f - powf(b2, (float)step);
   note_launch();
-  adam_kernel<<<cdiv((int)n, 256), 256, 0, st>>>(w, g, m, v, n, lr, b1, b2, c1, c2, 1e-8f);
+  adam_kernel<<<cdiv((int)n, 256), 256, 0, st>>>(w, g, m, v, n, lr, b1, b2, c1, c2, 1e-8f, skip);
 }
 
 }  // namespace dnnmg

@@ -91,3 +91,22 @@ def test_batched_cycle_matches_single_cycles(precision, tol, nu1, nu2, modes):
         assert rel(got, ref) < tol, rel(got, ref)
     for _ in range(10):
         assert torch.equal(B.vcycle(bvec), first)
+
+
+@pytest.mark.parametrize("ob,more", [((2, 1), {}), (None, {}), ((1, 1), dict(nu=0.001, dt=2.0)),
+                                     ((13, 1), dict(nu=0.02, dt=1e-3)),
+                                     ((6, 2, 1), dict(nu=0.001, dt=0.5))])
+def test_coarse_inverse_solves_the_coarse_system(ob, more):
+    """The coarse inverse by elimination of node columns, checked on the device
+    to 2e-12 per entry of A Ainv - 1 (the band LU takes over otherwise): with 891 unknowns the residual of a solve stays
+    below 891 * 2e-12 of the right-hand side's largest entry."""
+    dn = lib()
+    o = ob or (-1, -1)
+    kw = dict(dict(nu=0.01, dt=0.01), **more)
+    c = dn.Context(level_solve=2, precision=0, obstacle_i0=o[0], obstacle_j0=o[1],
+                   obstacle_level=1 if len(o) > 2 else 0, **kw)
+    c.linearize(torch.from_numpy(seeded_state(mesh.Level(2, obstacle=ob), 9)).cuda())
+    n = mesh.Level(1, obstacle=ob).ndof
+    b = torch.randn(n, generator=torch.Generator().manual_seed(2), dtype=torch.float64).cuda()
+    r = c.apply(1, c.vcycle(1, b)) - b
+    assert float(r.abs().max() / b.abs().max()) < 891 * 2e-12
