@@ -471,10 +471,10 @@ int dnnmg_vcycle_plan(const dnnmg_ctx* ctx, int level, int* split_level, int* sp
  * lock-step with the algorithm of a single context (Newton, FGMRES, one
  * V-cycle per Krylov step; DNN-MG steps add the network correction of
  * Algorithm 1 with one network evaluation over the patches of all problems).
- * Every stage (a Vanka colour pass on level k, a defect, a transfer, a
- * Krylov vector operation, ...) is one kernel launch over a work list of
- * the blocks of all problems that take part in it; problems that have
- * converged are masked.  One FGMRES iteration is replayed as a CUDA graph.
+ * The V-cycles of all problems are one cooperative launch, every other stage
+ * (a setup, a residual, a Krylov vector operation, ...) is one kernel launch
+ * over a work list of the blocks of all problems that take part in it;
+ * problems that have converged are masked.  One FGMRES iteration is replayed as a CUDA graph.
  *
  * Problems may differ in nu, dt, theta, alpha0, the obstacle and
  * level_solve; all other fields must be equal.  DNN-MG needs

@@ -1,9 +1,9 @@
 // Batched engine (internal): many independent channel problems of uneven
-// size stepped in lock-step, one kernel launch per V-cycle stage for all of
-// them.
+// size stepped in lock-step: the whole V-cycle of all of them is one cooperative
+// launch (batch_vcycle.cu), every other stage one launch.
 //
 // Every level of every problem is described by a BLev record in device
-// memory.  A stage kernel is launched over a work list of (problem, block)
+// memory.  A stage works through a work list of (problem, block)
 // pairs, built once at setup for that stage's level and block shape, so a
 // launch covers exactly the tiles or node blocks of the problems that have
 // the level and no block idles.  Problems that have converged are masked by

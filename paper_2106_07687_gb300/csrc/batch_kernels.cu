@@ -1,5 +1,6 @@
-// Batched stage kernels: one launch covers one stage (a Vanka colour pass, a
-// defect, a transfer, a vector operation, ...) of every problem of a batch.
+// Batched stage kernels: one launch covers one stage (a setup, a residual, a
+// vector operation, ...) of every problem of a batch (the V-cycle is in
+// batch_vcycle.cu).
 // Each block takes its (problem, block) pair from the stage's work list,
 // returns at once if the problem is masked, loads the problem's level record
 // and constants and runs the same per-node, per-tile or per-cell body as the
