@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(walk_threads<T>(), 1)
                                        nullptr, C.g.nn, tag0 + f.tcin, 0u, W.state},
                             iterate(F), i, j, valid, budget);
           else
-            prolong_node<T>(F.g, C.g, PlanarX<T>{C.x, nullptr, C.g.nn}, iterate(F), i, j, valid,
+            prolong_node<T>(F.g, C.g, PlanarX<T>{C.x, C.g.nn}, iterate(F), i, j, valid,
                             budget);
         });
         break;

@@ -244,7 +244,7 @@ __device__ __forceinline__ void walk_phases(const VLevel<T>* glv, const OpTable<
           if (f.tcin)
             prolong_node<T>(g, c, xc, x, i, j, valid, budget);
           else
-            prolong_node<T>(g, c, PlanarX<T>{C.x, nullptr, c.nn}, x, i, j, valid, budget);
+            prolong_node<T>(g, c, PlanarX<T>{C.x, c.nn}, x, i, j, valid, budget);
         }
         break;
       }

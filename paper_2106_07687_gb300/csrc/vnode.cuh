@@ -297,8 +297,8 @@ struct NodeLevel {
 };
 
 // ---- the iterate of a level ------------------------------------------------------------
-// PlanarX: [3][nn] arrays; a grid-wide barrier separates the phases that write
-// and read it.
+// PlanarX: [3][nn] arrays (the coarsest level's solution); a barrier lies between
+// the phases that write and read it.
 // TaggedX: every node's values carry the number of the update that wrote them,
 // in the same 16-byte word (FP32: u, v, p, tag; FP64: three words of a value and
 // a tag), which is stored and loaded as one access.  A reader waits until the
@@ -317,7 +317,6 @@ constexpr int kTagPolls = 1 << 21;
 template <typename T>
 struct PlanarX {
   const T* in;
-  T* out;
   int nn;
   template <int N, class F>
   __device__ __forceinline__ void load(const int (&n)[N], const bool (&)[N], T (&u)[N], T (&v)[N],
@@ -327,10 +326,6 @@ struct PlanarX {
       u[r] = __ldcg(in + n[r]), v[r] = __ldcg(in + nn + n[r]), p[r] = __ldcg(in + 2 * nn + n[r]);
     other_loads();
   }
-  __device__ __forceinline__ void store(int n, T u, T v, T p) const {
-    out[n] = u, out[nn + n] = v, out[2 * nn + n] = p;
-  }
-  __device__ __forceinline__ void store_one(int n, int c, T v) const { out[c * nn + n] = v; }
 };
 
 // (no clobber of memory: nothing but these two touches a tagged buffer, and a
