@@ -252,22 +252,31 @@ __device__ __forceinline__ void gauss_data(const T bu[4], const T bv[4], GaussDa
 // from interpolations along x and then y.  56 operations instead of 96, for the
 // types whose arithmetic bounds the operator kernels (FP64, double-float).
 template <typename T>
-__device__ __forceinline__ void gauss_data_shared(const T bu[4], const T bv[4], GaussData<T>& gd) {
+__device__ __forceinline__ void gauss_values(const T b[4], T v[4]) {
   const T G[2] = {T(kG0), T(kG1)}, F[2] = {T(1) - T(kG0), T(1) - T(kG1)};
-  auto field = [&](const T b[4], T v[4], T vx[4], T vy[4]) {
-    const T d0 = b[1] - b[0], d1 = b[3] - b[2], e0 = b[2] - b[0], e1 = b[3] - b[1];
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const T x = F[k] * d0 + G[k] * d1, y = F[k] * e0 + G[k] * e1;
-      const T lo = F[k] * b[0] + G[k] * b[1], hi = F[k] * b[2] + G[k] * b[3];
-      vx[2 * k] = vx[2 * k + 1] = x;  // points of one height
-      vy[k] = vy[2 + k] = y;          // points of one abscissa
-      v[k] = F[0] * lo + G[0] * hi;
-      v[2 + k] = F[1] * lo + G[1] * hi;
-    }
-  };
-  field(bu, gd.Bu, gd.Bux, gd.Buy);
-  field(bv, gd.Bv, gd.Bvx, gd.Bvy);
+  for (int k = 0; k < 2; ++k) {
+    const T lo = F[k] * b[0] + G[k] * b[1], hi = F[k] * b[2] + G[k] * b[3];
+    v[k] = F[0] * lo + G[0] * hi;
+    v[2 + k] = F[1] * lo + G[1] * hi;
+  }
+}
+template <typename T>
+__device__ __forceinline__ void gauss_derivatives(const T b[4], T vx[4], T vy[4]) {
+  const T G[2] = {T(kG0), T(kG1)}, F[2] = {T(1) - T(kG0), T(1) - T(kG1)};
+  const T d0 = b[1] - b[0], d1 = b[3] - b[2], e0 = b[2] - b[0], e1 = b[3] - b[1];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    vx[2 * k] = vx[2 * k + 1] = F[k] * d0 + G[k] * d1;  // points of one height
+    vy[k] = vy[2 + k] = F[k] * e0 + G[k] * e1;          // points of one abscissa
+  }
+}
+template <typename T>
+__device__ __forceinline__ void gauss_data_shared(const T bu[4], const T bv[4], GaussData<T>& gd) {
+  gauss_values<T>(bu, gd.Bu);
+  gauss_values<T>(bv, gd.Bv);
+  gauss_derivatives<T>(bu, gd.Bux, gd.Buy);
+  gauss_derivatives<T>(bv, gd.Bvx, gd.Bvy);
 }
 
 // Element Jacobian A'_T(vbar) entries between local nodes al (row) and be

@@ -112,7 +112,10 @@ __device__ __forceinline__ void assemble_node(const Grid& g, const Sten<T>& s,
       load_cell<T, false>(g, vb, ci, cj, 0, bu);
       load_cell<T, false>(g, vb + g.nn, ci, cj, 0, bv);
       GaussData<T> gd;
-      gauss_data<T>(bu, bv, gd);
+      if constexpr (sizeof(T) == 8)
+        gauss_data_shared<T>(bu, bv, gd);
+      else
+        gauss_data<T>(bu, bv, gd);
 #pragma unroll
       for (int b = 0; b < 4; ++b) {
         T J[3][3];
