@@ -329,7 +329,7 @@ int Batch<T>::init() {
       if (k >= 2) {
         l.inv = mem_.alloc<T>((size_t)4 * 144 * vanka_slots(g));
         l.cf = mem_.alloc<T>((size_t)kCoefs<T> * g.nn);
-        // no cycle has the number 0 the tags start with
+        // the words start with a number that no update has taken
         const size_t words = 2 * (size_t)kTagWords<T> * g.nn;
         l.xt = mem_.alloc<ulonglong2>(words);
         if (l.xt) cudaMemsetAsync(l.xt, 0, words * sizeof(ulonglong2), st_);
@@ -522,6 +522,7 @@ int Batch<T>::init() {
   walk_.Ainv = Ainv_;
   walk_.astride = astride_;
   walk_.state = status_ + n_;
+  walk_.numbers = vcycle_numbers(c0_.nu1, c0_.nu2);
   for (int k = 2; k <= Lmax_; ++k) {
     auto g = [&](int p, int l) -> const Grid& { return hl_[p][l].g; };
     walk_.defect[k] = level_items(k, [&](int p) { return vcycle_defect_tiles(g(p, k)); });

@@ -88,10 +88,11 @@ struct BWalk {
   int nprob, nL, mode, n1;  // mode: every problem's stabilisation form, -1 if they differ
   const double* Ainv;       // coarse inverses, `astride` doubles apart, n1 unknowns
   long long astride;
-  int* state;               // a status word and the cycle's number (see launch_vcycle_persistent)
+  int* state;               // a status word and the cycle's first number
+  unsigned numbers;         // by which a cycle advances it (see launch_vcycle_persistent)
   Work pass[kBLevels], defect[kBLevels], zero[kBLevels], restr[kBLevels], prol[kBLevels];
 };
-// one cycle over nph phases (build_batch_phases) of every active problem
+// one cycle over nph phases (vcycle_phases) of every active problem
 template <typename T>
 void bk_vcycle(const BWalk<T>& W, const Phase* ph, int nph, const T* topb, T* topx, T omega,
                const int* act, cudaStream_t st);

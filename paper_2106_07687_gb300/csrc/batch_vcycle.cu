@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(walk_threads<T>(), 1)
   const BLev<T>* rec = in_smem ? srec : W.lev;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int w0 = blockIdx.x + gridDim.x * w, nw = gridDim.x * NW;
-  const unsigned cycle = __ldcg(reinterpret_cast<unsigned*>(W.state) + 1), tag0 = cycle << 8;
+  const unsigned tag0 = __ldcg(reinterpret_cast<unsigned*>(W.state) + 1);
   int budget = kTagPolls;
   for (int p = p0; p < p1; ++p) {
     Phase f{};
@@ -177,10 +177,12 @@ __global__ void __launch_bounds__(walk_threads<T>(), 1)
   // every block has read the number before its first barrier (a cycle with a
   // phase that uses it has one)
   if (bump && blockIdx.x == 0 && threadIdx.x == 0)
-    *(reinterpret_cast<volatile unsigned*>(W.state) + 1) = cycle + 1;
+    *(reinterpret_cast<volatile unsigned*>(W.state) + 1) = tag0 + W.numbers;
 }
 
-__global__ void next_cycle_kernel(int* state) { state[1] += 1; }
+__global__ void next_cycle_kernel(int* state, unsigned numbers) {
+  state[1] = (int)((unsigned)state[1] + numbers);
+}
 
 template <typename T>
 size_t walk_bytes(int nprob, int nL, int n1) {
@@ -221,7 +223,7 @@ void bk_vcycle(const BWalk<T>& W, const Phase* ph, int nph, const T* topb, T* to
                                                      0);
   }
   note_launch();
-  next_cycle_kernel<<<1, 1, 0, st>>>(W.state);
+  next_cycle_kernel<<<1, 1, 0, st>>>(W.state, W.numbers);
 }
 
 template void bk_vcycle<float>(const BWalk<float>&, const Phase*, int, const float*, float*, float,

@@ -80,7 +80,7 @@ class Solver final : public SolverBase {
     coarse_work_ = c_->mem.alloc<double>(coarse_factor_doubles(g0));
     ainv_ = c_->mem.alloc<double>((size_t)9 * g0.nn * g0.nn);
     status_ = c_->mem.alloc<int>(4);
-    // setup status (0, 1), wait status (2) and the number of the next cycle (3)
+    // setup status (0, 1), wait status (2) and the next cycle's first number (3)
     if (status_) {
       cudaMemsetAsync(status_, 0, 3 * sizeof(int), st_);  // fresh memory is not zero
       cudaMemsetAsync(status_ + 3, 1, sizeof(int), st_);
@@ -108,7 +108,8 @@ class Solver final : public SolverBase {
     if (cfg.persistent_vcycle != 0) {
       std::vector<VLevel<T>> hv(K_ + 1);
       for (int k = 0; k <= K_; ++k) {
-        // the iterate's tagged buffers; no cycle has the number 0 they start with
+        // the iterate's tagged buffers, whose words start with a number that no
+        // update has taken
         const size_t words = 2 * (size_t)kTagWords<T> * lv_[k].g.nn;
         ulonglong2* xt = k > 0 ? c_->mem.alloc<ulonglong2>(words) : nullptr;
         if (xt) cudaMemsetAsync(xt, 0, words * sizeof(ulonglong2), st_);
@@ -563,18 +564,19 @@ class Solver final : public SolverBase {
         (split_mode_ == 0 ? vgrid_ > 0 : cluster_ > 0)) {
       const int p = c_->prof.begin(DNNMG_STAGE_VCYCLE, lv_[k].level, st_);
       int rc;
+      const unsigned numbers = vcycle_numbers(c_->cfg.nu1, c_->cfg.nu2);
       if (split_mode_ == 0) {
         // at most one block per warp tile of the sub-cycle's top level
         int blocks = std::max(64, vcycle_warp_tiles(lv_[k].g));
         if (coop_cap_ > 0 && blocks > coop_cap_) blocks = coop_cap_;
         blocks = blocks > vgrid_ ? vgrid_ : blocks;
         rc = launch_vcycle_persistent<T>(dlv_, dtab_, dph_ + ph_off_[k], ph_n_[k], k, b, x, ainv_,
-                                         (T)c_->cfg.omega, status_ + 2, blocks, coarse_nd_, st_,
-                                         skip);
+                                         (T)c_->cfg.omega, status_ + 2, numbers, blocks,
+                                         coarse_nd_, st_, skip);
       } else {
         rc = launch_vcycle_cluster<T>(dlv_, dtab_, dph_ + ph_off_[k], ph_n_[k], k, b, x, ainv_,
-                                      (T)c_->cfg.omega, status_ + 2, cluster_, coarse_nd_,
-                                      st_);
+                                      (T)c_->cfg.omega, status_ + 2, numbers, cluster_,
+                                      coarse_nd_, st_);
       }
       c_->prof.end(p, st_);
       if (rc == 0) return;

@@ -83,18 +83,19 @@ __device__ __forceinline__ void for_items(int count, F f) {
 // arrays (a grid-wide barrier for the cooperative launch, the cluster barrier for
 // the single-cluster launch).  Threads of all blocks split every node-wise
 // phase; the warp tiles of a colour pass or defect go round-robin over the
-// blocks first.  state: the status word and the cycle's number.
+// blocks first.  state: the status word and the cycle's first number.
 template <typename T, class Sync>
 __device__ __forceinline__ void walk_phases(const VLevel<T>* glv, const OpTable<T>* gtab,
                                             const Phase* gph, int nph, int top, const T* topb,
                                             T* topx, const double* __restrict__ Ainv, T omega,
-                                            int* state, WalkSmem<T>& S, Sync sync) {
+                                            int* state, unsigned numbers, WalkSmem<T>& S,
+                                            Sync sync) {
   constexpr int NT = walk_threads<T>();
   double* sbuf = reinterpret_cast<double*>(S.tile);  // the coarse right-hand side
   copy_ints(S.lv, glv, top + 1);
   copy_ints(S.ph, gph, nph);
   copy_ints(&S.tab, gtab, 1);
-  const unsigned cycle = __ldcg(reinterpret_cast<unsigned*>(state) + 1), tag0 = cycle << 8;
+  const unsigned tag0 = __ldcg(reinterpret_cast<unsigned*>(state) + 1);
   __syncthreads();
   for (int p = threadIdx.x; p < nph; p += NT) {
     const Phase f = S.ph[p];
@@ -258,20 +259,20 @@ __device__ __forceinline__ void walk_phases(const VLevel<T>* glv, const OpTable<
   // every block has read the number before its first barrier (a cycle with a
   // phase that uses it has one)
   if (blockIdx.x == 0 && threadIdx.x == 0)
-    *(reinterpret_cast<volatile unsigned*>(state) + 1) = cycle + 1;
+    *(reinterpret_cast<volatile unsigned*>(state) + 1) = tag0 + numbers;
 }
 
 template <typename T>
 __global__ void __launch_bounds__(walk_threads<T>(), 1)
     vcycle_kernel(const VLevel<T>* lv, const OpTable<T>* tab, const Phase* ph, int nph, int top,
                   const T* topb, T* topx, const double* __restrict__ Ainv, T omega, int* state,
-                  const int* skip) {
+                  unsigned numbers, const int* skip) {
   // a speculative FGMRES iteration after the cycle stopped: every block
   // reads the same flag (set before this launch) and returns before any barrier
   if (skip && *skip) return;
   extern __shared__ __align__(16) uint8_t dyn[];
   cg::grid_group grid = cg::this_grid();
-  walk_phases<T>(lv, tab, ph, nph, top, topb, topx, Ainv, omega, state,
+  walk_phases<T>(lv, tab, ph, nph, top, topb, topx, Ainv, omega, state, numbers,
                  *reinterpret_cast<WalkSmem<T>*>(dyn), [&] { grid.sync(); });
 }
 
@@ -282,10 +283,10 @@ template <typename T>
 __global__ void __launch_bounds__(walk_threads<T>(), 1)
     vcycle_cluster_kernel(const VLevel<T>* lv, const OpTable<T>* tab, const Phase* ph, int nph,
                           int top, const T* topb, T* topx, const double* __restrict__ Ainv,
-                          T omega, int* state) {
+                          T omega, int* state, unsigned numbers) {
   extern __shared__ __align__(16) uint8_t dyn[];
   cg::cluster_group cl = cg::this_cluster();
-  walk_phases<T>(lv, tab, ph, nph, top, topb, topx, Ainv, omega, state,
+  walk_phases<T>(lv, tab, ph, nph, top, topb, topx, Ainv, omega, state, numbers,
                  *reinterpret_cast<WalkSmem<T>*>(dyn), [&] { cl.sync(); });
 }
 
@@ -390,11 +391,11 @@ int vcycle_grid(int coarse_nd) {
 template <typename T>
 int launch_vcycle_persistent(const VLevel<T>* lv, const OpTable<T>* tab, const Phase* ph, int nph,
                              int top, const T* topb, T* topx, const double* Ainv, T omega,
-                             int* state, int grid, int coarse_nd, cudaStream_t st,
-                             const int* skip) {
+                             int* state, unsigned numbers, int grid, int coarse_nd,
+                             cudaStream_t st, const int* skip) {
   void* args[] = {(void*)&lv,   (void*)&tab,  (void*)&ph,   (void*)&nph,   (void*)&top,
                   (void*)&topb, (void*)&topx, (void*)&Ainv, (void*)&omega, (void*)&state,
-                  (void*)&skip};
+                  (void*)&numbers, (void*)&skip};
   note_launch();
   const cudaError_t e =
       cudaLaunchCooperativeKernel((void*)vcycle_kernel<T>, dim3(grid), dim3(walk_threads<T>()),
@@ -440,7 +441,8 @@ int vcycle_cluster_size(int coarse_nd) {
 template <typename T>
 int launch_vcycle_cluster(const VLevel<T>* lv, const OpTable<T>* tab, const Phase* ph, int nph,
                           int top, const T* topb, T* topx, const double* Ainv, T omega,
-                          int* state, int cluster, int coarse_nd, cudaStream_t st) {
+                          int* state, unsigned numbers, int cluster, int coarse_nd,
+                          cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -455,7 +457,7 @@ int launch_vcycle_cluster(const VLevel<T>* lv, const OpTable<T>* tab, const Phas
   cfg.numAttrs = 1;
   note_launch();
   const cudaError_t e = cudaLaunchKernelEx(&cfg, vcycle_cluster_kernel<T>, lv, tab, ph, nph, top,
-                                           topb, topx, Ainv, omega, state);
+                                           topb, topx, Ainv, omega, state, numbers);
   return e == cudaSuccess ? 0 : 1;
 }
 
@@ -463,12 +465,12 @@ int launch_vcycle_cluster(const VLevel<T>* lv, const OpTable<T>* tab, const Phas
   template void launch_assemble_blocks<T>(const AsmLevel<T>*, int, int, cudaStream_t);           \
   template int vcycle_grid<T>(int);                                                              \
   template int launch_vcycle_persistent<T>(const VLevel<T>*, const OpTable<T>*, const Phase*,    \
-                                           int, int, const T*, T*, const double*, T, int*, int,  \
-                                           int, cudaStream_t, const int*);                       \
+                                           int, int, const T*, T*, const double*, T, int*,       \
+                                           unsigned, int, int, cudaStream_t, const int*);        \
   template int vcycle_cluster_size<T>(int);                                                      \
   template int launch_vcycle_cluster<T>(const VLevel<T>*, const OpTable<T>*, const Phase*, int,  \
-                                        int, const T*, T*, const double*, T, int*, int, int,     \
-                                        cudaStream_t);
+                                        int, const T*, T*, const double*, T, int*, unsigned,     \
+                                        int, int, cudaStream_t);
 DNNMG_INST(float)
 DNNMG_INST(double)
 #undef DNNMG_INST

@@ -54,6 +54,13 @@ struct Phase {
   int tin = 0, tout = 0, cin = 0, tcin = 0, last = 0;
 };
 
+// How far a cycle advances the numbers of the updates: a level's iterate takes
+// the numbers 0 (its start from zero) to 4 (nu1 + nu2) + 1 (every colour pass and
+// the prolongation) above the cycle's first.
+inline unsigned vcycle_numbers(int nu1, int nu2) {
+  return 4u * ((unsigned)nu1 + (unsigned)nu2) + 2u;
+}
+
 // phase list of one V(nu1, nu2) cycle with top level `top`, x zeroed first
 std::vector<Phase> vcycle_phases(int top, int nu1, int nu2);
 // whether a launch of nphases phases over nlevels levels fits the kernels'
@@ -76,15 +83,18 @@ int vcycle_cluster_size(int coarse_nd);
 template <typename T>
 int launch_vcycle_cluster(const VLevel<T>* lv, const OpTable<T>* tab, const Phase* ph, int nph,
                           int top, const T* topb, T* topx, const double* Ainv, T omega,
-                          int* state, int cluster, int coarse_nd, cudaStream_t st);
+                          int* state, unsigned numbers, int cluster, int coarse_nd,
+                          cudaStream_t st);
 // state: two device words, a status word (8: a wait for an update hit its bound)
-// and the cycle's number, which the launch counts up (starts above 0).
+// and the cycle's first number, which the launch advances by `numbers`
+// (vcycle_numbers; the word starts above 0).
 // returns 0 on success; with skip, nothing runs when *skip != 0 at the
 // launch's start
 template <typename T>
 int launch_vcycle_persistent(const VLevel<T>* lv, const OpTable<T>* tab, const Phase* ph, int nph,
                              int top, const T* topb, T* topx, const double* Ainv, T omega,
-                             int* state, int grid, int coarse_nd, cudaStream_t st,
+                             int* state, unsigned numbers, int grid, int coarse_nd,
+                             cudaStream_t st,
                              const int* skip = nullptr);
 
 }  // namespace dnnmg

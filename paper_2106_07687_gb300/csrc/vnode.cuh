@@ -309,8 +309,10 @@ struct NodeLevel {
 // the barrier's chain (stores acknowledged, an atomic, a poll) and the load
 // behind it become one store and one polled load.  Two buffers suffice: the
 // tile that overwrites a node has waited for the values of every tile that read
-// the node's previous ones (they lie within its own two-node halo).  Tags never
-// repeat: they hold the cycle's number, kept on the device.  The wait is
+// the node's previous ones (they lie within its own two-node halo).  The numbers
+// run on from cycle to cycle (vcycle_numbers per cycle, whatever its sweeps), in a
+// word on the device: they come round after 2^32 updates, 238 million V(2,2)
+// cycles, in which every word that a cycle reads is rewritten.  The wait is
 // bounded (kTagPolls rounds over a warp's whole run; then bit 8 of *status is
 // set and the warp stops waiting).  All lanes of the warp call load; other_loads
 // is run once, behind the first round's loads, to issue what the tile reads
