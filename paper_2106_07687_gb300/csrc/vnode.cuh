@@ -239,7 +239,10 @@ __device__ __forceinline__ void vanka_setup_cell(const Grid& g, const uint16_t* 
     const unsigned mx = __reduce_max_sync(mask, key);
     const int p = (__ffs(__ballot_sync(mask, key == mx && !used) & mask) - 1) & 15;
     pcol[k] = p;
-    ok = ok && mx != 0u;  // the same in every lane of the group
+    // a pivot that is neither zero nor NaN (whose bits lie above infinity's; the
+    // same in every lane of the group)
+    constexpr unsigned kInf = sizeof(T) == 4 ? 0x7F800000u : 0x7FF00000u;
+    ok = ok && mx != 0u && mx <= kInf;
     if (ok) {
       const bool piv = lane == p;
       const T ip = pivot_recip(__shfl_sync(mask, A[k], p, 16));

@@ -1,4 +1,5 @@
-"""V-cycles at the edges of what the calls accept: very many smoothing sweeps."""
+"""V-cycles at the edges of what the calls accept: very many smoothing sweeps, and
+linearisation points that are not finite."""
 import pytest
 
 from oracle import mesh
@@ -47,3 +48,33 @@ def test_batched_cycle_with_many_sweeps(precision, tol, nu1, nu2):
                                                                            rel(got, ref64))
     for k in range(20):
         assert torch.equal(B.vcycle(rhs[k % 2]), first[k % 2])
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("node", [(7, 5), (8, 8), (38, 19)])
+def test_linearisation_at_a_non_finite_state_is_an_error(precision, node, bad):
+    """A velocity that is not finite makes local matrices without an inverse, on the
+    finest level only ((7, 5): a node of no coarser level) or on all of them, and
+    linearize reports it, for one problem and in a batch."""
+    dn = lib()
+    L = 3
+    lev = mesh.Level(L, obstacle=(5, 1))
+    good = torch.from_numpy(seeded_state(lev, 3)).cuda()
+    x = good.clone()
+    x[node[1] * lev.nnx + node[0]] = bad
+    kw = dict(level_solve=L, precision=precision, obstacle_i0=5, obstacle_j0=1, nu=0.01, dt=0.01)
+    c = dn.Context(**kw)
+    B = dn.Batch([dn.default_config(**kw), dn.default_config(**kw)])
+    for tries in range(2):  # the first linearisation, and one after a good one
+        with pytest.raises(dn.DnnmgError) as e:
+            c.linearize(x)
+        assert e.value.code == dn.ERR_NUMERICAL
+        B.set_state(0, good)
+        B.set_state(1, x)
+        with pytest.raises(dn.DnnmgError) as e:
+            B.linearize()
+        assert e.value.code == dn.ERR_NUMERICAL
+        B.set_state(1, good)
+        B.linearize()
+        c.linearize(good)
