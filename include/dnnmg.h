@@ -188,7 +188,8 @@ int dnnmg_set_state(dnnmg_ctx* ctx, const double* x);
  * inverses, coarse-level LU and inverse).  Needed before dnnmg_apply() and
  * dnnmg_vcycle(); dnnmg_step() does it itself.
  * Errors: DNNMG_ERR_NUMERICAL if a local Vanka matrix or the coarse matrix
- * is singular. */
+ * is singular, DNNMG_ERR_TIMEOUT (once) if a wait inside a V-cycle launched
+ * earlier hit its bound; the linearisation is then complete. */
 int dnnmg_linearize(dnnmg_ctx* ctx, const double* x);
 
 /* y = A'(vbar) w on level `level` (coarse <= level <= L) at the current
@@ -200,7 +201,9 @@ int dnnmg_apply(dnnmg_ctx* ctx, int level, const void* w, void* y, int precision
 /* One V(nu1, nu2) cycle (Sec. 2.2; cell-wise Vanka smoother, bilinear
  * transfers, direct coarse solve) on level `level` for A'(vbar) x = b,
  * starting from x = 0.  b, x: device [3][nn] arrays of the context's
- * precision (see dnnmg_apply).  b should vanish on constrained DOFs. */
+ * precision (see dnnmg_apply).  b should vanish on constrained DOFs.
+ * The call does not wait for the cycle: a wait inside it that hit its bound is
+ * reported by the next dnnmg_linearize() or dnnmg_step(). */
 int dnnmg_vcycle(dnnmg_ctx* ctx, int level, const void* b, void* x, int precision);
 
 /* r = f - A_n(x) (Eqs. 4-5) on level L in FP64, zero on constrained DOFs.
@@ -215,7 +218,8 @@ int dnnmg_residual(dnnmg_ctx* ctx, const double* x, const double* f, double* r);
  * the step is recomputed without the network right-hand side (Sec. 3.3).
  * stats (host pointer, may be NULL) receives the step statistics.
  * Returns DNNMG_ERR_NOT_CONVERGED if Newton hit newton_max (the step is still
- * taken), DNNMG_ERR_NUMERICAL on NaN/Inf. */
+ * taken), DNNMG_ERR_NUMERICAL on NaN/Inf, DNNMG_ERR_TIMEOUT if a wait inside a
+ * V-cycle or the network hit its bound. */
 int dnnmg_step(dnnmg_ctx* ctx, int mode, dnnmg_step_stats* stats);
 
 /* One time step with the level-L state exchanged through HOST memory (the
@@ -464,6 +468,12 @@ int dnnmg_vcycle_split(const dnnmg_ctx* ctx);
 int dnnmg_vcycle_plan(const dnnmg_ctx* ctx, int level, int* split_level, int* split_mode,
                       int* pass_shape);
 
+/* Bound of the waits inside the context's V-cycles: a warp polls at most `polls`
+ * times per phase for the values it needs, then goes on without them and the
+ * cycle is reported (see dnnmg_vcycle).  The default, 2^21, is over a second;
+ * with 0 every cycle gives up at once and is reported.  Synchronous. */
+int dnnmg_vcycle_polls(dnnmg_ctx* ctx, int polls);
+
 /* ------------------------------------------------------------------------
  * Batched problems
  *
@@ -516,7 +526,8 @@ int dnnmg_batch_vcycle(dnnmg_batch* b, const void* rhs, void* x);
  * that problem's own device vectors ([3][nn] of its level, batch precision),
  * not the concatenated ones.  The instance form of dnnmg_vcycle.
  * Errors: DNNMG_ERR_ARG (inst out of range), DNNMG_ERR_STATE (not
- * linearised). */
+ * linearised), DNNMG_ERR_TIMEOUT (a wait inside the cycle hit its bound; also
+ * dnnmg_batch_vcycle and dnnmg_batch_step). */
 int dnnmg_batch_vcycle_inst(dnnmg_batch* b, int inst, const void* rhs, void* x);
 /* One time step of every problem; stats[0..n) (nullable) receive each
  * problem's counts and status (ms: the batch's step time).  Returns
@@ -529,6 +540,8 @@ int dnnmg_batch_set_feature_stats(dnnmg_batch* b, const float* mean, const float
 /* corrected fine velocity of problem `inst` after a DNN-MG step ([2][..] of
  * level L + replaced_levels, device) */
 int dnnmg_batch_get_fine_velocity(dnnmg_batch* b, int inst, double* v);
+/* the batch's form of dnnmg_vcycle_polls */
+int dnnmg_batch_vcycle_polls(dnnmg_batch* b, int polls);
 /* on != 0 (default): replay FGMRES iterations as CUDA graphs */
 int dnnmg_batch_graphs(dnnmg_batch* b, int on);
 /* stage timers as dnnmg_profile / dnnmg_profile_read (levels are absolute) */

@@ -75,6 +75,12 @@ class Batch final : public BatchBase {
   int set_feature_stats(const float* mean, const float* stdv);
   int get_fine_velocity(int p, double* v);
   Prof& prof() { return prof_; }
+  int set_polls(int polls) {
+    sync_in();
+    cudaMemcpyAsync(status_ + n_ + 2, &polls, sizeof(int), cudaMemcpyHostToDevice, st_);
+    cudaStreamSynchronize(st_);
+    return check("vcycle_polls");
+  }
   int set_graphs(int on) {
     use_graphs_ = on != 0;
     return DNNMG_OK;
@@ -157,6 +163,7 @@ class Batch final : public BatchBase {
   }
 
   void vcycle_all(const T* b, T* x, const int* act);
+  int wait_status(int word);
   int read_status(std::vector<int>& status);
   void fgmres_iteration(int j);
   int linearize_masked(const int* act, bool coarse, bool precond);
@@ -393,7 +400,7 @@ int Batch<T>::init() {
   cact_ = mem_.alloc<int>(n_);
   nact_ = mem_.alloc<int>(n_);
   sel_ = mem_.alloc<int>(n_);
-  status_ = mem_.alloc<int>(n_ + 2);  // and the cycles' state words
+  status_ = mem_.alloc<int>(n_ + 3);  // and the cycles' state words
   // vector blocks
   std::vector<int> vinst(nblk), vfirst(n_), vcount(n_);
   for (int p = 0; p < n_; ++p) {
@@ -563,8 +570,8 @@ int Batch<T>::init() {
     cudaStreamSynchronize(st_);
   }
   for (int* a : {kcnt_, its_, gact_, cact_, nact_, sel_, status_}) cudaMemsetAsync(a, 0, sizeof(int) * n_, st_);
-  cudaMemsetAsync(status_ + n_, 0, sizeof(int), st_);
-  cudaMemsetAsync(status_ + n_ + 1, 1, sizeof(int), st_);
+  const int words[3] = {0, 1, kTagPolls};
+  cudaMemcpyAsync(status_ + n_, words, sizeof(words), cudaMemcpyHostToDevice, st_);
   for (double* a : {resid_, target_, nrm_}) cudaMemsetAsync(a, 0, sizeof(double) * n_, st_);
   const double one = 1.0;
   cudaMemcpyAsync(one_, &one, sizeof(double), cudaMemcpyHostToDevice, st_);
@@ -585,14 +592,20 @@ void Batch<T>::vcycle_all(const T* b, T* x, const int* act) {
   prof_.end(p, st_);
 }
 
-// The setups' status words, and an error when a wait of an earlier cycle hit its
-// bound (reported once).
+// An error when a wait of a cycle hit its bound (`word`: the cycles' status word),
+// reported once.
+template <typename T>
+int Batch<T>::wait_status(int word) {
+  if (!word) return DNNMG_OK;
+  cudaMemsetAsync(status_ + n_, 0, sizeof(int), st_);
+  return fail(DNNMG_ERR_TIMEOUT, "a wait inside a V-cycle timed out");
+}
+
+// The setups' status words, and the cycles' (wait_status).
 template <typename T>
 int Batch<T>::read_status(std::vector<int>& status) {
   if (int rc = sync_read(status_, status.data(), sizeof(int) * (n_ + 1))) return rc;
-  if (!status[n_]) return DNNMG_OK;
-  cudaMemsetAsync(status_ + n_, 0, sizeof(int), st_);
-  return fail(DNNMG_ERR_TIMEOUT, "a wait for an update of the cycle timed out");
+  return wait_status(status[n_]);
 }
 
 // Linearise the active problems at their current state: the FGMRES matvec
@@ -788,6 +801,14 @@ int Batch<T>::newton(const std::vector<int>& mask, std::vector<dnnmg_step_stats>
   std::vector<int> gits(n_, 0), nits(n_, 0);
   for (int q = 0; q < n_; ++q)
     if (act[q]) s[q].res0 = nrm[q];
+  // the status of these solves' cycles, read when they end; NaN may come from a
+  // cycle whose wait hit its bound, which is then the error
+  auto late = [&](int rc) {
+    int word = 0;
+    if (int r2 = sync_read(status_ + n_, &word, sizeof(int))) return r2;
+    if (int r2 = wait_status(word)) return r2;
+    return rc;
+  };
   int it = 0;
   while (true) {
     bool any = false;
@@ -818,7 +839,7 @@ int Batch<T>::newton(const std::vector<int>& mask, std::vector<dnnmg_step_stats>
         }
       if (changed) act_d = upload_mask(act, nact_);
     }
-    if (int rc = solve(act_d, act, gits)) return rc;
+    if (int rc = solve(act_d, act, gits)) return late(rc);
     p = prof_.begin(DNNMG_STAGE_RESIDUAL, Lmax_, st_);
     bk_residual64<T>(v_, 0, x64_, f64_, r64_, top_.w(), act_d, st_);
     prof_.end(p, st_);
@@ -838,7 +859,7 @@ int Batch<T>::newton(const std::vector<int>& mask, std::vector<dnnmg_step_stats>
     s[q].res_final = nrm[q];
     if (s[q].status == DNNMG_OK && nrm[q] > c0_.newton_tol) s[q].status = DNNMG_ERR_NOT_CONVERGED;
   }
-  return check("newton");
+  return late(check("newton"));
 }
 
 // the network correction of Algorithm 1 for every problem after the level-L solves.
@@ -960,7 +981,8 @@ int Batch<T>::vcycle_one(int p, const void* b, void* x) {
   cudaMemcpyAsync(bb + off_[p], b, sizeof(T) * n3, cudaMemcpyDeviceToDevice, st_);
   vcycle_all(bb, xx, act);
   cudaMemcpyAsync(x, xx + off_[p], sizeof(T) * n3, cudaMemcpyDeviceToDevice, st_);
-  cudaStreamSynchronize(st_);
+  std::vector<int> status(n_ + 1);
+  if (int rc = read_status(status)) return rc;
   return check("vcycle_one");
 }
 
@@ -1145,6 +1167,11 @@ int dnnmg_batch_set_feature_stats(dnnmg_batch* b, const float* mean_host, const 
 int dnnmg_batch_get_fine_velocity(dnnmg_batch* b, int inst, double* v) {
   if (!b || !v || inst < 0 || inst >= (int)b->cfg.size()) return DNNMG_ERR_ARG;
   return with_engine(b, [&](auto& e) { return e.get_fine_velocity(inst, v); });
+}
+
+int dnnmg_batch_vcycle_polls(dnnmg_batch* b, int polls) {
+  if (!b || polls < 0) return DNNMG_ERR_ARG;
+  return with_engine(b, [&](auto& e) { return e.set_polls(polls); });
 }
 
 int dnnmg_batch_graphs(dnnmg_batch* b, int on) {

@@ -88,8 +88,8 @@ struct BWalk {
   int nprob, nL, mode, n1;  // mode: every problem's stabilisation form, -1 if they differ
   const double* Ainv;       // coarse inverses, `astride` doubles apart, n1 unknowns
   long long astride;
-  int* state;               // a status word and the cycle's first number
-  unsigned numbers;         // by which a cycle advances it (see launch_vcycle_persistent)
+  int* state;               // the cycle's state words (see launch_vcycle_persistent)
+  unsigned numbers;
   Work pass[kBLevels], defect[kBLevels], zero[kBLevels], restr[kBLevels], prol[kBLevels];
 };
 // one cycle over nph phases (vcycle_phases) of every active problem

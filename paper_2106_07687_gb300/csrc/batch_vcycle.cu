@@ -48,8 +48,10 @@ __global__ void __launch_bounds__(walk_threads<T>(), 1)
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int w0 = blockIdx.x + gridDim.x * w, nw = gridDim.x * NW;
   const unsigned tag0 = __ldcg(reinterpret_cast<unsigned*>(W.state) + 1);
-  int budget = kTagPolls;
+  const int polls = __ldcg(W.state + 2);
+  int budget = polls;
   for (int p = p0; p < p1; ++p) {
+    if (budget > 0) budget = polls;
     Phase f{};
     f.type = __ldg(&ph[p].type), f.level = __ldg(&ph[p].level), f.colour = __ldg(&ph[p].colour);
     f.in = __ldg(&ph[p].in), f.out = __ldg(&ph[p].out);

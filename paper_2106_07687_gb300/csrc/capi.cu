@@ -465,6 +465,11 @@ int dnnmg_vcycle_plan(const dnnmg_ctx* ctx, int level, int* split_level, int* sp
   return DNNMG_OK;
 }
 
+int dnnmg_vcycle_polls(dnnmg_ctx* ctx, int polls) {
+  if (!ctx || !ctx->solver || polls < 0) return DNNMG_ERR_ARG;
+  return ctx->solver->set_polls(polls);
+}
+
 size_t dnnmg_num_params(const dnnmg_ctx* ctx) { return ctx ? ctx->nd.num_params() : 0; }
 
 int dnnmg_net_dims(const dnnmg_ctx* ctx, int* c_in, int* c_out) {

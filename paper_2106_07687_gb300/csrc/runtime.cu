@@ -79,11 +79,12 @@ class Solver final : public SolverBase {
     if (part_solid_) pieces_ = make_patch_pieces(g0.h, cfg);
     coarse_work_ = c_->mem.alloc<double>(coarse_factor_doubles(g0));
     ainv_ = c_->mem.alloc<double>((size_t)9 * g0.nn * g0.nn);
-    status_ = c_->mem.alloc<int>(4);
-    // setup status (0, 1), wait status (2) and the next cycle's first number (3)
+    status_ = c_->mem.alloc<int>(5);
+    // setup status (0, 1), wait status (2), the next cycle's first number (3) and
+    // the bound of a warp's polls per phase (4)
     if (status_) {
-      cudaMemsetAsync(status_, 0, 3 * sizeof(int), st_);  // fresh memory is not zero
-      cudaMemsetAsync(status_ + 3, 1, sizeof(int), st_);
+      const int words[5] = {0, 0, 0, 1, kTagPolls};
+      cudaMemcpyAsync(status_, words, sizeof(words), cudaMemcpyHostToDevice, st_);
     }
     m_ = cfg.gmres_m;
     n_ = 3 * (size_t)lv_[K_].g.nn;
@@ -216,11 +217,12 @@ class Solver final : public SolverBase {
       linearized_ = true;
       return c_->check("linearize");
     }
-    int status = 0;
-    cudaMemcpyAsync(c_->h_scalars, status_, sizeof(int), cudaMemcpyDeviceToHost, st_);
+    int words[4] = {0, 0, 0, 0}, status = 0;
+    cudaMemcpyAsync(c_->h_scalars, status_, sizeof(words), cudaMemcpyDeviceToHost, st_);
     if (int rc = c_->check("linearize")) return rc;
     cudaStreamSynchronize(st_);
-    std::memcpy(&status, c_->h_scalars, sizeof(int));
+    std::memcpy(words, c_->h_scalars, sizeof(words));
+    const int late = status_from(words, &status);  // of cycles launched before
     linearized_ = true;
     if (!tuned_) {
       tune_split();
@@ -228,7 +230,14 @@ class Solver final : public SolverBase {
     }
     if (status & 1) return c_->fail(DNNMG_ERR_NUMERICAL, "singular local Vanka matrix");
     if (status & 2) return c_->fail(DNNMG_ERR_NUMERICAL, "singular coarse-level matrix");
+    if (late) return c_->fail(DNNMG_ERR_TIMEOUT, "a wait inside an earlier V-cycle timed out");
     return DNNMG_OK;
+  }
+
+  int set_polls(int polls) override {
+    cudaMemcpyAsync(status_ + 4, &polls, sizeof(int), cudaMemcpyHostToDevice, st_);
+    cudaStreamSynchronize(st_);
+    return c_->check("vcycle_polls");
   }
 
   int apply(int k, const void* w, void* y) override {
@@ -1389,6 +1398,12 @@ int dnnmg_ctx::residual_norm_end(unsigned long long t, double* nrm) {
 }
 
 int dnnmg_ctx::newton(const double* f, dnnmg_step_stats* s) {
+  // NaN may come from a cycle whose wait hit its bound: that is then the error
+  auto numerical = [&](int rc) {
+    return rc == DNNMG_ERR_NUMERICAL && solver->device_status() > 0
+               ? fail(DNNMG_ERR_TIMEOUT, "a wait inside a V-cycle timed out")
+               : rc;
+  };
   const unsigned long long t0 = residual_norm_begin(f);
   // the linearisations' singularity flags are read once, after the loop
   solver->clear_setup_status();
@@ -1405,7 +1420,8 @@ int dnnmg_ctx::newton(const double* f, dnnmg_step_stats* s) {
   s->res0 = nrm;
   int it = 0, gits = 0;
   while (nrm > cfg.newton_tol && it < cfg.newton_max) {
-    if (!std::isfinite(nrm)) return fail(DNNMG_ERR_NUMERICAL, "non-finite Newton residual");
+    if (!std::isfinite(nrm))
+      return numerical(fail(DNNMG_ERR_NUMERICAL, "non-finite Newton residual"));
     // the coarse-level factorisation is refreshed at the first Newton step of
     // every coarse_refresh-th time step (a lagged preconditioner component)
     const bool refresh = it == 0 && steps_taken % cfg.coarse_refresh == 0;
@@ -1415,7 +1431,7 @@ int dnnmg_ctx::newton(const double* f, dnnmg_step_stats* s) {
     if (!(it == 0 && lin0))
       if (int rc = solver->linearize(x64, refresh, precond, false)) return rc;
     int its = 0;
-    if (int rc = solver->solve(r64, x64, cfg.eps_damp, &its)) return rc;
+    if (int rc = solver->solve(r64, x64, cfg.eps_damp, &its)) return numerical(rc);
     gits += its;
     // the smoothers' and setups' status words travel with this norm
     if (int rc = residual_norm_end(residual_norm_begin(f, true), &nrm)) return rc;
@@ -1430,7 +1446,7 @@ int dnnmg_ctx::newton(const double* f, dnnmg_step_stats* s) {
   for (int i = 0; i < 4; ++i) words[i] = mail_h->iv[i];
   // after an iteration the status words came with the last norm; else read them now
   if (const int ds = it > 0 ? solver->status_from(words, &setup) : solver->device_status(&setup))
-    return ds < 0 ? check("newton") : fail(DNNMG_ERR_TIMEOUT, "a colour pass's inverse copy timed out");
+    return ds < 0 ? check("newton") : fail(DNNMG_ERR_TIMEOUT, "a wait inside a V-cycle timed out");
   if (setup & 1) return fail(DNNMG_ERR_NUMERICAL, "singular local Vanka matrix");
   if (setup & 2) return fail(DNNMG_ERR_NUMERICAL, "singular coarse-level matrix");
   if (!std::isfinite(nrm)) return fail(DNNMG_ERR_NUMERICAL, "non-finite Newton residual");

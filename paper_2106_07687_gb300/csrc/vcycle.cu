@@ -62,6 +62,7 @@ struct WalkSmem {
   VLevel<T> lv[kMaxVLevels];
   Phase ph[kMaxPhases];
   PassRec<T> rec[kMaxPhases];
+  int polls;  // a warp's bound per phase
   alignas(16) WarpTile<T> tile[walk_threads<T>() / 32];
 };
 
@@ -83,7 +84,7 @@ __device__ __forceinline__ void for_items(int count, F f) {
 // arrays (a grid-wide barrier for the cooperative launch, the cluster barrier for
 // the single-cluster launch).  Threads of all blocks split every node-wise
 // phase; the warp tiles of a colour pass or defect go round-robin over the
-// blocks first.  state: the status word and the cycle's first number.
+// blocks first.  state: see launch_vcycle_persistent.
 template <typename T, class Sync>
 __device__ __forceinline__ void walk_phases(const VLevel<T>* glv, const OpTable<T>* gtab,
                                             const Phase* gph, int nph, int top, const T* topb,
@@ -96,6 +97,8 @@ __device__ __forceinline__ void walk_phases(const VLevel<T>* glv, const OpTable<
   copy_ints(S.ph, gph, nph);
   copy_ints(&S.tab, gtab, 1);
   const unsigned tag0 = __ldcg(reinterpret_cast<unsigned*>(state) + 1);
+  int budget = __ldcg(state + 2);
+  if (threadIdx.x == 0) S.polls = budget;
   __syncthreads();
   for (int p = threadIdx.x; p < nph; p += NT) {
     const Phase f = S.ph[p];
@@ -135,8 +138,8 @@ __device__ __forceinline__ void walk_phases(const VLevel<T>* glv, const OpTable<
   __syncthreads();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int w0 = blockIdx.x + gridDim.x * w, nw = gridDim.x * (NT / 32);
-  int budget = kTagPolls;
   for (int p = 0; p < nph; ++p) {
+    if (budget > 0) budget = S.polls;
     const PassRec<T>& R = S.rec[p];
     const int type = R.type;
     if (type == kPhasePass || type == kPhaseDefect) {

@@ -85,9 +85,10 @@ int launch_vcycle_cluster(const VLevel<T>* lv, const OpTable<T>* tab, const Phas
                           int top, const T* topb, T* topx, const double* Ainv, T omega,
                           int* state, unsigned numbers, int cluster, int coarse_nd,
                           cudaStream_t st);
-// state: two device words, a status word (8: a wait for an update hit its bound)
-// and the cycle's first number, which the launch advances by `numbers`
-// (vcycle_numbers; the word starts above 0).
+// state: three device words, a status word (8: a wait for an update hit its
+// bound), the cycle's first number, which the launch advances by `numbers`
+// (vcycle_numbers; the word starts above 0), and the bound of a warp's polls per
+// phase (kTagPolls).
 // returns 0 on success; with skip, nothing runs when *skip != 0 at the
 // launch's start
 template <typename T>

@@ -95,6 +95,7 @@ def _declare(lib):
         "dnnmg_kernel_launches": ([], ctypes.c_uint64),
         "dnnmg_vcycle_split": ([P], ctypes.c_int),
         "dnnmg_vcycle_plan": ([P, ctypes.c_int, P, P, P], ctypes.c_int),
+        "dnnmg_vcycle_polls": ([P, ctypes.c_int], ctypes.c_int),
         "dnnmg_gather_batch": ([P, P, P, P, ctypes.c_int, ctypes.c_int, ctypes.c_int64, P, P],
                                ctypes.c_int),
         "dnnmg_batch_setup": ([P, ctypes.c_int, P, P], ctypes.c_int),
@@ -111,6 +112,7 @@ def _declare(lib):
         "dnnmg_batch_set_weights": ([P, P], ctypes.c_int),
         "dnnmg_batch_set_feature_stats": ([P, P, P], ctypes.c_int),
         "dnnmg_batch_get_fine_velocity": ([P, ctypes.c_int, P], ctypes.c_int),
+        "dnnmg_batch_vcycle_polls": ([P, ctypes.c_int], ctypes.c_int),
         "dnnmg_batch_graphs": ([P, ctypes.c_int], ctypes.c_int),
         "dnnmg_batch_profile": ([P, ctypes.c_int], ctypes.c_int),
         "dnnmg_batch_profile_read": ([P, ctypes.c_int, ctypes.c_int, P, P], ctypes.c_int),

@@ -1,5 +1,5 @@
-"""V-cycles at the edges of what the calls accept: very many smoothing sweeps, and
-linearisation points that are not finite."""
+"""V-cycles at the edges of what the calls accept: very many smoothing sweeps,
+linearisation points that are not finite, and waits that hit their bound."""
 import pytest
 
 from oracle import mesh
@@ -78,3 +78,73 @@ def test_linearisation_at_a_non_finite_state_is_an_error(precision, node, bad):
         B.set_state(1, good)
         B.linearize()
         c.linearize(good)
+
+
+DEFAULT_POLLS = 1 << 21
+
+
+def _timeout(dn, call):
+    with pytest.raises(dn.DnnmgError) as e:
+        call()
+    assert e.value.code == dn.ERR_TIMEOUT
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_cycle_whose_waits_run_out_is_reported(precision, mode):
+    """With no polls allowed every wait gives up (the kernel still runs to its end):
+    the next linearisation and the step itself say so, once, and cycles with the
+    default bound give the same values as before."""
+    dn = lib()
+    L = 3
+    lev = mesh.Level(L, obstacle=(2, 1))
+    x = torch.from_numpy(seeded_state(lev, 5)).cuda()
+    c = dn.Context(level_solve=L, precision=precision, obstacle_i0=2, obstacle_j0=1, nu=0.01, dt=0.01,
+                   persistent_vcycle=L, persistent_mode=mode)
+    c.linearize(x)
+    b = torch.randn(lev.ndof, generator=torch.Generator().manual_seed(1),
+                    dtype=torch.float64).to(c.vdtype).cuda()
+    ref = c.vcycle(L, b).clone()
+    c.linearize(x)  # nothing to report
+    c._check(c.lib.dnnmg_vcycle_polls(c.h, 0))
+    c.vcycle(L, b)
+    _timeout(dn, lambda: c.linearize(x))
+    c.linearize(x)  # reported once
+    _timeout(dn, c.step)
+    c._check(c.lib.dnnmg_vcycle_polls(c.h, DEFAULT_POLLS))
+    c.linearize(x)
+    assert torch.equal(c.vcycle(L, b), ref)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("graphs", [0, 1])
+def test_batched_cycle_whose_waits_run_out_is_reported(precision, graphs):
+    dn = lib()
+    levels = (2, 3)
+    B = dn.Batch([dn.default_config(level_solve=L, precision=precision, obstacle_i0=2, obstacle_j0=1,
+                                    nu=0.01, dt=0.01) for L in levels])
+    B._check(B.lib.dnnmg_batch_graphs(B.h, graphs))
+    states = [torch.from_numpy(seeded_state(mesh.Level(L, obstacle=(2, 1)), 6 + L)).cuda()
+              for L in levels]
+    b = torch.randn(B.length, generator=torch.Generator().manual_seed(2),
+                    dtype=torch.float64).to(B.vdtype).cuda()
+
+    def start():
+        for p, x in enumerate(states):
+            B.set_state(p, x)
+        B.linearize()
+
+    start()
+    off = B.layout(1)[1]
+    b1 = b[off:off + mesh.Level(3).ndof].clone()
+    ref, ref1 = B.vcycle(b).clone(), B.vcycle_inst(1, b1).clone()
+    for _ in range(2):  # eager iterations first, then graphs
+        B.step()
+    B._check(B.lib.dnnmg_batch_vcycle_polls(B.h, 0))
+    start()
+    for call in (lambda: B.vcycle(b), lambda: B.vcycle_inst(1, b1), B.step):
+        _timeout(dn, call)
+    B._check(B.lib.dnnmg_batch_vcycle_polls(B.h, DEFAULT_POLLS))
+    start()
+    assert torch.equal(B.vcycle(b), ref) and torch.equal(B.vcycle_inst(1, b1), ref1)
+    B.step()
