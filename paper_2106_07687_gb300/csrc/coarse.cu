@@ -6,6 +6,7 @@
 
 #include "coarse_body.cuh"
 #include "kernels.h"
+#include "recip.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -65,16 +66,6 @@ enum { kBlkD, kBlkL, kBlkU, kBlkL2, kBlkU2, kBlkC1, kBlkC2, kBlkZ, kBlkP, kBlkQ,
 __host__ __device__ inline bool columns_supported(const Grid& g) { return 3 * g.nny == kCB; }
 __host__ __device__ inline size_t column_blocks_doubles(const Grid& g) {
   return (size_t)kBlkKinds * g.nnx * kCBB + 2 * (size_t)band_of(g).n;
-}
-
-// 1 / d by Newton's iteration from the hardware's approximation (about 20
-// bits): two steps reach the rounding error.
-__device__ __forceinline__ double recip64(double d) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-#pragma unroll
-  for (int k = 0; k < 2; ++k) y = fma(y, fma(-d, y, 1.0), y);
-  return y;
 }
 
 // Invert the 27 x 27 block whose entry (r, c) is load(r, c) into out (row

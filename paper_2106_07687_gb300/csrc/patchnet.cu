@@ -30,6 +30,7 @@
 #include "kernels.h"
 #include "krylov_body.cuh"
 #include "patchnet.cuh"
+#include "recip.cuh"
 #include "umma.cuh"
 
 namespace dnnmg {
@@ -48,18 +49,8 @@ __device__ __forceinline__ uint16_t f2bf(float v) {
   return __bfloat16_as_ushort(__float2bfloat16_rn(v));
 }
 
-// 1 / x for x >= 1 without the branch of the compiled division, which kept
-// the gates of a thread's units from overlapping: one Newton step on the
-// hardware approximation (P. Markstein, "Computation of elementary functions
-// on the IBM RISC System/6000 processor", 1990).  Equal to 1.0f / x for every
-// float in [1, 2^125) (all of them compared); above, where x may be infinite,
-// the approximation itself.
-__device__ __forceinline__ float recip_ge1(float x) {
-  float y;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  const float r = __fmaf_rn(y, __fmaf_rn(-x, y, 1.0f), y);
-  return x < 0x1p125f ? r : y;
-}
+// the compiled division branches, which kept the gates of a thread's units from
+// overlapping
 __device__ __forceinline__ float sigmoidf_(float x) { return recip_ge1(1.0f + __expf(-x)); }
 
 // two values as BF16, lo in the low half

@@ -15,6 +15,7 @@
 // of 8 x 4 nodes by itself: no block barrier, and a level of few nodes still
 // spreads over all SMs.
 #pragma once
+#include "recip.cuh"
 #include "vanka_body.cuh"
 
 namespace dnnmg {
@@ -145,17 +146,8 @@ __device__ __forceinline__ void assemble_node(const Grid& g, const Sten<T>& s,
 }
 
 // ---- setup of the local inverses -------------------------------------------------------
-// 1 / d; in FP64 by Newton's iteration from the hardware's approximation
-// (about 20 bits; two steps reach the rounding error), because every FP64
-// instruction takes 64 cycles of a warp's scheduler
 __device__ __forceinline__ float pivot_recip(float d) { return 1.0f / d; }
-__device__ __forceinline__ double pivot_recip(double d) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-#pragma unroll
-  for (int k = 0; k < 2; ++k) y = fma(y, fma(-d, y, 1.0), y);
-  return y;
-}
+__device__ __forceinline__ double pivot_recip(double d) { return recip64_any(d); }
 
 // Inverse of the restriction of the level's Jacobian to the 12 unknowns of
 // the fluid cell of `slot` in `colour` (its 4 nodes x u, v, p), with identity
