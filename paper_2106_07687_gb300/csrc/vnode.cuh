@@ -220,21 +220,25 @@ __device__ __forceinline__ void vanka_setup_cell(const Grid& g, const uint16_t* 
 #pragma unroll
   for (int k = 0; k < 12; ++k) {
     // the bit patterns of non-negative numbers order like the numbers: one
-    // maximum over the half-warp (FP64: of the high words), then the lowest
-    // unused lane that holds it
-    unsigned key;
+    // maximum over the half-warp (FP64: of the high words, then of the low words
+    // beside the largest), then the lowest unused lane that holds it
+    unsigned key, low = 0u, mlow = 0u;
     if constexpr (sizeof(T) == 4)
       key = __float_as_uint(A[k]) & 0x7FFFFFFFu;
     else
       key = (unsigned)__double2hiint(A[k]) & 0x7FFFFFFFu;
     if (used) key = 0u;
     const unsigned mx = __reduce_max_sync(mask, key);
-    const int p = (__ffs(__ballot_sync(mask, key == mx && !used) & mask) - 1) & 15;
+    if constexpr (sizeof(T) == 8) {
+      low = key == mx && !used ? (unsigned)__double2loint(A[k]) : 0u;
+      mlow = __reduce_max_sync(mask, low);
+    }
+    const int p = (__ffs(__ballot_sync(mask, key == mx && low == mlow && !used) & mask) - 1) & 15;
     pcol[k] = p;
     // a pivot that is neither zero nor NaN (whose bits lie above infinity's; the
     // same in every lane of the group)
     constexpr unsigned kInf = sizeof(T) == 4 ? 0x7F800000u : 0x7FF00000u;
-    ok = ok && mx != 0u && mx <= kInf;
+    ok = ok && (mx | mlow) != 0u && mx <= kInf;
     if (ok) {
       const bool piv = lane == p;
       const T ip = pivot_recip(__shfl_sync(mask, A[k], p, 16));
