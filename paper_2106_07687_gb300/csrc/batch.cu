@@ -307,6 +307,15 @@ int Batch<T>::init() {
   std::vector<Sten<T>> hsT((size_t)n_ * nL_);
   std::vector<Sten<double>> hs64((size_t)n_ * nL_), hsx((size_t)n_ * nL_);
   std::vector<BPar> hpar(n_);
+  // kinds of coefficient tables: the stabilisation form and alpha0 / nu
+  std::map<std::pair<int, double>, int> kinds;
+  std::vector<int> kind(n_), kind_of;
+  for (int p = 0; p < n_; ++p) {
+    const auto at = kinds.emplace(std::make_pair(cf[p].lps_mode, cf[p].alpha0 / cf[p].nu),
+                                  (int)kinds.size());
+    if (at.second) kind_of.push_back(p);
+    kind[p] = at.first->second;
+  }
   for (int p = 0; p < n_; ++p) {
     const dnnmg_config& c = cf[p];
     for (int k = 1; k <= L_[p] + R_; ++k) {
@@ -331,7 +340,10 @@ int Batch<T>::init() {
       l.vb = mem_.alloc<T>(n2);
       l.vb64 = mem_.alloc<double>(n2);
       l.h = (T)g.h;
-      l.hs = (T)(g.h * g.h * c.alpha0 / c.nu);
+      const double hs = g.h * g.h * c.alpha0 / c.nu;
+      l.hs = (T)hs;
+      l.hslo = (T)(hs - (double)l.hs);
+      l.kind = kind[p];
       l.mode = c.lps_mode;
       if (k >= 2) {
         l.inv = mem_.alloc<T>((size_t)4 * 144 * vanka_slots(g));
@@ -503,21 +515,22 @@ int Batch<T>::init() {
   cudaMemcpyAsync(ds64, hs64.data(), sizeof(Sten<double>) * hs64.size(), cudaMemcpyHostToDevice, st_);
   cudaMemcpyAsync(dsx, hsx.data(), sizeof(Sten<double>) * hsx.size(), cudaMemcpyHostToDevice, st_);
   cudaMemcpyAsync(dpar, hpar.data(), sizeof(BPar) * n_, cudaMemcpyHostToDevice, st_);
-  // coefficient tables of the stabilisation forms, and the cycle's items
-  OpTable<T>* dtab = mem_.alloc<OpTable<T>>(3);
+  // coefficient tables of the stabilisation forms (the cycle's, one of which lies in
+  // shared memory for all problems) and of the kinds, and the cycle's items
+  const size_t ntab = 3 + kind_of.size();
+  OpTable<T>* dtab = mem_.alloc<OpTable<T>>(ntab);
   if (!mem_.ok()) return fail(DNNMG_ERR_CUDA, "device allocation failed");
   {
-    std::vector<OpTable<T>> tab(3);
-    for (int mode = 0; mode < 3; ++mode) {
-      dnnmg_config one = c0_;
-      one.nu = one.alpha0 = 1.0;
-      one.lps_mode = mode;
-      fill_op_table<T>(make_sten<double>(1.0, one), tab[mode]);
+    std::vector<OpTable<T>> tab(ntab);
+    for (size_t t = 0; t < ntab; ++t) {
+      dnnmg_config one = t < 3 ? c0_ : cf[kind_of[t - 3]];
+      if (t < 3) one.nu = one.alpha0 = 1.0, one.lps_mode = (int)t;
+      fill_op_table<T>(make_sten<double>(1.0, one), tab[t]);
     }
-    cudaMemcpyAsync(dtab, tab.data(), sizeof(OpTable<T>) * 3, cudaMemcpyHostToDevice, st_);
+    cudaMemcpyAsync(dtab, tab.data(), sizeof(OpTable<T>) * ntab, cudaMemcpyHostToDevice, st_);
     cudaStreamSynchronize(st_);
   }
-  v_ = BView<T>{dl, dsT, ds64, dsx, dpar, dtab, nL_};
+  v_ = BView<T>{dl, dsT, ds64, dsx, dpar, dtab + 3, nL_};
   walk_.lev = dl;
   walk_.tab = dtab;
   walk_.nprob = n_;

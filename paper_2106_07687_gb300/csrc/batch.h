@@ -40,10 +40,12 @@ struct BLev {
   double* vb64;                  // FP64 linearisation point (velocity)
   T* cf;                         // assembled velocity blocks (vnode.cuh)
   const uint16_t* pat;           // node patterns
-  T h, hs;                       // mesh width; h^2 alpha0 / nu, the stabilisation's scale
+  T h, hs, hslo;                 // mesh width; h^2 alpha0 / nu, the stabilisation's scale, and
+                                 // what hs lacks of it in FP32
+  int kind;                      // table of the problem's own alpha0 / nu (the setup's)
   long long off;                 // offset of the problem in the top-level vectors
   int top;                       // 1 on the problem's finest solved level
-  int mode;                      // stabilisation form (index of the coefficient table)
+  int mode;                      // stabilisation form (table for alpha0 / nu = 1, the cycle's)
 };
 
 // Per-problem scalars read by the batched kernels.
@@ -66,7 +68,7 @@ struct BView {
   const Sten<double>* s64;   // FP64 constants (residual, coarse assembly)
   const Sten<double>* sx;    // explicit theta-scheme bracket (FP64)
   const BPar* par;           // [problem]
-  const OpTable<T>* tab;     // per stabilisation form, for h = nu = alpha0 = 1
+  const OpTable<T>* tab;     // per kind (stabilisation form and alpha0 / nu), for h = 1
   int nL;
 };
 

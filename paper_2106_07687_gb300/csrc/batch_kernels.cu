@@ -191,8 +191,8 @@ __global__ void __launch_bounds__(kSetupThreads)
   if (masked(act, wk.x)) return;
   const BLev<T> L = lev_of(v, wk.x, k);
   const int nsb = cdiv(vanka_slots(L.g), kSetupCells);
-  vanka_setup_cell<T>(L.g, L.pat, L.cf, v.tab[L.mode], L.h, L.hs, L.inv, status + wk.x, wk.y / nsb,
-                      (wk.y % nsb) * kSetupCells + threadIdx.x / 16);
+  vanka_setup_cell<T>(L.g, L.pat, L.cf, v.tab[L.kind], L.h, L.h * L.h, L.inv, status + wk.x,
+                      wk.y / nsb, (wk.y % nsb) * kSetupCells + threadIdx.x / 16);
 }
 
 template <typename T>

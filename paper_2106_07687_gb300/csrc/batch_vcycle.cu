@@ -23,7 +23,7 @@ namespace dnnmg {
 
 namespace {
 
-constexpr int kRecBytes = 96 * 1024;  // level records kept in shared memory, at most
+constexpr int kRecBytes = 104 * 1024;  // level records kept in shared memory, at most
 
 template <typename T>
 struct BWalkSmem {
@@ -70,7 +70,8 @@ __global__ void __launch_bounds__(walk_threads<T>(), 1)
       return W.mode >= 0 ? S.tab : W.tab[L.mode];
     };
     auto node_level = [&](const BLev<T>& L) {
-      return NodeLevel<T>{L.g.nx, L.g.ny, L.g.nnx, L.g.nn, L.pat, L.cf, L.h, L.hs};
+      return NodeLevel<T, sizeof(T) == 4>{L.g.nx, L.g.ny, L.g.nnx, L.g.nn,
+                                          L.pat,  L.cf,   L.h,     L.hs,   L.hslo};
     };
     auto iterate = [&](const BLev<T>& L) {
       const size_t words = (size_t)kTagWords<T> * L.g.nn;

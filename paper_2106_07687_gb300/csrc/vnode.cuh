@@ -289,13 +289,16 @@ struct WarpTile {
   T w[3][kWSY][kWPitch];
 };
 
-// Level data of the node-wise kernels.
-template <typename T>
+// Level data of the node-wise kernels.  With SPLIT the stabilisation's scale is a
+// sum of two (a batch's FP32 levels, whose table is scaled by alpha0 / nu).
+template <typename T, bool SPLIT = false>
 struct NodeLevel {
+  static constexpr bool kSplit = SPLIT;
   int nx, ny, nnx, nn;
   const uint16_t* pat;  // node patterns
   const T* cf;          // assembled velocity blocks
-  T h, h2;              // mesh width and its square
+  T h, h2;              // mesh width and the scale of the stabilisation's table
+  T h2lo = T(0);        // what h2 lacks of the exact scale
 };
 
 // ---- the iterate of a level ------------------------------------------------------------
@@ -428,8 +431,8 @@ struct TaggedX {
 
 // Stage the nodes around tile (i0, j0), three per lane, and load this lane's own
 // node `own` (its unmasked values; -1: none).
-template <typename T, bool OWN, class X, class F>
-__device__ __forceinline__ void stage_warp_tile(const NodeLevel<T>& L, const X& x, int i0, int j0,
+template <typename T, bool OWN, class NL, class X, class F>
+__device__ __forceinline__ void stage_warp_tile(const NL& L, const X& x, int i0, int j0,
                                                 int lane, int own, WarpTile<T>& S, T& xu, T& xv,
                                                 T& xp, int& budget, F other_loads) {
   static_assert(kWSX * kWSY == 96, "three nodes per lane");
@@ -462,8 +465,8 @@ __device__ __forceinline__ void stage_warp_tile(const NodeLevel<T>& L, const X& 
 
 // Rows of A'(vbar) at the staged node (li, lj) with pattern pt, coefficients c
 // and class cls = (i & 1) + 2 (j & 1); constrained rows are the caller's.
-template <typename T>
-__device__ __forceinline__ void node_rows_assembled(const NodeLevel<T>& L, const OpTable<T>& tab,
+template <typename T, class NL>
+__device__ __forceinline__ void node_rows_assembled(const NL& L, const OpTable<T>& tab,
                                                     const WarpTile<T>& S, const T c[36], int li,
                                                     int lj, int pt, int cls, T& ru, T& rv, T& rp) {
   const T(*gd)[4] = tab.gd[pt & 15];
@@ -500,13 +503,15 @@ __device__ __forceinline__ void node_rows_assembled(const NodeLevel<T>& L, const
   }
   ru = u0 + L.h * u1;
   rv = v0 + L.h * v1;
-  rp = L.h * (d0 + d1) + L.h2 * (((s[0] + s[1]) + (s[3] + s[4])) + s[2]);
+  const T sum = ((s[0] + s[1]) + (s[3] + s[4])) + s[2];
+  rp = L.h * (d0 + d1) + L.h2 * sum;
+  if constexpr (NL::kSplit) rp += L.h2lo * sum;
 }
 
 // One colour pass (see vanka_body.cuh) on the warp's 4 x 2 colour cells (bx,
 // by).  Lane 4 q + a owns node a of cell q.
-template <typename T, class X>
-__device__ __forceinline__ void warp_pass_tile(const NodeLevel<T>& L, const OpTable<T>& tab,
+template <typename T, class NL, class X>
+__device__ __forceinline__ void warp_pass_tile(const NL& L, const OpTable<T>& tab,
                                                int colour, const T* b, const X& x, const T* inv,
                                                int pitch, int nslots, T omega, int bx, int by,
                                                int lane, WarpTile<T>& S, int& budget) {
@@ -651,8 +656,8 @@ __device__ __forceinline__ T quad_sum(T v) {
 }
 
 // Stage the 8 x 6 nodes around tile (i0, j0) and load this lane's own node.
-template <typename T, bool OWN, class X, class F>
-__device__ __forceinline__ void stage_split_tile(const NodeLevel<T>& L, const X& x, int i0, int j0,
+template <typename T, bool OWN, class NL, class X, class F>
+__device__ __forceinline__ void stage_split_tile(const NL& L, const X& x, int i0, int j0,
                                                  int lane, int own, WarpTile<T>& S, T& xu, T& xv,
                                                  T& xp, int& budget, F other_loads) {
   constexpr int N = OWN ? 3 : 2;
@@ -684,8 +689,8 @@ __device__ __forceinline__ void stage_split_tile(const NodeLevel<T>& L, const X&
 }
 
 // this lane's coefficients: neighbours s, s + 4 and (s = 0) 8
-template <typename T>
-__device__ __forceinline__ void load_split_blocks(const NodeLevel<T>& L, int n, int s, T c[12]) {
+template <typename T, class NL>
+__device__ __forceinline__ void load_split_blocks(const NL& L, int n, int s, T c[12]) {
   using V = typename Vec16<T>::type;
   constexpr int NV = 4 / kVec16<T>;
   const V* p = reinterpret_cast<const V*>(L.cf);
@@ -698,8 +703,8 @@ __device__ __forceinline__ void load_split_blocks(const NodeLevel<T>& L, int n, 
   }
 }
 
-template <typename T>
-__device__ __forceinline__ void node_rows_split(const NodeLevel<T>& L, const OpTable<T>& tab,
+template <typename T, class NL>
+__device__ __forceinline__ void node_rows_split(const NL& L, const OpTable<T>& tab,
                                                 const WarpTile<T>& S, const T c[12], int li, int lj,
                                                 int pt, int cls, int s, T& ru, T& rv, T& rp) {
   T u0 = 0, v0 = 0, u1 = 0, v1 = 0, d0 = 0, ls = 0;
@@ -731,8 +736,8 @@ __device__ __forceinline__ void node_rows_split(const NodeLevel<T>& L, const OpT
 }
 
 // One colour pass on the warp's 2 x 1 colour cells (bx, by).
-template <typename T, class X>
-__device__ __forceinline__ void split_pass_tile(const NodeLevel<T>& L, const OpTable<T>& tab,
+template <typename T, class NL, class X>
+__device__ __forceinline__ void split_pass_tile(const NL& L, const OpTable<T>& tab,
                                                 int colour, const T* b, const X& x, const T* inv,
                                                 int pitch, int nslots, T omega, int bx, int by,
                                                 int lane, WarpTile<T>& S, int& budget) {
@@ -775,8 +780,8 @@ __device__ __forceinline__ void split_pass_tile(const NodeLevel<T>& L, const OpT
 }
 
 // d = b - A'(vbar) x, zero on constrained unknowns, on the warp's 4 x 2 nodes.
-template <typename T, class X>
-__device__ __forceinline__ void split_defect_tile(const NodeLevel<T>& L, const OpTable<T>& tab,
+template <typename T, class NL, class X>
+__device__ __forceinline__ void split_defect_tile(const NL& L, const OpTable<T>& tab,
                                                   const T* b, const X& x, T* d, int bx, int by,
                                                   int lane, WarpTile<T>& S, int& budget) {
   const int i0 = kSX * bx, j0 = kSY * by, m = lane >> 2, s = lane & 3;
@@ -801,8 +806,8 @@ __device__ __forceinline__ void split_defect_tile(const NodeLevel<T>& L, const O
 }
 
 // d = b - A'(vbar) x, zero on constrained unknowns, on the warp's 8 x 4 nodes.
-template <typename T, class X>
-__device__ __forceinline__ void warp_defect_tile(const NodeLevel<T>& L, const OpTable<T>& tab,
+template <typename T, class NL, class X>
+__device__ __forceinline__ void warp_defect_tile(const NL& L, const OpTable<T>& tab,
                                                  const T* b, const X& x, T* d, int bx, int by,
                                                  int lane, WarpTile<T>& S, int& budget) {
   const int i0 = kWX * bx, j0 = kWY * by, li = lane % kWX, lj = lane / kWX;

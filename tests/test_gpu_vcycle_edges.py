@@ -148,3 +148,39 @@ def test_batched_cycle_whose_waits_run_out_is_reported(precision, graphs):
     start()
     assert torch.equal(B.vcycle(b), ref) and torch.equal(B.vcycle_inst(1, b1), ref1)
     B.step()
+
+
+def test_batched_fp32_stabilisation_is_rounded_once():
+    """A batch scales one stabilisation table by every problem's alpha0 / nu.  At
+    alpha0 / nu = 1 + 3 2^-24 (times a power of two) FP32 rounds that scale up by
+    2^-24, and the table's entries (multiples of 1/6) by 2^-25: entries rounded twice
+    are 8.9e-8 too large, entries rounded once at most 2^-24 = 6.0e-8.  The error
+    of the FP32 cycle along its derivative to alpha0, for right-hand sides of rough
+    pressures, on which the stabilisation acts; the median of eight, because other
+    roundings project on it too."""
+    dn = lib()
+    L = 4
+    lev = mesh.Level(L, obstacle=(2, 1))
+    x = torch.from_numpy(seeded_state(lev, 8)).cuda()
+    cons = torch.from_numpy(lev.cons).cuda()
+    alpha0, eta = 0.125 * (1 + 3 * 2.0 ** -24), 1e-3
+    kw = dict(level_solve=L, obstacle_i0=2, obstacle_j0=1, nu=2.0 ** -7, dt=2.0 ** -7, lps_mode=1)
+    exact, moved = (dn.Context(precision=0, alpha0=a, **kw) for a in (alpha0, alpha0 * (1 + eta)))
+    for c in (exact, moved):
+        c.linearize(x)
+    B = dn.Batch([dn.default_config(precision=1, alpha0=alpha0, **kw)])
+    B.set_state(0, x)
+    B.linearize()
+    along = []
+    for seed in range(8):
+        g = torch.Generator().manual_seed(seed)
+        rough = torch.zeros(lev.ndof, dtype=torch.float64, device="cuda")
+        rough[2 * lev.nn:] = torch.randn(lev.nn, generator=g, dtype=torch.float64).cuda()
+        rough[cons] = 0
+        b = torch.zeros(B.length, device="cuda")
+        b[: lev.ndof] = exact.apply(L, rough).float()
+        ref = exact.vcycle(L, b[: lev.ndof].double())
+        deriv = (moved.vcycle(L, b[: lev.ndof].double()) - ref) / eta
+        err = B.vcycle(b)[: lev.ndof].double() - ref
+        along.append(abs(float(err @ deriv / (deriv @ deriv))))
+    assert sorted(along)[4] < 2.0 ** -24, along
