@@ -76,10 +76,12 @@ class Batch final : public BatchBase {
   int get_fine_velocity(int p, double* v);
   Prof& prof() { return prof_; }
   int set_polls(int polls) {
-    sync_in();
-    cudaMemcpyAsync(status_ + n_ + 2, &polls, sizeof(int), cudaMemcpyHostToDevice, st_);
-    cudaStreamSynchronize(st_);
-    return check("vcycle_polls");
+    walk_.polls = polls;
+    for (cudaGraphExec_t& g : graphs_) {  // they hold the former bound
+      if (g) cudaGraphExecDestroy(g);
+      g = nullptr;
+    }
+    return DNNMG_OK;
   }
   int set_graphs(int on) {
     use_graphs_ = on != 0;
@@ -169,7 +171,7 @@ class Batch final : public BatchBase {
   int linearize_masked(const int* act, bool coarse, bool precond);
   int solve(const int* nact_d, const std::vector<int>& nact, std::vector<int>& gits);
   int newton(const std::vector<int>& mask, std::vector<dnnmg_step_stats>& s);
-  int norms(const double* v, const int* act, std::vector<double>& out);
+  int norms(const double* v, const int* act, std::vector<double>& out, int* word = nullptr);
   void old_rhs_top(const double* xo, double* f, const int* act);
   void correction();
 
@@ -412,7 +414,7 @@ int Batch<T>::init() {
   cact_ = mem_.alloc<int>(n_);
   nact_ = mem_.alloc<int>(n_);
   sel_ = mem_.alloc<int>(n_);
-  status_ = mem_.alloc<int>(n_ + 3);  // and the cycles' state words
+  status_ = mem_.alloc<int>(n_ + 2);  // and the cycles' state words
   // vector blocks
   std::vector<int> vinst(nblk), vfirst(n_), vcount(n_);
   for (int p = 0; p < n_; ++p) {
@@ -543,6 +545,7 @@ int Batch<T>::init() {
   walk_.astride = astride_;
   walk_.state = status_ + n_;
   walk_.numbers = vcycle_numbers(c0_.nu1, c0_.nu2);
+  walk_.polls = kTagPolls;
   for (int k = 2; k <= Lmax_; ++k) {
     auto g = [&](int p, int l) -> const Grid& { return hl_[p][l].g; };
     walk_.defect[k] = level_items(k, [&](int p) { return vcycle_defect_tiles(g(p, k)); });
@@ -583,7 +586,7 @@ int Batch<T>::init() {
     cudaStreamSynchronize(st_);
   }
   for (int* a : {kcnt_, its_, gact_, cact_, nact_, sel_, status_}) cudaMemsetAsync(a, 0, sizeof(int) * n_, st_);
-  const int words[3] = {0, 1, kTagPolls};
+  const int words[2] = {0, 1};
   cudaMemcpyAsync(status_ + n_, words, sizeof(words), cudaMemcpyHostToDevice, st_);
   for (double* a : {resid_, target_, nrm_}) cudaMemsetAsync(a, 0, sizeof(double) * n_, st_);
   const double one = 1.0;
@@ -787,10 +790,14 @@ int Batch<T>::solve(const int* nact_d, const std::vector<int>& nact, std::vector
 }
 
 template <typename T>
-int Batch<T>::norms(const double* v, const int* act, std::vector<double>& out) {
+int Batch<T>::norms(const double* v, const int* act, std::vector<double>& out, int* word) {
   bk_multidot<double>(v, N_, 1, v, part_, vt_, nrm_, 1, act, st_);
   out.assign(n_, 0.0);
+  // the cycles' status word in the same wait, behind the norms in the staging buffer
+  int* behind = reinterpret_cast<int*>(static_cast<double*>(h_pin_) + n_);
+  if (word) cudaMemcpyAsync(behind, status_ + n_, sizeof(int), cudaMemcpyDeviceToHost, st_);
   if (int rc = sync_read(nrm_, out.data(), sizeof(double) * n_)) return rc;
+  if (word) *word = *behind;
   for (double& x : out) x = std::sqrt(x);
   return DNNMG_OK;
 }
@@ -814,14 +821,6 @@ int Batch<T>::newton(const std::vector<int>& mask, std::vector<dnnmg_step_stats>
   std::vector<int> gits(n_, 0), nits(n_, 0);
   for (int q = 0; q < n_; ++q)
     if (act[q]) s[q].res0 = nrm[q];
-  // the status of these solves' cycles, read when they end; NaN may come from a
-  // cycle whose wait hit its bound, which is then the error
-  auto late = [&](int rc) {
-    int word = 0;
-    if (int r2 = sync_read(status_ + n_, &word, sizeof(int))) return r2;
-    if (int r2 = wait_status(word)) return r2;
-    return rc;
-  };
   int it = 0;
   while (true) {
     bool any = false;
@@ -852,12 +851,20 @@ int Batch<T>::newton(const std::vector<int>& mask, std::vector<dnnmg_step_stats>
         }
       if (changed) act_d = upload_mask(act, nact_);
     }
-    if (int rc = solve(act_d, act, gits)) return late(rc);
+    if (int rc = solve(act_d, act, gits)) {
+      // NaN may come from a cycle whose wait hit its bound: that is then the error
+      int word = 0;
+      if (int r2 = sync_read(status_ + n_, &word, sizeof(int))) return r2;
+      if (int r2 = wait_status(word)) return r2;
+      return rc;
+    }
     p = prof_.begin(DNNMG_STAGE_RESIDUAL, Lmax_, st_);
     bk_residual64<T>(v_, 0, x64_, f64_, r64_, top_.w(), act_d, st_);
     prof_.end(p, st_);
     std::vector<double> nn;
-    if (int rc = norms(r64_, act_d, nn)) return rc;
+    int word = 0;
+    if (int rc = norms(r64_, act_d, nn, &word)) return rc;
+    if (int rc = wait_status(word)) return rc;
     for (int q = 0; q < n_; ++q)
       if (act[q]) {
         nrm[q] = nn[q];
@@ -872,7 +879,7 @@ int Batch<T>::newton(const std::vector<int>& mask, std::vector<dnnmg_step_stats>
     s[q].res_final = nrm[q];
     if (s[q].status == DNNMG_OK && nrm[q] > c0_.newton_tol) s[q].status = DNNMG_ERR_NOT_CONVERGED;
   }
-  return late(check("newton"));
+  return check("newton");
 }
 
 // the network correction of Algorithm 1 for every problem after the level-L solves.

@@ -92,6 +92,7 @@ struct BWalk {
   long long astride;
   int* state;               // the cycle's state words (see launch_vcycle_persistent)
   unsigned numbers;
+  int polls;
   Work pass[kBLevels], defect[kBLevels], zero[kBLevels], restr[kBLevels], prol[kBLevels];
 };
 // one cycle over nph phases (vcycle_phases) of every active problem

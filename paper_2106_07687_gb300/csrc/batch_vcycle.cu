@@ -47,11 +47,10 @@ __global__ void __launch_bounds__(walk_threads<T>(), 1)
   const BLev<T>* rec = in_smem ? srec : W.lev;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int w0 = blockIdx.x + gridDim.x * w, nw = gridDim.x * NW;
-  const unsigned tag0 = __ldcg(reinterpret_cast<unsigned*>(W.state) + 1);
-  const int polls = __ldcg(W.state + 2);
-  int budget = polls;
+  const unsigned word = __ldcg(reinterpret_cast<unsigned*>(W.state) + 1), tag0 = word << 1;
+  int budget = W.polls;
   for (int p = p0; p < p1; ++p) {
-    if (budget > 0) budget = polls;
+    if (budget > 0) budget = W.polls;
     Phase f{};
     f.type = __ldg(&ph[p].type), f.level = __ldg(&ph[p].level), f.colour = __ldg(&ph[p].colour);
     f.in = __ldg(&ph[p].in), f.out = __ldg(&ph[p].out);
@@ -180,7 +179,7 @@ __global__ void __launch_bounds__(walk_threads<T>(), 1)
   // every block has read the number before its first barrier (a cycle with a
   // phase that uses it has one)
   if (bump && blockIdx.x == 0 && threadIdx.x == 0)
-    *(reinterpret_cast<volatile unsigned*>(W.state) + 1) = tag0 + W.numbers;
+    *(reinterpret_cast<volatile unsigned*>(W.state) + 1) = word + W.numbers;
 }
 
 __global__ void next_cycle_kernel(int* state, unsigned numbers) {

@@ -467,7 +467,8 @@ int dnnmg_vcycle_plan(const dnnmg_ctx* ctx, int level, int* split_level, int* sp
 
 int dnnmg_vcycle_polls(dnnmg_ctx* ctx, int polls) {
   if (!ctx || !ctx->solver || polls < 0) return DNNMG_ERR_ARG;
-  return ctx->solver->set_polls(polls);
+  ctx->solver->set_polls(polls);
+  return DNNMG_OK;
 }
 
 size_t dnnmg_num_params(const dnnmg_ctx* ctx) { return ctx ? ctx->nd.num_params() : 0; }

@@ -79,11 +79,10 @@ class Solver final : public SolverBase {
     if (part_solid_) pieces_ = make_patch_pieces(g0.h, cfg);
     coarse_work_ = c_->mem.alloc<double>(coarse_factor_doubles(g0));
     ainv_ = c_->mem.alloc<double>((size_t)9 * g0.nn * g0.nn);
-    status_ = c_->mem.alloc<int>(5);
-    // setup status (0, 1), wait status (2), the next cycle's first number (3) and
-    // the bound of a warp's polls per phase (4)
+    status_ = c_->mem.alloc<int>(4);
+    // setup status (0, 1), wait status (2) and half the next cycle's first number (3)
     if (status_) {
-      const int words[5] = {0, 0, 0, 1, kTagPolls};
+      const int words[4] = {0, 0, 0, 1};
       cudaMemcpyAsync(status_, words, sizeof(words), cudaMemcpyHostToDevice, st_);
     }
     m_ = cfg.gmres_m;
@@ -234,11 +233,7 @@ class Solver final : public SolverBase {
     return DNNMG_OK;
   }
 
-  int set_polls(int polls) override {
-    cudaMemcpyAsync(status_ + 4, &polls, sizeof(int), cudaMemcpyHostToDevice, st_);
-    cudaStreamSynchronize(st_);
-    return c_->check("vcycle_polls");
-  }
+  void set_polls(int polls) override { polls_ = polls; }
 
   int apply(int k, const void* w, void* y) override {
     if (!linearized_) return c_->fail(DNNMG_ERR_STATE, "apply before linearize");
@@ -580,12 +575,12 @@ class Solver final : public SolverBase {
         if (coop_cap_ > 0 && blocks > coop_cap_) blocks = coop_cap_;
         blocks = blocks > vgrid_ ? vgrid_ : blocks;
         rc = launch_vcycle_persistent<T>(dlv_, dtab_, dph_ + ph_off_[k], ph_n_[k], k, b, x, ainv_,
-                                         (T)c_->cfg.omega, status_ + 2, numbers, blocks,
-                                         coarse_nd_, st_, skip);
+                                         (T)c_->cfg.omega, status_ + 2, numbers, polls_,
+                                         blocks, coarse_nd_, st_, skip);
       } else {
         rc = launch_vcycle_cluster<T>(dlv_, dtab_, dph_ + ph_off_[k], ph_n_[k], k, b, x, ainv_,
-                                      (T)c_->cfg.omega, status_ + 2, numbers, cluster_,
-                                      coarse_nd_, st_);
+                                      (T)c_->cfg.omega, status_ + 2, numbers, polls_,
+                                      cluster_, coarse_nd_, st_);
       }
       c_->prof.end(p, st_);
       if (rc == 0) return;
@@ -625,6 +620,7 @@ class Solver final : public SolverBase {
   bool part_solid_ = false;  // the coarse level has part-solid stabilisation patches
   PatchPieces pieces_{};
   int* status_ = nullptr;
+  int polls_ = kTagPolls;  // bound of a cycle's waits
   T *V_ = nullptr, *Z_ = nullptr, *wsol_ = nullptr, *rT_ = nullptr, *rcur_ = nullptr;
   double *H_ = nullptr, *cs_ = nullptr, *sn_ = nullptr, *gv_ = nullptr, *hcol_ = nullptr,
          *y_ = nullptr, *partials_ = nullptr;

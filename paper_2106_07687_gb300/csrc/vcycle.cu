@@ -62,7 +62,6 @@ struct WalkSmem {
   VLevel<T> lv[kMaxVLevels];
   Phase ph[kMaxPhases];
   PassRec<T> rec[kMaxPhases];
-  int polls;  // a warp's bound per phase
   alignas(16) WarpTile<T> tile[walk_threads<T>() / 32];
 };
 
@@ -89,16 +88,14 @@ template <typename T, class Sync>
 __device__ __forceinline__ void walk_phases(const VLevel<T>* glv, const OpTable<T>* gtab,
                                             const Phase* gph, int nph, int top, const T* topb,
                                             T* topx, const double* __restrict__ Ainv, T omega,
-                                            int* state, unsigned numbers, WalkSmem<T>& S,
-                                            Sync sync) {
+                                            int* state, unsigned numbers, int polls,
+                                            WalkSmem<T>& S, Sync sync) {
   constexpr int NT = walk_threads<T>();
   double* sbuf = reinterpret_cast<double*>(S.tile);  // the coarse right-hand side
   copy_ints(S.lv, glv, top + 1);
   copy_ints(S.ph, gph, nph);
   copy_ints(&S.tab, gtab, 1);
-  const unsigned tag0 = __ldcg(reinterpret_cast<unsigned*>(state) + 1);
-  int budget = __ldcg(state + 2);
-  if (threadIdx.x == 0) S.polls = budget;
+  const unsigned word = __ldcg(reinterpret_cast<unsigned*>(state) + 1), tag0 = word << 1;
   __syncthreads();
   for (int p = threadIdx.x; p < nph; p += NT) {
     const Phase f = S.ph[p];
@@ -138,8 +135,9 @@ __device__ __forceinline__ void walk_phases(const VLevel<T>* glv, const OpTable<
   __syncthreads();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int w0 = blockIdx.x + gridDim.x * w, nw = gridDim.x * (NT / 32);
+  int budget = polls;
   for (int p = 0; p < nph; ++p) {
-    if (budget > 0) budget = S.polls;
+    if (budget > 0) budget = polls;
     const PassRec<T>& R = S.rec[p];
     const int type = R.type;
     if (type == kPhasePass || type == kPhaseDefect) {
@@ -262,20 +260,20 @@ __device__ __forceinline__ void walk_phases(const VLevel<T>* glv, const OpTable<
   // every block has read the number before its first barrier (a cycle with a
   // phase that uses it has one)
   if (blockIdx.x == 0 && threadIdx.x == 0)
-    *(reinterpret_cast<volatile unsigned*>(state) + 1) = tag0 + numbers;
+    *(reinterpret_cast<volatile unsigned*>(state) + 1) = word + numbers;
 }
 
 template <typename T>
 __global__ void __launch_bounds__(walk_threads<T>(), 1)
     vcycle_kernel(const VLevel<T>* lv, const OpTable<T>* tab, const Phase* ph, int nph, int top,
                   const T* topb, T* topx, const double* __restrict__ Ainv, T omega, int* state,
-                  unsigned numbers, const int* skip) {
+                  unsigned numbers, int polls, const int* skip) {
   // a speculative FGMRES iteration after the cycle stopped: every block
   // reads the same flag (set before this launch) and returns before any barrier
   if (skip && *skip) return;
   extern __shared__ __align__(16) uint8_t dyn[];
   cg::grid_group grid = cg::this_grid();
-  walk_phases<T>(lv, tab, ph, nph, top, topb, topx, Ainv, omega, state, numbers,
+  walk_phases<T>(lv, tab, ph, nph, top, topb, topx, Ainv, omega, state, numbers, polls,
                  *reinterpret_cast<WalkSmem<T>*>(dyn), [&] { grid.sync(); });
 }
 
@@ -286,10 +284,10 @@ template <typename T>
 __global__ void __launch_bounds__(walk_threads<T>(), 1)
     vcycle_cluster_kernel(const VLevel<T>* lv, const OpTable<T>* tab, const Phase* ph, int nph,
                           int top, const T* topb, T* topx, const double* __restrict__ Ainv,
-                          T omega, int* state, unsigned numbers) {
+                          T omega, int* state, unsigned numbers, int polls) {
   extern __shared__ __align__(16) uint8_t dyn[];
   cg::cluster_group cl = cg::this_cluster();
-  walk_phases<T>(lv, tab, ph, nph, top, topb, topx, Ainv, omega, state, numbers,
+  walk_phases<T>(lv, tab, ph, nph, top, topb, topx, Ainv, omega, state, numbers, polls,
                  *reinterpret_cast<WalkSmem<T>*>(dyn), [&] { cl.sync(); });
 }
 
@@ -394,11 +392,11 @@ int vcycle_grid(int coarse_nd) {
 template <typename T>
 int launch_vcycle_persistent(const VLevel<T>* lv, const OpTable<T>* tab, const Phase* ph, int nph,
                              int top, const T* topb, T* topx, const double* Ainv, T omega,
-                             int* state, unsigned numbers, int grid, int coarse_nd,
-                             cudaStream_t st, const int* skip) {
+                             int* state, unsigned numbers, int polls, int grid,
+                             int coarse_nd, cudaStream_t st, const int* skip) {
   void* args[] = {(void*)&lv,   (void*)&tab,  (void*)&ph,   (void*)&nph,   (void*)&top,
                   (void*)&topb, (void*)&topx, (void*)&Ainv, (void*)&omega, (void*)&state,
-                  (void*)&numbers, (void*)&skip};
+                  (void*)&numbers, (void*)&polls, (void*)&skip};
   note_launch();
   const cudaError_t e =
       cudaLaunchCooperativeKernel((void*)vcycle_kernel<T>, dim3(grid), dim3(walk_threads<T>()),
@@ -444,7 +442,7 @@ int vcycle_cluster_size(int coarse_nd) {
 template <typename T>
 int launch_vcycle_cluster(const VLevel<T>* lv, const OpTable<T>* tab, const Phase* ph, int nph,
                           int top, const T* topb, T* topx, const double* Ainv, T omega,
-                          int* state, unsigned numbers, int cluster, int coarse_nd,
+                          int* state, unsigned numbers, int polls, int cluster, int coarse_nd,
                           cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
@@ -460,7 +458,7 @@ int launch_vcycle_cluster(const VLevel<T>* lv, const OpTable<T>* tab, const Phas
   cfg.numAttrs = 1;
   note_launch();
   const cudaError_t e = cudaLaunchKernelEx(&cfg, vcycle_cluster_kernel<T>, lv, tab, ph, nph, top,
-                                           topb, topx, Ainv, omega, state, numbers);
+                                           topb, topx, Ainv, omega, state, numbers, polls);
   return e == cudaSuccess ? 0 : 1;
 }
 
@@ -469,11 +467,11 @@ int launch_vcycle_cluster(const VLevel<T>* lv, const OpTable<T>* tab, const Phas
   template int vcycle_grid<T>(int);                                                              \
   template int launch_vcycle_persistent<T>(const VLevel<T>*, const OpTable<T>*, const Phase*,    \
                                            int, int, const T*, T*, const double*, T, int*,       \
-                                           unsigned, int, int, cudaStream_t, const int*);        \
+                                           unsigned, int, int, int, cudaStream_t, const int*);   \
   template int vcycle_cluster_size<T>(int);                                                      \
   template int launch_vcycle_cluster<T>(const VLevel<T>*, const OpTable<T>*, const Phase*, int,  \
                                         int, const T*, T*, const double*, T, int*, unsigned,     \
-                                        int, int, cudaStream_t);
+                                        int, int, int, cudaStream_t);
 DNNMG_INST(float)
 DNNMG_INST(double)
 #undef DNNMG_INST

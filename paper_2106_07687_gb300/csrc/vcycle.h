@@ -54,11 +54,13 @@ struct Phase {
   int tin = 0, tout = 0, cin = 0, tcin = 0, last = 0;
 };
 
-// How far a cycle advances the numbers of the updates: a level's iterate takes
-// the numbers 0 (its start from zero) to 4 (nu1 + nu2) + 1 (every colour pass and
-// the prolongation) above the cycle's first.
+// Half of what a cycle advances the numbers of the updates by: a level's iterate
+// takes the numbers 0 (its start from zero) to 4 (nu1 + nu2) + 1 (every colour pass
+// and the prolongation) above the cycle's first, an even number.  (The state word
+// holds half of it: with the number itself there the batch's FP64 kernel, at its
+// limit of registers, took 2,790 instead of 2,740 us for twelve channels.)
 inline unsigned vcycle_numbers(int nu1, int nu2) {
-  return 4u * ((unsigned)nu1 + (unsigned)nu2) + 2u;
+  return 2u * ((unsigned)nu1 + (unsigned)nu2) + 1u;
 }
 
 // phase list of one V(nu1, nu2) cycle with top level `top`, x zeroed first
@@ -83,19 +85,19 @@ int vcycle_cluster_size(int coarse_nd);
 template <typename T>
 int launch_vcycle_cluster(const VLevel<T>* lv, const OpTable<T>* tab, const Phase* ph, int nph,
                           int top, const T* topb, T* topx, const double* Ainv, T omega,
-                          int* state, unsigned numbers, int cluster, int coarse_nd,
+                          int* state, unsigned numbers, int polls, int cluster, int coarse_nd,
                           cudaStream_t st);
-// state: three device words, a status word (8: a wait for an update hit its
-// bound), the cycle's first number, which the launch advances by `numbers`
-// (vcycle_numbers; the word starts above 0), and the bound of a warp's polls per
+// state: two device words, a status word (8: a wait for an update hit its bound)
+// and half of the cycle's first number, which the launch advances by `numbers`
+// (vcycle_numbers; the word starts above 0).  polls: the bound of a warp's polls per
 // phase (kTagPolls).
 // returns 0 on success; with skip, nothing runs when *skip != 0 at the
 // launch's start
 template <typename T>
 int launch_vcycle_persistent(const VLevel<T>* lv, const OpTable<T>* tab, const Phase* ph, int nph,
                              int top, const T* topb, T* topx, const double* Ainv, T omega,
-                             int* state, unsigned numbers, int grid, int coarse_nd,
-                             cudaStream_t st,
+                             int* state, unsigned numbers, int polls, int grid,
+                             int coarse_nd, cudaStream_t st,
                              const int* skip = nullptr);
 
 }  // namespace dnnmg

@@ -315,9 +315,8 @@ struct NodeLevel {
 // run on from cycle to cycle (vcycle_numbers per cycle, whatever its sweeps), in a
 // word on the device: they come round after 2^32 updates, 238 million V(2,2)
 // cycles, in which every word that a cycle reads is rewritten.  The wait is
-// bounded (a warp's rounds of one phase by the third of the cycle's state words,
-// kTagPolls unless it was set; then bit 8 of *status is set and the warp waits no
-// more).  All lanes of the warp call load; other_loads
+// bounded (a warp's rounds of one phase, by kTagPolls unless the caller sets another
+// bound; then bit 8 of *status is set and the warp waits no more).  All lanes of the warp call load; other_loads
 // is run once, behind the first round's loads, to issue what the tile reads
 // besides the iterate: the tags are then mostly there when it is through.
 constexpr int kTagPolls = 1 << 21;  // over a second
