@@ -354,12 +354,10 @@ int Batch<T>::init() {
         const size_t words = 2 * (size_t)kTagWords<T> * g.nn;
         l.xt = mem_.alloc<ulonglong2>(words);
         if (l.xt) cudaMemsetAsync(l.xt, 0, words * sizeof(ulonglong2), st_);
-        const std::vector<uint16_t> pat = node_patterns(hl_[p][k]);
-        uint16_t* dp = mem_.alloc<uint16_t>(pat.size());
+        uint16_t* pat = mem_.alloc<uint16_t>(g.nn);
         if (!mem_.ok()) return fail(DNNMG_ERR_CUDA, "device allocation failed");
-        cudaMemcpyAsync(dp, pat.data(), sizeof(uint16_t) * pat.size(), cudaMemcpyHostToDevice, st_);
-        cudaStreamSynchronize(st_);
-        l.pat = dp;
+        launch_node_patterns(g, pat, st_);
+        l.pat = pat;
       }
     }
     BPar& pr = hpar[p];

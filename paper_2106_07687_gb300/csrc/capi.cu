@@ -14,7 +14,6 @@
 #include "dnnmg_step.h"
 #include "coarse_body.cuh"
 #include "runtime.h"
-#include "vnode.cuh"
 
 using namespace dnnmg;
 
@@ -71,29 +70,6 @@ HostLevel make_level(int ell, int oi0, int oj0, int olev) {
       L.flags[(size_t)j * g.nnx + i] = f;
     }
   return L;
-}
-
-std::vector<uint16_t> node_patterns(const HostLevel& L) {
-  const Grid& g = L.g;
-  std::vector<uint16_t> pat(g.nn, 0);
-  for (int j = 0; j <= g.ny; ++j)
-    for (int i = 0; i <= g.nx; ++i) {
-      unsigned p = 0;
-      for (int b = 0; b < 4; ++b) {
-        const int ci = i - 1 + (b & 1), cj = j - 1 + (b >> 1);
-        if (ci >= 0 && cj >= 0 && ci < g.nx && cj < g.ny && !L.solid[(size_t)cj * g.nx + ci])
-          p |= 1u << b;
-        const int PI = (i >> 1) - (b & 1), PJ = (j >> 1) - (b >> 1);
-        if (PI >= 0 && PJ >= 0 && PI < g.nx / 2 && PJ < g.ny / 2 && i - 2 * PI <= 2 &&
-            j - 2 * PJ <= 2 && !L.solid[(size_t)(2 * PJ) * g.nx + 2 * PI])
-          p |= 1u << (kPatPatch + b);
-      }
-      const uint8_t f = L.flags[(size_t)j * g.nnx + i];
-      if (f & kVDir) p |= kPatVDir;
-      if (f & kPFix) p |= kPatPFix;
-      pat[(size_t)j * g.nnx + i] = (uint16_t)p;
-    }
-  return pat;
 }
 
 // Q1 element constants from 1D tensor products on a cell of width h:

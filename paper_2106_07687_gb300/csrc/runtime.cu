@@ -46,13 +46,10 @@ class Solver final : public SolverBase {
       l.vb64 = c_->mem.alloc<double>(n2);
       if (k > 0) {
         l.inv = c_->mem.alloc<T>((size_t)4 * 144 * vanka_slots(l.g));
-        const std::vector<uint16_t> pat = node_patterns(c_->lv[l.level]);
         l.cf = c_->mem.alloc<T>(kCoefs<T> * (size_t)l.g.nn);
-        l.pat = c_->mem.alloc<uint16_t>(pat.size());
+        l.pat = c_->mem.alloc<uint16_t>(l.g.nn);
         if (!c_->mem.ok()) return c_->fail(DNNMG_ERR_CUDA, "device allocation failed");
-        cudaMemcpyAsync(l.pat, pat.data(), sizeof(uint16_t) * pat.size(), cudaMemcpyHostToDevice,
-                        st_);
-        cudaStreamSynchronize(st_);
+        launch_node_patterns(l.g, l.pat, st_);
       }
     }
     dasm_ = c_->mem.alloc<AsmLevel<T>>(K_ + 1);

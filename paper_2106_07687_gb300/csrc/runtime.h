@@ -19,8 +19,6 @@ struct HostLevel {
 };
 
 HostLevel make_level(int ell, int oi0, int oj0, int olev);
-// patterns of the level's nodes (vnode.cuh)
-std::vector<uint16_t> node_patterns(const HostLevel& L);
 // whether some 2h stabilisation patch of the level is part solid
 bool part_solid_patches(const HostLevel& L);
 struct PatchPieces;
@@ -39,20 +37,38 @@ class DevMem {
   ~DevMem() {
     for (void* p : ptrs_) cudaFree(p);
   }
+  // 256-byte aligned; the small buffers of a hierarchy share blocks (a batch of
+  // twelve channels makes 800 of them)
   template <typename T>
   T* alloc(size_t n) {
-    void* p = nullptr;
-    if (cudaMalloc(&p, n * sizeof(T) + 16) != cudaSuccess) {
-      ok_ = false;
-      return nullptr;
+    const size_t bytes = (n * sizeof(T) + 16 + 255) / 256 * 256;
+    if (bytes > kBlock / 4) return static_cast<T*>(take(bytes));
+    if (bytes > left_) {
+      next_ = static_cast<uint8_t*>(take(kBlock));
+      left_ = next_ ? kBlock : 0;
+      if (!next_) return nullptr;
     }
-    ptrs_.push_back(p);
+    void* p = next_;
+    next_ += bytes;
+    left_ -= bytes;
     return static_cast<T*>(p);
   }
   bool ok() const { return ok_; }
 
  private:
+  static constexpr size_t kBlock = 1 << 20;
+  void* take(size_t bytes) {
+    void* p = nullptr;
+    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+      ok_ = false;
+      return nullptr;
+    }
+    ptrs_.push_back(p);
+    return p;
+  }
   std::vector<void*> ptrs_;
+  uint8_t* next_ = nullptr;  // the current block's free part
+  size_t left_ = 0;
   bool ok_ = true;
 };
 

@@ -301,6 +301,26 @@ __global__ void __launch_bounds__(128)
   assemble_node<T>(lv[k].g, lv[k].s, lv[k].vb, lv[k].cf, t - lv[k].first);
 }
 
+__global__ void __launch_bounds__(256) node_patterns_kernel(Grid g, uint16_t* __restrict__ pat) {
+  const int n = blockIdx.x * blockDim.x + threadIdx.x;
+  if (n >= g.nn) return;
+  const int i = n % g.nnx, j = n / g.nnx;
+  unsigned p = 0;
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    const int ci = i - 1 + (b & 1), cj = j - 1 + (b >> 1);
+    if (ci >= 0 && cj >= 0 && ci < g.nx && cj < g.ny && !g.solid[cj * g.nx + ci]) p |= 1u << b;
+    const int PI = (i >> 1) - (b & 1), PJ = (j >> 1) - (b >> 1);
+    if (PI >= 0 && PJ >= 0 && PI < g.nx / 2 && PJ < g.ny / 2 && i - 2 * PI <= 2 &&
+        j - 2 * PJ <= 2 && !g.solid[(2 * PJ) * g.nx + 2 * PI])
+      p |= 1u << (kPatPatch + b);
+  }
+  const uint8_t f = g.flags[n];
+  if (f & kVDir) p |= kPatVDir;
+  if (f & kPFix) p |= kPatPFix;
+  pat[n] = (uint16_t)p;
+}
+
 // phases of the cycle of level k; returns the buffer and number of its final
 // iterate (0: the coarsest level's solution)
 std::pair<int, int> build_phases(int k, int nu1, int nu2, std::vector<Phase>& out) {
@@ -344,6 +364,11 @@ size_t walk_smem(int coarse_nd) {
   return head + std::max(tiles, sizeof(double) * coarse_nd);
 }
 }  // namespace
+
+void launch_node_patterns(const Grid& g, uint16_t* pat, cudaStream_t st) {
+  note_launch();
+  node_patterns_kernel<<<cdiv(g.nn, 256), 256, 0, st>>>(g, pat);
+}
 
 template <typename T>
 void launch_assemble_blocks(const AsmLevel<T>* lv, int nlev, int nodes, cudaStream_t st) {

@@ -28,6 +28,8 @@ struct AsmLevel {
   T* cf;
   int first;
 };
+// patterns of a level's nodes (vnode.cuh)
+void launch_node_patterns(const Grid& g, uint16_t* pat, cudaStream_t st);
 // velocity blocks of the first nlev levels of `lv` (device array), `nodes`
 // nodes in all, in one launch
 template <typename T>
