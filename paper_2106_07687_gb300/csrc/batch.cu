@@ -50,7 +50,11 @@ class Batch final : public BatchBase {
     if (st_) cudaStreamSynchronize(st_);
     for (auto& g : graphs_)
       if (g) cudaGraphExecDestroy(g);
+    if (side_) cudaStreamSynchronize(side_);
     if (st_) cudaStreamDestroy(st_);
+    if (side_) cudaStreamDestroy(side_);
+    if (fork_ev_) cudaEventDestroy(fork_ev_);
+    if (join_ev_) cudaEventDestroy(join_ev_);
     if (h_pin_) cudaFreeHost(h_pin_);
     if (h_mask_) cudaFreeHost(h_mask_);
     if (ev0_) cudaEventDestroy(ev0_);
@@ -177,6 +181,8 @@ class Batch final : public BatchBase {
 
   dnnmg_batch* B_;
   cudaStream_t ust_ = nullptr, st_ = nullptr;
+  cudaStream_t side_ = nullptr;  // setups beside the coarse factorisation
+  cudaEvent_t fork_ev_ = nullptr, join_ev_ = nullptr;
   int n_ = 0, Lmax_ = 0, nL_ = 0, R_ = 0, m_ = 0, n1_ = 0;
   dnnmg_config c0_{};
   std::vector<int> L_;
@@ -265,7 +271,10 @@ int Batch<T>::init() {
     Lmax_ = std::max(Lmax_, L_[p]);
   }
   nL_ = Lmax_ + std::max(2, R_ + 1);
-  if (cudaStreamCreateWithFlags(&st_, cudaStreamNonBlocking) != cudaSuccess)
+  if (cudaStreamCreateWithFlags(&st_, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaStreamCreateWithFlags(&side_, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaEventCreateWithFlags(&fork_ev_, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&join_ev_, cudaEventDisableTiming) != cudaSuccess)
     return fail(DNNMG_ERR_CUDA, "stream creation failed");
   if (cudaMallocHost(&h_pin_, (size_t)n_ * (2 * m_ + 4) * sizeof(double) + 4096) != cudaSuccess ||
       cudaMallocHost(reinterpret_cast<void**>(&h_mask_), sizeof(int) * n_) != cudaSuccess)
@@ -632,21 +641,29 @@ int Batch<T>::linearize_masked(const int* act, bool coarse, bool precond) {
   bk_top_vb<T>(v_, x64_, top_.w(), act, st_);
   for (int k = Lmax_; k >= 2; --k) bk_inject_vb<T>(v_, k, node1_[k - 1].w(), act, st_);
   cudaMemsetAsync(status_, 0, sizeof(int) * n_, st_);
-  for (int k = 1; k <= Lmax_; ++k) {
-    bk_cast_vb<T>(v_, k, node0_[k].w(), act, st_);
-    if (k >= 2) {
-      const int p = prof_.begin(DNNMG_STAGE_VANKA_SETUP, k, st_);
-      bk_assemble<T>(v_, k, node0_[k].w(), act, st_);
-      bk_setup<T>(v_, k, status_, setup_[k].w(), act, st_);
-      prof_.end(p, st_);
-    }
+  for (int k = 1; k <= Lmax_; ++k) bk_cast_vb<T>(v_, k, node0_[k].w(), act, st_);
+  // the blocks and setups beside the coarse factorisation (one block per problem for
+  // 4 ms), unless the stages are being timed
+  const bool factor = coarse || !coarse_done_, beside = factor && !prof_.on();
+  const cudaStream_t ss = beside ? side_ : st_;
+  if (beside) {
+    cudaEventRecord(fork_ev_, st_);
+    cudaStreamWaitEvent(side_, fork_ev_, 0);
   }
-  if (coarse || !coarse_done_) {
+  for (int k = 2; k <= Lmax_; ++k) {
+    const int p = prof_.begin(DNNMG_STAGE_VANKA_SETUP, k, ss);
+    bk_assemble<T>(v_, k, node0_[k].w(), act, ss);
+    bk_setup<T>(v_, k, status_, setup_[k].w(), act, ss);
+    prof_.end(p, ss);
+  }
+  if (beside) cudaEventRecord(join_ev_, side_);
+  if (factor) {
     const int p = prof_.begin(DNNMG_STAGE_COARSE_FACTOR, 1, st_);
     bk_coarse_factor<T>(v_, n_, n1_, cwork_, cstride_, bandsz_, Ainv_, astride_, status_, act, st_);
     prof_.end(p, st_);
     coarse_done_ = true;
   }
+  if (beside) cudaStreamWaitEvent(st_, join_ev_, 0);
   linearized_ = true;
   return check("linearize");
 }
