@@ -811,7 +811,7 @@ int dnnmg_ctx::init_train() {
     ghT[l] = mem.alloc<uint16_t>((size_t)MG * K);
   }
   tb.loss_partial = mem.alloc<double>(tr_blocks_max);
-  loss_dev = mem.alloc<float>(4);
+  loss_dev = mem.alloc<double>(1);
   grad = mem.alloc<float>(nd.num_params());
   adam_m = mem.alloc<float>(nd.num_params());
   adam_v = mem.alloc<float>(nd.num_params());
@@ -914,11 +914,15 @@ int dnnmg_ctx::train_grad_impl(const uint16_t* Xd, const float* Yd, int B, int T
   return check("train");
 }
 
-// The loss and the status with one wait, behind everything the call launched.
+// The loss and the status in one post, behind everything the call launched.  (A copy
+// to pinned memory ahead of the post is complete for the device when the post runs,
+// but the host may see the post first.)
 int dnnmg_ctx::train_finish(const char* what, float* loss) {
-  cudaMemcpyAsync(h_scalars, loss_dev, sizeof(float), cudaMemcpyDeviceToHost, st);
-  if (int rc = net_check(what)) return rc;
-  if (loss) std::memcpy(loss, h_scalars, sizeof(float));
+  if (int rc = check(what)) return rc;
+  const unsigned long long t = mail_ticket();
+  launch_post(mail_d, t, loss_dev, 1, 1, net_status, 0, 1, st);
+  if (int rc = net_wait(t, what)) return rc;
+  if (loss) *loss = (float)mail_h->v[1];
   return check(what);
 }
 

@@ -228,7 +228,8 @@ struct dnnmg_ctx {
   double* stat_partial = nullptr;  // [128][C_in][2] feature-statistics partials
   // training workspace (capacity cfg.train_batch x cfg.train_seq)
   dnnmg::TrainBufs tb{};
-  float *loss_dev = nullptr, *grad = nullptr, *adam_m = nullptr,
+  double* loss_dev = nullptr;
+  float *grad = nullptr, *adam_m = nullptr,
         *adam_v = nullptr, *cpart = nullptr;
   uint16_t *da1T = nullptr, *wT = nullptr;
   uint16_t* giT[dnnmg::kMaxLayers] = {};  // gate gradients of each layer (input side)

@@ -608,7 +608,7 @@ __global__ void wgrad_reduce_kernel(WGradArgs a, const float* __restrict__ Cpart
   }
 }
 
-__global__ void loss_kernel(const double* __restrict__ part, int n, double inv, float* out) {
+__global__ void loss_kernel(const double* __restrict__ part, int n, double inv, double* out) {
   __shared__ double sh[32];
   double acc = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) acc += part[i];
@@ -618,7 +618,7 @@ __global__ void loss_kernel(const double* __restrict__ part, int n, double inv, 
   if (threadIdx.x == 0) {
     double s = 0.0;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += sh[w];
-    *out = (float)(s * inv);
+    *out = s * inv;
   }
 }
 
@@ -759,7 +759,7 @@ size_t wgrad_partials(const WGradJob* jobs, int njobs, int K, int splits) {
   return n;
 }
 
-void launch_loss(const double* part, int n, double inv, float* out, cudaStream_t st) {
+void launch_loss(const double* part, int n, double inv, double* out, cudaStream_t st) {
   note_launch();
   loss_kernel<<<1, 256, 0, st>>>(part, n, inv, out);
 }

@@ -76,7 +76,7 @@ struct WGradArgs {
 int launch_wgrad(const WGradJob* jobs, int njobs, int K, int splits, float* Cpart, int* status,
                  cudaStream_t st);
 size_t wgrad_partials(const WGradJob* jobs, int njobs, int K, int splits);
-void launch_loss(const double* part, int n, double inv, float* out, cudaStream_t st);
+void launch_loss(const double* part, int n, double inv, double* out, cudaStream_t st);
 // nothing happens when *skip != 0
 void launch_adam(float* w, const float* g, float* m, float* v, size_t n, float lr, int step,
                  const int* skip, cudaStream_t st);

@@ -53,3 +53,21 @@ def test_loss_of_targets_that_are_not_finite(bad):
     ctx._check(ctx.lib.dnnmg_train_grad(ctx.h, X.data_ptr(), Y.data_ptr(), B, T, None,
                                         ctypes.byref(loss)))
     assert np.isnan(loss.value) if np.isnan(bad) else loss.value == float("inf")
+
+
+@pytest.mark.parametrize("B,T", [(16, 1), (16, 4)])
+def test_loss_is_that_of_the_call(B, T):
+    """The host reads the loss of the call it waits for, in short calls whose
+    targets change from one to the next (zero weights: the mean of their squares)."""
+    dn = lib()
+    for _ in range(20):  # first calls of new contexts too
+        ctx = dn.Context(level_solve=2, train_batch=B, train_seq=T)
+        ctx.set_weights(torch.zeros(ctx.num_params()))
+        X = torch.zeros(B, T, 40, dtype=torch.bfloat16, device="cuda")
+        Y = [torch.full((B, T, 18), float(k), device="cuda") for k in range(1, 6)]
+        torch.cuda.synchronize()
+        loss = ctypes.c_float()
+        for k in range(200):
+            ctx._check(ctx.lib.dnnmg_train_grad(ctx.h, X.data_ptr(), Y[k % 5].data_ptr(), B, T, None,
+                                                ctypes.byref(loss)))
+            assert loss.value == (k % 5 + 1) ** 2, (k, loss.value)
