@@ -203,7 +203,7 @@ void bk_vcycle(const BWalk<T>& W, const Phase* ph, int nph, const T* topb, T* to
   int dev = 0, sms = 0, per = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaFuncSetAttribute(bvcycle_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaFuncSetAttribute(bvcycle_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, bvcycle_kernel<T>, walk_threads<T>(),
                                                     smem) != cudaSuccess)
     per = 0;

@@ -142,6 +142,11 @@ void launch_vanka_pass_stream(const void* map, const Grid& g, const Sten<float>&
 constexpr int kSetupThreads = 128;
 constexpr int kSetupCells = kSetupThreads / 16;
 
+// Limit to set as a kernel's dynamic shared memory when its launches differ in size:
+// the most that a block can have.  Another thread may set the same kernel's limit
+// between this one's call and its launch, so the value must not depend on the launch.
+constexpr int kSmemLimit = 227 * 1024;
+
 // Coarse direct solve (coarse.cu) -------------------------------------------
 // Assemble the banded Jacobian of the coarsest level (FP64), factor it with
 // partial pivoting and form the explicit inverse Ainv (ndof x ndof, FP64,

@@ -43,7 +43,7 @@ constexpr uint32_t kWaitPolls = 1u << 22;  // bound of every mbarrier wait
 constexpr int kTile = 128;
 constexpr int kFwdWG = 4;                      // warpgroups of the forward kernel
 constexpr int kFwdThreads = kTile * kFwdWG;
-constexpr size_t kSmemMax = 227 * 1024;
+constexpr size_t kSmemMax = kSmemLimit;
 
 __device__ __forceinline__ uint16_t f2bf(float v) {
   return __bfloat16_as_ushort(__float2bfloat16_rn(v));
@@ -718,7 +718,8 @@ int launch_forward_groups(const NetDims& d, const PackedNet& pk, const FwdArgs& 
   const PackLayout L = PackLayout::of(d);
   const FwdSmem S = FwdSmem::of(d, L.total, G);
   cudaFuncSetAttribute(patchnet_forward_kernel<TRAIN, H, NL, G>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S.total);
+                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       TRAIN ? kSmemLimit - 1024 : kSmemLimit);  // beside its static part
   note_launch();
   patchnet_forward_kernel<TRAIN, H, NL, G>
       <<<blocks, kFwdThreads, S.total, st>>>(d, L, pk.w, pk.bias, a);

@@ -674,7 +674,7 @@ void launch_backward_shape(const NetDims& d, const uint16_t* wT, const BwdArgs& 
   const BwdPack W = BwdPack::of(d);
   const BwdSmem S = BwdSmem::of(d, W.total);
   cudaFuncSetAttribute(patchnet_backward_kernel<H, NL>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S.total);
+                       cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
   note_launch();
   patchnet_backward_kernel<H, NL><<<nblocks, kBwdThreads, S.total, st>>>(d, W, wT, a);
 }
