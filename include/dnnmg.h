@@ -468,6 +468,11 @@ int dnnmg_vcycle_split(const dnnmg_ctx* ctx);
 int dnnmg_vcycle_plan(const dnnmg_ctx* ctx, int level, int* split_level, int* split_mode,
                       int* pass_shape);
 
+/* How the coarse inverse in use was formed: 0 by elimination of node columns, 1 by
+ * the banded LU (where the elimination's check asked for it, and from the start with
+ * part-solid patches), -1 before the first linearisation.  Synchronous. */
+int dnnmg_coarse_lu(dnnmg_ctx* ctx);
+
 /* Bound of the waits inside the context's V-cycles: a warp polls at most `polls`
  * times per phase for the values it needs, then goes on without them and the
  * cycle is reported (see dnnmg_vcycle).  The default, 2^21, is over a second;

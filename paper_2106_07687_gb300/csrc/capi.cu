@@ -441,6 +441,10 @@ int dnnmg_vcycle_plan(const dnnmg_ctx* ctx, int level, int* split_level, int* sp
   return DNNMG_OK;
 }
 
+int dnnmg_coarse_lu(dnnmg_ctx* ctx) {
+  return ctx && ctx->solver ? ctx->solver->coarse_lu() : -1;
+}
+
 int dnnmg_vcycle_polls(dnnmg_ctx* ctx, int polls) {
   if (!ctx || !ctx->solver || polls < 0) return DNNMG_ERR_ARG;
   ctx->solver->set_polls(polls);

@@ -651,8 +651,9 @@ size_t coarse_factor_doubles(const Grid& g) {
   return coarse_work_doubles(g) + (columns_supported(g) ? column_blocks_doubles(g) + 1 : 0);
 }
 
-void launch_coarse_factor(const Grid& g, const Sten<double>& s, const double* vb, double* work,
-                          double* Ainv, int* status, cudaStream_t st, const PatchPieces* pp) {
+const int* launch_coarse_factor(const Grid& g, const Sten<double>& s, const double* vb,
+                                double* work, double* Ainv, int* status, cudaStream_t st,
+                                const PatchPieces* pp) {
   const Band bd = band_of(g);
   double* ab = work;
   int* piv = reinterpret_cast<int*>(work + (size_t)bd.n * bd.W);
@@ -695,6 +696,7 @@ void launch_coarse_factor(const Grid& g, const Sten<double>& s, const double* vb
   note_launch();
   band_inverse_kernel<<<cdiv(bd.n, kInvWarps), 32 * kInvWarps, smem, st>>>(g, ab, piv, rd, Ainv,
                                                                            need);
+  return need;
 }
 
 template <typename T>

@@ -231,6 +231,14 @@ class Solver final : public SolverBase {
   }
 
   void set_polls(int polls) override { polls_ = polls; }
+  int coarse_lu() override {
+    if (!coarse_done_ || !coarse_lu_) return coarse_done_ ? 1 : -1;
+    cudaMemcpyAsync(c_->h_scalars, coarse_lu_, sizeof(int), cudaMemcpyDeviceToHost, st_);
+    if (cudaStreamSynchronize(st_) != cudaSuccess) return -1;
+    int lu = 0;
+    std::memcpy(&lu, c_->h_scalars, sizeof(int));
+    return lu != 0;
+  }
 
   int apply(int k, const void* w, void* y) override {
     if (!linearized_) return c_->fail(DNNMG_ERR_STATE, "apply before linearize");
@@ -420,8 +428,8 @@ class Solver final : public SolverBase {
   }
 
   void factor_coarse() {
-    launch_coarse_factor(lv_[0].g, lv_[0].s64, lv_[0].vb64, coarse_work_, ainv_, status_, st_,
-                         part_solid_ ? &pieces_ : nullptr);
+    coarse_lu_ = launch_coarse_factor(lv_[0].g, lv_[0].s64, lv_[0].vb64, coarse_work_, ainv_,
+                                      status_, st_, part_solid_ ? &pieces_ : nullptr);
   }
 
   // The constants of the assembled operator: every level's assembly record and
@@ -618,6 +626,7 @@ class Solver final : public SolverBase {
   PatchPieces pieces_{};
   int* status_ = nullptr;
   int polls_ = kTagPolls;  // bound of a cycle's waits
+  const int* coarse_lu_ = nullptr;  // see launch_coarse_factor
   T *V_ = nullptr, *Z_ = nullptr, *wsol_ = nullptr, *rT_ = nullptr, *rcur_ = nullptr;
   double *H_ = nullptr, *cs_ = nullptr, *sn_ = nullptr, *gv_ = nullptr, *hcol_ = nullptr,
          *y_ = nullptr, *partials_ = nullptr;

@@ -153,6 +153,7 @@ class SolverBase {
   virtual int apply(int k, const void* w, void* y) = 0;
   virtual int vcycle(int k, const void* b, void* x) = 0;
   virtual void set_polls(int polls) = 0;
+  virtual int coarse_lu() = 0;
   // FGMRES on the finest level: w64 += eps * A'^{-1} r64 (approximately)
   virtual int solve(const double* r64, double* x64, double eps, int* its) = 0;
   virtual int precision() const = 0;

@@ -95,6 +95,7 @@ def _declare(lib):
         "dnnmg_kernel_launches": ([], ctypes.c_uint64),
         "dnnmg_vcycle_split": ([P], ctypes.c_int),
         "dnnmg_vcycle_plan": ([P, ctypes.c_int, P, P, P], ctypes.c_int),
+        "dnnmg_coarse_lu": ([P], ctypes.c_int),
         "dnnmg_vcycle_polls": ([P, ctypes.c_int], ctypes.c_int),
         "dnnmg_gather_batch": ([P, P, P, P, ctypes.c_int, ctypes.c_int, ctypes.c_int64, P, P],
                                ctypes.c_int),
