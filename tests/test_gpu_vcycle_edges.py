@@ -184,3 +184,31 @@ def test_batched_fp32_stabilisation_is_rounded_once():
         err = B.vcycle(b)[: lev.ndof].double() - ref
         along.append(abs(float(err @ deriv / (deriv @ deriv))))
     assert sorted(along)[4] < 2.0 ** -24, along
+
+
+@pytest.mark.parametrize("L,precision,tol", [(6, 0, 1e-10), (6, 1, 2e-5), (7, 1, 2e-5), (8, 1, 2e-5)])
+def test_persistent_cycle_of_large_levels(L, precision, tol):
+    """Where a level's tiles outnumber the warps and its index arithmetic grows (4.2 M
+    nodes on level 8): the persistent cycle against that of one launch per stage, with
+    the bars they have on the smaller levels."""
+    dn = lib()
+    nnx, nny = (16 << L) + 1, (4 << L) + 1
+    y = torch.linspace(0, 1, nny, dtype=torch.float64, device="cuda")[:, None]
+    x = torch.linspace(0, 4, nnx, dtype=torch.float64, device="cuda")[None, :]
+    s = torch.zeros(3, nny, nnx, dtype=torch.float64, device="cuda")
+    s[0] = 6 * y * (1 - y) * (1 + 0.2 * torch.sin(2 * x))
+    s[1] = 0.2 * torch.sin(3 * x) * torch.sin(3.14159265358979 * y)
+    g = torch.Generator(device="cuda").manual_seed(L)
+    b = torch.randn(s.numel(), generator=g, dtype=torch.float64, device="cuda")
+    common = dict(level_solve=L, precision=precision, obstacle_i0=3, obstacle_j0=1, nu=0.0065,
+                  dt=0.005, gmres_m=2)
+    out = []
+    for kw in (dict(persistent_vcycle=0), dict(persistent_vcycle=L, persistent_mode=0)):
+        c = dn.Context(**common, **kw)
+        c.linearize(s.reshape(-1))
+        assert c.lib.dnnmg_vcycle_split(c.h) == kw["persistent_vcycle"]
+        out.append(c.vcycle(L, b.to(c.vdtype)).double())
+        again = c.vcycle(L, b.to(c.vdtype)).double()
+        assert torch.equal(again, out[-1])
+        c.close()
+    assert 0 < float((out[1] - out[0]).norm() / out[0].norm()) < tol
