@@ -606,8 +606,7 @@ int Batch<T>::init() {
 }
 
 // One V(nu1, nu2) cycle of every active problem on its own finest level (b, x
-// in the top-level layout); x is read only without pre-smoothing, and is then
-// zero on entry.
+// in the top-level layout); x is only written, all of it but the padding.
 template <typename T>
 void Batch<T>::vcycle_all(const T* b, T* x, const int* act) {
   const int p = prof_.begin(DNNMG_STAGE_VCYCLE, Lmax_, st_);
@@ -702,7 +701,6 @@ void Batch<T>::fgmres_iteration(int j) {
   T* zj = Z_ + (size_t)j * N_;
   T* w = V_ + (size_t)(j + 1) * N_;
   const int hs = 2 * m_ + 4;
-  if (c0_.nu1 == 0) launch_fill<T>(zj, T(0), N_, st_);
   vcycle_all(vj, zj, gact_);
   int p = prof_.begin(DNNMG_STAGE_APPLY, Lmax_, st_);
   bk_apply<T>(v_, zj, vbJ_, w, top_.w(), gact_, st_);
