@@ -474,9 +474,10 @@ int dnnmg_vcycle_plan(const dnnmg_ctx* ctx, int level, int* split_level, int* sp
 int dnnmg_coarse_lu(dnnmg_ctx* ctx);
 
 /* Bound of the waits inside the context's V-cycles: a warp polls at most `polls`
- * times per phase for the values it needs, then goes on without them and the
- * cycle is reported (see dnnmg_vcycle).  The default, 2^21, is over a second;
- * with 0 every cycle launched from then on gives up at once and is reported. */
+ * times for the values it needs (in a batch, between two of the cycle's grid
+ * barriers), then goes on without them and the cycle is reported (see
+ * dnnmg_vcycle).  The default, 2^21, is over a second; with 0 every cycle
+ * launched from then on gives up at once and is reported. */
 int dnnmg_vcycle_polls(dnnmg_ctx* ctx, int polls);
 
 /* ------------------------------------------------------------------------

@@ -189,7 +189,7 @@ class Batch final : public BatchBase {
   std::vector<std::vector<HostLevel>> hl_;
   std::vector<long long> off_, offF_, offM_;  // top, fine (L + R) and, for R = 2, L + 1
   long long N_ = 0, NF_ = 0, NM_ = 0;
-  DevMem mem_;
+  DevMem mem_{true};
   std::vector<BLev<T>> hlev_;
   BView<T> v_{};
   // work lists
@@ -208,7 +208,7 @@ class Batch final : public BatchBase {
   double *H_ = nullptr, *cs_ = nullptr, *sn_ = nullptr, *gv_ = nullptr, *hcol_ = nullptr,
          *y_ = nullptr, *resid_ = nullptr, *target_ = nullptr, *one_ = nullptr, *nrm_ = nullptr;
   int *kcnt_ = nullptr, *its_ = nullptr, *gact_ = nullptr, *cact_ = nullptr, *nact_ = nullptr,
-      *sel_ = nullptr, *status_ = nullptr;
+      *sel_ = nullptr, *status_ = nullptr;  // status_: setups' words, then the cycles' state
   // coarse level
   double *cwork_ = nullptr, *Ainv_ = nullptr;
   long long cstride_ = 0, bandsz_ = 0, astride_ = 0;
@@ -413,7 +413,9 @@ int Batch<T>::init() {
   y_ = mem_.alloc<double>((size_t)n_ * (m_ + 1));
   resid_ = mem_.alloc<double>(n_);
   target_ = mem_.alloc<double>(n_);
-  nrm_ = mem_.alloc<double>(n_);
+  // the norms, and behind them the status words, which the host reads with them
+  nrm_ = mem_.alloc<double>(n_ + (n_ + 3) / 2);
+  status_ = nrm_ ? reinterpret_cast<int*>(nrm_ + n_) : nullptr;
   one_ = mem_.alloc<double>(1);
   kcnt_ = mem_.alloc<int>(n_);
   its_ = mem_.alloc<int>(n_);
@@ -421,7 +423,6 @@ int Batch<T>::init() {
   cact_ = mem_.alloc<int>(n_);
   nact_ = mem_.alloc<int>(n_);
   sel_ = mem_.alloc<int>(n_);
-  status_ = mem_.alloc<int>(n_ + 2);  // and the cycles' state words
   // vector blocks
   std::vector<int> vinst(nblk), vfirst(n_), vcount(n_);
   for (int p = 0; p < n_; ++p) {
@@ -806,11 +807,15 @@ template <typename T>
 int Batch<T>::norms(const double* v, const int* act, std::vector<double>& out, int* word) {
   bk_multidot<double>(v, N_, 1, v, part_, vt_, nrm_, 1, act, st_);
   out.assign(n_, 0.0);
-  // the cycles' status word in the same wait, behind the norms in the staging buffer
-  int* behind = reinterpret_cast<int*>(static_cast<double*>(h_pin_) + n_);
-  if (word) cudaMemcpyAsync(behind, status_ + n_, sizeof(int), cudaMemcpyDeviceToHost, st_);
-  if (int rc = sync_read(nrm_, out.data(), sizeof(double) * n_)) return rc;
-  if (word) *word = *behind;
+  if (!word) {
+    if (int rc = sync_read(nrm_, out.data(), sizeof(double) * n_)) return rc;
+  } else {  // and the status words behind them
+    std::vector<double> both(n_ + (n_ + 2) / 2);
+    if (int rc = sync_read(nrm_, both.data(), sizeof(double) * n_ + sizeof(int) * (n_ + 1)))
+      return rc;
+    std::copy(both.begin(), both.begin() + n_, out.begin());
+    std::memcpy(word, reinterpret_cast<const int*>(both.data() + n_) + n_, sizeof(int));
+  }
   for (double& x : out) x = std::sqrt(x);
   return DNNMG_OK;
 }

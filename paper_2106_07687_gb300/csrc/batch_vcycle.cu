@@ -50,7 +50,6 @@ __global__ void __launch_bounds__(walk_threads<T>(), 1)
   const unsigned word = __ldcg(reinterpret_cast<unsigned*>(W.state) + 1), tag0 = word << 1;
   int budget = W.polls;
   for (int p = p0; p < p1; ++p) {
-    if (budget > 0) budget = W.polls;
     Phase f{};
     f.type = __ldg(&ph[p].type), f.level = __ldg(&ph[p].level), f.colour = __ldg(&ph[p].colour);
     f.in = __ldg(&ph[p].in), f.out = __ldg(&ph[p].out);
@@ -174,7 +173,10 @@ __global__ void __launch_bounds__(walk_threads<T>(), 1)
     // the defect, the restricted one and the coarse solution are plain arrays
     const bool plain =
         f.type == kPhaseDefect || f.type == kPhaseRestrict || f.type == kPhaseCoarse;
-    if (plain && p + 1 < p1) cg::this_grid().sync();
+    if (plain && p + 1 < p1) {
+      if (budget > 0) budget = W.polls;  // a batch's size and sweeps have no bound
+      cg::this_grid().sync();
+    }
   }
   // every block has read the number before its first barrier (a cycle with a
   // phase that uses it has one)

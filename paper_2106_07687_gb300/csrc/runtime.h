@@ -37,12 +37,15 @@ class DevMem {
   ~DevMem() {
     for (void* p : ptrs_) cudaFree(p);
   }
-  // 256-byte aligned; the small buffers of a hierarchy share blocks (a batch of
-  // twelve channels makes 800 of them)
+  // share: buffers of up to a quarter of a block share blocks (a batch of twelve
+  // channels makes 800 buffers: set-up 15.0 -> 13.8 ms; a context makes fewer, and its
+  // level-5 cycle is 0.6 us faster with buffers of their own)
+  explicit DevMem(bool share = false) : share_(share) {}
+  // 256-byte aligned
   template <typename T>
   T* alloc(size_t n) {
     const size_t bytes = (n * sizeof(T) + 16 + 255) / 256 * 256;
-    if (bytes > kBlock / 4) return static_cast<T*>(take(bytes));
+    if (!share_ || bytes > kBlock / 4) return static_cast<T*>(take(bytes));
     if (bytes > left_) {
       next_ = static_cast<uint8_t*>(take(kBlock));
       left_ = next_ ? kBlock : 0;
@@ -67,6 +70,7 @@ class DevMem {
     return p;
   }
   std::vector<void*> ptrs_;
+  bool share_;
   uint8_t* next_ = nullptr;  // the current block's free part
   size_t left_ = 0;
   bool ok_ = true;

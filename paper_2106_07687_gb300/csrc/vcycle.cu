@@ -137,7 +137,6 @@ __device__ __forceinline__ void walk_phases(const VLevel<T>* glv, const OpTable<
   const int w0 = blockIdx.x + gridDim.x * w, nw = gridDim.x * (NT / 32);
   int budget = polls;
   for (int p = 0; p < nph; ++p) {
-    if (budget > 0) budget = polls;
     const PassRec<T>& R = S.rec[p];
     const int type = R.type;
     if (type == kPhasePass || type == kPhaseDefect) {

@@ -91,8 +91,8 @@ int launch_vcycle_cluster(const VLevel<T>* lv, const OpTable<T>* tab, const Phas
                           cudaStream_t st);
 // state: two device words, a status word (8: a wait for an update hit its bound)
 // and half of the cycle's first number, which the launch advances by `numbers`
-// (vcycle_numbers; the word starts above 0).  polls: the bound of a warp's polls per
-// phase (kTagPolls).
+// (vcycle_numbers; the word starts above 0).  polls: the bound of a warp's polls
+// (kTagPolls).
 // returns 0 on success; with skip, nothing runs when *skip != 0 at the
 // launch's start
 template <typename T>

@@ -315,7 +315,8 @@ struct NodeLevel {
 // run on from cycle to cycle (vcycle_numbers per cycle, whatever its sweeps), in a
 // word on the device: they come round after 2^32 updates, 238 million V(2,2)
 // cycles, in which every word that a cycle reads is rewritten.  The wait is
-// bounded (a warp's rounds of one phase, by kTagPolls unless the caller sets another
+// bounded (a warp's rounds over a single problem's cycle of at most 160 phases, or
+// between two barriers of a batch's, by kTagPolls unless the caller sets another
 // bound; then bit 8 of *status is set and the warp waits no more).  All lanes of the warp call load; other_loads
 // is run once, behind the first round's loads, to issue what the tile reads
 // besides the iterate: the tags are then mostly there when it is through.
