@@ -6,7 +6,7 @@
 // nodes) items, one warp each, with the same warp bodies and the same numbered
 // updates of the iterate instead of barriers (vnode.cuh).  One FP32 cycle of
 // twelve channels on levels 3 to 5: 77 launches with cell-by-cell tiles 1,338
-// us, this with a barrier per phase 704 us, with numbered updates 577 us; a pass
+// us, this with a barrier per phase 704 us, with numbered updates 563 us; a pass
 // of the top level moves 80 MB of inverses and blocks (265 k nodes, 12 us).
 // Where the grid cannot be resident the same kernel is launched once per phase.
 #include <algorithm>
